@@ -29,6 +29,8 @@ struct ProbHost {
   void* B = nullptr;
   void* Ahl = nullptr;   // split tiles (BSE_C128_DF)
   void* Bhl = nullptr;
+  int4 *Afx = nullptr, *Bfx = nullptr;   // complex128 tiles in fixed point and their scales
+  int* texp = nullptr;
   float* tmax = nullptr;   // mixed PH path: per-tile bound on |U|, |V| (device)
   void* UV = nullptr;      // mixed PH path: {U_re, V_re, U_im, V_im} records of the packed tiles
   std::vector<float> htmax;
@@ -102,6 +104,8 @@ struct bse_handle {
   std::vector<KState> hstate;
   TileJob* djobs = nullptr;
   int njobs = 0;
+  int nfx = 0;           // complex128: the first nfx jobs are fixed-point tiles, in nq bands each
+  int nq = 0;            // (0: the handle has no fixed-point tiles)
   std::vector<TileJob> hjobs;
   // mixed PH path: the tile jobs split by precision for the current solve
   bool mixed = false;        // BSE_C64_MIXED with B
@@ -283,6 +287,9 @@ struct Driver {
                            h->maxnT, mode, nullptr, shape, h->prod_err, s);
     else if (h->df)
       launch_product_df(h->dprobs, h->djobs, h->njobs, h->count, h->maxnT, mode, nullptr, h->ph != 0, h->split,
+                        shape, s);
+    else if (h->nq > 0)
+      launch_product_fx(h->dprobs, h->djobs, h->njobs, h->nfx, h->nq, h->count, h->maxnT, mode, nullptr, h->ph != 0,
                         shape, s);
     else
       launch_product<ST, R>(h->dprobs, h->djobs, h->njobs, h->count, h->maxnT, mode, 1, nullptr, h->ph != 0,
@@ -510,7 +517,8 @@ struct Driver {
       const int rc = dalloc((void**)&h->gbar, sizeof(GridBar));
       if (rc) return rc;
     }
-    const int r = launch_steps_persist<ST, R>(h->dprobs, h->djobs, h->njobs, h->ph != 0, steps, h->gbar, h->stream);
+    const int r = launch_steps_persist<ST, R>(h->dprobs, h->djobs, h->njobs, h->nfx, h->ph != 0, steps, h->gbar,
+                                              h->stream);
     if (r < 0) return BSE_ECUDA;
     return r;
   }
@@ -707,7 +715,7 @@ int alloc_solve(bse_handle* h, int ncv) {
     if (h->ph && (rc = dalloc(&q.P2, es * (size_t)q.Npad * ncv))) return rc;
     if ((rc = dalloc(&q.w, es * (size_t)q.Npad))) return rc;
     if ((rc = dalloc(&q.pw, es * (size_t)q.Npad))) return rc;
-    if ((rc = dalloc(&q.part, cs * (size_t)q.nT * q.nT * TS))) return rc;
+    if ((rc = dalloc(&q.part, cs * (size_t)q.nT * q.nT * TS * std::max(1, h->nq)))) return rc;
     if (h->mixed) {
       if ((rc = dalloc(&q.xs, sizeof(float4) * (size_t)q.Npad))) return rc;
       if ((rc = dalloc((void**)&q.Vs, sizeof(float4) * (size_t)q.Npad * nbas))) return rc;
@@ -798,6 +806,8 @@ int upload_probs(bse_handle* h) {
     d.jwld = 2 * q.ncv + 2;
     d.S2 = q.S2;
     d.Vs = q.Vs; d.Ps = q.Ps; d.ws = q.ws;
+    d.Afx = q.Afx; d.Bfx = q.Bfx; d.texp = q.texp;
+    d.nq = h->nq;
   }
   CK(cudaMemcpyAsync(h->dprobs, h->hprobs.data(), sizeof(Prob) * h->count, cudaMemcpyHostToDevice,
                      h->stream));
@@ -840,6 +850,39 @@ int split_mixed_jobs(bse_handle* h, double tol, double tau_opt) {
     CK(cudaMemcpyAsync(h->djobs_coarse, coarse.data(), sizeof(TileJob) * coarse.size(), cudaMemcpyHostToDevice,
                        h->stream));
   CK(cudaStreamSynchronize(h->stream));    // the host vectors go out of scope
+  return BSE_OK;
+}
+
+// The fixed-point copy of a complex128 handle's tiles (fx_phases.cuh), which doubles its packed
+// storage: made when it takes at most a third of the device memory that is free (a handle that
+// nearly fills the GPU, or one that finds it nearly full, keeps the FP64 product alone), and
+// dropped again when any allocation fails.  The jobs are reordered: fixed-point tiles first.
+int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
+  size_t need = 0, freeb = 0, totalb = 0;
+  for (const ProbHost& q : h->p) need += (size_t)q.ntiles * TS * TS * sizeof(int4) * (h->ph ? 2 : 1);
+  if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess) { cudaGetLastError(); return BSE_OK; }
+  if (need > freeb / 3) return BSE_OK;
+  std::vector<std::vector<int>> ex(h->count);
+  int rc = BSE_OK;
+  for (int i = 0; i < h->count && rc == BSE_OK; ++i) {
+    ProbHost& q = h->p[i];
+    const size_t bytes = (size_t)q.ntiles * TS * TS * sizeof(int4);
+    if ((rc = dalloc((void**)&q.Afx, bytes)) || (h->ph && (rc = dalloc((void**)&q.Bfx, bytes))) ||
+        (rc = dalloc((void**)&q.texp, sizeof(int) * (size_t)q.ntiles)))
+      break;
+    launch_fx_pack((const double2*)q.A, (const double2*)q.B, q.N, q.nT, q.Afx, q.Bfx, q.texp, h->stream);
+    ex[i].resize(q.ntiles);
+    CK(cudaMemcpyAsync(ex[i].data(), q.texp, sizeof(int) * (size_t)q.ntiles, cudaMemcpyDeviceToHost, h->stream));
+  }
+  CK(cudaStreamSynchronize(h->stream));
+  if (rc != BSE_OK) {
+    for (ProbHost& q : h->p) { dfreet(q.Afx); dfreet(q.Bfx); dfreet(q.texp); }
+    return rc == BSE_ENOMEM ? BSE_OK : rc;
+  }
+  const auto mid = std::stable_partition(jobs.begin(), jobs.end(),
+                                         [&](const TileJob& j) { return ex[j.prob][j.t] >= 0; });
+  h->nfx = (int)(mid - jobs.begin());
+  h->nq = fx_bands(h->nfx);
   return BSE_OK;
 }
 
@@ -983,6 +1026,7 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
 void setup_tuner(bse_handle* h) {
   const int occ = h->mixed ? product_mx_occupancy()
                  : h->df  ? product_df_occupancy(h->ph != 0, h->split)
+                 : h->nfx > 0 ? product_fx_occupancy(h->ph != 0)
                           : (h->vs == sizeof(float2) ? product_occupancy<float2, float>(h->ph != 0)
                                                      : product_occupancy<double2, double>(h->ph != 0));
   const bool batch = h->count > 1;
@@ -998,7 +1042,7 @@ void setup_tuner(bse_handle* h) {
   h->tseen.assign(n, 0);
   h->tnext = 0;
   h->shape = ProdShape{0, batch ? 1 : 0};
-  h->tkey = TuneKey{h->dtype * 2 + h->ph, h->njobs, h->count};
+  h->tkey = TuneKey{h->dtype * 2 + h->ph + (h->nfx > 0 ? 16 : 0), h->njobs, h->count};
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tuned.find(h->tkey);
   h->tuned = it != g_tuned.end();
@@ -1086,6 +1130,9 @@ int apply_impl(bse_handle* h, int op, int k, const void* X, void* Y) {
     if (h->df && h->split)   // complex128 handle: the solver's double-FP32 product
       launch_product_df(h->dprobs, h->djobs, h->njobs, 1, h->maxnT, PM_GENERIC, &io, hasB && op != BSE_OP_A,
                         true, h->shape, h->stream);
+    else if (h->nq > 0)
+      launch_product_fx(h->dprobs, h->djobs, h->njobs, h->nfx, h->nq, 1, h->maxnT, PM_GENERIC, &io, hasB, h->shape,
+                        h->stream);
     else
       launch_product<ST, R>(h->dprobs, h->djobs, h->njobs, 1, h->maxnT, PM_GENERIC, 1, &io,
                             hasB && op != BSE_OP_A, h->shape, h->stream);
@@ -1251,6 +1298,8 @@ int haydock_impl(bse_handle* h, const void* d, int where, int m, int sign, int n
     io.sB = sB;
     if (h->df)
       launch_product_df(h->dprobs, h->djobs, h->njobs, 1, h->maxnT, PM_GENERIC, &io, ph, h->split, h->shape, s);
+    else if (h->nq > 0)
+      launch_product_fx(h->dprobs, h->djobs, h->njobs, h->nfx, h->nq, 1, h->maxnT, PM_GENERIC, &io, ph, h->shape, s);
     else
       launch_product<ST, R>(h->dprobs, h->djobs, h->njobs, 1, h->maxnT, PM_GENERIC, 1, &io, ph, h->shape, s);
   };
@@ -1469,6 +1518,7 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
     rc = dalloc((void**)&h->prod_err, sizeof(int));
     if (rc == BSE_OK && cudaMemsetAsync(h->prod_err, 0, sizeof(int), h->stream) != cudaSuccess) rc = BSE_ECUDA;
   }
+  if (rc == BSE_OK && dtype == BSE_C128) rc = setup_fx(h, jobs);
   if (rc == BSE_OK) {
     h->njobs = (int)jobs.size();
     rc = dalloc((void**)&h->djobs, sizeof(TileJob) * jobs.size());
@@ -1673,6 +1723,9 @@ int bse_destroy(bse_handle* h) {
     dfree(q.B);
     dfree(q.Ahl);
     dfree(q.Bhl);
+    dfreet(q.Afx);
+    dfreet(q.Bfx);
+    dfreet(q.texp);
     dfreet(q.tmax);
     dfree(q.UV);
   }

@@ -159,6 +159,14 @@ struct Prob {
   float4* Vs;
   float4* Ps;
   float4* ws;
+  // complex128 tiles in fixed point (fx_phases.cuh; null where the FP64 product runs alone):
+  // int4 limbs {re_hi, re_lo, im_hi, im_lo} per packed element of A and B (P and Q on PH
+  // handles), diagonal left out; the biased exponent of each tile's scale (-1: the tile is on
+  // the FP64 kernel); and the bands per tile, whose column sums take nq planes of `part`
+  const int4* Afx;
+  const int4* Bfx;
+  const int* texp;
+  int nq;
 };
 
 // Jobs of the tiled product: problem, tile row I, tile column J, tile index.
@@ -243,6 +251,21 @@ void launch_tile_bound(const float2* A, const float2* B, int64_t ntiles, float* 
 // sums the float4 (hi, lo) partial-sum slots of the double-FP32 kernels in FP64 (k_product.cu)
 void launch_prod_reduce_d(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s);
 
+// complex128 products with fixed-point tiles (k_product_fx.cu): `jobs` lists the nfx fixed-point
+// tiles first, then the ones of the FP64 kernel
+void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, int nq, int nprob, int maxnT,
+                       int mode, const GenericIO* io_host, bool hasB, ProdShape shape, cudaStream_t s);
+int product_fx_occupancy(bool hasB);
+// limbs and scales of packed complex128 tiles; texp[t] = -1 for tiles left to the FP64 kernel
+void launch_fx_pack(const double2* A, const double2* B, int64_t N, int nT, int4* Afx, int4* Bfx, int* texp,
+                    cudaStream_t s);
+int fx_bands(int ntiles);      // bands per tile for a handle of that many tiles
+void launch_prod_reduce_f64(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s);
+// the FP64 tile kernel alone (k_product.cu)
+void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, GenericIO io, bool hasB,
+                      ProdShape shape, cudaStream_t s);
+int num_sms();
+
 // bounded-wait self-test (k_adjoint_tc.cu): 0 on success, -1 on a CUDA error
 int selftest_bounded_wait(int arrive, int* expired_host);
 
@@ -287,8 +310,8 @@ struct GridBar {
   int pad;
 };
 template <typename ST, typename R>
-int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, bool ph, int steps, GridBar* gb,
-                         cudaStream_t s);
+int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, bool ph, int steps,
+                         GridBar* gb, cudaStream_t s);
 
 // dense structure-preserving diagonalisation (k_dense.cu): the nev lowest positive omega of
 // problem 0 of a PH handle and their right eigenvectors in Z (ld 2 Npad); returns 0, 1 (M_r not

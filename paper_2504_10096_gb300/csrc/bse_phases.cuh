@@ -264,45 +264,66 @@ __device__ __forceinline__ void prod_tiles_body(const Prob* __restrict__ probs, 
   }
 }
 
-// y[I*TS + r] = sum_J part[I][J][r]; grid (maxnT, nprob).
+// y[I*TS + r] = sum_J part[I][J][r].  A unit is 32 rows of a block row: 8 warps, lane = row, warp
+// g sums the slots J = g, g + 8, ... in order, and the eight group sums are added in group order
+// (a fixed rounding order).  FP64 adds cost 64 clocks per warp and scheduler on this GPU, so the
+// rows are spread over four times as many CTAs as there are block rows.
 constexpr int REDUCE_GROUPS = 8;
+constexpr int REDUCE_ROWS = 32;
+constexpr int REDUCE_UNITS = TS / REDUCE_ROWS;       // units of a block row
 
-// One unit: block row I of problem ip, with any multiple of TS threads (each thread takes
-// the groups g = threadIdx.x / TS + k blockDim.x / TS); grp: (REDUCE_GROUPS - 1) x TS entries
-// of shared memory.  The group sums and their order are those of the REDUCE_GROUPS * TS
-// thread launch, so the result is the same bits for any thread count.
+// One unit: rows 32 (u % 4) ... of block row u / 4 of problem ip; grp: REDUCE_GROUPS x 32 entries
+// of shared memory.
 template <typename ST, typename R, bool COH = false>
 __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs, int mode, const GenericIO& io,
-                                                 int I, int ip, typename Acc<R>::T (*grp)[TS]) {
+                                                 int u, int ip, typename Acc<R>::T (*grp)[REDUCE_ROWS]) {
   using CT = typename Acc<R>::T;
   const Prob& p = probs[ip];
+  const int I = u / REDUCE_UNITS;
   if (I >= p.nT) return;
   const ST* x; ST* y; R sB;
   if (!prod_operands<ST, R>(p, mode, io, x, y, sB)) return;
-  // REDUCE_GROUPS groups of 128 threads sum the slots J = g, g + G, ... in
-  // order; the group sums are then added in group order (fixed rounding order)
-  const int r = threadIdx.x & (TS - 1);
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int r = (u % REDUCE_UNITS) * REDUCE_ROWS + lane;
   const CT* part = (const CT*)p.part + (int64_t)I * p.nT * TS;
-  CT acc0 = czero<CT>();
-  for (int g = threadIdx.x >> 7; g < REDUCE_GROUPS; g += blockDim.x >> 7) {
-    CT acc = czero<CT>();
-    int J = g;
-    for (; J + 3 * REDUCE_GROUPS < p.nT; J += 4 * REDUCE_GROUPS) {   // four loads in flight, then the sums
-      CT v[4];
+  CT acc = czero<CT>();
+  int J = g;
+  for (; J + 3 * REDUCE_GROUPS < p.nT; J += 4 * REDUCE_GROUPS) {   // four loads in flight, then the sums
+    CT v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = ldp<COH>(part + (int64_t)(J + u * REDUCE_GROUPS) * TS + r);
+    for (int k = 0; k < 4; ++k) v[k] = ldp<COH>(part + (int64_t)(J + k * REDUCE_GROUPS) * TS + r);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc = cadd(acc, v[u]);
-    }
-    for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, ldp<COH>(part + (int64_t)J * TS + r));
-    if (g > 0) grp[g - 1][r] = acc;
-    else acc0 = acc;
+    for (int k = 0; k < 4; ++k) acc = cadd(acc, v[k]);
   }
+  for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, ldp<COH>(part + (int64_t)J * TS + r));
+  if constexpr (std::is_same<CT, double2>::value) {
+    // fixed-point tiles: the column sums of a tile's further bands, planes 1 ... nq - 1
+    const int nb = p.nq - 1;
+    for (int k = g; k < nb * I; k += REDUCE_GROUPS) {
+      const int q = 1 + k / I, Jq = k - (q - 1) * I;
+      if (p.texp[(int64_t)Jq * p.nT - (int64_t)Jq * (Jq - 1) / 2 + (I - Jq)] < 0) continue;
+      acc = cadd(acc, ldp<COH>(part + ((int64_t)q * p.nT * p.nT + Jq) * TS + r));
+    }
+  }
+  grp[g][lane] = acc;
   __syncthreads();
-  if (threadIdx.x < TS) {
+  if (g == 0) {
 #pragma unroll
-    for (int q = 0; q < REDUCE_GROUPS - 1; ++q) acc0 = cadd(acc0, grp[q][r]);
-    y[(int64_t)I * TS + r] = ccvt<ST>(acc0);
+    for (int q = 1; q < REDUCE_GROUPS; ++q) acc = cadd(acc, grp[q][lane]);
+    const int64_t row = (int64_t)I * TS + r;
+    if constexpr (std::is_same<CT, double2>::value) {
+      // ... and the diagonal entry, which a fixed-point diagonal tile leaves out
+      const int64_t t = (int64_t)I * p.nT - (int64_t)I * (I - 1) / 2;
+      if (p.nq > 0 && p.texp[t] >= 0) {
+        const int64_t d = t * (TS * TS) + r * (TS + 1);
+        const CT xv = ldp<COH>((const CT*)x + row);
+        const CT u = ((const CT*)(p.ph && sB < (R)0 ? p.B : p.A))[d];
+        const CT v = p.ph ? ((const CT*)(sB < (R)0 ? p.A : p.B))[d] : u;
+        acc.x = fma(u.x, xv.x, acc.x); acc.x = fma(-v.y, xv.y, acc.x);
+        acc.y = fma(u.y, xv.x, acc.y); acc.y = fma(v.x, xv.y, acc.y);
+      }
+    }
+    y[row] = ccvt<ST>(acc);
   }
   __syncthreads();                     // grp is rewritten by the next unit
 }

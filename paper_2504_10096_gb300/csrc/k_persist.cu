@@ -17,7 +17,7 @@
 // cooperative, so all CTAs are resident together.
 #include <algorithm>
 
-#include "bse_phases.cuh"
+#include "fx_phases.cuh"
 
 namespace bse {
 namespace {
@@ -64,7 +64,7 @@ __device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned int nblk, unsign
 
 template <typename ST, typename R, bool HASB>
 __global__ void __launch_bounds__(PS_THREADS, 1)
-k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int steps,
+k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int nfx, int steps,
                 GridBar* gb) {
   using CT = typename Acc<R>::T;
   extern __shared__ __align__(16) unsigned char psm[];
@@ -80,7 +80,7 @@ k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
   CT* xc = reinterpret_cast<CT*>(psm);
   CT* xr = xc + TS;
   CT(*pred)[TS] = reinterpret_cast<CT(*)[TS]>(xr + TS);
-  CT(*grp)[TS] = reinterpret_cast<CT(*)[TS]>(psm);
+  CT(*grp)[REDUCE_ROWS] = reinterpret_cast<CT(*)[REDUCE_ROWS]>(psm);
   double2(*dred)[4] = reinterpret_cast<double2(*)[4]>(psm);
   ST* cf = reinterpret_cast<ST*>(psm);
   ST(*ured)[32] = reinterpret_cast<ST(*)[32]>(cf + 2 * MAXM + 2);
@@ -91,11 +91,19 @@ k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
   const int nrow = (int)((p.Npad + PS_THREADS - 1) / PS_THREADS);
   const int ncp = (p.ncol + 1) / 2;
   const int m1 = HASB ? PM_STEP_MMINUS : PM_STEP_A;
+  // the tiles of a product: the fixed-point ones (complex128), then the others
+  auto tiles = [&](int mode) {
+    if constexpr (std::is_same<ST, double2>::value)
+      if (nfx > 0)
+        fx_tiles_body<HASB, true>(probs, jobs, nfx, p.nq, mode, io, 1, bid, nblk, *reinterpret_cast<FxShared*>(psm));
+    if (njobs > nfx)
+      prod_tiles_body<ST, R, HASB, true>(probs, jobs + nfx, njobs - nfx, mode, io, 1, bid, nblk, xc, xr, pred);
+  };
   for (int s = 0; s < steps; ++s) {
     if (!kactive(st)) break;                          // the same state in every CTA
-    prod_tiles_body<ST, R, HASB, true>(probs, jobs, njobs, m1, io, 1, bid, nblk, xc, xr, pred);
+    tiles(m1);
     if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    for (int I = bid; I < nT; I += nblk) prod_reduce_body<ST, R, true>(probs, m1, io, I, 0, grp);
+    for (int u = bid; u < REDUCE_UNITS * nT; u += nblk) prod_reduce_body<ST, R, true>(probs, m1, io, u, 0, grp);
     if (!grid_sync(gb, nblk, gen, &s_ok)) return;
     for (int pass = 0; pass < 2; ++pass) {
       for (int u = bid; u < ncp * nrb; u += nblk) {
@@ -110,9 +118,9 @@ k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
       if (!grid_sync(gb, nblk, gen, &s_ok)) return;
     }
     if (HASB) {
-      prod_tiles_body<ST, R, HASB, true>(probs, jobs, njobs, PM_STEP_MPLUS, io, 1, bid, nblk, xc, xr, pred);
+      tiles(PM_STEP_MPLUS);
       if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-      for (int I = bid; I < nT; I += nblk) prod_reduce_body<ST, R, true>(probs, PM_STEP_MPLUS, io, I, 0, grp);
+      for (int u = bid; u < REDUCE_UNITS * nT; u += nblk) prod_reduce_body<ST, R, true>(probs, PM_STEP_MPLUS, io, u, 0, grp);
       if (!grid_sync(gb, nblk, gen, &s_ok)) return;
     }
     if (nrb == 1) {
@@ -136,9 +144,10 @@ template <typename ST, typename R, bool HASB>
 size_t persist_smem() {
   using CT = typename Acc<R>::T;
   const size_t prod = (size_t)10 * TS * sizeof(CT);
-  const size_t red = (size_t)(REDUCE_GROUPS - 1) * TS * sizeof(CT);
+  const size_t red = (size_t)REDUCE_GROUPS * REDUCE_ROWS * sizeof(CT);
+  const size_t fx = std::is_same<ST, double2>::value ? sizeof(FxShared) : 0;
   const size_t upd = (size_t)(2 * MAXM + 2) * sizeof(ST) + (size_t)8 * 32 * sizeof(ST);
-  return std::max(std::max(prod, red), std::max(upd, (size_t)(9 * sizeof(double) + 8 * sizeof(double2))));
+  return std::max(std::max(std::max(prod, red), fx), std::max(upd, (size_t)(9 * sizeof(double) + 8 * sizeof(double2))));
 }
 
 template <typename ST, typename R, bool HASB>
@@ -160,12 +169,13 @@ int persist_grid() {
 }
 
 template <typename ST, typename R, bool HASB>
-int launch_persist_t(const Prob* dprobs, const TileJob* jobs, int njobs, int steps, GridBar* gb, cudaStream_t s) {
+int launch_persist_t(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, int steps, GridBar* gb,
+                     cudaStream_t s) {
   const int grid = persist_grid<ST, R, HASB>();
   if (grid <= 0) return 1;
   if (cudaMemsetAsync(gb, 0, sizeof(GridBar), s) != cudaSuccess) return -1;
   const size_t sm = persist_smem<ST, R, HASB>();
-  void* args[] = {(void*)&dprobs, (void*)&jobs, (void*)&njobs, (void*)&steps, (void*)&gb};
+  void* args[] = {(void*)&dprobs, (void*)&jobs, (void*)&njobs, (void*)&nfx, (void*)&steps, (void*)&gb};
   count_launch();
   const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_steps_persist<ST, R, HASB>, dim3(grid),
                                                     dim3(PS_THREADS), args, sm, s);
@@ -179,15 +189,15 @@ int launch_persist_t(const Prob* dprobs, const TileJob* jobs, int njobs, int ste
 }  // namespace
 
 template <typename ST, typename R>
-int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, bool ph, int steps, GridBar* gb,
-                         cudaStream_t s) {
-  return ph ? launch_persist_t<ST, R, true>(dprobs, jobs, njobs, steps, gb, s)
-            : launch_persist_t<ST, R, false>(dprobs, jobs, njobs, steps, gb, s);
+int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, bool ph, int steps,
+                         GridBar* gb, cudaStream_t s) {
+  return ph ? launch_persist_t<ST, R, true>(dprobs, jobs, njobs, nfx, steps, gb, s)
+            : launch_persist_t<ST, R, false>(dprobs, jobs, njobs, nfx, steps, gb, s);
 }
 
-template int launch_steps_persist<double2, double>(const Prob*, const TileJob*, int, bool, int, GridBar*,
+template int launch_steps_persist<double2, double>(const Prob*, const TileJob*, int, int, bool, int, GridBar*,
                                                    cudaStream_t);
-template int launch_steps_persist<float2, float>(const Prob*, const TileJob*, int, bool, int, GridBar*,
+template int launch_steps_persist<float2, float>(const Prob*, const TileJob*, int, int, bool, int, GridBar*,
                                                  cudaStream_t);
 
 }  // namespace bse

@@ -43,27 +43,28 @@ k_prod_tiles(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, i
   prod_tiles_body<ST, R, HASB>(probs, jobs, njobs, mode, io, strided, blockIdx.x, gridDim.x, xc, xr, red);
 }
 
-// y[I*TS + r] = sum_J part[I][J][r]; grid (maxnT, nprob) (prod_reduce_body).
+// y[I*TS + r] = sum_J part[I][J][r]; grid (REDUCE_UNITS maxnT, nprob) (prod_reduce_body).
 template <typename ST, typename R>
-__global__ void __launch_bounds__(REDUCE_GROUPS * TS)
+__global__ void __launch_bounds__(REDUCE_GROUPS * REDUCE_ROWS)
 k_prod_reduce(const Prob* __restrict__ probs, int mode, GenericIO io) {
   using CT = typename Acc<R>::T;
-  __shared__ CT grp[REDUCE_GROUPS - 1][TS];
+  __shared__ CT grp[REDUCE_GROUPS][REDUCE_ROWS];
   prod_reduce_body<ST, R>(probs, mode, io, blockIdx.x, blockIdx.y, grp);
 }
 
 // Same reduction for the double-FP32 kernels, whose slots hold (hi, lo) float
 // pairs {re_hi, re_lo, im_hi, im_lo}: each slot is widened to FP64 and the slots
 // are summed in FP64 in the fixed order above.
-__global__ void __launch_bounds__(REDUCE_GROUPS * TS)
+__global__ void __launch_bounds__(REDUCE_GROUPS * REDUCE_ROWS)
 k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
-  __shared__ double2 grp[REDUCE_GROUPS - 1][TS];
+  __shared__ double2 grp[REDUCE_GROUPS][REDUCE_ROWS];
   const Prob& p = probs[blockIdx.y];
-  const int I = blockIdx.x;
+  const int I = blockIdx.x / REDUCE_UNITS;
   if (I >= p.nT) return;
   const double2* x; double2* y; double sB;
   if (!prod_operands<double2, double>(p, mode, io, x, y, sB)) return;
-  const int r = threadIdx.x & (TS - 1), g = threadIdx.x >> 7;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int r = (blockIdx.x % REDUCE_UNITS) * REDUCE_ROWS + lane;
   const float4* part = (const float4*)p.part + (int64_t)I * p.nT * TS;
   double2 acc = make_double2(0.0, 0.0);
   auto wide = [](float4 v) { return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w); };
@@ -76,11 +77,11 @@ k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
     for (int u = 0; u < 4; ++u) acc = cadd(acc, wide(v[u]));
   }
   for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, wide(part[(int64_t)J * TS + r]));
-  if (g > 0) grp[g - 1][r] = acc;
+  grp[g][lane] = acc;
   __syncthreads();
   if (g == 0) {
 #pragma unroll
-    for (int q = 0; q < REDUCE_GROUPS - 1; ++q) acc = cadd(acc, grp[q][r]);
+    for (int q = 1; q < REDUCE_GROUPS; ++q) acc = cadd(acc, grp[q][lane]);
     y[(int64_t)I * TS + r] = acc;
     if (p.ws && y == (double2*)p.w) p.ws[(int64_t)I * TS + r] = dsplit(acc);   // its double-FP32 shadow
   }
@@ -285,7 +286,7 @@ void launch_pq_combine(double2* a, double2* b, int64_t n, cudaStream_t s) {
 
 // ---------------------------------------------------------------- launchers
 static int g_num_sms = 0;
-static int num_sms() {
+int num_sms() {
   if (!g_num_sms) {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -332,11 +333,27 @@ void launch_product(const Prob* dprobs, const TileJob* jobs, int njobs, int npro
     k_prod_tiles<ST, R, true><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
   else
     k_prod_tiles<ST, R, false><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
-  k_prod_reduce<ST, R><<<dim3(maxnT, nprob), REDUCE_GROUPS * TS, 0, s>>>(dprobs, mode, io);
+  k_prod_reduce<ST, R><<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode, io);
 }
 
 void launch_prod_reduce_d(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s) {
-  k_prod_reduce_dfc<<<dim3(maxnT, nprob), REDUCE_GROUPS * TS, 0, s>>>(dprobs, mode, io);
+  k_prod_reduce_dfc<<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode, io);
+}
+
+void launch_prod_reduce_f64(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s) {
+  count_launch();
+  k_prod_reduce<double2, double><<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode,
+                                                                                                      io);
+}
+
+void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, GenericIO io, bool hasB,
+                      ProdShape shape, cudaStream_t s) {
+  count_launch();
+  const int grid = product_grid(product_occupancy<double2, double>(hasB), shape, njobs);
+  if (hasB)
+    k_prod_tiles<double2, double, true><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+  else
+    k_prod_tiles<double2, double, false><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
 }
 
 template void launch_product<double2, double>(const Prob*, const TileJob*, int, int, int, int, int,

@@ -1,0 +1,129 @@
+// Kernels of the fixed-point complex128 product (fx_phases.cuh): the tile kernel and the packing
+// of the limbs.
+#include <algorithm>
+
+#include "fx_phases.cuh"
+
+namespace bse {
+namespace {
+
+template <bool HASB>
+__global__ void __launch_bounds__(FX_THREADS, 1)
+k_prod_tiles_fx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int nq, int mode,
+                GenericIO io, int strided) {
+  __shared__ FxShared sh;
+  fx_tiles_body<HASB, false>(probs, jobs, njobs, nq, mode, io, strided, blockIdx.x, gridDim.x, sh);
+}
+
+// v / 2^(e - 1022) as a float (magnitude below 1, truncated; small values flush to zero)
+__device__ __forceinline__ float fx_ratio(double v, int e) {
+  const unsigned int h = (unsigned int)__double2hiint(v), l = (unsigned int)__double2loint(v);
+  const int ev = (int)((h >> 20) & 0x7ffu) - e + 126;
+  const unsigned int m = ((h & 0xfffffu) << 3) | (l >> 29);
+  return ev > 0 ? __uint_as_float(((unsigned int)ev << 23) | m) : 0.f;
+}
+
+// One CTA per tile (I, J >= I): the scale from the largest component, the choice between the
+// fixed-point and the FP64 kernel, and the limbs (zeros on the matrix diagonal).  The tile's
+// second reading comes from L2.
+template <bool HASB>
+__global__ void __launch_bounds__(256)
+k_fx_pack(const double2* __restrict__ A, const double2* __restrict__ B, int64_t N, int nT, int4* __restrict__ Af,
+          int4* __restrict__ Bf, int* __restrict__ texp) {
+  const int I = blockIdx.y, J = blockIdx.x;
+  if (J < I) return;
+  const int64_t t = (int64_t)I * nT - (int64_t)I * (I - 1) / 2 + (J - I);
+  const double2* a = A + t * (TS * TS);
+  const double2* b = HASB ? B + t * (TS * TS) : nullptr;
+  __shared__ unsigned int smx[8];
+  __shared__ float ssq[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto off_diag = [&](int e) { return I != J || (e >> 7) != (e & (TS - 1)); };
+  // high words of the magnitudes; 1 for a subnormal that has none
+  auto mag = [](double v) { return max(hi_abs(v), __double2loint(v) ? 1u : 0u); };
+  unsigned int m = 0;
+  for (int e = tid; e < TS * TS; e += 256) {
+    if (!off_diag(e)) continue;
+    const double2 v = a[e];
+    m = max(m, max(mag(v.x), mag(v.y)));
+    if (HASB) {
+      const double2 w = b[e];
+      m = max(m, max(mag(w.x), mag(w.y)));
+    }
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) smx[warp] = m;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) m = max(m, smx[w]);
+  const int ex = max(64, (int)(m >> 20));
+  float s = 0.f;
+  for (int e = tid; e < TS * TS; e += 256) {
+    double2 v = a[e], w = HASB ? b[e] : make_double2(0.0, 0.0);
+    if (!off_diag(e)) v = w = make_double2(0.0, 0.0);
+    Af[t * (TS * TS) + e] = fx_entry(v, ex);
+    if (HASB) Bf[t * (TS * TS) + e] = fx_entry(w, ex);
+    const float f0 = fx_ratio(v.x, ex), f1 = fx_ratio(v.y, ex), f2 = fx_ratio(w.x, ex), f3 = fx_ratio(w.y, ex);
+    s += f0 * f0 + f1 * f1 + f2 * f2 + f3 * f3;
+  }
+#pragma unroll
+  for (int k = 16; k >= 1; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+  if (lane == 0) ssq[warp] = s;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < 8; ++w) s += ssq[w];
+    // entries inside the matrix; the peak is at least half the scale, 2^-2 of it squared
+    const int64_t nr = min((int64_t)TS, N - (int64_t)I * TS), nc = min((int64_t)TS, N - (int64_t)J * TS);
+    const float count = (float)(nr * nc) * (HASB ? 4.f : 2.f);
+    const bool in_range = ex >= 256 && ex <= 1792;
+    texp[t] = m == 0 || (in_range && count <= FX_PEAK * FX_PEAK * s) ? ex : -1;
+  }
+}
+
+}  // namespace
+
+// Bands per tile: the fewest row steps on the busiest SM, a unit of TS / nq rows costing about 16
+// rows more (staging, the column sums).
+int fx_bands(int ntiles) {
+  int best = 1;
+  int64_t cost = INT64_MAX;
+  for (int nq = 1; nq <= 8; nq *= 2) {
+    const int64_t c = (((int64_t)ntiles * nq + num_sms() - 1) / num_sms()) * (TS / nq + 16);
+    if (c < cost) { cost = c; best = nq; }
+  }
+  return best;
+}
+
+int product_fx_occupancy(bool hasB) {
+  static int occ[2] = {0, 0};
+  const int ib = hasB ? 1 : 0;
+  if (!occ[ib]) {
+    int o = 0;
+    if (hasB) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_fx<true>, FX_THREADS, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_fx<false>, FX_THREADS, 0);
+    occ[ib] = o > 0 ? o : 1;
+  }
+  return occ[ib];
+}
+
+void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, int nq, int nprob, int maxnT,
+                       int mode, const GenericIO* io_host, bool hasB, ProdShape shape, cudaStream_t s) {
+  GenericIO io{};
+  if (io_host) io = *io_host;
+  if (nfx > 0) {
+    count_launch();
+    const int grid = product_grid(product_fx_occupancy(hasB), shape, nfx * nq);
+    if (hasB) k_prod_tiles_fx<true><<<grid, FX_THREADS, 0, s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
+    else k_prod_tiles_fx<false><<<grid, FX_THREADS, 0, s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
+  }
+  if (njobs > nfx) launch_tiles_f64(dprobs, jobs + nfx, njobs - nfx, mode, io, hasB, shape, s);
+  launch_prod_reduce_f64(dprobs, nprob, maxnT, mode, io, s);
+}
+
+void launch_fx_pack(const double2* A, const double2* B, int64_t N, int nT, int4* Afx, int4* Bfx, int* texp,
+                    cudaStream_t s) {
+  count_launch();
+  if (B) k_fx_pack<true><<<dim3(nT, nT), 256, 0, s>>>(A, B, N, nT, Afx, Bfx, texp);
+  else k_fx_pack<false><<<dim3(nT, nT), 256, 0, s>>>(A, B, N, nT, Afx, nullptr, texp);
+}
+
+}  // namespace bse
