@@ -41,6 +41,7 @@ struct ProbHost {
   void* part = nullptr;
   void* xs = nullptr;        // mixed PH path: pre-split product vector and chunk maxima
   float* xmax = nullptr;
+  double* npart = nullptr;   // norm partial sums, then the normalisation's ticket
   double *cpart = nullptr, *coef = nullptr, *small = nullptr, *S = nullptr;
   // Gruning variant: odd basis W, Z = M- W, their restart scratch, the projected tree and the
   // odd-side Ritz coefficients (allocated by the first solve that asks for the variant)
@@ -114,7 +115,7 @@ struct bse_handle {
   int njobs_fine = 0, njobs_coarse = 0;
   int maxnT = 0;
   int64_t maxNpad = 0;
-  int maxnrb = 1;
+  int slab = 32;         // rows of a Gram-Schmidt update unit
   int ncv = 0;
   int nev = 0;
   bool solved = false;
@@ -199,7 +200,7 @@ bool is_c64(int dtype) { return dtype == BSE_C64 || dtype == BSE_C64_MIXED; }
 void free_solve_buffers(ProbHost& q) {
   dfree(q.V); dfree(q.P); dfree(q.V2); dfree(q.P2); dfree(q.w); dfree(q.pw); dfree(q.part); dfree(q.xs);
   dfreet(q.xmax);
-  dfreet(q.cpart); dfreet(q.coef); dfreet(q.small); dfreet(q.S);
+  dfreet(q.cpart); dfreet(q.npart); dfreet(q.coef); dfreet(q.small); dfreet(q.S);
   dfree(q.W); dfree(q.Zo); dfree(q.W2); dfree(q.Z2); dfreet(q.jw); dfreet(q.S2);
   dfreet(q.Vs); dfreet(q.Ps); dfreet(q.ws);
   q.ncv = 0;
@@ -342,12 +343,11 @@ struct Driver {
 
   void cgs(int pass, int half = 0) {
     const int ncol = h->ncv + 1 + h->ncv;
-    launch_step_cgs<ST>(h->dprobs, h->count, h->ph, h->maxnrb, h->maxNpad, ncol, pass, half, h->mixed && h->ph,
-                        s);
+    launch_step_cgs<ST>(h->dprobs, h->count, h->ph, h->maxNpad, h->slab, ncol, pass, half, h->mixed && h->ph, s);
   }
 
   void normalize(int start, int half, cudaStream_t st) {
-    launch_step_normalize<ST>(h->dprobs, h->count, h->ph, h->maxnrb, h->maxNpad, start, half, st);
+    launch_step_normalize<ST>(h->dprobs, h->count, h->ph, h->maxNpad, start, half, st);
   }
 
   void step() {
@@ -707,7 +707,6 @@ int alloc_solve(bse_handle* h, int ncv) {
     free_solve_buffers(q);
     const int ncol = 2 * ncv + 1;          // stride of the CGS partial sums and coefficients
     const int nbas = ncv + 1;              // basis columns of V and P
-    const int nrb = nrb_of(q.Npad);
     int rc;
     if ((rc = dalloc(&q.V, es * (size_t)q.Npad * nbas))) return rc;
     if (h->ph && (rc = dalloc(&q.P, es * (size_t)q.Npad * nbas))) return rc;
@@ -725,7 +724,9 @@ int alloc_solve(bse_handle* h, int ncv) {
       CK(cudaMemsetAsync(q.Ps, 0, sizeof(float4) * (size_t)q.Npad * nbas, h->stream));
       if ((rc = dalloc((void**)&q.xmax, sizeof(float) * (size_t)q.nT))) return rc;
     }
-    if ((rc = dalloc((void**)&q.cpart, sizeof(double2) * (size_t)nrb * ncol))) return rc;
+    if ((rc = dalloc((void**)&q.cpart, sizeof(double2) * (size_t)DOT_CHUNKS * ncol))) return rc;
+    if ((rc = dalloc((void**)&q.npart, sizeof(double) * (size_t)(q.Npad / 8) + 16))) return rc;
+    CK(cudaMemsetAsync(q.npart, 0, sizeof(double) * (size_t)(q.Npad / 8) + 16, h->stream));
     if ((rc = dalloc((void**)&q.coef, sizeof(double2) * 2 * (size_t)ncol))) return rc;
     if ((rc = dalloc((void**)&q.small, sizeof(double) * 6 * (size_t)(ncv + 1)))) return rc;
     if ((rc = dalloc((void**)&q.S, sizeof(double) * (size_t)ncv * ncv))) return rc;
@@ -778,11 +779,14 @@ int upload_probs(bse_handle* h) {
     d.Npad = q.Npad;
     d.ph = h->ph;
     d.ncv = q.ncv;
+    d.slab = h->slab;
     d.ncol = 2 * q.ncv + 1;
     d.A = q.A;
     d.B = q.B;
     d.V = q.V; d.P = q.P; d.V2 = q.V2; d.P2 = q.P2; d.w = q.w; d.pw = q.pw; d.part = q.part;
     d.cpart = q.cpart;
+    d.npart = q.npart;
+    d.tick = q.npart ? (unsigned int*)(q.npart + q.Npad / 8) : nullptr;
     d.coef = q.coef;
     const int64_t m1 = q.ncv + 1;
     d.theta = q.small;
@@ -792,7 +796,6 @@ int upload_probs(bse_handle* h) {
     d.ritz = q.small + 4 * m1;
     d.rest = q.small + 5 * m1;
     d.S = q.S;
-    d.nrb = nrb_of(q.Npad);
     d.st = h->dstate + i;
     d.Ahl = q.Ahl;
     d.Bhl = q.Bhl;
@@ -808,6 +811,7 @@ int upload_probs(bse_handle* h) {
     d.Vs = q.Vs; d.Ps = q.Ps; d.ws = q.ws;
     d.Afx = q.Afx; d.Bfx = q.Bfx; d.texp = q.texp;
     d.nq = h->nq;
+    d.err = h->prod_err;
   }
   CK(cudaMemcpyAsync(h->dprobs, h->hprobs.data(), sizeof(Prob) * h->count, cudaMemcpyHostToDevice,
                      h->stream));
@@ -1026,7 +1030,7 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
 void setup_tuner(bse_handle* h) {
   const int occ = h->mixed ? product_mx_occupancy()
                  : h->df  ? product_df_occupancy(h->ph != 0, h->split)
-                 : h->nfx > 0 ? product_fx_occupancy(h->ph != 0)
+                 : h->nfx > 0 ? product_fx_occupancy()
                           : (h->vs == sizeof(float2) ? product_occupancy<float2, float>(h->ph != 0)
                                                      : product_occupancy<double2, double>(h->ph != 0));
   const bool batch = h->count > 1;
@@ -1103,6 +1107,14 @@ __global__ void k_cvt_pad(const ST* __restrict__ X, int64_t N, int64_t Npad, int
   out[(int64_t)c * Npad + r] = r < N ? ccvt<CT>(X[(int64_t)c * N + r]) : czero<CT>();
 }
 
+// waits for the handle's stream; BSE_ETIMEOUT if a product kernel's bounded wait expired
+int sync_product(bse_handle* h) {
+  int perr = 0;
+  if (h->prod_err) CK(cudaMemcpyAsync(&perr, h->prod_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return perr ? BSE_ETIMEOUT : BSE_OK;
+}
+
 template <typename ST>
 int apply_impl(bse_handle* h, int op, int k, const void* X, void* Y) {
   using R = typename std::conditional<std::is_same<ST, float2>::value, float, double>::type;
@@ -1138,8 +1150,7 @@ int apply_impl(bse_handle* h, int op, int k, const void* X, void* Y) {
                             hasB && op != BSE_OP_A, h->shape, h->stream);
     CK(cudaMemcpyAsync(Y, q.pw, h->es * (size_t)N, cudaMemcpyDeviceToDevice, h->stream));
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(h->stream));
-    return BSE_OK;
+    return sync_product(h);
   }
   const int kc = op == BSE_OP_H ? 2 * k : k;
   const size_t need = sizeof(CT) * (size_t)Npad * kc * 3 + 1024;
@@ -1371,7 +1382,7 @@ int haydock_impl(bse_handle* h, const void* d, int where, int m, int sign, int n
     CK(cudaMemcpyAsync(hal.data(), alpha, sizeof(double) * m, cudaMemcpyDeviceToHost, s0));
     CK(cudaMemcpyAsync(hbe.data(), beta, sizeof(double) * m, cudaMemcpyDeviceToHost, s0));
   }
-  CK(cudaStreamSynchronize(s0));
+  if ((rc = sync_product(h))) return rc;
   CK(cudaGetLastError());
   float ms = 0.f;
   cudaEventElapsedTime(&ms, e0, e1);
@@ -1462,7 +1473,6 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
     q.ntiles = (int64_t)q.nT * (q.nT + 1) / 2;
     h->maxnT = std::max(h->maxnT, q.nT);
     h->maxNpad = std::max(h->maxNpad, q.Npad);
-    h->maxnrb = std::max(h->maxnrb, nrb_of(q.Npad));
     const size_t bytes = h->es * (size_t)q.ntiles * TS * TS;
     if ((rc = dalloc(&q.A, bytes))) break;
     if (h->ph && (rc = dalloc(&q.B, bytes))) break;
@@ -1513,12 +1523,15 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
       }
   }
   if (rc == BSE_OK && jobs.size() > 2147483647ull) rc = BSE_EINVAL;
-  if (rc == BSE_OK && h->mixed) {
-    h->hjobs = jobs;
+  int64_t rows = 0;      // update units: about one per SM, when the problems allow it
+  for (const ProbHost& q : h->p) rows += q.Npad;
+  while (h->slab > 8 && rows / (h->slab / 2) <= num_sms()) h->slab /= 2;
+  if (rc == BSE_OK && dtype == BSE_C128) rc = setup_fx(h, jobs);
+  if (rc == BSE_OK && h->mixed) h->hjobs = jobs;
+  if (rc == BSE_OK && (h->mixed || h->nfx > 0)) {
     rc = dalloc((void**)&h->prod_err, sizeof(int));
     if (rc == BSE_OK && cudaMemsetAsync(h->prod_err, 0, sizeof(int), h->stream) != cudaSuccess) rc = BSE_ECUDA;
   }
-  if (rc == BSE_OK && dtype == BSE_C128) rc = setup_fx(h, jobs);
   if (rc == BSE_OK) {
     h->njobs = (int)jobs.size();
     rc = dalloc((void**)&h->djobs, sizeof(TileJob) * jobs.size());
@@ -1672,10 +1685,7 @@ int bse_apply_mixed(bse_handle* h, int op, double tile_tau, const void* X, void*
                        PM_GENERIC, &io, h->shape, h->prod_err, h->stream);
   CK(cudaMemcpyAsync(Y, q.pw, sizeof(double2) * (size_t)q.N, cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaGetLastError());
-  int perr = 0;
-  CK(cudaMemcpyAsync(&perr, h->prod_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  if (perr) return BSE_ETIMEOUT;
+  if ((rc = sync_product(h))) return rc;
   h->stats.tiles_fine = h->njobs_fine;
   h->stats.tiles_coarse = h->njobs_coarse;
   return BSE_OK;

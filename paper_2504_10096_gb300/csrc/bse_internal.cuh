@@ -18,7 +18,8 @@ namespace bse {
 
 constexpr int TS = 128;            // tile edge of the packed storage
 constexpr int PROD_THREADS = 256;  // 16 x 16 threads per tile
-constexpr int ROWBLK = 2048;       // rows per CTA in the tall-skinny reductions
+constexpr int ROWBLK = 2048;       // rows per CTA in the tall-skinny reductions of the post-processing
+constexpr int DOT_CHUNKS = 8;      // row chunks of the Gram-Schmidt dots, at most (4, 16: slower)
 constexpr int MAXM = 1024;         // largest Krylov subspace supported
 
 // ---------------------------------------------------------------- complex
@@ -108,6 +109,7 @@ struct Prob {
   int64_t Npad;       // nT * TS
   int ph;             // 1 for the pseudo-Hermitian form
   int ncv;
+  int slab;           // rows of a slab of the Gram-Schmidt updates: 8, 16 or 32
   int ncol;           // stride of the CGS partial sums and coefficients: 2 ncv + 1
                       // (PH: ncv + 1 K-inner products and ncv + 1 twin coefficients)
   const void* A;      // packed tiles
@@ -119,7 +121,9 @@ struct Prob {
   void* w;            // Npad work vectors
   void* pw;
   void* part;         // product partials nT * nT * TS * KMAXP (compute type)
-  double* cpart;      // CGS / norm partials: nrb * ncol complex
+  double* cpart;      // CGS partial dots: DOT_CHUNKS x ncol (TDA: complex)
+  double* npart;      // partial sums of a new vector's squared norm (norm_parts of them)
+  unsigned int* tick; // CTAs of a normalisation that are done (reset by the last one)
   double* coef;       // 2 * ncol complex (pass 1, pass 2)
   double* theta;      // [ncv + 1] Ritz values of kept vectors
   double* barrow;     // [ncv + 1] arrow couplings
@@ -128,7 +132,6 @@ struct Prob {
   double* ritz;       // [ncv] Ritz values of the active block
   double* rest;       // [ncv] Ritz estimates
   double* S;          // ncv x ncv, column-major, ld ncv
-  int nrb;            // row blocks of the tall-skinny reductions
   KState* st;
   // complex128 path with double-FP32 products: the packed tiles split into
   // (hi, lo) float pairs, float4 {re_hi, im_hi, re_lo, im_lo} per element
@@ -167,6 +170,7 @@ struct Prob {
   const int4* Bfx;
   const int* texp;
   int nq;
+  int* err;           // raised by a product kernel whose bounded wait expired
 };
 
 // Jobs of the tiled product: problem, tile row I, tile column J, tile index.
@@ -255,7 +259,7 @@ void launch_prod_reduce_d(const Prob* dprobs, int nprob, int maxnT, int mode, Ge
 // tiles first, then the ones of the FP64 kernel
 void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, int nq, int nprob, int maxnT,
                        int mode, const GenericIO* io_host, bool hasB, ProdShape shape, cudaStream_t s);
-int product_fx_occupancy(bool hasB);
+int product_fx_occupancy();
 // limbs and scales of packed complex128 tiles; texp[t] = -1 for tiles left to the FP64 kernel
 void launch_fx_pack(const double2* A, const double2* B, int64_t N, int nT, int4* Afx, int4* Bfx, int* texp,
                     cudaStream_t s);
@@ -304,10 +308,8 @@ int launch_adjoint_tc(const double2* Z, int64_t ldz, int64_t Npad, int64_t N, in
 // barrier.  Returns 0 (launched), 1 (not available: no cooperative launch; the caller uses the
 // per-phase kernels) or -1 (CUDA error).  A barrier wait that expires sets gb->err.
 struct GridBar {
-  unsigned int count;
-  unsigned int gen;
+  unsigned int count;   // arrivals of the launch so far
   int err;
-  int pad;
 };
 template <typename ST, typename R>
 int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, bool ph, int steps,
@@ -325,11 +327,11 @@ int dense_shao(const Prob* dprobs, int64_t N, int64_t Npad, bool tiles64, bool p
 // normalisation: 0 the folded (or TDA) step, 1 the odd half of a Gruning step (against W
 // and the twins i V), 2 its even half and its fresh vectors (against V and the twins i W)
 template <typename ST>
-void launch_step_cgs(const Prob* dprobs, int nprob, int ph, int maxnrb, int64_t maxNpad,
-                     int ncol, int pass, int half, bool dfs, cudaStream_t s);
+void launch_step_cgs(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int slab, int ncol, int pass, int half,
+                     bool dfs, cudaStream_t s);
 template <typename ST>
-void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int maxnrb, int64_t maxNpad,
-                           int start, int half, cudaStream_t s);
+void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int start, int half,
+                           cudaStream_t s);
 template <typename ST>
 void launch_start_vector(const Prob* dprobs, int nprob, int64_t maxNpad, uint64_t seed,
                          const void* v0, cudaStream_t s);

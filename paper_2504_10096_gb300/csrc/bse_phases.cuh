@@ -264,6 +264,22 @@ __device__ __forceinline__ void prod_tiles_body(const Prob* __restrict__ probs, 
   }
 }
 
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+  return v;
+}
+
+// The products whose result closes a Krylov vector: their reduction leaves the partial sums of the
+// squared norm Re(w^H M w) (one per 32 rows), so that the normalisation needs no pass of its own.
+__device__ __forceinline__ bool prod_is_norm(int mode) {
+  return mode == PM_STEP_MPLUS || mode == PM_START_MPLUS || mode == PM_STEP_MMINUS_W;
+}
+template <typename ST>
+__device__ __forceinline__ double norm_term(ST a, ST b) {
+  return (double)a.x * (double)b.x + (double)a.y * (double)b.y;
+}
+
 // y[I*TS + r] = sum_J part[I][J][r].  A unit is 32 rows of a block row: 8 warps, lane = row, warp
 // g sums the slots J = g, g + 8, ... in order, and the eight group sums are added in group order
 // (a fixed rounding order).  FP64 adds cost 64 clocks per warp and scheduler on this GPU, so the
@@ -323,153 +339,123 @@ __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs,
         acc.y = fma(u.y, xv.x, acc.y); acc.y = fma(v.x, xv.y, acc.y);
       }
     }
-    y[row] = ccvt<ST>(acc);
+    const ST yv = ccvt<ST>(acc);
+    y[row] = yv;
+    if (prod_is_norm(mode)) {          // the squared norm's partial sum Re(w^H M w)
+      const double s = norm_term(ldp<COH>(x + row), yv);
+      const double t = warp_sum_d(s);
+      if (lane == 0) p.npart[u] = t;
+    }
   }
   __syncthreads();                     // grp is rewritten by the next unit
 }
 
 // ---------------------------------------------------------------- CGS2 dots
-// PH: cpart[rb][c] = sum_{rows in block rb} Re(conj(Dm[row, c]) x[row]) for c < nm and
+// PH: cpart[k][c] = sum_{rows in chunk k} Re(conj(Dm[row, c]) x[row]) for c < nm and
 // Im(conj(Dt[row, c']) x[row]) for c = nm + c' (the twin coefficients), nm + nt in all;
-// TDA: the complex conj(V[row, c]) x[row], c <= j.  grid (ceil(maxcols/2), maxnrb, nprob),
-// 8 warps: two columns per CTA, four warps per column, each warp a quarter of the block
-// rows; the four partial sums meet in shared memory (fixed order).
-// One unit: column pair bx, row block rb of problem ip (the kernel's blockIdx (x, y, z));
-// red: 2 x 4 double2 of shared memory.
+// TDA: the complex conj(V[row, c]) x[row], c <= j.  A warp-wide FP64 instruction takes 64 clocks
+// of its scheduler, so the work is cut into one-warp tasks (a column on a chunk of rows) that
+// spread evenly over all schedulers of the GPU; at most DOT_CHUNKS chunks, whole tiles each.
+__host__ __device__ __forceinline__ int dot_chunk_tiles(int nT) { return (nT + DOT_CHUNKS - 1) / DOT_CHUNKS; }
+__host__ __device__ __forceinline__ int dot_chunks(int nT) {
+  return (nT + dot_chunk_tiles(nT) - 1) / dot_chunk_tiles(nT);
+}
+
+// One task (a warp): column c of the set, chunk k.
 template <typename ST, bool COH>
-__device__ __forceinline__ void cgs_dot_body(const Prob* __restrict__ probs, int ph, int newvec, int half, int pass,
-                                             int bx, int rb, int ip, double2 (*red)[4]) {
+__device__ __forceinline__ void cgs_dot_task(const Prob& p, const KState* st, const CgsSet& cs, int ph, int newvec,
+                                             int half, int pass, int c, int k) {
   using R = typename RealOf<ST>::T;
-  const Prob& p = probs[ip];
-  const KState* st = p.st;
-  if (!kphase(st, newvec)) return;
-  if (rb >= p.nrb) return;
-  const CgsSet cs = cgs_set(p, st, ph, half);
-  const int nset = cs.nm + cs.nt;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int hw = warp >> 2, quarter = warp & 3;
-  const int c = bx * 2 + hw;
-  if (bx * 2 >= nset) return;                     // whole CTA
-  double2 a = mk(0.0, 0.0);
-  if (c < nset) {
-    const bool twin = c >= cs.nm;                         // warp-uniform
-    const int col = twin ? c - cs.nm : c;
-    const ST* Q = (const ST*)(twin ? cs.dt : cs.dm) + (int64_t)col * p.Npad;
-    const ST* w = cgs_src<ST>(p, st, half, pass, newvec);
-    const int64_t r0 = (int64_t)rb * ROWBLK + quarter * (ROWBLK / 4);
-    const int64_t r1 = min((int64_t)p.Npad, r0 + ROWBLK / 4);
-    // rounds of 8 rows per lane: all 16 loads of a round are issued before its arithmetic
-    int64_t r = r0 + lane;
-    if (ph) {   // real coefficients: Re(conj(q) x), or Im(conj(q) x) = Re(conj(q) (-i x)) for twins
-      R a1 = 0, a2 = 0;   // two chains (x and y products) for more ILP
-      for (; r + 7 * 32 < r1; r += 8 * 32) {
-        ST q[8], x[8];
+  const int lane = threadIdx.x & 31;
+  const bool twin = c >= cs.nm;                         // warp-uniform
+  const int col = twin ? c - cs.nm : c;
+  const int64_t rows = (int64_t)dot_chunk_tiles(p.nT) * TS;
+  const int64_t r0 = k * rows, r1 = min(p.Npad, r0 + rows);
+  const ST* Q = (const ST*)(twin ? cs.dt : cs.dm) + (int64_t)col * p.Npad;
+  const ST* w = cgs_src<ST>(p, st, half, pass, newvec);
+  int64_t r = r0 + lane;
+  if (ph) {   // real coefficients: Re(conj(q) x), or Im(conj(q) x) = Re(conj(q) (-i x)) for twins
+    R a1 = 0, a2 = 0;   // two chains (x and y products)
+    for (; r < r1; r += 4 * 32) {                       // whole tiles: four rows per lane and round
+      ST q[4], x[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          q[u] = ldv<COH>(Q + r + 32 * u);
-          x[u] = ldv<COH>(w + r + 32 * u);
-        }
-        if (twin) {
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const R t = x[u].x;
-            x[u].x = x[u].y;
-            x[u].y = -t;
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          a1 = fma(q[u].x, x[u].x, a1);
-          a2 = fma(q[u].y, x[u].y, a2);
-        }
+      for (int u = 0; u < 4; ++u) {
+        q[u] = ldv<COH>(Q + r + 32 * u);
+        x[u] = ldv<COH>(w + r + 32 * u);
       }
-      for (; r < r1; r += 32) {
-        const ST q = ldv<COH>(Q + r);
-        ST x = ldv<COH>(w + r);
-        if (twin) {
-          const R t = x.x;
-          x.x = x.y;
-          x.y = -t;
-        }
-        a1 = fma(q.x, x.x, a1);
-        a2 = fma(q.y, x.y, a2);
-      }
-      a = mk((double)a1 + (double)a2, 0.0);
-    } else {
-      ST acc = czero<ST>();
-      for (; r + 7 * 32 < r1; r += 8 * 32) {
-        ST q[8], x[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          q[u] = ldv<COH>(Q + r + 32 * u);
-          x[u] = ldv<COH>(w + r + 32 * u);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) cfmac(acc, q[u], x[u]);
+      for (int u = 0; u < 4; ++u) {
+        a1 = fma(q[u].x, twin ? x[u].y : x[u].x, a1);
+        a2 = fma(q[u].y, twin ? -x[u].x : x[u].y, a2);
       }
-      for (; r < r1; r += 32) cfmac(acc, ldv<COH>(Q + r), ldv<COH>(w + r));
-      a = mk((double)acc.x, (double)acc.y);
     }
+    const double t = warp_sum_d((double)a1 + (double)a2);
+    if (lane == 0) p.cpart[(int64_t)k * p.ncol + c] = t;
+  } else {
+    ST acc = czero<ST>();
+    for (; r < r1; r += 4 * 32) {
+      ST q[4], x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        q[u] = ldv<COH>(Q + r + 32 * u);
+        x[u] = ldv<COH>(w + r + 32 * u);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cfmac(acc, q[u], x[u]);
+    }
+    double2 a = mk((double)acc.x, (double)acc.y);
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) a = cadd(a, dshfl(a, m));
-  }
-  if (lane == 0) red[hw][quarter] = a;
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    const int cc = bx * 2 + threadIdx.x;
-    if (cc < nset) {
-      double2 t = red[threadIdx.x][0];
-#pragma unroll
-      for (int q = 1; q < 4; ++q) t = cadd(t, red[threadIdx.x][q]);
-      ((double2*)p.cpart)[(int64_t)rb * p.ncol + cc] = t;
-    }
+    if (lane == 0) ((double2*)p.cpart)[(int64_t)k * p.ncol + c] = a;
   }
 }
 
+// ---------------------------------------------------------------- CGS2 updates
 // w[row] = x[row] - sum_{c < nm} Um[row, c] coef[pass][c] (- i sum_{c'} Ut[row, c'] coef[pass][nm+c']
-// on the PH paths: the twin projection).  grid (ceil(maxNpad/32), nprob), 8 warps: lane = row of a
-// 32-row slab, warp w takes the set entries c = w mod 8 (six or eight loads in flight each),
-// and the eight partial sums meet in shared memory.  Spreading the columns over warps keeps
-// enough loads in flight when N is only a few hundred slabs; three CTAs per SM keep N = 10^4
-// (316 slabs) in one wave (ncu: at two per SM the last 12 CTAs ran as a second wave).
-// One unit: 32-row slab bx of problem ip; cf: 2 MAXM + 2 entries and red: 8 x 32 entries
-// of shared memory.
-template <typename ST, bool COH>
-__device__ __forceinline__ void cgs_update_body(const Prob* __restrict__ probs, int ph, int pass, int newvec,
-                                                int half, int bx, int ip, ST* cf, ST (*red)[32]) {
+// on the PH paths: the twin projection).  A unit is a slab of 8, 16 or 32 rows (Prob::slab: the
+// smallest that does not give more units than there are SMs; every unit sums the dots'
+// partial sums itself, so more of them cost more than they spread): a thread owns one row and every (256 / rows)-th
+// column of the set, and the partial sums meet in shared memory.
+// the sum of column c's partial dots over the chunks, in chunk order
+template <bool COH>
+__device__ __forceinline__ double2 cgs_coef(const Prob& p, int ph, int c, int nch) {
+  double2 sc = mk(0.0, 0.0);
+  if (ph) {
+    double v[DOT_CHUNKS];
+#pragma unroll
+    for (int k = 0; k < DOT_CHUNKS; ++k) v[k] = k < nch ? ldp<COH>(p.cpart + (int64_t)k * p.ncol + c) : 0.0;
+    sc.x = v[0];
+    for (int k = 1; k < nch; ++k) sc.x += v[k];
+  } else {
+    const double2* cp = (const double2*)p.cpart;
+    for (int k = 0; k < nch; ++k) sc = cadd(sc, ldp<COH>(cp + (int64_t)k * p.ncol + c));
+  }
+  return sc;
+}
+
+// One unit: slab bx of problem ip; cf: 2 MAXM + 2 entries and red: 8 x 32 entries of shared memory.
+template <typename ST, bool COH, int RS>
+__device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st, int ph, int pass, int newvec, int half,
+                                                int bx, ST* cf, ST (*red)[32]) {
   using R = typename RealOf<ST>::T;
-  const Prob& p = probs[ip];
-  const KState* st = p.st;
-  if (!kphase(st, newvec)) return;
-  const int64_t row = (int64_t)bx * 32 + (threadIdx.x & 31);
-  if ((int64_t)bx * 32 >= p.Npad) return;     // whole block (Npad is a multiple of 128)
+  constexpr int G = 256 / RS;                 // column groups
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const CgsSet cs = cgs_set(p, st, ph, half);
   const int nm = cs.nm;
   const int nset = nm + cs.nt;
-  // coefficients: the row-block partial sums of the dots, added in row-block order (PH: real
-  // part only); the first row slab also stores them for k_step_finish
-  const double2* cp = (const double2*)p.cpart;
+  const int nch = dot_chunks(p.nT);
+  // coefficients; the first slab also stores them for the step's end
   double2* coef = (double2*)p.coef + (int64_t)(pass & 1) * p.ncol;
-  for (int c = threadIdx.x; c < nset; c += blockDim.x) {
-    double2 sc = mk(0.0, 0.0);
-    int rb = 0;
-    for (; rb + 8 <= p.nrb; rb += 8) {      // eight loads in flight, then the sums in order
-      double2 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = ldp<COH>(cp + (int64_t)(rb + u) * p.ncol + c);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) sc = cadd(sc, v[u]);
-    }
-    for (; rb < p.nrb; ++rb) sc = cadd(sc, ldp<COH>(cp + (int64_t)rb * p.ncol + c));
-    if (ph) sc.y = 0.0;
+  for (int c = tid; c < nset; c += 256) {
+    const double2 sc = cgs_coef<COH>(p, ph, c, nch);
     cf[c] = ccvt<ST>(sc);
     if (bx == 0) coef[c] = sc;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
   const ST* vb = (const ST*)cs.um + row;
   const ST* pb = ph ? (const ST*)cs.ut + row : nullptr;
-  constexpr int U = sizeof(ST) == 16 ? 6 : 8;   // loads in flight per thread (registers for 3 CTAs/SM)
+  constexpr int U = sizeof(ST) == 16 ? 6 : 8;   // loads in flight per thread
   const int64_t ld = p.Npad;
   // entry cc of the set: Um[:, cc] for cc < nm, else the twin i Ut[:, cc - nm] (as (-t.y, t.x))
   auto colval = [&](int cc) -> ST {
@@ -481,97 +467,93 @@ __device__ __forceinline__ void cgs_update_body(const Prob* __restrict__ probs, 
     return t;
   };
   ST part = czero<ST>();
-  int c = warp;
+  int c = tid / RS;
   // all U loads of a round are issued before any of their arithmetic
   if (ph) {                                 // real coefficients (K-inner products, twin projections)
-    R ax[U], ay[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) ax[u] = ay[u] = (R)0;
-    for (; c + 8 * (U - 1) < nset; c += 8 * U) {
+    for (; c < nset; c += G * U) {
       ST v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) v[u] = colval(c + 8 * u);
+      for (int u = 0; u < U; ++u)
+        if (c + G * u < nset) v[u] = colval(c + G * u);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const R f = cf[c + 8 * u].x;
-        ax[u] = fma(v[u].x, f, ax[u]);
-        ay[u] = fma(v[u].y, f, ay[u]);
-      }
-    }
-    for (; c < nset; c += 8) {
-      const ST v = colval(c);
-      const R f = cf[c].x;
-      ax[0] = fma(v.x, f, ax[0]);
-      ay[0] = fma(v.y, f, ay[0]);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      part.x += ax[u];
-      part.y += ay[u];
+      for (int u = 0; u < U; ++u)
+        if (c + G * u < nset) {
+          const R f = cf[c + G * u].x;
+          part.x = fma(v[u].x, f, part.x);
+          part.y = fma(v[u].y, f, part.y);
+        }
     }
   } else {
-    ST acc[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) acc[u] = czero<ST>();
-    for (; c + 8 * (U - 1) < nset; c += 8 * U) {
+    for (; c < nset; c += G * U) {
       ST v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) v[u] = ldv<COH>(vb + (int64_t)(c + 8 * u) * ld);
+      for (int u = 0; u < U; ++u)
+        if (c + G * u < nset) v[u] = ldv<COH>(vb + (int64_t)(c + G * u) * ld);
 #pragma unroll
-      for (int u = 0; u < U; ++u) cfma(acc[u], v[u], cf[c + 8 * u]);
+      for (int u = 0; u < U; ++u)
+        if (c + G * u < nset) cfma(part, v[u], cf[c + G * u]);
     }
-    for (; c < nset; c += 8) cfma(acc[0], ldv<COH>(vb + (int64_t)c * ld), cf[c]);
-#pragma unroll
-    for (int u = 0; u < U; ++u) part = cadd(part, acc[u]);
   }
-  red[warp][lane] = part;
-  __syncthreads();
-  if (warp == 0) {
-    ST tot = red[0][lane];
 #pragma unroll
-    for (int q = 1; q < 8; ++q) tot = cadd(tot, red[q][lane]);
-    const ST* x = cgs_src<ST>(p, st, half, pass, newvec);
-    ST* w = (ST*)p.w;
-    w[row] = csub(ldp<COH>(x + row), tot);
+  for (int m = RS; m < 32; m <<= 1) part = cadd(part, shfl_xor_c(part, m));   // the warp's groups
+  if (lane < RS) red[warp][lane] = part;
+  __syncthreads();
+  // eight sums per row and component: a lane per sum
+  const ST* x = cgs_src<ST>(p, st, half, pass, newvec);
+  ST* w = (ST*)p.w;
+  double nrm = 0.0;
+#pragma unroll
+  for (int v = tid; v < RS * 16; v += 256) {
+    const int r = v >> 4, comp = (v >> 3) & 1;
+    const R* e = reinterpret_cast<const R*>(&red[v & 7][r]);
+    R t = e[comp];
+#pragma unroll
+    for (int m = 1; m < 8; m <<= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+    if ((v & 7) == 0) {
+      const int64_t o = ((int64_t)bx * RS + r) * 2 + comp;
+      const R nw = ldp<COH>((const R*)x + o) - t;
+      ((R*)w)[o] = nw;
+      nrm += (double)nw * (double)nw;
+    }
+  }
+  if (!ph && (pass & 1)) {                  // TDA: the squared norm's partial sum of the slab
+    nrm = warp_sum_d(nrm);
+    __syncthreads();
+    double* rd = reinterpret_cast<double*>(red);
+    if (lane == 0) rd[warp] = nrm;
+    __syncthreads();
+    if (tid == 0) {
+      double t = rd[0];
+      for (int q = 1; q < (RS * 16 < 256 ? RS * 16 / 32 : 8); ++q) t += rd[q];
+      p.npart[bx] = t;
+    }
+  }
+}
+
+template <typename ST, bool COH>
+__device__ __forceinline__ void cgs_update_unit(const Prob& p, const KState* st, int ph, int pass, int newvec, int half,
+                                                int bx, ST* cf, ST (*red)[32]) {
+  switch (p.slab) {
+    case 8: return cgs_update_slab<ST, COH, 8>(p, st, ph, pass, newvec, half, bx, cf, red);
+    case 16: return cgs_update_slab<ST, COH, 16>(p, st, ph, pass, newvec, half, bx, cf, red);
+    default: return cgs_update_slab<ST, COH, 32>(p, st, ph, pass, newvec, half, bx, cf, red);
   }
 }
 
 // ---------------------------------------------------------------- norms
-// cpart[rb].x = sum over rows of Re(conj(w) pw) (PH) or |w|^2 (TDA).
-// One unit: row block rb of problem ip; red: 8 doubles of shared memory.
-template <typename ST, bool COH = false>
-__device__ __forceinline__ void norm_partial_body(const Prob* __restrict__ probs, int ph, int start, int rb, int ip,
-                                                  double* red) {
-  const Prob& p = probs[ip];
-  const KState* st = p.st;
-  if (!kphase(st, start)) return;
-  if (rb >= p.nrb) return;
-  const ST* w = (const ST*)p.w;
-  const ST* pw = (const ST*)(ph ? p.pw : p.w);
-  const int64_t r0 = (int64_t)rb * ROWBLK;
-  const int64_t r1 = min((int64_t)p.Npad, r0 + ROWBLK);
-  double s = 0.0;
-  for (int64_t r = r0 + threadIdx.x; r < r1; r += 256) {
-    const ST a = ldp<COH>(w + r), b = ldp<COH>(pw + r);
-    s += (double)a.x * (double)b.x + (double)a.y * (double)b.y;
-  }
-#pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += red[i];
-    ((double2*)p.cpart)[rb] = mk(t, 0.0);
-  }
+// Partial sums of a new vector's squared norm: per 32 rows on the PH paths (the reduction of the
+// closing product), per slab of the last Gram-Schmidt update on the TDA path.
+__device__ __forceinline__ int norm_parts(const Prob& p, int ph) {
+  return (int)(p.Npad / (ph ? REDUCE_ROWS : p.slab));
 }
 
-template <bool COH = false>
-__device__ __forceinline__ double sum_norm_parts(const Prob& p) {
-  const double2* cp = (const double2*)p.cpart;
+// their sum in every lane of a warp, in a fixed order
+template <bool COH>
+__device__ __forceinline__ double norm_sum(const Prob& p, int ph) {
+  const int n = norm_parts(p, ph);
   double s = 0.0;
-  for (int rb = 0; rb < p.nrb; ++rb) s += ldp<COH>(cp + rb).x;
-  return s;
+  for (int i = threadIdx.x & 31; i < n; i += 32) s += ldp<COH>(p.npart + i);
+  return warp_sum_d(s);
 }
 
 // Where a normalised vector goes: V[:, j+1] (and P) for the folded / TDA step and the even
@@ -599,23 +581,10 @@ __device__ __forceinline__ void shadow_store(const Prob& p, const KState* st, in
   }
 }
 
-// X = w / beta, Y = pw / beta (norm_dest) when beta^2 is usable.
-// One unit: rows bx * blockDim.x ... of problem ip; sb2: one double of shared memory.
-template <typename ST, bool COH = false>
-__device__ __forceinline__ void normalize_body(const Prob* __restrict__ probs, int ph, int start, int half, int bx,
-                                               int ip, double* sb2) {
-  using R = typename RealOf<ST>::T;
-  const Prob& p = probs[ip];
-  const KState* st = p.st;
-  if (!kphase(st, start)) return;
-  if (threadIdx.x == 0) *sb2 = sum_norm_parts<COH>(p);
-  __syncthreads();
-  const double b2 = *sb2;
-  __syncthreads();                              // sb2 is rewritten by the next unit
-  if (!(b2 > 0.0) || !isfinite(b2)) return;   // k_step_finish records the outcome
-  const R inv = (R)(1.0 / sqrt(b2));
-  const int64_t row = (int64_t)bx * blockDim.x + threadIdx.x;
-  if (row >= p.Npad) return;
+// X = w / beta, Y = pw / beta (norm_dest) for one row, beta^2 = b2 > 0 and finite
+template <typename ST, bool COH>
+__device__ __forceinline__ void normalize_row(const Prob& p, const KState* st, int ph, int half, int64_t row,
+                                              typename RealOf<ST>::T inv) {
   ST *X, *Y;
   norm_dest<ST>(p, st, half, X, Y);
   const ST xv = cscale(ldp<COH>((const ST*)p.w + row), inv);
@@ -627,28 +596,31 @@ __device__ __forceinline__ void normalize_body(const Prob* __restrict__ probs, i
 
 // Record alpha_j, beta_j, advance j, given beta^2 = b2 of the new vector.  fresh = 0:
 // regular step; fresh = 1: a first or replacement vector was just normalised.
-__device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh, double b2) {
+// In a persistent launch every CTA keeps its own copy of the state and runs this on it; one of
+// them (`writer`) also stores alpha and beta.
+template <bool COH>
+__device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh, double b2, bool writer) {
   KState* st = p.st;
   const int j = st->j;
   if (!fresh) {
     const double2* coef = (const double2*)p.coef;
-    const double a = coef[j].x + coef[p.ncol + j].x;
+    const double a = ldp<COH>(&coef[j].x) + ldp<COH>(&coef[p.ncol + j].x);
     if (!isfinite(a) || !isfinite(b2)) { st->status = ST_NOTFINITE; return; }
-    p.alpha[j] = a;
+    if (writer) p.alpha[j] = a;
     st->passes += ph ? 2 : 1;
     st->steps += 1;
     // scale of the projected matrix for the breakdown test
     double scale = fabs(a);
     scale = fmax(scale, st->theta_scale);   // max |theta| of the kept Ritz values
-    if (j > 0) scale = fmax(scale, fabs(p.beta[j - 1]));
+    if (j > 0) scale = fmax(scale, fabs(ldp<COH>(p.beta + j - 1)));
     const double tiny = 1e-26 * scale * scale + 1e-300;
     if (ph && b2 < -1e6 * tiny) { st->status = ST_NOTPD; return; }
     if (b2 <= tiny) {                 // invariant subspace: the chain restarts
-      p.beta[j] = 0.0;                // with a fresh vector (host-driven)
+      if (writer) p.beta[j] = 0.0;    // with a fresh vector (host-driven)
       st->breakdown = 1;
       return;
     }
-    p.beta[j] = sqrt(b2);
+    if (writer) p.beta[j] = sqrt(b2);
     st->j = j + 1;
   } else {
     if (!isfinite(b2)) { st->status = ST_NOTFINITE; return; }
@@ -698,56 +670,11 @@ __device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh
   if (st->steps >= st->maxit && !st->done) { st->done = 1; st->status = ST_NOCONV; }
 }
 
-__device__ __forceinline__ void finish_one(const Prob& p, int ph, int fresh, int half, double b2) {
+template <bool COH>
+__device__ __forceinline__ void finish_one(const Prob& p, int ph, int fresh, int half, double b2, bool writer) {
   if (half) gk_finish_one(p, half, fresh, b2);
-  else step_finish_one(p, ph, fresh, b2);
+  else step_finish_one<COH>(p, ph, fresh, b2, writer);
 }
 
-
-// Problems of at most one reduction row block (Npad <= ROWBLK): the norm, the scaling of
-// the new basis vector and the state update in one CTA per problem (one launch instead of
-// three per Krylov step; the same arithmetic as k_norm_partial, k_normalize, k_step_finish).
-// One unit: problem ip; red: 8 doubles and sb2p: one double of shared memory.
-template <typename ST, bool COH = false>
-__device__ __forceinline__ void norm_fused_body(const Prob* __restrict__ probs, int ph, int start, int half, int ip,
-                                                double* red, double* sb2p) {
-  using R = typename RealOf<ST>::T;
-  double& sb2 = *sb2p;
-  const Prob& p = probs[ip];
-  const KState* st = p.st;
-  if (!kphase(st, start)) return;
-  const ST* w = (const ST*)p.w;
-  const ST* pw = (const ST*)(ph ? p.pw : p.w);
-  double s = 0.0;
-  for (int64_t r = threadIdx.x; r < p.Npad; r += 256) {
-    const ST a = ldp<COH>(w + r), b = ldp<COH>(pw + r);
-    s += (double)a.x * (double)b.x + (double)a.y * (double)b.y;
-  }
-#pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += red[i];
-    sb2 = t;
-  }
-  __syncthreads();
-  const double b2 = sb2;
-  if (b2 > 0.0 && isfinite(b2)) {
-    const R inv = (R)(1.0 / sqrt(b2));
-    ST *X, *Y;
-    norm_dest<ST>(p, st, half, X, Y);
-    for (int64_t r = threadIdx.x; r < p.Npad; r += 256) {
-      const ST xv = cscale(ldp<COH>(w + r), inv);
-      X[r] = xv;
-      ST yv = czero<ST>();
-      if (ph) Y[r] = yv = cscale(ldp<COH>((const ST*)p.pw + r), inv);
-      shadow_store<ST>(p, st, half, r, xv, yv);
-    }
-  }
-  __syncthreads();                     // every thread has read st->j
-  if (threadIdx.x == 0) finish_one(p, ph, start, half, b2);
-}
 
 }  // namespace bse

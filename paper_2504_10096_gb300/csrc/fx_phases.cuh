@@ -25,8 +25,9 @@
 //
 // Bounds: 3 integer multiply-adds per real FMA instead of one FMA of a two-lane FP64 pipe; 32
 // bytes per element pair either way, so the large products meet HBM instead of the FP64 pipe.
-// Measured, folded product: N = 8000 503 -> 228 us (HBM floor 154), N = 3000 75 -> 36 us,
-// N = 900 38 -> 6.7 us (36 tiles in bands).  Against extended precision, N = 127 ... 2500: 0.3 to
+// Measured, folded product: N = 8000 503 -> 171 us (6.05 TB/s), N = 3000 75 -> 28.5 us, N = 900
+// 38 -> 7.1 us (36 tiles in bands).  Sixteen warps per SM matter: the integer multiply-adds wait
+// on one another, and eight warps ran N = 8000 in 229 us.  Against extended precision, N = 127 ... 2500: 0.3 to
 // 1.2 units of 2^-53 normwise, the FP64 kernel 0.8 to 5.5.
 #pragma once
 
@@ -38,13 +39,52 @@ constexpr int FX_THREADS = 256;
 constexpr int FX_WARPS = FX_THREADS / 32;
 constexpr float FX_PEAK = 64.f;
 
-// shared memory of one unit
+constexpr long long FX_SPIN = 1ll << 24;      // polls of one wait for a row
+
+// Shared memory of a CTA.  Each warp streams its own rows of the tiles through a ring of row
+// buffers (a row of A and of B, 4 KiB, or of A alone, 2 KiB) with bulk asynchronous copies that
+// complete on the warp's own barriers, several rows ahead and across the units'
+// boundaries: 128 KiB in flight per SM and no block barrier in the row loop.
+template <int RING>                    // bytes of a warp's ring
 struct FxShared {
+  unsigned char ring[FX_WARPS][RING];
+  unsigned long long bar[FX_WARPS][8];
   int4 x[2][TS];                       // limbs of the column chunk J and the row chunk I
   int rows[TS][6];                     // three words of (re, im) per row of the unit
   int cols[FX_WARPS][6][TS];           // ... per column, one partial sum per warp
   unsigned int mx[2][TS / 32];
 };
+
+__device__ __forceinline__ uint32_t fx_s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// once per launch, before the first unit (all threads; the caller synchronises the block)
+template <int RING>
+__device__ __forceinline__ void fx_init(FxShared<RING>& sh) {
+  if (threadIdx.x < FX_WARPS * 8)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(fx_s32(&sh.bar[0][0] + threadIdx.x)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ bool fx_wait(uint32_t bar, uint32_t parity) {
+  for (long long i = 0; i < FX_SPIN; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void fx_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(bar)
+      : "memory");
+}
 
 __device__ __forceinline__ unsigned int hi_abs(double v) { return (unsigned int)__double2hiint(v) & 0x7fffffffu; }
 
@@ -117,148 +157,202 @@ __device__ __forceinline__ double fx_double(int w0, unsigned int w1, unsigned in
   return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
+// A warp's place in its stream of rows; it outlives one walk over the units (the barriers' phases
+// go on), so a kernel keeps one per warp for its whole life.
+struct FxPipe {
+  unsigned int issued = 0, used = 0;     // rows copied, rows consumed
+  bool ok = true;                        // no wait has expired
+};
+
 // Units of the fixed-point product: a tile, or a band of TS / nq of its rows.  A band's row sums
 // are whole rows of slot (I, J); its column sums go to plane q of the slots, which the reduction
 // adds.  Bands exist so that a problem of few tiles still occupies every SM.
-// One unit: job t, band q; `sh` is rewritten by the next unit.
-template <bool HASB, bool COH>
-__device__ __forceinline__ void fx_tile_unit(const Prob& p, const TileJob jb, const double2* x, bool pos, int q, int nq,
-                                             FxShared& sh) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool diag = jb.I == jb.J;
-  const int nrow = TS / nq, row0 = q * nrow;
-  const int4* At = (const int4*)(HASB && !pos ? p.Bfx : p.Afx) + (int64_t)jb.t * (TS * TS);
-  const int4* Bt = HASB ? (const int4*)(pos ? p.Bfx : p.Afx) + (int64_t)jb.t * (TS * TS) : nullptr;
-  __syncthreads();                       // shared memory of the previous unit is free
-  const double2 xv = ldp<COH>(x + (int64_t)(tid < TS ? jb.J : jb.I) * TS + (tid & (TS - 1)));
-  {
-    const unsigned int m = __reduce_max_sync(0xffffffffu, max(hi_abs(xv.x), hi_abs(xv.y)));
-    if (lane == 0) sh.mx[warp >> 2][warp & 3] = m;
-  }
-  for (int e = tid; e < FX_WARPS * 6 * TS / 4; e += FX_THREADS)
-    reinterpret_cast<int4*>(sh.cols)[e] = make_int4(0, 0, 0, 0);
-  __syncthreads();
-  auto chunk_exp = [&](int k) {
-    const unsigned int m = max(max(sh.mx[k][0], sh.mx[k][1]), max(sh.mx[k][2], sh.mx[k][3]));
-    return max(64, (int)(m >> 20));
-  };
-  const int ec = chunk_exp(0), er = chunk_exp(1);
-  sh.x[tid >> 7][tid & (TS - 1)] = fx_entry(xv, tid < TS ? ec : er);
-  __syncthreads();
-  int4 xc[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) xc[b] = sh.x[0][lane + 32 * b];
-  const int4* ar = At + (int64_t)(row0 + warp) * TS + lane;
-  const int4* br = HASB ? Bt + (int64_t)(row0 + warp) * TS + lane : nullptr;
-  const int npr = nrow / FX_WARPS;       // rows of this warp: row0 + warp + 8 a
-  int4 un[4], vn[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    un[b] = __ldg(ar + 32 * b);
-    if (HASB) vn[b] = __ldg(br + 32 * b);
-  }
-  for (int a0 = 0; a0 < npr; a0 += 8) {
-    const int a1 = min(npr, a0 + 8);     // a flush every eight rows: 16 terms per column sum
-    long long chh[4][2], chl[4][2];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) chh[b][0] = chh[b][1] = chl[b][0] = chl[b][1] = 0;
-#pragma unroll 1
-    for (int a = a0; a < a1; ++a) {
-      int4 u[4], v[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        u[b] = un[b];
-        v[b] = HASB ? vn[b] : un[b];
-      }
-      if (a + 1 < npr) {                 // the next row's loads run under this row's arithmetic
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          un[b] = __ldg(ar + (int64_t)(a + 1) * FX_WARPS * TS + 32 * b);
-          if (HASB) vn[b] = __ldg(br + (int64_t)(a + 1) * FX_WARPS * TS + 32 * b);
-        }
-      }
-      const int r = row0 + warp + FX_WARPS * a;
-      const int4 y = sh.x[1][r];
-      const int4 yn = make_int4(-y.x, -y.y, -y.z, -y.w);
-      // row (M_s x_J)_r: re = U_re x_re - V_im x_im, im = U_im x_re + V_re x_im
-      long long s1h = 0, s1l = 0, s2h = 0, s2l = 0, s3h = 0, s3l = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        fx_mac(s1h, s1l, u[b].x, u[b].y, xc[b].x, xc[b].y);
-        fx_mac(s2h, s2l, v[b].z, v[b].w, xc[b].z, xc[b].w);
-        fx_mac(s3h, s3l, u[b].z, u[b].w, xc[b].x, xc[b].y);
-        fx_mac(s3h, s3l, v[b].x, v[b].y, xc[b].z, xc[b].w);
-      }
-      if (!diag) {
-        // column (M_s^T x_I)_c: re = U_re y_re + U_im y_im, im = V_re y_im - V_im y_re
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          fx_mac(chh[b][0], chl[b][0], u[b].x, u[b].y, y.x, y.y);
-          fx_mac(chh[b][0], chl[b][0], u[b].z, u[b].w, y.z, y.w);
-          fx_mac(chh[b][1], chl[b][1], v[b].x, v[b].y, y.z, y.w);
-          fx_mac(chh[b][1], chl[b][1], v[b].z, v[b].w, yn.x, yn.y);
-        }
-      }
-      int w[6];
-      fx_words(s1h - s2h, s1l - s2l, w[0], w[1], w[2]);
-      fx_words(s3h, s3l, w[3], w[4], w[5]);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) w[k] = __reduce_add_sync(0xffffffffu, w[k]);
-      if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) sh.rows[r - row0][k] = w[k];
-      }
-    }
-    if (!diag) {
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          int w[3];
-          fx_words(chh[b][c], chl[b][c], w[0], w[1], w[2]);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) sh.cols[warp][3 * c + k][lane + 32 * b] += w[k];
-        }
-    }
-  }
-  __syncthreads();
-  const int eu = p.texp[jb.t];
-  double* part = (double*)p.part;
-  const int i = tid >> 1, c = tid & 1;
-  if (i < nrow) {
-    const int* w = sh.rows[i] + 3 * c;
-    part[(((int64_t)jb.I * p.nT + jb.J) * TS + row0 + i) * 2 + c] = fx_double(w[0], w[1], w[2], eu, ec);
-  }
-  if (!diag) {
-    int w[3] = {0, 0, 0};
-#pragma unroll
-    for (int wp = 0; wp < FX_WARPS; ++wp)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) w[k] += sh.cols[wp][3 * c + k][i];
-    part[(((int64_t)q * p.nT * p.nT + (int64_t)jb.J * p.nT + jb.I) * TS + i) * 2 + c] =
-        fx_double(w[0], w[1], w[2], eu, er);
-  }
-}
-
-// the unit walk of CTA bid of nblk over njobs * nq units
-template <bool HASB, bool COH>
+// The walk of CTA bid of nblk over njobs * nq units.  A wait that expires raises *err; the warp
+// then goes on without waiting (its reads stay inside the ring) and issues no further copy.
+template <bool HASB, bool COH, int RING>
 __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs,
                                               int njobs, int nq, int mode, const GenericIO& io, int strided, int bid,
-                                              int nblk, FxShared& sh) {
-  const int nunit = njobs * nq;
+                                              int nblk, FxShared<RING>& sh, FxPipe& pipe, int* err) {
+  constexpr unsigned int ROWB = TS * sizeof(int4);                     // bytes of one matrix's row
+  constexpr unsigned int DEPTH = RING / (HASB ? 2 * ROWB : ROWB);   // rows in the ring
+  const int lq = 31 - __clz(nq), nunit = njobs << lq;                  // nq is a power of two
   const int per = strided ? 1 : (nunit + nblk - 1) / nblk;
   const int u0 = strided ? bid : bid * per;
   const int u1 = strided ? nunit : min(nunit, u0 + per);
   const int du = strided ? nblk : 1;
-  for (int u = u0; u < u1; u += du) {
-    const TileJob jb = jobs[u / nq];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nrow = TS >> lq, npr = nrow / FX_WARPS;   // rows of a unit and of a warp: row0 + warp + 8 a
+  const uint32_t ring = fx_s32(sh.ring[warp]), bars = fx_s32(sh.bar[warp]);
+  const double2* x;
+  double2* y;
+  double sB = 0.0;
+  // the next unit from u on whose problem takes part, and its operand
+  auto next_unit = [&](int u, TileJob& jb) {
+    for (; u < u1; u += du) {
+      jb = jobs[u >> lq];
+      if (prod_operands<double2, double>(probs[jb.prob], mode, io, x, y, sB)) break;
+    }
+    return u;
+  };
+  auto x_value = [&](const TileJob& jb) {
+    return ldp<COH>(x + (int64_t)(tid < TS ? jb.J : jb.I) * TS + (tid & (TS - 1)));
+  };
+  TileJob jb{}, jn{}, jp{};
+  int un = next_unit(u0, jn);
+  double2 xn = make_double2(0.0, 0.0);
+  if (un < u1) xn = x_value(jn);
+  // producer: `left` rows of unit pu to copy, the next ones at srcA, srcB
+  int pu = un, left = 0;
+  const int4 *srcA = nullptr, *srcB = nullptr;
+  jp = jn;
+  auto source = [&]() {
+    if (pu >= u1) return;
+    const Prob& p = probs[jp.prob];
+    const int64_t off = (int64_t)jp.t * (TS * TS) + ((pu & (nq - 1)) * nrow + warp) * TS;
+    const bool pos = sB > 0.0;           // U, V = P, Q for the plus half, Q, P for the minus half
+    srcA = (HASB && !pos ? p.Bfx : p.Afx) + off;
+    if (HASB) srcB = (pos ? p.Bfx : p.Afx) + off;
+    left = pipe.ok ? npr : 0;
+  };
+  source();
+  auto produce = [&]() {
+    if (left == 0) return;
+    if (lane == 0) {
+      const unsigned int s = pipe.issued % DEPTH;
+      const uint32_t dst = ring + s * (RING / DEPTH), bar = bars + 8 * s;
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                   "r"(HASB ? 2 * ROWB : ROWB)
+                   : "memory");
+      fx_copy(dst, srcA, ROWB, bar);
+      if (HASB) fx_copy(dst + ROWB, srcB, ROWB, bar);
+    }
+    srcA += FX_WARPS * TS;
+    if (HASB) srcB += FX_WARPS * TS;
+    ++pipe.issued;
+    if (--left == 0) {
+      const double2* xs = x;             // the consumer's operand stays
+      pu = next_unit(pu + du, jp);
+      source();
+      x = xs;
+    }
+  };
+  for (unsigned int k = 0; k < DEPTH; ++k) produce();
+  while (un < u1) {
+    const int u = un;
+    jb = jn;
     const Prob& p = probs[jb.prob];
-    const double2* x;
-    double2* y;
-    double sB;
-    if (!prod_operands<double2, double>(p, mode, io, x, y, sB)) continue;   // uniform per CTA
-    fx_tile_unit<HASB, COH>(p, jb, x, sB > 0.0, u % nq, nq, sh);
+    const bool diag = jb.I == jb.J;
+    const int q = u & (nq - 1), row0 = q * nrow;
+    const double2 xv = xn;
+    un = next_unit(u + du, jn);
+    if (un < u1) xn = x_value(jn);       // arrives under this unit's arithmetic
+    __syncthreads();                     // the shared sums of the previous unit have been read
+    {
+      const unsigned int m = __reduce_max_sync(0xffffffffu, max(hi_abs(xv.x), hi_abs(xv.y)));
+      if (lane == 0) sh.mx[warp >> 2][warp & 3] = m;
+    }
+    __syncthreads();
+    auto chunk_exp = [&](int k) {
+      const unsigned int m = max(max(sh.mx[k][0], sh.mx[k][1]), max(sh.mx[k][2], sh.mx[k][3]));
+      return max(64, (int)(m >> 20));
+    };
+    const int ec = chunk_exp(0), er = chunk_exp(1);
+    sh.x[tid >> 7][tid & (TS - 1)] = fx_entry(xv, tid < TS ? ec : er);
+    __syncthreads();
+    int4 xc[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) xc[b] = sh.x[0][lane + 32 * b];
+    for (int a0 = 0; a0 < npr; a0 += 8) {
+      const int a1 = min(npr, a0 + 8);   // a flush every eight rows: 16 terms per column sum
+      long long chh[4][2], chl[4][2];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) chh[b][0] = chh[b][1] = chl[b][0] = chl[b][1] = 0;
+#pragma unroll 1
+      for (int a = a0; a < a1; ++a) {
+        const unsigned int s = pipe.used % DEPTH;
+        if (pipe.ok && __any_sync(0xffffffffu, !fx_wait(bars + 8 * s, (pipe.used / DEPTH) & 1))) {
+          if (lane == 0) atomicExch(err, 1);
+          pipe.ok = false;
+          left = 0;
+        }
+        const int4* rp = reinterpret_cast<const int4*>(sh.ring[warp] + s * (RING / DEPTH)) + lane;
+        int4 uu[4], vv[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          uu[b] = rp[32 * b];
+          vv[b] = HASB ? rp[TS + 32 * b] : uu[b];
+        }
+        ++pipe.used;
+        __syncwarp();                    // the row is in registers: its buffer may be refilled
+        produce();
+        const int r = row0 + warp + FX_WARPS * a;
+        const int4 y4 = sh.x[1][r];
+        const int ynh = -y4.x, ynl = -y4.y;
+        // row (M_s x_J)_r: re = U_re x_re - V_im x_im, im = U_im x_re + V_re x_im
+        long long s1h = 0, s1l = 0, s2h = 0, s2l = 0, s3h = 0, s3l = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          fx_mac(s1h, s1l, uu[b].x, uu[b].y, xc[b].x, xc[b].y);
+          fx_mac(s2h, s2l, vv[b].z, vv[b].w, xc[b].z, xc[b].w);
+          fx_mac(s3h, s3l, uu[b].z, uu[b].w, xc[b].x, xc[b].y);
+          fx_mac(s3h, s3l, vv[b].x, vv[b].y, xc[b].z, xc[b].w);
+        }
+        if (!diag) {
+          // column (M_s^T x_I)_c: re = U_re y_re + U_im y_im, im = V_re y_im - V_im y_re
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            fx_mac(chh[b][0], chl[b][0], uu[b].x, uu[b].y, y4.x, y4.y);
+            fx_mac(chh[b][0], chl[b][0], uu[b].z, uu[b].w, y4.z, y4.w);
+            fx_mac(chh[b][1], chl[b][1], vv[b].x, vv[b].y, y4.z, y4.w);
+            fx_mac(chh[b][1], chl[b][1], vv[b].z, vv[b].w, ynh, ynl);
+          }
+        }
+        int w[6];
+        fx_words(s1h - s2h, s1l - s2l, w[0], w[1], w[2]);
+        fx_words(s3h, s3l, w[3], w[4], w[5]);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w[k] = __reduce_add_sync(0xffffffffu, w[k]);
+        if (lane == 0) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) sh.rows[r - row0][k] = w[k];
+        }
+      }
+      if (!diag) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            int w[3];
+            fx_words(chh[b][c], chl[b][c], w[0], w[1], w[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              int& d = sh.cols[warp][3 * c + k][lane + 32 * b];
+              d = a0 == 0 ? w[k] : d + w[k];
+            }
+          }
+      }
+    }
+    __syncthreads();
+    const int eu = p.texp[jb.t];
+    double* part = (double*)p.part;
+    const int i = tid >> 1, c = tid & 1;
+    if (i < nrow) {
+      const int* w = sh.rows[i] + 3 * c;
+      part[(((int64_t)jb.I * p.nT + jb.J) * TS + row0 + i) * 2 + c] = fx_double(w[0], w[1], w[2], eu, ec);
+    }
+    if (!diag) {
+      int w[3] = {0, 0, 0};
+#pragma unroll
+      for (int wp = 0; wp < FX_WARPS; ++wp)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) w[k] += sh.cols[wp][3 * c + k][i];
+      part[(((int64_t)q * p.nT * p.nT + (int64_t)jb.J * p.nT + jb.I) * TS + i) * 2 + c] =
+          fx_double(w[0], w[1], w[2], eu, er);
+    }
   }
+  if (!pipe.ok && lane == 0)             // leave no copy in flight
+    for (unsigned int k = pipe.issued > DEPTH ? pipe.issued - DEPTH : 0; k < pipe.issued; ++k)
+      fx_wait(bars + 8 * (k % DEPTH), (k / DEPTH) & 1);
 }
 
 }  // namespace bse

@@ -49,11 +49,16 @@ namespace bse {
 
 // ---------------------------------------------------------------- one kernel per phase
 // The bodies (bse_phases.cuh) on the grids of the launchers below.
+// grid (ceil(maxcols/8), chunks, nprob): a warp per column and chunk
 template <typename ST>
 __global__ void __launch_bounds__(256)
 k_cgs_dot(const Prob* __restrict__ probs, int ph, int newvec, int half, int pass) {
-  __shared__ double2 red[2][4];
-  cgs_dot_body<ST, false>(probs, ph, newvec, half, pass, blockIdx.x, blockIdx.y, blockIdx.z, red);
+  const Prob& p = probs[blockIdx.z];
+  const KState* st = p.st;
+  if (!kphase(st, newvec) || (int)blockIdx.y >= dot_chunks(p.nT)) return;
+  const CgsSet cs = cgs_set(p, st, ph, half);
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (c < cs.nm + cs.nt) cgs_dot_task<ST, false>(p, st, cs, ph, newvec, half, pass, c, blockIdx.y);
 }
 
 // three CTAs per SM keep N = 10^4 (316 slabs of 32 rows) in one wave (ncu: at two per SM the
@@ -63,7 +68,10 @@ __global__ void __launch_bounds__(256, 3)
 k_cgs_update(const Prob* __restrict__ probs, int ph, int pass, int newvec, int half) {
   __shared__ ST cf[2 * MAXM + 2];
   __shared__ ST red[8][32];
-  cgs_update_body<ST, false>(probs, ph, pass, newvec, half, blockIdx.x, blockIdx.y, cf, red);
+  const Prob& p = probs[blockIdx.y];
+  const KState* st = p.st;
+  if (!kphase(st, newvec) || (int64_t)blockIdx.x * p.slab >= p.Npad) return;
+  cgs_update_unit<ST, false>(p, st, ph, pass, newvec, half, blockIdx.x, cf, red);
 }
 
 // ---------------------------------------------------------------- double-FP32 Gram-Schmidt
@@ -91,131 +99,96 @@ __device__ __forceinline__ void df_add(float& sh, float& sl, float bh, float bl)
   sl += err + bl;
 }
 
-// units and output as k_cgs_dot (folded step, half 0: Re(P^H w) and Im(V^H w))
+// tasks and output as k_cgs_dot (folded step, half 0: Re(P^H w) and Im(V^H w))
 __global__ void __launch_bounds__(256)
 k_cgs_dot_dfs(const Prob* __restrict__ probs, int newvec) {
-  __shared__ double red[2][4];
   const Prob& p = probs[blockIdx.z];
   const KState* st = p.st;
-  if (!kphase(st, newvec)) return;
-  const int rb = blockIdx.y;
-  if (rb >= p.nrb) return;
+  if (!kphase(st, newvec) || (int)blockIdx.y >= dot_chunks(p.nT)) return;
   const int j = st->j;
-  const int nset = 2 * (j + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int hw = warp >> 2, quarter = warp & 3;
-  const int c = blockIdx.x * 2 + hw;
-  if (blockIdx.x * 2 >= nset) return;                     // whole CTA
-  double a = 0.0;
-  if (c < nset) {
-    const bool twin = c > j;                              // warp-uniform
-    const int col = twin ? c - (j + 1) : c;
-    const float4* Q = (twin ? p.Vs : p.Ps) + (int64_t)col * p.Npad;
-    const float4* w = p.ws;
-    const int64_t r0 = (int64_t)rb * ROWBLK + quarter * (ROWBLK / 4);
-    const int64_t r1 = min((int64_t)p.Npad, r0 + ROWBLK / 4);
-    float sh = 0.f, sl = 0.f;
-    int64_t r = r0 + lane;
-    for (; r + 3 * 32 < r1; r += 4 * 32) {
-      float4 q[4], x[4];
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= 2 * (j + 1)) return;
+  const bool twin = c > j;                              // warp-uniform
+  const int col = twin ? c - (j + 1) : c;
+  const float4* Q = (twin ? p.Vs : p.Ps) + (int64_t)col * p.Npad;
+  const float4* w = p.ws;
+  const int64_t rows = (int64_t)dot_chunk_tiles(p.nT) * TS;
+  const int64_t r0 = blockIdx.y * rows, r1 = min(p.Npad, r0 + rows);
+  float sh = 0.f, sl = 0.f;
+  for (int64_t r = r0 + lane; r < r1; r += 4 * 32) {
+    float4 q[4], x[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        q[u] = __ldg(Q + r + 32 * u);
-        x[u] = __ldg(w + r + 32 * u);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (twin) {              // Im(conj(q) x) = q_re x_im - q_im x_re
-          df_madd(sh, sl, q[u].x, q[u].z, x[u].y, x[u].w);
-          df_madd(sh, sl, -q[u].y, -q[u].w, x[u].x, x[u].z);
-        } else {                 // Re(conj(q) x) = q_re x_re + q_im x_im
-          df_madd(sh, sl, q[u].x, q[u].z, x[u].x, x[u].z);
-          df_madd(sh, sl, q[u].y, q[u].w, x[u].y, x[u].w);
-        }
-      }
-    }
-    for (; r < r1; r += 32) {
-      const float4 q = __ldg(Q + r), x = __ldg(w + r);
-      if (twin) {
-        df_madd(sh, sl, q.x, q.z, x.y, x.w);
-        df_madd(sh, sl, -q.y, -q.w, x.x, x.z);
-      } else {
-        df_madd(sh, sl, q.x, q.z, x.x, x.z);
-        df_madd(sh, sl, q.y, q.w, x.y, x.w);
-      }
+    for (int u = 0; u < 4; ++u) {
+      q[u] = __ldg(Q + r + 32 * u);
+      x[u] = __ldg(w + r + 32 * u);
     }
 #pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, sh, m), ol = __shfl_xor_sync(0xffffffffu, sl, m);
-      df_add(sh, sl, oh, ol);
-    }
-    a = (double)sh + (double)sl;
-  }
-  if (lane == 0) red[hw][quarter] = a;
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    const int cc = blockIdx.x * 2 + threadIdx.x;
-    if (cc < nset) {
-      double t = red[threadIdx.x][0];
-#pragma unroll
-      for (int q = 1; q < 4; ++q) t += red[threadIdx.x][q];
-      ((double2*)p.cpart)[(int64_t)rb * p.ncol + cc] = mk(t, 0.0);
+    for (int u = 0; u < 4; ++u) {
+      if (twin) {              // Im(conj(q) x) = q_re x_im - q_im x_re
+        df_madd(sh, sl, q[u].x, q[u].z, x[u].y, x[u].w);
+        df_madd(sh, sl, -q[u].y, -q[u].w, x[u].x, x[u].z);
+      } else {                 // Re(conj(q) x) = q_re x_re + q_im x_im
+        df_madd(sh, sl, q[u].x, q[u].z, x[u].x, x[u].z);
+        df_madd(sh, sl, q[u].y, q[u].w, x[u].y, x[u].w);
+      }
     }
   }
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, sh, m), ol = __shfl_xor_sync(0xffffffffu, sl, m);
+    df_add(sh, sl, oh, ol);
+  }
+  if (lane == 0) p.cpart[(int64_t)blockIdx.y * p.ncol + c] = (double)sh + (double)sl;
 }
 
 // units as k_cgs_update: w = w - V c - i P d (c, d the pass's real coefficients), and ws
-__global__ void __launch_bounds__(256, 3)
-k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
-  __shared__ float2 cf[2 * MAXM + 2];
-  __shared__ float4 red[8][32];
-  const Prob& p = probs[blockIdx.y];
-  const KState* st = p.st;
-  if (!kphase(st, newvec)) return;
-  const int64_t row = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
-  if ((int64_t)blockIdx.x * 32 >= p.Npad) return;     // whole block (Npad is a multiple of 128)
-  const int nj = st->j + 1;
-  const int nset = 2 * nj;
-  const double2* cp = (const double2*)p.cpart;
+template <int RS>
+__device__ __forceinline__ void cgs_update_dfs_slab(const Prob& p, int nj, int pass, float2* cf, float4 (*red)[32]) {
+  constexpr int G = 256 / RS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bx = blockIdx.x;
+  const int nset = 2 * nj, nch = dot_chunks(p.nT);
   double2* coef = (double2*)p.coef + (int64_t)(pass & 1) * p.ncol;
-  for (int c = threadIdx.x; c < nset; c += blockDim.x) {
-    double sc = 0.0;
-    int rb = 0;
-    for (; rb + 8 <= p.nrb; rb += 8) {      // eight loads in flight, then the sums in order
-      double v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = cp[(int64_t)(rb + u) * p.ncol + c].x;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) sc += v[u];
-    }
-    for (; rb < p.nrb; ++rb) sc += cp[(int64_t)rb * p.ncol + c].x;
+  for (int c = tid; c < nset; c += 256) {
+    const double sc = cgs_coef<false>(p, 1, c, nch).x;
     const float h = (float)sc;
     cf[c] = make_float2(h, (float)(sc - (double)h));
-    if (blockIdx.x == 0) coef[c] = mk(sc, 0.0);
+    if (bx == 0) coef[c] = mk(sc, 0.0);
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
   // entry cc: V[:, cc] (cc < nj) or the twin i P[:, cc - nj] = (-P_im, P_re)
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-  for (int c = warp; c < nset; c += 8) {
-    const bool tw = c >= nj;
-    const float4 v = __ldg((tw ? p.Ps : p.Vs) + (int64_t)(tw ? c - nj : c) * p.Npad + row);
-    const float2 f = cf[c];
-    if (tw) {
-      df_madd(rh, rl, -v.y, -v.w, f.x, f.y);
-      df_madd(ih, il, v.x, v.z, f.x, f.y);
-    } else {
-      df_madd(rh, rl, v.x, v.z, f.x, f.y);
-      df_madd(ih, il, v.y, v.w, f.x, f.y);
+  for (int c0 = tid / RS; c0 < nset; c0 += 4 * G) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = c0 + G * u;
+      if (c < nset) v[u] = __ldg((c >= nj ? p.Ps : p.Vs) + (int64_t)(c >= nj ? c - nj : c) * p.Npad + row);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = c0 + G * u;
+      if (c >= nset) continue;
+      const float2 f = cf[c];
+      const float4 t = c >= nj ? make_float4(-v[u].y, v[u].x, -v[u].w, v[u].z) : v[u];
+      df_madd(rh, rl, t.x, t.z, f.x, f.y);
+      df_madd(ih, il, t.y, t.w, f.x, f.y);
     }
   }
-  red[warp][lane] = make_float4(rh, rl, ih, il);
+#pragma unroll
+  for (int m = RS; m < 32; m <<= 1) {         // the warp's column groups
+    const float orh = __shfl_xor_sync(0xffffffffu, rh, m), orl = __shfl_xor_sync(0xffffffffu, rl, m);
+    const float oih = __shfl_xor_sync(0xffffffffu, ih, m), oil = __shfl_xor_sync(0xffffffffu, il, m);
+    df_add(rh, rl, orh, orl);
+    df_add(ih, il, oih, oil);
+  }
+  if (lane < RS) red[warp][lane] = make_float4(rh, rl, ih, il);
   __syncthreads();
-  if (warp == 0) {
-    float4 t = red[0][lane];
+  if (tid < RS) {
+    float4 t = red[0][tid];
 #pragma unroll
     for (int q = 1; q < 8; ++q) {
-      const float4 o = red[q][lane];
+      const float4 o = red[q][tid];
       df_add(t.x, t.y, o.x, o.y);
       df_add(t.z, t.w, o.z, o.w);
     }
@@ -227,35 +200,44 @@ k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
   }
 }
 
-template <typename ST>
-__global__ void __launch_bounds__(256)
-k_norm_partial(const Prob* __restrict__ probs, int ph, int start) {
-  __shared__ double red[8];
-  norm_partial_body<ST>(probs, ph, start, blockIdx.x, blockIdx.y, red);
+__global__ void __launch_bounds__(256, 3)
+k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
+  __shared__ float2 cf[2 * MAXM + 2];
+  __shared__ float4 red[8][32];
+  const Prob& p = probs[blockIdx.y];
+  const KState* st = p.st;
+  if (!kphase(st, newvec) || (int64_t)blockIdx.x * p.slab >= p.Npad) return;
+  const int nj = st->j + 1;
+  switch (p.slab) {
+    case 8: return cgs_update_dfs_slab<8>(p, nj, pass, cf, red);
+    case 16: return cgs_update_dfs_slab<16>(p, nj, pass, cf, red);
+    default: return cgs_update_dfs_slab<32>(p, nj, pass, cf, red);
+  }
 }
 
+// The new basis vector and the step's end in one launch: every warp sums the norm's partial sums
+// itself, scales its rows, and the last CTA of a problem to finish (a ticket) updates its state,
+// which all the others have read by then.
 template <typename ST>
 __global__ void __launch_bounds__(256)
 k_normalize(const Prob* __restrict__ probs, int ph, int start, int half) {
-  __shared__ double sb2;
-  normalize_body<ST>(probs, ph, start, half, blockIdx.x, blockIdx.y, &sb2);
-}
-
-// One thread per problem.
-__global__ void k_step_finish(const Prob* __restrict__ probs, int nprob, int ph, int fresh, int half) {
-  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ip >= nprob) return;
-  const Prob& p = probs[ip];
-  if (!kphase(p.st, fresh)) return;
-  finish_one(p, ph, fresh, half, sum_norm_parts(p));
-}
-
-template <typename ST>
-__global__ void __launch_bounds__(256)
-k_norm_fused(const Prob* __restrict__ probs, int ph, int start, int half) {
-  __shared__ double red[8];
-  __shared__ double sb2;
-  norm_fused_body<ST>(probs, ph, start, half, blockIdx.x, red, &sb2);
+  using R = typename RealOf<ST>::T;
+  __shared__ unsigned int last;
+  const Prob& p = probs[blockIdx.y];
+  const KState* st = p.st;
+  const unsigned int nblk = (unsigned int)((p.Npad + 255) / 256);
+  if (blockIdx.x >= nblk || !kphase(st, start)) return;
+  const int64_t row = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const double b2 = norm_sum<false>(p, ph);
+  // a beta^2 that is no positive number is recorded by the step's end
+  if (row < p.Npad && b2 > 0.0 && isfinite(b2)) normalize_row<ST, false>(p, st, ph, half, row, (R)rsqrt(b2));
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(p.tick, 1u);
+  __syncthreads();
+  if (last != nblk - 1 || threadIdx.x != 0) return;
+  *p.tick = 0u;
+  finish_one<false>(p, ph, start, half, b2, true);
 }
 
 // ---------------------------------------------------------------- start vector
@@ -503,34 +485,30 @@ __global__ void k_restart_commit(const Prob* __restrict__ probs, int nprob, int 
 
 // ---------------------------------------------------------------- launchers
 template <typename ST>
-void launch_step_cgs(const Prob* dprobs, int nprob, int ph, int maxnrb, int64_t maxNpad, int ncol,
-                     int pass, int half, bool dfs, cudaStream_t s) {
+void launch_step_cgs(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int slab, int ncol, int pass, int half,
+                     bool dfs, cudaStream_t s) {
   // pass: 0/1 regular step passes; 2/3 the same for a fresh (replacement) vector
   count_launch(2);
   const int newvec = pass >= 2 ? 1 : 0;
   const int ps = pass & 1;
+  // a batch's smaller problems may have more chunks than its largest
+  const unsigned nch = nprob > 1 ? DOT_CHUNKS : (unsigned)dot_chunks((int)(maxNpad / TS));
+  const dim3 gd((ncol + 7) / 8, nch, nprob), gu((unsigned)(maxNpad / slab), nprob);
   if (dfs && ph && half == 0) {        // the double-FP32 shadows of the mixed path
-    k_cgs_dot_dfs<<<dim3((ncol + 1) / 2, maxnrb, nprob), 256, 0, s>>>(dprobs, newvec);
-    k_cgs_update_dfs<<<dim3((unsigned)((maxNpad + 31) / 32), nprob), 256, 0, s>>>(dprobs, ps, newvec);
+    k_cgs_dot_dfs<<<gd, 256, 0, s>>>(dprobs, newvec);
+    k_cgs_update_dfs<<<gu, 256, 0, s>>>(dprobs, ps, newvec);
     return;
   }
-  k_cgs_dot<ST><<<dim3((ncol + 1) / 2, maxnrb, nprob), 256, 0, s>>>(dprobs, ph, newvec, half, ps);
-  k_cgs_update<ST><<<dim3((unsigned)((maxNpad + 31) / 32), nprob), 256, 0, s>>>(dprobs, ph, ps, newvec, half);
+  k_cgs_dot<ST><<<gd, 256, 0, s>>>(dprobs, ph, newvec, half, ps);
+  k_cgs_update<ST><<<gu, 256, 0, s>>>(dprobs, ph, ps, newvec, half);
 }
 
 template <typename ST>
-void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int maxnrb, int64_t maxNpad,
-                           int start, int half, cudaStream_t s) {
-  if (maxnrb == 1) {
-    count_launch();
-    k_norm_fused<ST><<<nprob, 256, 0, s>>>(dprobs, ph, start, half);
-    return;
-  }
-  count_launch(3);
+void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int start, int half,
+                           cudaStream_t s) {
+  count_launch();
   // start: 0 regular step, 1 fresh (first or replacement) vector
-  k_norm_partial<ST><<<dim3(maxnrb, nprob), 256, 0, s>>>(dprobs, ph, start);
   k_normalize<ST><<<dim3((unsigned)((maxNpad + 255) / 256), nprob), 256, 0, s>>>(dprobs, ph, start, half);
-  k_step_finish<<<(nprob + 127) / 128, 128, 0, s>>>(dprobs, nprob, ph, start, half);
 }
 
 template <typename ST>
@@ -560,8 +538,8 @@ void launch_restart(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int 
 }
 
 #define INST(ST)                                                                                        \
-  template void launch_step_cgs<ST>(const Prob*, int, int, int, int64_t, int, int, int, bool, cudaStream_t); \
-  template void launch_step_normalize<ST>(const Prob*, int, int, int, int64_t, int, int, cudaStream_t); \
+  template void launch_step_cgs<ST>(const Prob*, int, int, int64_t, int, int, int, int, bool, cudaStream_t); \
+  template void launch_step_normalize<ST>(const Prob*, int, int, int64_t, int, int, cudaStream_t); \
   template void launch_start_vector<ST>(const Prob*, int, int64_t, uint64_t, const void*,              \
                                         cudaStream_t);                                                  \
   template void launch_restart<ST>(const Prob*, int, int, int64_t, int, bool, bool, cudaStream_t);

@@ -11,11 +11,12 @@
 // KState: the step loop stops when the subspace is full, a breakdown asks the host for a fresh
 // vector, or the problem is done; the restart itself stays with the per-phase kernels.
 //
-// The grid barrier counts arrivals with an atomic and releases a generation number; every
-// wait is bounded (about a second of polling), after which the CTA raises the barrier's error
-// flag and the whole launch returns, so a wait can never hang the device.  The launch is
+// The grid barrier counts arrivals; every wait is bounded (about a second of polling), after
+// which the CTA raises the barrier's error flag and returns, and the others' waits expire in turn,
+// so a wait can never hang the device.  The launch is
 // cooperative, so all CTAs are resident together.
 #include <algorithm>
+#include <cstddef>
 
 #include "fx_phases.cuh"
 
@@ -23,6 +24,9 @@ namespace bse {
 namespace {
 
 constexpr int PS_THREADS = 256;
+// One CTA per SM: two of 128 registers a thread spill in the product's row loop (measured, PH
+// N = 3000: 473 ms against 311; TDA N = 2000: 81 against 53).
+constexpr int PS_RING = 8192;              // two (TDA: four) tile rows per warp in flight (16 KiB: no faster)
 constexpr long long PS_SPIN = 1ll << 22;   // polls of one barrier wait
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
@@ -31,113 +35,125 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
   return v;
 }
 
-// All CTAs of the launch meet here; false (in every thread of the CTA) when some wait expired.
+// All CTAs of the launch meet here; false (in every thread of the CTA) when the wait expired.  The
+// arrivals of all barriers of a launch add up in one counter, so nothing is reset and a waiter
+// polls the counter itself: one release and the polls, 1.3 us where an arrival count that the last
+// CTA turns into a generation number, with a fence in every thread, took 2.2.
 __device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned int nblk, unsigned int& gen, int* s_ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    const unsigned int g = gen;
-    __threadfence();                                   // this CTA's writes before the arrival
-    if (atomicAdd(&gb->count, 1u) == nblk - 1) {
-      atomicExch(&gb->count, 0u);                      // nobody arrives again before the release
-      __threadfence();
-      atomicAdd(&gb->gen, 1u);                         // release generation g
-    } else {
-      long long i = 0;
-      while (ld_acquire_u32(&gb->gen) == g) {
-        if (++i > PS_SPIN) {
-          atomicExch(&gb->err, 1);
-          ok = 0;
-          break;
-        }
+    const unsigned int target = (gen + 1) * nblk;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->count) : "memory");
+    long long i = 0;
+    while ((int)(ld_acquire_u32(&gb->count) - target) < 0) {
+      if (++i > PS_SPIN) {
+        atomicExch(&gb->err, 1);
+        ok = 0;
+        break;
       }
     }
-    __threadfence();
-    gen = g + 1;
-    if (ok && *(volatile int*)&gb->err) ok = 0;
     *s_ok = ok;
   }
+  ++gen;
   __syncthreads();
-  __threadfence();                                     // every thread orders its later loads
   return *s_ok != 0;
+}
+
+// The FP64 tiles (a few, if any, beside fixed-point ones) stay out of line: their registers would be
+// spilled around the other phases.
+template <typename ST, typename R, bool HASB>
+__device__ __noinline__ void ps_tiles(const Prob* probs, const TileJob* jobs, int njobs, int mode, int bid, int nblk,
+                                      unsigned char* sm) {
+  using CT = typename Acc<R>::T;
+  CT* xc = reinterpret_cast<CT*>(sm);
+  CT(*red)[TS] = reinterpret_cast<CT(*)[TS]>(xc + 2 * TS);
+  prod_tiles_body<ST, R, HASB, true>(probs, jobs, njobs, mode, GenericIO{}, 1, bid, nblk, xc, xc + TS, red);
 }
 
 template <typename ST, typename R, bool HASB>
 __global__ void __launch_bounds__(PS_THREADS, 1)
 k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int nfx, int steps,
                 GridBar* gb) {
-  using CT = typename Acc<R>::T;
-  extern __shared__ __align__(16) unsigned char psm[];
+  constexpr bool FX = std::is_same<ST, double2>::value;
+  extern __shared__ __align__(128) unsigned char psm[];
   __shared__ int s_ok;
-  const int bid = blockIdx.x;
+  // every CTA keeps its own copy of the problem's description and state and advances the state
+  // itself (the same numbers everywhere): no read of it has to cross the GPU
+  __shared__ KState s_st;
+  __shared__ Prob s_p;
+  const int bid = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned int nblk = gridDim.x;
   unsigned int gen = 0;
-  const Prob& p = probs[0];
-  const KState* st = p.st;
+  KState* const gst = probs[0].st;
+  if (tid == 0) {
+    s_p = probs[0];
+    s_st = *gst;
+    s_p.st = &s_st;
+  }
   const int ph = HASB ? 1 : 0;
+  // the fixed-point product's row rings and barriers keep their place (complex128); the rest of
+  // the shared memory is carved per phase
+  FxPipe pipe;
+  unsigned char* rest = psm;
+  if constexpr (FX) {
+    fx_init(*reinterpret_cast<FxShared<PS_RING>*>(psm));
+    rest += offsetof(FxShared<PS_RING>, x);
+  }
+  __syncthreads();
+  const Prob& p = s_p;
+  const KState* st = &s_st;
+  const int nslab = (int)(p.Npad / p.slab), nch = dot_chunks(p.nT);
   const GenericIO io{};
-  // one shared-memory region, carved per phase
-  CT* xc = reinterpret_cast<CT*>(psm);
-  CT* xr = xc + TS;
-  CT(*pred)[TS] = reinterpret_cast<CT(*)[TS]>(xr + TS);
-  CT(*grp)[REDUCE_ROWS] = reinterpret_cast<CT(*)[REDUCE_ROWS]>(psm);
-  double2(*dred)[4] = reinterpret_cast<double2(*)[4]>(psm);
-  ST* cf = reinterpret_cast<ST*>(psm);
+  using CT = typename Acc<R>::T;
+  ST* cf = reinterpret_cast<ST*>(rest);
   ST(*ured)[32] = reinterpret_cast<ST(*)[32]>(cf + 2 * MAXM + 2);
-  double* nred = reinterpret_cast<double*>(psm);
-  double* sb2 = nred + 8;
-  const int nT = p.nT, nrb = p.nrb;
-  const int nslab = (int)(p.Npad / 32);
-  const int nrow = (int)((p.Npad + PS_THREADS - 1) / PS_THREADS);
-  const int ncp = (p.ncol + 1) / 2;
-  const int m1 = HASB ? PM_STEP_MMINUS : PM_STEP_A;
-  // the tiles of a product: the fixed-point ones (complex128), then the others
-  auto tiles = [&](int mode) {
-    if constexpr (std::is_same<ST, double2>::value)
-      if (nfx > 0)
-        fx_tiles_body<HASB, true>(probs, jobs, nfx, p.nq, mode, io, 1, bid, nblk, *reinterpret_cast<FxShared*>(psm));
-    if (njobs > nfx)
-      prod_tiles_body<ST, R, HASB, true>(probs, jobs + nfx, njobs - nfx, mode, io, 1, bid, nblk, xc, xr, pred);
-  };
+  CT(*grp)[REDUCE_ROWS] = reinterpret_cast<CT(*)[REDUCE_ROWS]>(rest);
   for (int s = 0; s < steps; ++s) {
     if (!kactive(st)) break;                          // the same state in every CTA
-    tiles(m1);
+#pragma unroll 1
+    for (int prod = 0; prod < (HASB ? 2 : 1); ++prod) {
+      const int mode = !HASB ? PM_STEP_A : (prod ? PM_STEP_MPLUS : PM_STEP_MMINUS);
+      // the tiles: the fixed-point ones (complex128), then the others
+      if constexpr (FX)
+        if (nfx > 0)
+          fx_tiles_body<HASB, true>(&s_p, jobs, nfx, p.nq, mode, io, 1, bid, nblk, *reinterpret_cast<FxShared<PS_RING>*>(psm),
+                                    pipe, p.err);
+      if (njobs > nfx) ps_tiles<ST, R, HASB>(&s_p, jobs + nfx, njobs - nfx, mode, bid, nblk, rest);
+      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
+      for (int u = bid; u < REDUCE_UNITS * p.nT; u += nblk) prod_reduce_body<ST, R, true>(&s_p, mode, io, u, 0, grp);
+      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
+      if (prod) break;
+      const CgsSet cs = cgs_set(p, st, ph, 0);
+      const int nset = cs.nm + cs.nt;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        // tasks go round the CTAs first: neighbours share an SM's schedulers as little as possible
+        for (int t = bid + nblk * warp; t < nset * nch; t += nblk * (PS_THREADS / 32))
+          cgs_dot_task<ST, true>(p, st, cs, ph, 0, 0, pass, t % nset, t / nset);
+        if (!grid_sync(gb, nblk, gen, &s_ok)) return;
+        for (int u = bid; u < nslab; u += nblk) {
+          cgs_update_unit<ST, true>(p, st, ph, pass, 0, 0, u, cf, ured);
+          __syncthreads();
+        }
+        if (!grid_sync(gb, nblk, gen, &s_ok)) return;
+      }
+    }
+    // the new basis vector and the end of the step: warps with rows of their own and warp 0
+    const int64_t r0 = ((int64_t)bid + (int64_t)nblk * warp) * 32;
+    double b2 = 0.0;
+    if (warp == 0 || r0 < p.Npad) b2 = norm_sum<true>(p, ph);
+    if (r0 < p.Npad && b2 > 0.0 && isfinite(b2)) {
+      const R inv = (R)rsqrt(b2);
+      for (int64_t r = r0; r < p.Npad; r += (int64_t)nblk * PS_THREADS)
+        normalize_row<ST, true>(p, st, ph, 0, r + lane, inv);
+    }
+    __syncthreads();                                  // every warp has read the state
+    if (tid == 0) finish_one<true>(s_p, ph, 0, 0, b2, bid == 0);
     if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    for (int u = bid; u < REDUCE_UNITS * nT; u += nblk) prod_reduce_body<ST, R, true>(probs, m1, io, u, 0, grp);
-    if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int u = bid; u < ncp * nrb; u += nblk) {
-        cgs_dot_body<ST, true>(probs, ph, 0, 0, pass, u % ncp, u / ncp, 0, dred);
-        __syncthreads();
-      }
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-      for (int u = bid; u < nslab; u += nblk) {
-        cgs_update_body<ST, true>(probs, ph, pass, 0, 0, u, 0, cf, ured);
-        __syncthreads();
-      }
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    }
-    if (HASB) {
-      tiles(PM_STEP_MPLUS);
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-      for (int u = bid; u < REDUCE_UNITS * nT; u += nblk) prod_reduce_body<ST, R, true>(probs, PM_STEP_MPLUS, io, u, 0, grp);
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    }
-    if (nrb == 1) {
-      if (bid == 0) norm_fused_body<ST, true>(probs, ph, 0, 0, 0, nred, sb2);
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    } else {
-      for (int rb = bid; rb < nrb; rb += nblk) {
-        norm_partial_body<ST, true>(probs, ph, 0, rb, 0, nred);
-        __syncthreads();
-      }
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-      for (int u = bid; u < nrow; u += nblk) normalize_body<ST, true>(probs, ph, 0, 0, u, 0, sb2);
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-      if (bid == 0 && threadIdx.x == 0 && kphase(st, 0)) finish_one(p, ph, 0, 0, sum_norm_parts<true>(p));
-      if (!grid_sync(gb, nblk, gen, &s_ok)) return;
-    }
   }
+  __syncthreads();
+  if (bid == 0 && tid == 0) *gst = s_st;
 }
 
 template <typename ST, typename R, bool HASB>
@@ -145,9 +161,10 @@ size_t persist_smem() {
   using CT = typename Acc<R>::T;
   const size_t prod = (size_t)10 * TS * sizeof(CT);
   const size_t red = (size_t)REDUCE_GROUPS * REDUCE_ROWS * sizeof(CT);
-  const size_t fx = std::is_same<ST, double2>::value ? sizeof(FxShared) : 0;
   const size_t upd = (size_t)(2 * MAXM + 2) * sizeof(ST) + (size_t)8 * 32 * sizeof(ST);
-  return std::max(std::max(std::max(prod, red), fx), std::max(upd, (size_t)(9 * sizeof(double) + 8 * sizeof(double2))));
+  const size_t rest = std::max(std::max(prod, red), upd);
+  if (!std::is_same<ST, double2>::value) return rest;
+  return std::max(sizeof(FxShared<PS_RING>), offsetof(FxShared<PS_RING>, x) + rest);
 }
 
 template <typename ST, typename R, bool HASB>

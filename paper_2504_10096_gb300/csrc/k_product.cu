@@ -84,6 +84,10 @@ k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
     for (int q = 1; q < REDUCE_GROUPS; ++q) acc = cadd(acc, grp[q][lane]);
     y[(int64_t)I * TS + r] = acc;
     if (p.ws && y == (double2*)p.w) p.ws[(int64_t)I * TS + r] = dsplit(acc);   // its double-FP32 shadow
+    if (prod_is_norm(mode)) {
+      const double t = warp_sum_d(norm_term(x[(int64_t)I * TS + r], acc));
+      if (lane == 0) p.npart[blockIdx.x] = t;
+    }
   }
 }
 

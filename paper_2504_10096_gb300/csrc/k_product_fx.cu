@@ -7,12 +7,18 @@
 namespace bse {
 namespace {
 
+constexpr int FX_RING = 8192;   // two (TDA: four) rows per warp, two CTAs per SM
+
 template <bool HASB>
-__global__ void __launch_bounds__(FX_THREADS, 1)
+__global__ void __launch_bounds__(FX_THREADS, 2)
 k_prod_tiles_fx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int nq, int mode,
                 GenericIO io, int strided) {
-  __shared__ FxShared sh;
-  fx_tiles_body<HASB, false>(probs, jobs, njobs, nq, mode, io, strided, blockIdx.x, gridDim.x, sh);
+  extern __shared__ __align__(128) unsigned char fxsm[];
+  FxShared<FX_RING>& sh = *reinterpret_cast<FxShared<FX_RING>*>(fxsm);
+  fx_init(sh);
+  __syncthreads();
+  FxPipe pipe;
+  fx_tiles_body<HASB, false>(probs, jobs, njobs, nq, mode, io, strided, blockIdx.x, gridDim.x, sh, pipe, probs[0].err);
 }
 
 // v / 2^(e - 1022) as a float (magnitude below 1, truncated; small values flush to zero)
@@ -93,16 +99,15 @@ int fx_bands(int ntiles) {
   return best;
 }
 
-int product_fx_occupancy(bool hasB) {
-  static int occ[2] = {0, 0};
-  const int ib = hasB ? 1 : 0;
-  if (!occ[ib]) {
-    int o = 0;
-    if (hasB) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_fx<true>, FX_THREADS, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_fx<false>, FX_THREADS, 0);
-    occ[ib] = o > 0 ? o : 1;
-  }
-  return occ[ib];
+// two CTAs per SM (96 KiB of shared memory and 128 registers a thread each)
+int product_fx_occupancy() {
+  static const bool set = [] {
+    cudaFuncSetAttribute(k_prod_tiles_fx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared<FX_RING>));
+    cudaFuncSetAttribute(k_prod_tiles_fx<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared<FX_RING>));
+    return true;
+  }();
+  (void)set;
+  return 2;
 }
 
 void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int nfx, int nq, int nprob, int maxnT,
@@ -111,9 +116,9 @@ void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int n
   if (io_host) io = *io_host;
   if (nfx > 0) {
     count_launch();
-    const int grid = product_grid(product_fx_occupancy(hasB), shape, nfx * nq);
-    if (hasB) k_prod_tiles_fx<true><<<grid, FX_THREADS, 0, s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
-    else k_prod_tiles_fx<false><<<grid, FX_THREADS, 0, s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
+    const int grid = product_grid(product_fx_occupancy(), shape, nfx * nq);
+    if (hasB) k_prod_tiles_fx<true><<<grid, FX_THREADS, sizeof(FxShared<FX_RING>), s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
+    else k_prod_tiles_fx<false><<<grid, FX_THREADS, sizeof(FxShared<FX_RING>), s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
   }
   if (njobs > nfx) launch_tiles_f64(dprobs, jobs + nfx, njobs - nfx, mode, io, hasB, shape, s);
   launch_prod_reduce_f64(dprobs, nprob, maxnT, mode, io, s);
