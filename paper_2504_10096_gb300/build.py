@@ -16,7 +16,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbse.so")
-SOURCES = ["k_product.cu", "k_product_df.cu", "k_product_fx.cu", "k_krylov.cu", "k_ritz.cu", "k_post.cu", "bse_api.cu",
+SOURCES = ["k_product.cu", "k_product_df.cu", "k_product_fx.cu", "k_block_fx.cu",
+           "k_krylov.cu", "k_ritz.cu", "k_post.cu", "bse_api.cu",
            "k_noalloc.cu", "k_adjoint_tc.cu", "k_haydock.cu", "k_peak.cu", "k_dense.cu", "k_persist.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

@@ -49,6 +49,7 @@ struct ProbHost {
   double *jw = nullptr, *S2 = nullptr;
   // mixed PH path: double-FP32 shadows of V, P and w for the Gram-Schmidt passes
   float4 *Vs = nullptr, *Ps = nullptr, *ws = nullptr;
+  bool block_fx = false;     // every tile has a fixed-point scale: block products take that kernel
   // results
   double2* Z = nullptr;
   int zcols = 0;
@@ -123,6 +124,8 @@ struct bse_handle {
   // post-processing scratch (single problem at a time)
   void* post = nullptr;
   size_t post_bytes = 0;
+  void* blk = nullptr;       // workspace of the fixed-point block product
+  size_t blk_bytes = 0;
   // adjoint tile list
   int2* adj_tiles = nullptr;
   int64_t adj_ntiles = 0;
@@ -237,6 +240,37 @@ int pack_matrix(bse_handle* h, const T* src, int64_t N, int nT, int herm, int wh
   cudaError_t e = cudaStreamSynchronize(h->stream);
   cudaFree(stage);
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return BSE_ECUDA;
+  return BSE_OK;
+}
+
+// Y = A XA + sB B XB (FP64 blocks of K columns, Npad rows) with the stored tiles of problem i
+int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB) {
+  ProbHost& q = h->p[i];
+  // (complex128 PH tiles hold P and Q, so they always go through the two-matrix form)
+  if (hasB == (h->ph != 0) && q.block_fx) {
+    const size_t need = block_fx_bytes(q.nT, K, hasB);
+    if (need > h->blk_bytes) {
+      dfree(h->blk);
+      h->blk_bytes = dalloc(&h->blk, need) == BSE_OK ? need : 0;
+    }
+    if (h->blk) {
+      BlockFx b{};
+      b.M0 = h->tiles64 ? (const void*)q.A : q.Afx;
+      b.M1 = hasB ? (h->tiles64 ? (const void*)q.B : q.Bfx) : nullptr;
+      b.texp = q.texp;
+      b.A = q.A;
+      b.B = q.B;
+      b.nT = q.nT;
+      launch_block_fx(b, hasB, h->tiles64, xa, xb, q.Npad, sB, y, q.Npad, K, h->blk, h->stream);
+      CK(cudaGetLastError());
+      return BSE_OK;
+    }
+  }
+  if (h->tiles64)
+    launch_rowblock<float2, double>(h->dprobs, i, q.nT, xa, xb, (int)q.Npad, sB, y, (int)q.Npad, K, hasB, h->stream);
+  else
+    launch_rowblock<double2, double>(h->dprobs, i, q.nT, xa, xb, (int)q.Npad, sB, y, (int)q.Npad, K, hasB, h->stream);
+  CK(cudaGetLastError());
   return BSE_OK;
 }
 
@@ -656,12 +690,7 @@ struct Driver {
     const void* xb = h->ph ? (const void*)XB : nullptr;
     const double sgn = h->ph ? 1.0 : 0.0;
     if (h->ph) launch_prepare_hz2(q.Z, ldz, Npad, k, XA, XB, h->stream);
-    if (h->tiles64)
-      launch_rowblock<float2, double>(h->dprobs, i, q.nT, xa, xb, (int)Npad, sgn, U, (int)Npad, kc, h->ph != 0,
-                                      h->stream);
-    else
-      launch_rowblock<double2, double>(h->dprobs, i, q.nT, xa, xb, (int)Npad, sgn, U, (int)Npad, kc, h->ph != 0,
-                                       h->stream);
+    if ((rc = block_product(h, i, (const double2*)xa, (const double2*)xb, sgn, U, kc, h->ph != 0))) return rc;
     launch_residuals2(q.Z, ldz, U, Npad, k, h->ph, part4, nrb, rho, z2, res, h->stream);
     CK(cudaGetLastError());
     std::vector<double> hr(k), hres(k);
@@ -883,10 +912,27 @@ int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
     for (ProbHost& q : h->p) { dfreet(q.Afx); dfreet(q.Bfx); dfreet(q.texp); }
     return rc == BSE_ENOMEM ? BSE_OK : rc;
   }
+  for (int i = 0; i < h->count; ++i) h->p[i].block_fx = *std::min_element(ex[i].begin(), ex[i].end()) >= 0;
   const auto mid = std::stable_partition(jobs.begin(), jobs.end(),
                                          [&](const TileJob& j) { return ex[j.prob][j.t] >= 0; });
   h->nfx = (int)(mid - jobs.begin());
   h->nq = fx_bands(h->nfx);
+  return BSE_OK;
+}
+
+// The scales of complex64 tiles, for the fixed-point block products (residuals in FP64 accuracy).
+int setup_scales64(bse_handle* h) {
+  std::vector<std::vector<int>> ex(h->count);
+  for (int i = 0; i < h->count; ++i) {
+    ProbHost& q = h->p[i];
+    const int rc = dalloc((void**)&q.texp, sizeof(int) * (size_t)q.ntiles);
+    if (rc) return rc;
+    launch_block_scale64((const float2*)q.A, (const float2*)q.B, q.N, q.nT, q.texp, h->stream);
+    ex[i].resize(q.ntiles);
+    CK(cudaMemcpyAsync(ex[i].data(), q.texp, sizeof(int) * (size_t)q.ntiles, cudaMemcpyDeviceToHost, h->stream));
+  }
+  CK(cudaStreamSynchronize(h->stream));
+  for (int i = 0; i < h->count; ++i) h->p[i].block_fx = *std::min_element(ex[i].begin(), ex[i].end()) >= 0;
   return BSE_OK;
 }
 
@@ -1182,8 +1228,12 @@ int apply_impl(bse_handle* h, int op, int k, const void* X, void* Y) {
     xb = nullptr;  // conj(XA)
   }
   // P, Q tiles always go through the unpacking variant (sB = 0 drops the B half)
-  launch_rowblock<ST, R>(h->dprobs, 0, q.nT, XA, xb, (int)Npad, sB, U, (int)Npad, kc,
-                         hasB && (op != BSE_OP_A || !h->tiles64), h->stream);
+  const bool two = hasB && (op != BSE_OP_A || !h->tiles64);
+  if constexpr (std::is_same<ST, double2>::value) {
+    if ((rc = block_product(h, 0, XA, (const double2*)xb, sB, U, kc, two))) return rc;
+  } else {
+    launch_rowblock<ST, R>(h->dprobs, 0, q.nT, XA, xb, (int)Npad, sB, U, (int)Npad, kc, two, h->stream);
+  }
   count_launch();
   k_hz_out<ST, CT><<<dim3((unsigned)((N + 255) / 256), k), 256, 0, h->stream>>>(U, N, Npad, k, op, (ST*)Y);
   CK(cudaGetLastError());
@@ -1527,6 +1577,7 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
   for (const ProbHost& q : h->p) rows += q.Npad;
   while (h->slab > 8 && rows / (h->slab / 2) <= num_sms()) h->slab /= 2;
   if (rc == BSE_OK && dtype == BSE_C128) rc = setup_fx(h, jobs);
+  if (rc == BSE_OK && h->tiles64) rc = setup_scales64(h);
   if (rc == BSE_OK && h->mixed) h->hjobs = jobs;
   if (rc == BSE_OK && (h->mixed || h->nfx > 0)) {
     rc = dalloc((void**)&h->prod_err, sizeof(int));
@@ -1746,6 +1797,7 @@ int bse_destroy(bse_handle* h) {
   dfreet(h->dstate);
   dfreet(h->djobs);
   dfree(h->post);
+  dfree(h->blk);
   dfreet(h->pj_work);
   dfreet(h->pj_flag);
   dfreet(h->gbar);

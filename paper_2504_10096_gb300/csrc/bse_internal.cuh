@@ -270,6 +270,23 @@ void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mo
                       ProdShape shape, cudaStream_t s);
 int num_sms();
 
+// blocks of columns in FP64 accuracy with fixed-point tiles (k_block_fx.cu): Y = A XA + sB B XB
+// (XB null: conj(XA)), Npad rows; `work` holds block_fx_bytes
+struct BlockFx {
+  const void* M0;     // limbs of A (P on PH handles), or complex64 A
+  const void* M1;     // ... of B (Q), or complex64 B; null without B
+  const int* texp;    // scale exponents of the tiles, all >= 0
+  const void* A;      // the packed tiles themselves (the diagonal's part is FP64)
+  const void* B;
+  int nT;
+};
+int block_fx_splits(int nT, int K);
+size_t block_fx_bytes(int nT, int K, bool hasB);
+void launch_block_fx(const BlockFx& q, bool hasB, bool tiles64, const double2* xa, const double2* xb, int64_t ldx,
+                     double sB, double2* y, int64_t ldy, int K, void* work, cudaStream_t s);
+// scale exponents of complex64 tiles, -1 for tiles a fixed-point product must not take
+void launch_block_scale64(const float2* A, const float2* B, int64_t N, int nT, int* texp, cudaStream_t s);
+
 // bounded-wait self-test (k_adjoint_tc.cu): 0 on success, -1 on a CUDA error
 int selftest_bounded_wait(int arrive, int* expired_host);
 

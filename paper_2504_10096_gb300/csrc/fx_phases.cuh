@@ -125,12 +125,9 @@ __device__ __forceinline__ void fx_words(long long hh, long long hl, int& w0, in
   w2 = (int)((((unsigned int)v & 0xfffu) << 14) | (lo >> 16));
 }
 
-// (w0 2^52 + w1 2^26 + w2) 2^(eu + ex - 2044 - 72) as a double (sums of words: w1, w2 unsigned);
-// eu, ex: biased exponents of the scales, 2047 (an infinity or a NaN in the chunk) gives a NaN
-__device__ __forceinline__ double fx_double(int w0, unsigned int w1, unsigned int w2, int eu, int ex) {
-  const unsigned long long l0 = ((unsigned long long)w1 << 26) + w2;
-  long long h = (long long)w0 + (long long)(l0 >> 52);
-  unsigned long long l = l0 & 0xfffffffffffffull;
+// (h 2^52 + l) 2^(eu + ex - 2044 - 72) as a double, |h| < 2^33 and 0 <= l < 2^52; eu, ex: biased
+// exponents of the scales, ex = 2047 (an infinity or a NaN in the chunk) gives a NaN
+__device__ __forceinline__ double fx_pack_double(long long h, unsigned long long l, int eu, int ex) {
   const bool neg = h < 0;
   if (neg) {
     h = -h - (l ? 1 : 0);
@@ -155,6 +152,11 @@ __device__ __forceinline__ double fx_double(int w0, unsigned int w1, unsigned in
   if (e > 2046) b = 0x7ff0000000000000ull;
   if (ex == 2047) b = 0x7ff8000000000000ull;
   return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+}
+// ... of words or sums of words: w0 2^52 + w1 2^26 + w2 (w1, w2 unsigned)
+__device__ __forceinline__ double fx_double(int w0, unsigned int w1, unsigned int w2, int eu, int ex) {
+  const unsigned long long l = ((unsigned long long)w1 << 26) + w2;
+  return fx_pack_double((long long)w0 + (long long)(l >> 52), l & 0xfffffffffffffull, eu, ex);
 }
 
 // A warp's place in its stream of rows; it outlives one walk over the units (the barriers' phases

@@ -96,3 +96,35 @@ def test_nan_and_inf_reach_the_result():
         Ab[5, 140] = bad
         y = _product(Ab, B, x, bse.BSE_OP_MPLUS)
         assert not np.isfinite(y[5]) and not np.isfinite(y[140])
+
+
+@pytest.mark.parametrize("form,n,k", [("ph", 1, 2), ("ph", 127, 3), ("ph", 129, 16), ("ph", 385, 17), ("ph", 700, 33),
+                                      ("tda", 2, 2), ("tda", 128, 15), ("tda", 513, 20)])
+def test_blocks_match_extended_precision(form, n, k):
+    """bse_apply on k columns (the fixed-point block kernel) at the edges of its 64 x 16 units; the
+    columns of very different size.  The PH form multiplies P = A + B and Q = A - B with
+    (XA +- XB) / 2, so its bound holds for the larger of the two vectors; one more rounding each for
+    P, Q and the half sums."""
+    from paper_2504_10096_gb300 import bse
+    A, B = problem(n, "c128", form=form, seed=n)
+    rng = np.random.default_rng(n)
+    rows = 2 * n if form == "ph" else n
+    X = (rng.standard_normal((rows, k)) + 1j * rng.standard_normal((rows, k))) * 10.0 ** rng.integers(-6, 7, k)
+    s = bse.Solver(torch.from_numpy(A).cuda(), None if B is None else torch.from_numpy(B).cuda())
+    L = np.clongdouble
+    a, b = A.astype(L), None if B is None else B.astype(L)
+    if form == "tda":
+        refs = {bse.BSE_OP_A: (X, a @ X.astype(L))}
+    else:
+        x1, x2 = X[:n].astype(L), X[n:].astype(L)
+        refs = {bse.BSE_OP_H: (X, np.vstack([a @ x1 + b @ x2, -(b.conj() @ x1 + a.conj() @ x2)])),
+                bse.BSE_OP_MPLUS: (X[:n], a @ x1 + b @ x1.conj()), bse.BSE_OP_A: (X[:n], a @ x1)}
+    for op, (V, ref) in refs.items():
+        y = s.apply(op, torch.from_numpy(np.ascontiguousarray(V)).cuda()).cpu().numpy()
+        for c in range(k):
+            big = np.abs(V[:n, c]) + (np.abs(V[n:, c]) if op == bse.BSE_OP_H else 0)
+            bnd = _bound(A, B, big.astype(complex)) * (1.0 if form == "tda" else 3.0)
+            err = np.abs(y[:, c] - ref[:, c]).astype(np.float64)
+            lim = np.concatenate([bnd, bnd]) if op == bse.BSE_OP_H else bnd
+            assert np.all(err <= lim), (op, c, float(np.max(err / lim)))
+    s.close()
