@@ -619,6 +619,9 @@ struct Driver {
       }
       if (steps > 0) {
         if ((rc = run_steps(steps))) return rc;
+        // the restart follows without a look at the state: it leaves every problem alone whose
+        // subspace is not full (breakdown, error, done)
+        if (!(h->ph && h->variant == VAR_PROJECTED)) run_restart();
         continue;
       }
       if (h->ph && h->variant == VAR_PROJECTED) {

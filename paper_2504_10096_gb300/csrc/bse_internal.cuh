@@ -93,6 +93,12 @@ struct KState {
   double theta_scale; // max |theta| over the kept vectors [k, l) (scale of the breakdown test)
 };
 
+// the subspace is full: the restart's kernels act on the problem (and on no other, so they can be
+// launched behind the steps without reading the state back)
+__device__ __forceinline__ bool restart_ready(const KState* st) {
+  return !st->done && st->status == ST_OK && !st->breakdown && st->j >= st->m;
+}
+
 // Structure-preserving Lanczos variants of the pseudo-Hermitian iteration
 // (Sec. 2.2.1 names three): VAR_SHAO, the folded recurrence on M- M+ in the
 // M+ inner product; VAR_GRUNING, the Lanczos recurrence of H itself in the

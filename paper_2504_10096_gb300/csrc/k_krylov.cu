@@ -419,67 +419,57 @@ k_restart_gemm_df(const Prob* __restrict__ probs, int which) {
 }
 
 // V[:, k0+i] = V2[:, i]; V[:, k0+nkeep] = V[:, m]; same for P; W[:, k0+i] = W2[:, i] and
-// Z from Z2 on the Gruning path (the odd basis has no extra column).
+// Z from Z2 on the Gruning path (the odd basis has no extra column); the double-FP32 shadows
+// follow.  grid (rows / 256, ncv + 1, nprob): a column per CTA row, none reads what another writes.
 template <typename ST>
 __global__ void k_restart_copy(const Prob* __restrict__ probs, int ph, int gk) {
-  const Prob& p = probs[blockIdx.y];
+  const Prob& p = probs[blockIdx.z];
   const KState* st = p.st;
   if (st->status != ST_OK || !st->r_go) return;   // decided in this restart only
-  const int k0 = st->r_k0, nkeep = st->r_nkeep, m = st->m;
+  const int k0 = st->r_k0, nkeep = st->r_nkeep, m = st->m, i = blockIdx.y;
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= p.Npad) return;
-  ST* V = (ST*)p.V;
-  const ST* V2 = (const ST*)p.V2;
-  const ST vm = V[(int64_t)m * p.Npad + row];
-  for (int i = 0; i < nkeep; ++i) V[(int64_t)(k0 + i) * p.Npad + row] = V2[(int64_t)i * p.Npad + row];
-  V[(int64_t)(k0 + nkeep) * p.Npad + row] = vm;
+  if (row >= p.Npad || i > nkeep) return;
+  const bool extra = i == nkeep;                  // the newest vector moves behind the kept ones
+  const int64_t dst = (int64_t)(k0 + i) * p.Npad + row, src2 = (int64_t)i * p.Npad + row;
+  const int64_t srcm = (int64_t)m * p.Npad + row;
+  const ST v = extra ? ((const ST*)p.V)[srcm] : ((const ST*)p.V2)[src2];
+  ((ST*)p.V)[dst] = v;
+  ST u = czero<ST>();
   if (ph) {
-    ST* P = (ST*)p.P;
-    const ST* P2 = (const ST*)p.P2;
-    const ST pm = P[(int64_t)m * p.Npad + row];
-    for (int i = 0; i < nkeep; ++i) P[(int64_t)(k0 + i) * p.Npad + row] = P2[(int64_t)i * p.Npad + row];
-    P[(int64_t)(k0 + nkeep) * p.Npad + row] = pm;
+    u = extra ? ((const ST*)p.P)[srcm] : ((const ST*)p.P2)[src2];
+    ((ST*)p.P)[dst] = u;
   }
   if constexpr (std::is_same<ST, double2>::value) {
-    if (p.Vs) {                         // the double-FP32 shadows follow
-      for (int i = 0; i < nkeep; ++i)
-        p.Vs[(int64_t)(k0 + i) * p.Npad + row] = dsplit(((const double2*)p.V2)[(int64_t)i * p.Npad + row]);
-      p.Vs[(int64_t)(k0 + nkeep) * p.Npad + row] = dsplit(vm);
-      if (ph) {
-        for (int i = 0; i < nkeep; ++i)
-          p.Ps[(int64_t)(k0 + i) * p.Npad + row] = dsplit(((const double2*)p.P2)[(int64_t)i * p.Npad + row]);
-        p.Ps[(int64_t)(k0 + nkeep) * p.Npad + row] = dsplit(((const double2*)p.P)[(int64_t)(k0 + nkeep) * p.Npad + row]);
-      }
+    if (p.Vs) {
+      p.Vs[dst] = dsplit(v);
+      if (ph) p.Ps[dst] = dsplit(u);
     }
   }
-  if (gk) {
-    ST* W = (ST*)p.W;
-    ST* Z = (ST*)p.Z;
-    const ST* W2 = (const ST*)p.W2;
-    const ST* Z2 = (const ST*)p.Z2;
-    for (int i = 0; i < nkeep; ++i) {
-      W[(int64_t)(k0 + i) * p.Npad + row] = W2[(int64_t)i * p.Npad + row];
-      Z[(int64_t)(k0 + i) * p.Npad + row] = Z2[(int64_t)i * p.Npad + row];
-    }
+  if (gk && !extra) {
+    ((ST*)p.W)[dst] = ((const ST*)p.W2)[src2];
+    ((ST*)p.Z)[dst] = ((const ST*)p.Z2)[src2];
   }
 }
 
-__global__ void k_restart_commit(const Prob* __restrict__ probs, int nprob, int ph) {
-  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ip >= nprob) return;
-  const Prob& p = probs[ip];
+// one warp per problem
+__global__ void __launch_bounds__(32) k_restart_commit(const Prob* __restrict__ probs) {
+  const Prob& p = probs[blockIdx.x];
   KState* st = p.st;
   if (st->status != ST_OK || !st->r_go) return;   // decided in this restart only
-  const int k0 = st->r_k0;
-  st->k = k0 + st->r_nl;
-  st->l = k0 + st->r_nkeep;
+  const int k0 = st->r_k0, k = k0 + st->r_nl, l = k0 + st->r_nkeep;
   double ts = 0.0;
-  for (int i = st->k; i < st->l; ++i) ts = fmax(ts, fabs(p.theta[i]));
+  for (int i = k + (int)threadIdx.x; i < l; i += 32) ts = fmax(ts, fabs(p.theta[i]));
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) ts = fmax(ts, __shfl_xor_sync(0xffffffffu, ts, m));
+  __syncwarp();
+  if (threadIdx.x != 0) return;
+  st->k = k;
+  st->l = l;
   st->theta_scale = ts;
-  st->j = st->l;
+  st->j = l;
   st->restarts += 1;
   st->r_go = 0;
-  if (st->k >= st->nev) st->done = 1;
+  if (k >= st->nev) st->done = 1;
   else if (st->steps >= st->maxit) { st->done = 1; st->status = ST_NOCONV; }
 }
 
@@ -533,8 +523,8 @@ void launch_restart(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int 
       k_restart_gemm<ST><<<dim3(gx, (ncv + 15) / 16, nprob), 256, 0, s>>>(dprobs, which);
   }
   const unsigned gr = (unsigned)((maxNpad + 255) / 256);
-  k_restart_copy<ST><<<dim3(gr, nprob), 256, 0, s>>>(dprobs, ph, gruning ? 1 : 0);
-  k_restart_commit<<<(nprob + 127) / 128, 128, 0, s>>>(dprobs, nprob, ph);
+  k_restart_copy<ST><<<dim3(gr, ncv + 1, nprob), 256, 0, s>>>(dprobs, ph, gruning ? 1 : 0);
+  k_restart_commit<<<nprob, 32, 0, s>>>(dprobs);
 }
 
 #define INST(ST)                                                                                        \
