@@ -616,8 +616,9 @@ __device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh
     const double tiny = 1e-26 * scale * scale + 1e-300;
     if (ph && b2 < -1e6 * tiny) { st->status = ST_NOTPD; return; }
     if (b2 <= tiny) {                 // invariant subspace: the chain restarts
-      if (writer) p.beta[j] = 0.0;    // with a fresh vector (host-driven)
-      st->breakdown = 1;
+      if (writer) p.beta[j] = 0.0;    // with a fresh vector (host-driven), unless the subspace is full
+      if (j + 1 < st->m) st->breakdown = 1;     // (then its Ritz pairs are exact and all lock; a fresh
+      else st->j = j + 1;                       // vector may not even exist: m = N)
       return;
     }
     if (writer) p.beta[j] = sqrt(b2);
@@ -660,8 +661,9 @@ __device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh
     st->passes += 2;
     st->steps += 1;
     if (b2 <= tiny) {                   // invariant subspace: the chain restarts
-      p.beta[j] = 0.0;                  // with a fresh vector (host-driven)
-      st->breakdown = 1;
+      p.beta[j] = 0.0;                  // with a fresh vector (host-driven), unless the subspace is full
+      if (j + 1 < st->m) st->breakdown = 1;
+      else st->j = j + 1;
       return;
     }
     p.beta[j] = sqrt(b2);

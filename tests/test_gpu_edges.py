@@ -108,3 +108,19 @@ def test_caller_ncv_equal_to_nev(form):
     assert nconv == nev
     np.testing.assert_allclose(vals, ref, rtol=1e-9, atol=0)
     s.close()
+
+
+@pytest.mark.parametrize("form", ["ph", "tda"])
+@pytest.mark.parametrize("n", [1, 2, 3])
+def test_whole_space_needs_no_next_vector(form, n):
+    """nev = N: the last step of the only cycle finds an invariant subspace, and what is left of a fresh
+    vector may be exactly zero, which used to end some of these solves with ENOTPD or ENOTFINITE."""
+    from paper_2504_10096_gb300 import bse
+    for seed in range(24):
+        A, B = problem(n, "c128", form=form, seed=seed, n_g=8)
+        s = _solver(A, B) if form == "ph" else bse.Solver(torch.from_numpy(A).cuda())
+        vals, _, nconv = s.solve(n, tol=1e-12)
+        ref = O.ph_lowest(A, B, n)[0] if form == "ph" else O.tda_lowest(A, n)[0]
+        assert nconv == n
+        np.testing.assert_allclose(vals, ref, rtol=1e-11, atol=0)
+        s.close()
