@@ -35,7 +35,8 @@ def _stale(obj, src):
         return True
     t = os.path.getmtime(obj)
     deps = [src, os.path.join(CSRC, "bse_internal.cuh"), os.path.join(CSRC, "bse_phases.cuh"),
-            os.path.join(CSRC, "fx_phases.cuh"),
+            os.path.join(CSRC, "fx_phases.cuh"), os.path.join(CSRC, "tree_solve.cuh"),
+            os.path.join(CSRC, "grid_sync.cuh"),
             os.path.join(HERE, "..", "include", "bse.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -501,6 +501,7 @@ struct Driver {
       const int nw = std::min(st.r_pkeep - st.k, n);
       const int rc = projected_ritz(h->dprobs, i, n, nw, h->pj_work, h->pj_flag, h->stream);
       if (rc < 0) return BSE_ECUDA;
+      if (rc == 2) return BSE_ETIMEOUT;
     }
     launch_lock_decide_form(h->dprobs, h->count, h->ph, h->stream);
     launch_restart<ST>(h->dprobs, h->count, h->ph, h->maxNpad, h->ncv, false, h->mixed, h->stream);
@@ -1684,6 +1685,7 @@ int bse_solve_dense(bse_handle* h, int nev, double tol, double* eval_out, void* 
     const int r = dense_shao(h->dprobs, q.N, q.Npad, h->tiles64, !h->tiles64, nev, (double*)work, h->adj_err, q.Z,
                              nullptr, h->stream);
     if (r < 0) return BSE_ECUDA;
+    if (r == 2) return BSE_ETIMEOUT;
     if (r > 0) status = BSE_ENOTPD;
     if ((rc = drv.finish(0, nev, tol, false))) return rc;
     if (evec_out && (rc = drv.store(0, evec_out))) return rc;
@@ -1693,6 +1695,7 @@ int bse_solve_dense(bse_handle* h, int nev, double tol, double* eval_out, void* 
     const int r = dense_shao(h->dprobs, q.N, q.Npad, h->tiles64, !h->tiles64, nev, (double*)work, h->adj_err, q.Z,
                              nullptr, h->stream);
     if (r < 0) return BSE_ECUDA;
+    if (r == 2) return BSE_ETIMEOUT;
     if (r > 0) status = BSE_ENOTPD;
     if ((rc = drv.finish(0, nev, tol, false))) return rc;
     if (evec_out && (rc = drv.store(0, evec_out))) return rc;

@@ -340,7 +340,7 @@ int launch_steps_persist(const Prob* dprobs, const TileJob* jobs, int njobs, int
 
 // dense structure-preserving diagonalisation (k_dense.cu): the nev lowest positive omega of
 // problem 0 of a PH handle and their right eigenvectors in Z (ld 2 Npad); returns 0, 1 (M_r not
-// positive definite) or -1 (CUDA error); `work` holds dense_scratch_doubles(N, nev) doubles
+// positive definite), 2 (a bounded wait expired) or -1 (CUDA error); `work` holds dense_scratch_doubles(N, nev) doubles
 size_t dense_scratch_doubles(int64_t N, int nev);
 int dense_shao(const Prob* dprobs, int64_t N, int64_t Npad, bool tiles64, bool pq, int nev, double* work,
                int* dflag, double2* Z, double* lam_out, cudaStream_t s);

@@ -9,8 +9,8 @@
 // this file and all FP64 on the CUDA cores (GB300's FP64 tensor rate is far
 // below its FP64 FMA rate, so no tensor-core path is used):
 //   1. assemble M_r (order n = 2N, column-major) from the handle's packed tiles;
-//   2. blocked right-looking Cholesky (64-column panels: diagonal block in one
-//      CTA, panel solve, trailing symmetric rank-64 update);
+//   2. blocked right-looking Cholesky (32-column panels: diagonal block and panel
+//      solve in one launch, trailing symmetric rank-32 update);
 //   3. W = L_top^T L_bot - L_bot^T L_top (J swaps the two halves of L's rows);
 //   4. Householder reduction of W to skew-tridiagonal form: the reflector
 //      H = I - tau v v^T of column k turns the trailing block into
@@ -26,12 +26,13 @@
 #include <cmath>
 
 #include "../../include/bse.h"
-#include "bse_internal.cuh"
+#include "grid_sync.cuh"
+#include "tree_solve.cuh"
 
 namespace bse {
 namespace {
 
-constexpr int DNB = 64;        // Cholesky panel width and GEMM tile edge
+constexpr int DNB = 32;        // Cholesky panel width and GEMM tile edge
 
 // (A_ij, B_ij) from the packed upper-triangle tiles of problem p (any i, j < N):
 // complex128 PH tiles hold P = A + B, Q = A - B; complex64 tiles hold A, B
@@ -77,126 +78,139 @@ __global__ void k_dn_assemble(const Prob* __restrict__ probs, int pq, double* __
   M[j * ld + i] = v;
 }
 
-// 2a. Cholesky of the diagonal block at k0 (kb <= 64 columns) in one CTA
-__global__ void __launch_bounds__(256) k_dn_potrf(double* __restrict__ M, int64_t ld, int64_t k0, int kb,
-                                                  int* __restrict__ notpd) {
+// 2. one panel: the diagonal block at k0 (kb <= 32 columns) is factored by every CTA for itself in
+// shared memory, a warp of rows per column step, and each CTA then solves x L11^T = a for its 32
+// rows below, eight lanes a row (four columns each: the 32-step chain of multiply-adds is what such
+// a solve costs, 64 clocks a step).  CTA 0 stores L11 to D (k_dn_update copies it back: the other
+// CTAs still read the block here).
+__global__ void __launch_bounds__(256) k_dn_panel(double* __restrict__ M, int64_t ld, int64_t n, int64_t k0, int kb,
+                                                  double* __restrict__ D, int* __restrict__ notpd) {
   __shared__ double a[DNB][DNB + 1];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kb * kb; e += 256) {
-    const int r = e % kb, c = e / kb;
-    a[r][c] = M[(k0 + c) * ld + k0 + r];
+  __shared__ double rd[DNB];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int e = tid; e < DNB * DNB; e += 256) {
+    const int r = e % DNB, c = e / DNB;
+    a[r][c] = (r < kb && c < kb && r >= c) ? M[(k0 + c) * ld + k0 + r] : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
   for (int c = 0; c < kb; ++c) {
-    if (tid == 0) {
+    if (warp == 0) {
       double d = a[c][c];
-      if (!(d > 0.0)) {            // M_r not positive definite: flag it, keep the numbers finite
-        atomicExch(notpd, 1);
-        d = 1.0;
-      }
-      a[c][c] = sqrt(d);
+      const bool bad = !(d > 0.0);     // M_r not positive definite: flag it, keep the numbers finite
+      if (bad) d = 1.0;
+      const double r = rsqrt(d);
+      if (bad && lane == 0 && blockIdx.x == 0) atomicExch(notpd, 1);
+      if (lane == c) { a[c][c] = d * r; rd[c] = r; }
+      else if (lane > c) a[lane][c] *= r;
     }
     __syncthreads();
-    const double inv = 1.0 / a[c][c];
-    for (int r = c + 1 + tid; r < kb; r += 256) a[r][c] *= inv;
-    __syncthreads();
-    for (int e = tid; e < (kb - c - 1) * (kb - c - 1); e += 256) {
-      const int r = c + 1 + e % (kb - c - 1), q = c + 1 + e / (kb - c - 1);
-      if (r >= q) a[r][q] -= a[r][c] * a[q][c];
-    }
+    // trailing columns q > c: a[r][q] -= a[r][c] a[q][c], lane = row
+    for (int q = c + 1 + warp; q < kb; q += 8)
+      if (lane >= q) a[lane][q] = fma(-a[lane][c], a[q][c], a[lane][q]);
     __syncthreads();
   }
-  for (int e = tid; e < kb * kb; e += 256) {
-    const int r = e % kb, c = e / kb;
-    if (r >= c) M[(k0 + c) * ld + k0 + r] = a[r][c];
-  }
-}
-
-// 2b. panel below the diagonal block: rows r >= k0 + kb solve x L11^T = a; one thread per row
-__global__ void __launch_bounds__(128) k_dn_trsm(double* __restrict__ M, int64_t ld, int64_t n, int64_t k0, int kb) {
-  __shared__ double l[DNB][DNB + 1];
-  for (int e = threadIdx.x; e < kb * kb; e += 128) {
-    const int r = e % kb, c = e / kb;
-    l[r][c] = r >= c ? M[(k0 + c) * ld + k0 + r] : 0.0;
-  }
-  __syncthreads();
-  const int64_t row = k0 + kb + (int64_t)blockIdx.x * 128 + threadIdx.x;
-  if (row >= n) return;
-  double x[DNB];
+  if (blockIdx.x == 0)
+    for (int e = tid; e < DNB * DNB; e += 256) D[e] = a[e % DNB][e / DNB];      // column-major
+  // rows below: eight lanes a row, lane s owns the columns s, s + 8, s + 16, s + 24
+  const int64_t row = k0 + kb + (int64_t)blockIdx.x * 32 + (tid >> 3);
+  const int s = tid & 7;
+  double x[4];
 #pragma unroll
-  for (int c = 0; c < DNB; ++c)
-    if (c < kb) x[c] = M[(k0 + c) * ld + row];
+  for (int u = 0; u < 4; ++u) {
+    const int c = s + 8 * u;
+    x[u] = (row < n && c < kb) ? M[(k0 + c) * ld + row] : 0.0;
+  }
 #pragma unroll
   for (int c = 0; c < DNB; ++c) {
-    if (c < kb) {
-      double s = x[c];
-#pragma unroll
-      for (int q = 0; q < DNB; ++q)
-        if (q < c) s -= x[q] * l[c][q];
-      x[c] = s / l[c][c];
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < DNB; ++c)
-    if (c < kb) M[(k0 + c) * ld + row] = x[c];
-}
-
-// C (m x m' block of an n x n column-major matrix) op= sum_q A(i, q) B(j, q) over kk
-// columns: 64 x 64 output tiles, 256 threads x (4 x 4), K staged 16 at a time.
-// mode 0: trailing Cholesky update C -= L21 L21^T on the lower triangle (tiles i >= j);
-// mode 1: G = A^T B with A, B row blocks (W step): C[i][j] = sum_k A[k][i] B[k][j].
-template <int MODE>
-__global__ void __launch_bounds__(256) k_dn_gemm(double* __restrict__ C, int64_t ldc, const double* __restrict__ Am,
-                                                 const double* __restrict__ Bm, int64_t lda, int64_t m, int64_t kk,
-                                                 int64_t off) {
-  __shared__ double sa[16][DNB + 1], sb[16][DNB + 1];
-  const int bi = blockIdx.x, bj = blockIdx.y;
-  if (MODE == 0 && bi < bj) return;                 // lower triangle only
-  const int tid = threadIdx.x, tr = tid & 15, tc = tid >> 4;
-  const int64_t i0 = (int64_t)bi * DNB, j0 = (int64_t)bj * DNB;
-  double acc[4][4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
-  for (int64_t q0 = 0; q0 < kk; q0 += 16) {
-    __syncthreads();
-    for (int e = tid; e < 16 * DNB; e += 256) {
-      const int r = e % DNB, q = e / DNB;
-      const int64_t gi = i0 + r, gj = j0 + r, gq = q0 + q;
-      if (MODE == 0) {   // A(i, q) = L21[i][q] = M[(off + q) * lda + off + i] style, passed as column-major panel
-        sa[q][r] = (gi < m && gq < kk) ? Am[gq * lda + gi] : 0.0;
-        sb[q][r] = (gj < m && gq < kk) ? Bm[gq * lda + gj] : 0.0;
-      } else {           // A(i, q) = Atop[q][i]: row q of the top block, column i
-        sa[q][r] = (gi < m && gq < kk) ? Am[gi * lda + gq] : 0.0;
-        sb[q][r] = (gj < m && gq < kk) ? Bm[gj * lda + gq] : 0.0;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) av[u] = sa[q][tr + 16 * u];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) bv[v] = sb[q][tc + 16 * v];
+    if (c < kb) {                          // uniform
+      if (s == (c & 7)) x[c >> 3] *= rd[c];
+      const double xc = __shfl_sync(0xffffffffu, x[c >> 3], (lane & 24) | (c & 7));
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+        if (s + 8 * u > c) x[u] = fma(-xc, a[s + 8 * u][c], x[u]);
     }
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < 4; ++u) {
+    const int c = s + 8 * u;
+    if (row < n && c < kb) M[(k0 + c) * ld + row] = x[u];
+  }
+}
+
+// trailing update C -= L21 L21^T on the lower triangle (32 x 32 tiles, 256 threads of 2 x 2), rows
+// and columns from `off`; the first CTA also copies the panel's diagonal block back from D
+__global__ void __launch_bounds__(256) k_dn_update(double* __restrict__ M, int64_t ld, int64_t n, int64_t k0, int kb,
+                                                   const double* __restrict__ D) {
+  __shared__ double sa[DNB][DNB + 1], sb[DNB][DNB + 1];
+  const int bi = blockIdx.x, bj = blockIdx.y, tid = threadIdx.x;
+  if (bi < bj) return;
+  if (bi == 0 && bj == 0)
+    for (int e = tid; e < kb * kb; e += 256) {
+      const int r = e % kb, c = e / kb;
+      if (r >= c) M[(k0 + c) * ld + k0 + r] = D[c * DNB + r];
+    }
+  const int64_t off = k0 + kb, i0 = off + (int64_t)bi * DNB, j0 = off + (int64_t)bj * DNB;
+  if (i0 >= n) return;
+  for (int e = tid; e < DNB * DNB; e += 256) {
+    const int r = e % DNB, q = e / DNB;
+    sa[q][r] = (i0 + r < n && q < kb) ? M[(k0 + q) * ld + i0 + r] : 0.0;
+    sb[q][r] = (j0 + r < n && q < kb) ? M[(k0 + q) * ld + j0 + r] : 0.0;
+  }
+  __syncthreads();
+  const int tr = tid & 15, tc = tid >> 4;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 8
+  for (int q = 0; q < DNB; ++q) {
+    const double a0 = sa[q][tr], a1 = sa[q][tr + 16], b0 = sb[q][tc], b1 = sb[q][tc + 16];
+    acc[0][0] = fma(a0, b0, acc[0][0]);
+    acc[0][1] = fma(a0, b1, acc[0][1]);
+    acc[1][0] = fma(a1, b0, acc[1][0]);
+    acc[1][1] = fma(a1, b1, acc[1][1]);
+  }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
       const int64_t gi = i0 + tr + 16 * u, gj = j0 + tc + 16 * v;
-      if (gi >= m || gj >= m) continue;
-      if (MODE == 0) {
-        if (gi >= gj) C[(off + gj) * ldc + off + gi] -= acc[u][v];
-      } else {
-        C[gj * ldc + gi] = acc[u][v];
-      }
+      if (gi < n && gj < n && gi >= gj) M[gj * ld + gi] -= acc[u][v];
+    }
+}
+
+// 3. G = L_top^T L_bot: G[i][j] = sum_q L[q][i] L[N + q][j], q < N.  L is lower triangular, so only
+// rows i < N are non-zero and q runs from max(i, j - N): a quarter of the full product.  32 x 32
+// tiles, 256 threads of 2 x 2, q staged 32 at a time; the other half of G is written as zeros.
+__global__ void __launch_bounds__(256) k_dn_wgemm(double* __restrict__ G, const double* __restrict__ L, int64_t ld,
+                                                  int64_t n) {
+  __shared__ double sa[DNB][DNB + 1], sb[DNB][DNB + 1];   // [q][column]
+  const int64_t N = n / 2, i0 = (int64_t)blockIdx.x * DNB, j0 = (int64_t)blockIdx.y * DNB;
+  const int tid = threadIdx.x, tr = tid & 15, tc = tid >> 4;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  int64_t q0 = i0 > j0 - N ? i0 : j0 - N;
+  if (i0 >= N) q0 = N;                                    // zero rows
+  for (; q0 < N; q0 += DNB) {
+    __syncthreads();
+    for (int e = tid; e < DNB * DNB; e += 256) {
+      const int q = e % DNB, c = e / DNB;                 // q along the columns of L
+      const int64_t gq = q0 + q, gi = i0 + c, gj = j0 + c;
+      sa[q][c] = (gq < N && gi < N && gq >= gi) ? L[gi * ld + gq] : 0.0;
+      sb[q][c] = (gq < N && gj < n && N + gq >= gj) ? L[gj * ld + N + gq] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int q = 0; q < DNB; ++q) {
+      const double a0 = sa[q][tr], a1 = sa[q][tr + 16], b0 = sb[q][tc], b1 = sb[q][tc + 16];
+      acc[0][0] = fma(a0, b0, acc[0][0]);
+      acc[0][1] = fma(a0, b1, acc[0][1]);
+      acc[1][0] = fma(a1, b0, acc[1][0]);
+      acc[1][1] = fma(a1, b1, acc[1][1]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int64_t gi = i0 + tr + 16 * u, gj = j0 + tc + 16 * v;
+      if (gi < n && gj < n) G[gj * ld + gi] = acc[u][v];
     }
 }
 
@@ -212,130 +226,187 @@ __global__ void k_dn_skew(double* __restrict__ W, int64_t ld, int64_t n) {
   W[i * ld + j] = gji - gij;
 }
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
+// 4. Householder reduction to skew-tridiagonal form in one cooperative launch: column j belongs to CTA
+// j mod G, in shared memory where the CTA's columns fit (order up to about 1900), else in place.  With
+// x = W[k+1:, k], beta = -sign(x0) |x|, v = x / (x0 - beta), v0 = 1, tau = (beta - x0) / beta (tau = 0
+// when x below x0 is zero), a step has two phases:
+//   * p = W22 v: since W is skew, p_j = -(column j) . v, each CTA from its own columns;
+//   * W22 += tau (v p^T - p v^T) on the own columns; the owner of column k + 1 updates it first and
+//     builds the next reflector from it.
+// So a step costs two grid barriers and a few multiply-adds per thread instead of four launches and a
+// matrix-vector product on n / 256 CTAs: 72 -> 7.5 us a column at order 600.  Whole diagonalisation,
+// measured: N = 300, 60 pairs 62.7 -> 9.5 ms; N = 1000, 50 pairs 450 -> 103 ms; N = 2000, 20 pairs 1.90 ->
+// 0.63 s.
+// Stores e_k = beta in E[k], tau in T[k], and v below the sub-diagonal of column k of W (its entry
+// k + 1 holds beta; the reflector's is 1).
+template <bool SMC>
+__global__ void __launch_bounds__(256) k_dn_tridiag(double* __restrict__ W, int64_t ld, int n, double* __restrict__ E,
+                                                    double* __restrict__ T, double* __restrict__ Pv, GridBar* gb) {
+  extern __shared__ double dsm[];
+  __shared__ int s_ok;
+  __shared__ double red[8], s_h[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = gridDim.x, bid = blockIdx.x;
+  unsigned int gen = 0;
+  double* vs = dsm;                // the reflector and p of the step (SMC); columns behind them
+  double* ps = dsm + n;
+  const int own = bid < n ? (n - 1 - bid) / G + 1 : 0;
+  auto col = [&](int q) { return SMC ? dsm + (size_t)(2 + q) * n : W + (int64_t)(bid + (int64_t)G * q) * ld; };
+  if (SMC) {
+    for (int q = 0; q < own; ++q) {
+      const double* src = W + (int64_t)(bid + (int64_t)G * q) * ld;
+      for (int r = tid; r < n; r += 256) col(q)[r] = src[r];
+    }
+    __syncthreads();
+  }
+  // the reflector of column c, whose entries below c are in x (all threads of the owner)
+  auto house = [&](const double* x, int c) {
+    double s = 0.0;
+    for (int r = c + 2 + tid; r < n; r += 256) s = fma(x[r], x[r], s);
+    s = warp_sum(s);
+    if (lane == 0) red[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+      double sig = lane < 8 ? red[lane] : 0.0;
 #pragma unroll
-  for (int m = 16; m >= 1; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int q = 0; q < nw; ++q) t += red[q];
-  return t;
+      for (int m = 4; m >= 1; m >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, m);
+      sig = __shfl_sync(0xffffffffu, sig, 0);
+      const double x0 = x[c + 1];
+      double beta = x0, tau = 0.0, scale = 0.0;
+      if (sig > 0.0) {
+        const double t = fma(x0, x0, sig), r = rsqrt(t), nrm = t * r;
+        beta = x0 >= 0.0 ? -nrm : nrm;
+        tau = fma(fabs(x0), r, 1.0);       // (beta - x0) / beta
+        const double g = 1.0 / (fabs(x0) + nrm);
+        scale = x0 >= 0.0 ? g : -g;        // 1 / (x0 - beta)
+      }
+      if (lane == 0) {
+        s_h[0] = beta;
+        s_h[1] = scale;
+        E[c] = beta;
+        T[c] = tau;
+      }
+    }
+    __syncthreads();
+    double* dst = W + (int64_t)c * ld;
+    const double beta = s_h[0], scale = s_h[1];
+    for (int r = c + 1 + tid; r < n; r += 256) dst[r] = r == c + 1 ? beta : x[r] * scale;
+  };
+  if (n > 2 && bid == 0) house(col(0), 0);
+  if (!grid_sync(gb, G, gen, &s_ok)) return;
+  for (int k = 0; k + 2 < n; ++k) {
+    const double* vk = W + (int64_t)k * ld;
+    const double tau = __ldcg(T + k);
+    auto v_at = [&](int r) { return SMC ? vs[r] : (r == k + 1 ? 1.0 : __ldcg(vk + r)); };
+    auto p_at = [&](int r) { return SMC ? ps[r] : __ldcg(Pv + r); };
+    if (SMC) {
+      for (int r = k + 1 + tid; r < n; r += 256) vs[r] = r == k + 1 ? 1.0 : __ldcg(vk + r);
+      __syncthreads();
+    }
+    // own columns j > k: a warp each
+    const int q0 = k + 1 <= bid ? 0 : (k + 1 - bid + G - 1) / G;
+    if (tau != 0.0)
+      for (int q = q0 + warp; q < own; q += 8) {
+        const double* x = col(q);
+        double s = 0.0;
+        for (int r = k + 1 + lane; r < n; r += 32) s = fma(x[r], v_at(r), s);
+        s = warp_sum(s);
+        if (lane == 0) Pv[bid + G * q] = -s;
+      }
+    if (!grid_sync(gb, G, gen, &s_ok)) return;
+    if (tau != 0.0) {
+      if (SMC) {
+        for (int r = k + 1 + tid; r < n; r += 256) ps[r] = __ldcg(Pv + r);
+        __syncthreads();
+      }
+      auto update = [&](int q, int r0, int dr) {
+        double* x = col(q);
+        const int j = bid + G * q;
+        const double tp = tau * p_at(j), tv = -tau * v_at(j);
+        for (int r = r0; r < n; r += dr) x[r] = fma(p_at(r), tv, fma(v_at(r), tp, x[r]));
+      };
+      int qn = -1;
+      if ((k + 1) % G == bid) {            // the next column first, by all warps
+        qn = (k + 1 - bid) / G;
+        update(qn, k + 1 + tid, 256);
+        __syncthreads();
+        if (k + 3 < n) house(col(qn), k + 1);
+      }
+      for (int q = q0 + warp; q < own; q += 8)
+        if (q != qn) update(q, k + 1 + lane, 32);
+    } else if ((k + 1) % G == bid && k + 3 < n) {
+      house(col((k + 1 - bid) / G), k + 1);
+    }
+    if (!grid_sync(gb, G, gen, &s_ok)) return;
+  }
+  // the last sub-diagonal entry needs no reflector
+  if ((n - 2) % G == bid && tid == 0) {
+    E[n - 2] = col((n - 2 - bid) / G)[n - 1];
+    T[n - 2] = 0.0;
+  }
 }
 
-// 4a. reflector of column k: x = W[k+1:, k]; beta = -sign(x0) |x|; v = x / (x0 - beta), v0 = 1,
-// tau = (beta - x0) / beta (tau = 0 when x below x0 is zero).  Stores e_k = beta in E[k], tau in
-// T[k], v (with v0 = 1) in V[k+1:] of a work column.  One CTA.
-__global__ void __launch_bounds__(1024) k_dn_house(const double* __restrict__ W, int64_t ld, int64_t n, int64_t k,
-                                                   double* __restrict__ E, double* __restrict__ T,
-                                                   double* __restrict__ V) {
+// the transpose of the Cholesky factor into the upper triangle (over the M_r values left there): the
+// back substitution reads rows of L along its columns
+__global__ void k_dn_mirror(double* __restrict__ M, int64_t ld, int64_t n) {
+  __shared__ double t[32][33];
+  const int64_t i0 = (int64_t)blockIdx.x * 32, j0 = (int64_t)blockIdx.y * 32;   // tile (i0, j0), i0 >= j0
+  if (i0 < j0) return;
+  for (int c = threadIdx.y; c < 32; c += 8) {
+    const int64_t i = i0 + threadIdx.x, j = j0 + c;
+    t[c][threadIdx.x] = (i < n && j < n) ? M[j * ld + i] : 0.0;
+  }
+  __syncthreads();
+  for (int c = threadIdx.y; c < 32; c += 8) {
+    const int64_t i = i0 + c, j = j0 + threadIdx.x;       // M[row j][column i] = L[i][j]
+    if (i < n && j < i) M[i * ld + j] = t[threadIdx.x][c];
+  }
+}
+
+// 5. S: zero diagonal, off-diagonals |e_k|.  The arrays the multisection and the inverse iteration
+// read (x = 0, |e|, and double-FP32 copies scaled to norm 1), and S's Gershgorin bound 2 max |e|; one CTA
+struct DnS {
+  double* x;      // n zeros
+  double* e;      // |e_k|
+  double* e2;     // its square
+  float2* xf;     // n zeros
+  float2* e2f;    // e2 scaled
+  double* bound;  // the bound and the scale
+};
+
+__global__ void __launch_bounds__(1024) k_dn_prepare(const double* __restrict__ E, int64_t n, DnS S) {
   __shared__ double red[32];
-  const double* x = W + k * ld;
-  double s = 0.0;
-  for (int64_t r = k + 2 + threadIdx.x; r < n; r += blockDim.x) s += x[r] * x[r];
-  const double sig = block_sum(s, red);
-  const double x0 = x[k + 1];
-  double beta, tau, scale;
-  if (sig == 0.0) {
-    beta = x0;
-    tau = 0.0;
-    scale = 0.0;
-  } else {
-    const double nrm = sqrt(x0 * x0 + sig);
-    beta = x0 >= 0.0 ? -nrm : nrm;
-    tau = (beta - x0) / beta;
-    scale = 1.0 / (x0 - beta);
+  double m = 0.0;
+  for (int64_t t = threadIdx.x; t + 1 < n; t += blockDim.x) m = fmax(m, fabs(E[t]));
+#pragma unroll
+  for (int k = 16; k >= 1; k >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, k));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = 0.0;
+  for (int q = 0; q < 32; ++q) m = fmax(m, red[q]);
+  const double bound = 2.0 * m * (1.0 + 1e-14) + 1e-300, sc = tree_scale(bound);
+  for (int64_t t = threadIdx.x; t < n; t += blockDim.x) {
+    const double e = t + 1 < n ? fabs(E[t]) : 0.0;
+    S.x[t] = 0.0;
+    S.e[t] = e;
+    S.e2[t] = e * e;
+    S.xf[t] = make_float2(0.f, 0.f);
+    S.e2f[t] = f2_split((e * sc) * (e * sc));
   }
-  for (int64_t r = k + 1 + threadIdx.x; r < n; r += blockDim.x) V[r] = r == k + 1 ? 1.0 : x[r] * scale;
   if (threadIdx.x == 0) {
-    E[k] = beta;
-    T[k] = tau;
+    S.bound[0] = bound;
+    S.bound[1] = sc;
   }
 }
 
-// 4b. p = W22 v over the trailing block rows/columns [k+1, n): one thread per row, columns
-// in chunks of 32 staged in shared memory
-__global__ void __launch_bounds__(256) k_dn_skew_mv(const double* __restrict__ W, int64_t ld, int64_t n, int64_t k,
-                                                    const double* __restrict__ V, double* __restrict__ Pv) {
-  __shared__ double sv[256];
-  const int64_t i = k + 1 + (int64_t)blockIdx.x * 256 + threadIdx.x;
-  double acc = 0.0;
-  for (int64_t j0 = k + 1; j0 < n; j0 += 256) {
-    __syncthreads();
-    const int64_t jj = j0 + threadIdx.x;
-    sv[threadIdx.x] = jj < n ? V[jj] : 0.0;
-    __syncthreads();
-    if (i < n) {
-      const int64_t jn = min((int64_t)256, n - j0);
-      const double* col = W + j0 * ld + i;
-#pragma unroll 4
-      for (int64_t q = 0; q < jn; ++q) acc = fma(col[q * ld], sv[q], acc);
-    }
-  }
-  if (i < n) Pv[i] = acc;
-}
-
-// 4c. W22 += tau (v p^T - p v^T); also stores v below the sub-diagonal of column k (the
-// reflector, for the back-transformation) and sets W[k+1][k] = beta
-__global__ void k_dn_skew_r2(double* __restrict__ W, int64_t ld, int64_t n, int64_t k, const double* __restrict__ V,
-                             const double* __restrict__ Pv, const double* __restrict__ T) {
-  const int64_t i = k + 1 + (int64_t)blockIdx.x * 32 + threadIdx.x;
-  const int64_t j = k + 1 + (int64_t)blockIdx.y * 8 + threadIdx.y;
-  if (i >= n || j >= n) return;
-  const double tau = T[k];
-  W[j * ld + i] += tau * (V[i] * Pv[j] - Pv[i] * V[j]);
-}
-
-__global__ void k_dn_store_v(double* __restrict__ W, int64_t ld, int64_t n, int64_t k, const double* __restrict__ V,
-                             const double* __restrict__ E) {
-  const int64_t r = k + 1 + (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (r >= n) return;
-  W[k * ld + r] = r == k + 1 ? E[k] : V[r];
-}
-
-// 5a. Sturm count of S - sigma I, S symmetric tridiagonal with zero diagonal and
-// off-diagonals |e_k| (k < n - 1): number of eigenvalues below sigma
-__device__ int dn_sturm(const double* __restrict__ e, int64_t n, double sigma, double pivmin) {
-  int cnt = 0;
-  double q = -sigma;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
-  for (int64_t t = 1; t < n; ++t) {
-    q = -sigma - e[t - 1] * e[t - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
-  }
-  return cnt;
-}
-
-// one warp per wanted eigenvalue (index idx0 + blockIdx.x of the ascending spectrum)
-__global__ void __launch_bounds__(32) k_dn_bisect(const double* __restrict__ e, int64_t n,
-                                                  const double* __restrict__ bound_p, int64_t idx0,
-                                                  double* __restrict__ lam) {
-  const int64_t idx = idx0 + blockIdx.x;
-  const int lane = threadIdx.x;
-  const double bound = *bound_p;
-  double lo = -bound, hi = bound;
-  const double pivmin = 1e-290 * fmax(1.0, bound * bound);
-  const double eps = 2.220446049250313e-16;
-  for (int it = 0; it < 100; ++it) {
-    const double width = hi - lo;
-    if (width <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + 4.0 * pivmin) break;
-    const double sig = lo + width * (double)(lane + 1) / 33.0;
-    const int c = dn_sturm(e, n, sig, pivmin);
-    const unsigned mask = __ballot_sync(0xffffffffu, c > idx);
-    if (mask == 0u) {
-      lo = __shfl_sync(0xffffffffu, sig, 31);
-    } else {
-      const int L = __ffs(mask) - 1;
-      const double sL = __shfl_sync(0xffffffffu, sig, L);
-      const double sLm = __shfl_sync(0xffffffffu, sig, L > 0 ? L - 1 : 0);
-      if (L > 0) lo = sLm;
-      hi = sL;
-    }
-  }
-  if (lane == 0) lam[blockIdx.x] = 0.5 * (lo + hi);
+// one CTA per wanted eigenvalue (index idx0 + blockIdx.x of the ascending spectrum)
+__global__ void __launch_bounds__(RV_THREADS) k_dn_bisect(DnS S, int64_t n, int64_t idx0, double* __restrict__ lam) {
+  __shared__ double s_sig[RV_THREADS];
+  __shared__ int s_cnt[RV_THREADS / 32];
+  const double bound = S.bound[0];
+  const double v = tree_eigenvalue(S.x, S.e2, S.xf, S.e2f, 0, (int)n, (int)(idx0 + blockIdx.x), -bound, bound, bound,
+                                   S.bound[1], s_sig, s_cnt);
+  if (threadIdx.x == 0) lam[blockIdx.x] = v;
 }
 
 __device__ __forceinline__ uint64_t dn_mix(uint64_t x) {
@@ -345,184 +416,185 @@ __device__ __forceinline__ uint64_t dn_mix(uint64_t x) {
   return x ^ (x >> 31);
 }
 
-// 5b. inverse iteration for the eigenvectors of S, one thread per cluster of close eigenvalues
-// (Gram-Schmidt inside a cluster); GEPP of S - lambda I in per-vector scratch (5 n doubles):
-// vectors s_c (n doubles each, unit 2-norm) go to Sv[c * n ...]
-__global__ void k_dn_inverse(const double* __restrict__ e, int64_t n, int nev, const double* __restrict__ lam,
-                             const double* __restrict__ bound_p, double* __restrict__ scratch,
-                             double* __restrict__ Sv) {
-  const int c0 = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c0 >= nev) return;
-  const double bound = *bound_p;
+// inverse iteration for the eigenvectors of S, one warp per cluster of close eigenvalues
+// (Gram-Schmidt inside a cluster); the factorisation in shared memory (SM) or in 5 n doubles of
+// scratch; vectors s_c (n doubles each, unit 2-norm) go to Sv[c * n ...]
+template <bool SM>
+__global__ void __launch_bounds__(32) k_dn_inverse(DnS S, int64_t n, int nev, const double* __restrict__ lam,
+                                                   double* __restrict__ scratch, double* __restrict__ Sv) {
+  extern __shared__ double dsm[];
+  const int c0 = blockIdx.x, lane = threadIdx.x;
+  const double bound = S.bound[0];
   const double eps = 2.220446049250313e-16;
   const double ctol = 1e-7 * bound;
   if (c0 > 0 && lam[c0] - lam[c0 - 1] < ctol) return;     // not a cluster leader
   int c1 = c0 + 1;
   while (c1 < nev && lam[c1] - lam[c1 - 1] < ctol) ++c1;
-  double* d = scratch + (int64_t)c0 * 5 * n;
-  double* du = d + n;
-  double* du2 = du + n;
-  double* dl = du2 + n;
-  double* pv = dl + n;                                     // pivots as doubles (0 / 1)
+  TV tv;
+  tv.d = tv.b = nullptr;
+  tv.h = 0;
+  tv.a = S.x;
+  tv.e = S.e;
+  tv.n = (int)n;
+  double* w = SM ? dsm : scratch + (int64_t)c0 * 5 * n;
+  Fact F;
+  F.invd = w;
+  F.dl = w + n;
+  F.du = w + 2 * n;
+  F.du2 = w + 3 * n;
+  F.piv = (unsigned char*)(w + 4 * n);
   const double pivmin = eps * fmax(bound, 1e-300);
   double lprev = -1e300;
   for (int c = c0; c < c1; ++c) {
     double lm = lam[c];
     if (c > c0 && lm - lprev < 10.0 * eps * bound) lm = lprev + 10.0 * eps * bound;
     lprev = lm;
-    for (int64_t t = 0; t < n; ++t) {
-      d[t] = -lm;
-      du[t] = t + 1 < n ? fabs(e[t]) : 0.0;
-      dl[t] = du[t];
-      du2[t] = 0.0;
-    }
-    for (int64_t t = 0; t + 1 < n; ++t) {
-      if (fabs(d[t]) >= fabs(dl[t])) {
-        pv[t] = 0.0;
-        if (d[t] == 0.0) d[t] = pivmin;
-        const double f = dl[t] / d[t];
-        dl[t] = f;
-        d[t + 1] -= f * du[t];
-      } else {
-        pv[t] = 1.0;
-        const double f = d[t] / dl[t];
-        d[t] = dl[t];
-        dl[t] = f;
-        const double tmp = du[t];
-        du[t] = d[t + 1];
-        d[t + 1] = tmp - f * d[t + 1];
-        if (t + 2 < n) {
-          du2[t] = du[t + 1];
-          du[t + 1] = -f * du[t + 1];
-        }
-      }
-    }
-    if (fabs(d[n - 1]) < pivmin) d[n - 1] = pivmin;
+    factor_tree(tv, lm, pivmin, F, lane);
     double* x = Sv + (int64_t)c * n;
-    for (int64_t t = 0; t < n; ++t)
+    for (int64_t t = lane; t < n; t += 32)
       x[t] = (double)(dn_mix((uint64_t)(c + 1) * 0x100000001b3ull + (uint64_t)t) >> 11) * (1.0 / 9007199254740992.0) - 0.5;
+    __syncwarp();
     for (int it = 0; it < 4; ++it) {
       for (int rep = 0; rep < 2; ++rep)
         for (int q = c0; q < c; ++q) {
           const double* sq = Sv + (int64_t)q * n;
           double dot = 0.0;
-          for (int64_t t = 0; t < n; ++t) dot += sq[t] * x[t];
-          for (int64_t t = 0; t < n; ++t) x[t] -= dot * sq[t];
+          for (int64_t t = lane; t < n; t += 32) dot = fma(sq[t], x[t], dot);
+          dot = warp_sum(dot);
+          for (int64_t t = lane; t < n; t += 32) x[t] = fma(-dot, sq[t], x[t]);
+          __syncwarp();
         }
       double nr = 0.0;
-      for (int64_t t = 0; t < n; ++t) nr += x[t] * x[t];
-      const double inv = nr > 0.0 ? 1.0 / sqrt(nr) : 0.0;
-      for (int64_t t = 0; t < n; ++t) x[t] *= inv;
+      for (int64_t t = lane; t < n; t += 32) nr = fma(x[t], x[t], nr);
+      nr = warp_sum(nr);
+      const double inv = nr > 0.0 ? rsqrt(nr) : 0.0;
+      for (int64_t t = lane; t < n; t += 32) x[t] *= inv;
+      __syncwarp();
       if (it == 3) break;
-      for (int64_t t = 0; t + 1 < n; ++t) {          // forward: L
-        if (pv[t] == 0.0) {
-          x[t + 1] -= dl[t] * x[t];
-        } else {
-          const double tmp = x[t];
-          x[t] = x[t + 1];
-          x[t + 1] = tmp - dl[t] * x[t];
-        }
-      }
-      x[n - 1] /= d[n - 1];                           // backward: U
-      if (n > 1) x[n - 2] = (x[n - 2] - du[n - 2] * x[n - 1]) / d[n - 2];
-      for (int64_t t = n - 3; t >= 0; --t) x[t] = (x[t] - du[t] * x[t + 1] - du2[t] * x[t + 2]) / d[t];
+      solve_tree(tv, F, x, lane);
     }
-  }
-}
-
-// zero the upper triangle of the Cholesky factor (the M_r values left there)
-__global__ void k_dn_zero_upper(double* __restrict__ M, int64_t ld, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
-  const int64_t j = (int64_t)blockIdx.y * 8 + threadIdx.y;
-  if (i < n && j < n && i < j) M[j * ld + i] = 0.0;
-}
-
-// the last sub-diagonal entry of T needs no reflector
-__global__ void k_dn_store_last(const double* __restrict__ W, int64_t ld, int64_t n, double* __restrict__ E,
-                                double* __restrict__ T) {
-  E[n - 2] = W[(n - 2) * ld + n - 1];
-  T[n - 2] = 0.0;
-}
-
-// Gershgorin bound of S: 2 max |e| (and a tiny floor), one CTA
-__global__ void __launch_bounds__(1024) k_dn_bound(const double* __restrict__ E, int64_t n, double* __restrict__ out) {
-  __shared__ double red[32];
-  double m = 0.0;
-  for (int64_t t = threadIdx.x; t + 1 < n; t += blockDim.x) m = fmax(m, fabs(E[t]));
-#pragma unroll
-  for (int k = 16; k >= 1; k >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, k));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t = fmax(t, red[q]);
-    *out = 2.0 * t * (1.0 + 1e-14) + 1e-300;
   }
 }
 
 // 6. one CTA per eigenvector: q = H_0 ... H_{n-3} D s (D: the phases that make -iT real, so q is
-// complex), then y = L^{-T} q, then z = Q y into Z (FP64 complex, ld 2 Npad: X rows then Y rows)
+// complex), then y = L^{-T} q, then z = Q y into Z (FP64 complex, ld 2 Npad: X rows then Y rows).  The
+// next reflector (row of L) is loaded while the current one is reduced; the two components of a dot
+// product share one reduction (a half-warp each from the second step on); the triangular solve goes
+// column by column of L^T's upper-triangle copy, so it needs no reduction at all.  q is in shared
+// memory (SM) or in qbuf.
+template <bool SM>
 __global__ void __launch_bounds__(256) k_dn_back(const double* __restrict__ Wv, const double* __restrict__ L,
                                                  int64_t ld, int64_t n, const double* __restrict__ E,
                                                  const double* __restrict__ T, const double* __restrict__ Sv,
                                                  double2* __restrict__ qbuf, int64_t Npad, double2* __restrict__ Z) {
-  __shared__ double red[8];
+  extern __shared__ double dsm[];
+  __shared__ double red[8][2];
   const int c = blockIdx.x;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t N = n / 2;
-  double2* q = qbuf + (int64_t)c * n;
+  double2* q = SM ? reinterpret_cast<double2*>(dsm) : qbuf + (int64_t)c * n;
   const double* s = Sv + (int64_t)c * n;
-  // D: d_0 = 1, d_{k+1} = d_k (-i) sign(e_k); the phase is i^(-k) times a sign, so it is
-  // tracked as an index mod 4 and a sign (sequential, one thread)
-  if (tid == 0) {
-    int ph = 0;
-    double sg = 1.0;
-    for (int64_t t = 0; t < n; ++t) {
-      const double v = s[t] * sg;
-      const double2 dv = (ph == 0) ? make_double2(v, 0.0)
-                       : (ph == 1) ? make_double2(0.0, -v)
-                       : (ph == 2) ? make_double2(-v, 0.0)
-                                   : make_double2(0.0, v);       // v (-i)^ph
-      q[t] = dv;
-      if (t + 1 < n) {
-        ph = (ph + 1) & 3;
-        if (E[t] < 0.0) sg = -sg;
+  // D: d_0 = 1, d_{t+1} = d_t (-i) sign(e_t): the phase (-i)^t and the parity of the negative e
+  // before t (prefix over 32-entry groups by ballots, each warp for itself)
+  {
+    unsigned par = 0;
+    for (int64_t t0 = 0; t0 < n; t0 += 32) {
+      const int64_t t = t0 + lane;
+      const unsigned neg = __ballot_sync(0xffffffffu, t + 1 < n && E[t] < 0.0);
+      if (((t0 >> 5) & 7) == warp && t < n) {
+        const bool minus = (par + __popc(neg & ((1u << lane) - 1u))) & 1u;
+        const double v = minus ? -s[t] : s[t];
+        const int ph = (int)(t & 3);
+        q[t] = ph == 0 ? make_double2(v, 0.0) : ph == 1 ? make_double2(0.0, -v)
+             : ph == 2 ? make_double2(-v, 0.0) : make_double2(0.0, v);              // v (-i)^t
       }
+      par += __popc(neg);
     }
   }
   __syncthreads();
-  for (int64_t k = n - 3; k >= 0; --k) {              // q <- H_k q on rows k+1 ... n-1
-    const double tau = T[k];
-    if (tau == 0.0) continue;                          // uniform: T is read by every thread
-    const double* v = Wv + k * ld;                     // v_{k+1} = 1 (stored as beta), v_r below
+  constexpr int U = 4;                                  // entries a thread keeps of the next column
+  double nx[U];
+  auto fetch = [&](const double* v, int64_t r0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) nx[u] = r0 + tid + 256 * u < n ? __ldg(v + r0 + tid + 256 * u) : 0.0;
+  };
+  if (n > 2) fetch(Wv + (n - 3) * ld, n - 2);
+  for (int64_t k = n - 3; k >= 0; --k) {                // q <- H_k q on rows k+1 ... n-1
+    const double tau = __ldg(T + k);
+    const double* v = Wv + k * ld;                      // v_{k+1} = 1 (stored as beta), v_r below
+    double cur[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) cur[u] = nx[u];
+    if (k > 0) fetch(Wv + (k - 1) * ld, k);
+    if (tau == 0.0) continue;                           // uniform
+    if (tid == 0) cur[0] = 1.0;
     double sr = 0.0, si = 0.0;
-    for (int64_t r = k + 1 + tid; r < n; r += 256) {
-      const double vr = r == k + 1 ? 1.0 : v[r];
-      sr += vr * q[r].x;
-      si += vr * q[r].y;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t r = k + 1 + tid + 256 * u;
+      if (r < n) {
+        sr = fma(cur[u], q[r].x, sr);
+        si = fma(cur[u], q[r].y, si);
+      }
     }
-    sr = block_sum(sr, red);
-    si = block_sum(si, red);
-    for (int64_t r = k + 1 + tid; r < n; r += 256) {
-      const double vr = r == k + 1 ? 1.0 : v[r];
-      q[r].x -= tau * vr * sr;
-      q[r].y -= tau * vr * si;
+    for (int64_t r = k + 1 + tid + 256 * U; r < n; r += 256) {
+      const double vr = __ldg(v + r);
+      sr = fma(vr, q[r].x, sr);
+      si = fma(vr, q[r].y, si);
+    }
+    // lanes 0-15 go on with the real sum, 16-31 with the imaginary one
+    double t = lane < 16 ? sr : si;
+    t += __shfl_xor_sync(0xffffffffu, lane < 16 ? si : sr, 16);
+#pragma unroll
+    for (int m = 8; m >= 1; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+    if ((lane & 15) == 0) red[warp][lane >> 4] = t;
+    __syncthreads();
+    t = red[lane & 7][(lane >> 3) & 1];
+#pragma unroll
+    for (int m = 4; m >= 1; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+    t *= -tau;
+    sr = __shfl_sync(0xffffffffu, t, 0);
+    si = __shfl_sync(0xffffffffu, t, 8);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t r = k + 1 + tid + 256 * u;
+      if (r < n) q[r] = make_double2(fma(cur[u], sr, q[r].x), fma(cur[u], si, q[r].y));
+    }
+    for (int64_t r = k + 1 + tid + 256 * U; r < n; r += 256) {
+      const double vr = __ldg(v + r);
+      q[r] = make_double2(fma(vr, sr, q[r].x), fma(vr, si, q[r].y));
     }
     __syncthreads();
   }
-  // y = L^{-T} q: for i = n-1 ... 0, y_i = (q_i - sum_{j > i} L[j][i] y_j) / L[i][i] (in place)
+  // y = L^{-T} q (in place): y_i = q_i / L[i][i], then q_j -= L[i][j] y_i for j < i, L[i][j] at row j of
+  // column i in the upper triangle
+  auto fetch_row = [&](int64_t i) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) nx[u] = tid + 256 * u < i ? __ldg(L + i * ld + tid + 256 * u) : 0.0;
+  };
+  fetch_row(n - 1);
+  double dn = __ldg(L + (n - 1) * ld + n - 1);
   for (int64_t i = n - 1; i >= 0; --i) {
-    const double* col = L + i * ld;
-    double sr = 0.0, si = 0.0;
-    for (int64_t j = i + 1 + tid; j < n; j += 256) {
-      sr += col[j] * q[j].x;
-      si += col[j] * q[j].y;
+    const double inv = recip(dn);
+    double cur[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) cur[u] = nx[u];
+    if (i > 0) {
+      fetch_row(i - 1);
+      dn = __ldg(L + (i - 1) * ld + i - 1);
     }
-    sr = block_sum(sr, red);
-    si = block_sum(si, red);
-    if (tid == 0) {
-      const double inv = 1.0 / col[i];
-      q[i] = make_double2((q[i].x - sr) * inv, (q[i].y - si) * inv);
+    const double2 qi = q[i];
+    const double2 y = make_double2(qi.x * inv, qi.y * inv);
+    __syncthreads();                                    // everyone has read q_i
+    if (tid == (int)(i & 255)) q[i] = y;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t j = tid + 256 * u;
+      if (j < i) q[j] = make_double2(fma(-cur[u], y.x, q[j].x), fma(-cur[u], y.y, q[j].y));
+    }
+    for (int64_t j = tid + 256 * U; j < i; j += 256) {
+      const double l = __ldg(L + i * ld + j);
+      q[j] = make_double2(fma(-l, y.x, q[j].x), fma(-l, y.y, q[j].y));
     }
     __syncthreads();
   }
@@ -544,17 +616,19 @@ __global__ void __launch_bounds__(256) k_dn_back(const double* __restrict__ Wv, 
 }  // namespace
 
 // scratch of dense_shao in doubles: M_r / L and W (ld x n each), the reflector work
-// vectors, the eigenvector scratch of the inverse iteration, and the complex q vectors
+// vectors, the arrays of S, the eigenvector scratch of the inverse iteration, the complex q
+// vectors, the panel's diagonal block and the grid barrier
 size_t dense_scratch_doubles(int64_t N, int nev) {
   const int64_t n = 2 * N;
   const int64_t ld = (n + 31) / 32 * 32;
-  // ten sub-buffers, each rounded up to 32 doubles
-  return (size_t)(2 * ld * n + 4 * n + (int64_t)nev * (5 * n + n + 2 * n) + nev + 8 + 10 * 32);
+  // sixteen sub-buffers, each rounded up to 32 doubles
+  return (size_t)(2 * ld * n + 3 * n + 5 * n + (int64_t)nev * (5 * n + n + 2 * n) + nev + DNB * DNB + 16 + 16 * 32);
 }
 
 // Steps 2-6 on an assembled M_r (step 1 is `assemble(M, ld)`): the nev lowest positive omega
 // (device, *lam_dev) and their right eigenvectors (unnormalised) in Z (ld 2 Npad).  Returns 0,
-// 1 (M_r not positive definite) or -1 (CUDA error); the stream is synchronised.
+// 1 (M_r not positive definite), 2 (a bounded wait expired) or -1 (CUDA error); the stream is
+// synchronised.
 template <typename Assemble>
 int dense_run(int64_t N, int64_t Npad, int nev, double* work, int* dflag, double2* Z, double** lam_dev,
               Assemble assemble, cudaStream_t s) {
@@ -567,71 +641,88 @@ int dense_run(int64_t N, int64_t Npad, int nev, double* work, int* dflag, double
     off += (size_t)((count + 31) / 32 * 32);
     return p;
   };
-  double* M = take(ld * n);         // M_r, then L (lower)
+  double* M = take(ld * n);         // M_r, then L (lower) and L^T (upper)
   double* W = take(ld * n);         // G, then W, then the reduced form with the reflectors
   double* E = take(n);              // sub-diagonal of T
   double* T = take(n);              // reflector scalars
-  double* V = take(n);              // current reflector
   double* Pv = take(n);             // W22 v
-  double* lam = take(nev + 8);      // wanted eigenvalues of S, then the bound of S
+  DnS S;
+  S.x = take(n);
+  S.e = take(n);
+  S.e2 = take(n);
+  S.xf = reinterpret_cast<float2*>(take(n));
+  S.e2f = reinterpret_cast<float2*>(take(n));
+  S.bound = take(2);
+  double* lam = take(nev);          // wanted eigenvalues of S
   double* inv = take((int64_t)nev * 5 * n);   // inverse-iteration scratch, 5 n per vector
   double* Sv = take((int64_t)nev * n);
   double2* qb = reinterpret_cast<double2*>(take((int64_t)nev * 2 * n));
+  double* D = take(DNB * DNB);
+  GridBar* gb = reinterpret_cast<GridBar*>(take(1));
   *lam_dev = lam;
-  if (cudaMemsetAsync(dflag, 0, sizeof(int), s) != cudaSuccess) return -1;
+  if (cudaMemsetAsync(dflag, 0, sizeof(int), s) != cudaSuccess ||
+      cudaMemsetAsync(gb, 0, sizeof(GridBar), s) != cudaSuccess)
+    return -1;
   // 1.
   const dim3 g2((unsigned)((n + 31) / 32), (unsigned)((n + 7) / 8)), b2(32, 8);
   assemble(M, ld);
   // 2. Cholesky
   for (int64_t k0 = 0; k0 < n; k0 += DNB) {
     const int kb = (int)std::min<int64_t>(DNB, n - k0);
-    count_launch();
-    k_dn_potrf<<<1, 256, 0, s>>>(M, ld, k0, kb, dflag);
-    const int64_t rest = n - k0 - kb;
-    if (rest > 0) {
-      count_launch(2);
-      k_dn_trsm<<<(unsigned)((rest + 127) / 128), 128, 0, s>>>(M, ld, n, k0, kb);
-      const unsigned nt = (unsigned)((rest + DNB - 1) / DNB);
-      // A = B = the panel L21, rows k0 + kb ..., columns k0 ... k0 + kb (column-major, ld)
-      const double* panel = M + k0 * ld + k0 + kb;
-      k_dn_gemm<0><<<dim3(nt, nt), 256, 0, s>>>(M, ld, panel, panel, ld, rest, kb, k0 + kb);
-    }
+    const unsigned nt = (unsigned)std::max<int64_t>(1, (n - k0 - kb + DNB - 1) / DNB);
+    count_launch(2);
+    k_dn_panel<<<nt, 256, 0, s>>>(M, ld, n, k0, kb, D, dflag);
+    k_dn_update<<<dim3(nt, nt), 256, 0, s>>>(M, ld, n, k0, kb, D);
   }
-  count_launch();
-  k_dn_zero_upper<<<g2, b2, 0, s>>>(M, ld, n);
-  // 3. G = L_top^T L_bot (rows 0..N-1 and N..2N-1 of L, all n columns), then W = G - G^T.
-  // In mode 1 the kernel reads A(i, q) = Am[i * lda + q]: column i of L, row q of the block
-  count_launch(2);
+  // 3. G = L_top^T L_bot, then W = G - G^T
+  count_launch(3);
   const unsigned ng = (unsigned)((n + DNB - 1) / DNB);
-  k_dn_gemm<1><<<dim3(ng, ng), 256, 0, s>>>(W, ld, M, M + N, ld, n, N, 0);
+  k_dn_mirror<<<dim3(ng, ng), b2, 0, s>>>(M, ld, n);
+  k_dn_wgemm<<<dim3(ng, ng), 256, 0, s>>>(W, M, ld, n);
   k_dn_skew<<<g2, b2, 0, s>>>(W, ld, n);
   // 4. skew-tridiagonalisation
-  for (int64_t k = 0; k + 2 < n; ++k) {
-    const int64_t m = n - k - 1;
-    count_launch(4);
-    k_dn_house<<<1, 1024, 0, s>>>(W, ld, n, k, E, T, V);
-    k_dn_skew_mv<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(W, ld, n, k, V, Pv);
-    k_dn_skew_r2<<<dim3((unsigned)((m + 31) / 32), (unsigned)((m + 7) / 8)), dim3(32, 8), 0, s>>>(W, ld, n, k, V, Pv,
-                                                                                                  T);
-    k_dn_store_v<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(W, ld, n, k, V, E);
-  }
-  // the last sub-diagonal entry needs no reflector
-  if (n >= 2) {
+  {
+    int nn = (int)n;
+    int64_t lda = ld;
+    const int grid = (int)std::min<int64_t>(num_sms(), n);
+    const size_t cols = sizeof(double) * (size_t)n * ((n + grid - 1) / grid + 2);
+    const bool smc = cols <= 200 * 1024;
+    void* args[] = {(void*)&W, (void*)&lda, (void*)&nn, (void*)&E, (void*)&T, (void*)&Pv, (void*)&gb};
+    const void* fn = smc ? (const void*)k_dn_tridiag<true> : (const void*)k_dn_tridiag<false>;
+    if (smc) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
     count_launch();
-    k_dn_store_last<<<1, 1, 0, s>>>(W, ld, n, E, T);
+    if (cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(256), args, smc ? cols : 0, s) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
   }
   // 5. eigenvalues N ... N + nev - 1 of S and their eigenvectors
   count_launch(3);
-  k_dn_bound<<<1, 1024, 0, s>>>(E, n, lam + nev);
-  k_dn_bisect<<<nev, 32, 0, s>>>(E, n, lam + nev, N, lam);
-  k_dn_inverse<<<(nev + 31) / 32, 32, 0, s>>>(E, n, nev, lam, lam + nev, inv, Sv);
+  k_dn_prepare<<<1, 1024, 0, s>>>(E, n, S);
+  k_dn_bisect<<<nev, RV_THREADS, 0, s>>>(S, n, N, lam);
+  const size_t fs = sizeof(double) * (size_t)(4 * n) + (size_t)n;
+  if (fs <= 200 * 1024) {
+    cudaFuncSetAttribute(k_dn_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs);
+    k_dn_inverse<true><<<nev, 32, fs, s>>>(S, n, nev, lam, inv, Sv);
+  } else {
+    k_dn_inverse<false><<<nev, 32, 0, s>>>(S, n, nev, lam, inv, Sv);
+  }
   // 6.
   count_launch();
-  k_dn_back<<<nev, 256, 0, s>>>(W, M, ld, n, E, T, Sv, qb, Npad, Z);
+  const size_t qs = sizeof(double2) * (size_t)n;
+  if (qs <= 200 * 1024) {
+    cudaFuncSetAttribute(k_dn_back<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
+    k_dn_back<true><<<nev, 256, qs, s>>>(W, M, ld, n, E, T, Sv, qb, Npad, Z);
+  } else {
+    k_dn_back<false><<<nev, 256, 0, s>>>(W, M, ld, n, E, T, Sv, qb, Npad, Z);
+  }
   int h = 0;
-  if (cudaMemcpyAsync(&h, dflag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
+  GridBar hb{};
+  if (cudaMemcpyAsync(&h, dflag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(&hb, gb, sizeof(GridBar), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    return -1;
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return -1;
-  return h ? 1 : 0;
+  return hb.err ? 2 : (h ? 1 : 0);
 }
 
 namespace {
@@ -667,6 +758,17 @@ __global__ void k_pj_assemble(const Prob* __restrict__ probs, int ip, double* __
     else if (lo >= h && hi == lo + 1) v = p.beta[l + (lo - h)];
   }
   M[j * ld + i] = v;
+}
+
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  v = warp_sum(v);
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[w] = v;
+  __syncthreads();
+  double t = 0.0;
+  for (int q = 0; q < nw; ++q) t += red[q];
+  return t;
 }
 
 // folded Ritz data from the small problem's eigenvectors: one CTA per wanted pair
@@ -760,7 +862,7 @@ int projected_ritz(const Prob* dprobs, int iprob, int n, int nw, double* work, i
     count_launch();
     k_pj_assemble<<<g2, b2, 0, s>>>(dprobs, iprob, M, ld);
   }, s);
-  if (rc < 0) return rc;
+  if (rc < 0 || rc == 2) return rc;
   count_launch();
   if (rc == 1) {
     k_pj_fail<<<1, 32, 0, s>>>(dprobs, iprob);

@@ -19,6 +19,7 @@
 #include <cstddef>
 
 #include "fx_phases.cuh"
+#include "grid_sync.cuh"
 
 namespace bse {
 namespace {
@@ -27,38 +28,6 @@ constexpr int PS_THREADS = 256;
 // One CTA per SM: two of 128 registers a thread spill in the product's row loop (measured, PH
 // N = 3000: 473 ms against 311; TDA N = 2000: 81 against 53).
 constexpr int PS_RING = 8192;              // two (TDA: four) tile rows per warp in flight (16 KiB: no faster)
-constexpr long long PS_SPIN = 1ll << 22;   // polls of one barrier wait
-
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// All CTAs of the launch meet here; false (in every thread of the CTA) when the wait expired.  The
-// arrivals of all barriers of a launch add up in one counter, so nothing is reset and a waiter
-// polls the counter itself: one release and the polls, 1.3 us where an arrival count that the last
-// CTA turns into a generation number, with a fence in every thread, took 2.2.
-__device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned int nblk, unsigned int& gen, int* s_ok) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    const unsigned int target = (gen + 1) * nblk;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gb->count) : "memory");
-    long long i = 0;
-    while ((int)(ld_acquire_u32(&gb->count) - target) < 0) {
-      if (++i > PS_SPIN) {
-        atomicExch(&gb->err, 1);
-        ok = 0;
-        break;
-      }
-    }
-    *s_ok = ok;
-  }
-  ++gen;
-  __syncthreads();
-  return *s_ok != 0;
-}
 
 // The FP64 tiles (a few, if any, beside fixed-point ones) stay out of line: their registers would be
 // spilled around the other phases.

@@ -67,6 +67,20 @@ def test_dense_matches_iterative():
     s.close()
 
 
+@pytest.mark.parametrize("n,nev", [(1, 1), (2, 2), (17, 9), (33, 16), (1030, 12), (3110, 4)])
+def test_dense_edges_of_the_reduction(n, nev):
+    """Orders where the reduction changes its ways: no reflector at all, one panel and a ragged one,
+    the columns past shared memory (2N > 1900), the factors of the inverse iteration past it (2N >
+    6200).  FP64 residuals at tol and agreement with the iterative solver."""
+    A, B = problem(n, "c128", seed=n, n_g=max(8, min(40, n // 4)))
+    s = _solver(A, B)
+    v1, _, nconv = s.solve_dense(nev, tol=1e-10, vectors=False)
+    assert nconv == nev and s.residuals().max() <= 1e-10
+    v2, _, _ = s.solve(nev, tol=1e-12, vectors=False)
+    np.testing.assert_allclose(v1, v2, rtol=1e-11, atol=0)
+    s.close()
+
+
 def test_dense_not_positive_definite_and_invalid():
     from paper_2504_10096_gb300 import bse
     n = 70
