@@ -67,3 +67,22 @@ def test_noalloc_rejects_oversize():
                                dummy.data_ptr(), dummy.data_ptr(), 0)
     assert rc == bse.BSE_EINVAL
     assert "invalid" in bse.bse_strerror(rc)
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("n", [1, 100, 129, 600, 1300, 2100, 2900])
+def test_noalloc_bands(dtype, n):
+    """Orders whose tiles are cut into 8, 4, 2 and 1 bands of rows, element by element."""
+    from paper_2504_10096_gb300 import bse
+    A, B = problem(n, dtype, seed=n + 5, n_g=32)
+    At, Bt = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    xh = rand_block(n, 1, dtype, seed=9)
+    x = torch.from_numpy(xh[:, 0]).cuda()
+    code = bse.BSE_C128 if dtype == "c128" else bse.BSE_C64
+    for op, f, name in ((bse.BSE_OP_A, lambda: O.apply_a(A, xh), "a"),
+                        (bse.BSE_OP_MMINUS, lambda: O.apply_mminus(A, B, xh), "mminus")):
+        y = torch.full_like(x, float("nan"))
+        rc = bse.bse_apply_noalloc(n, At.data_ptr(), Bt.data_ptr(), code, op, x.data_ptr(), y.data_ptr(),
+                                   torch.cuda.current_stream().cuda_stream)
+        assert rc == bse.BSE_OK
+        assert_elementwise(y.cpu().numpy(), f()[:, 0], product_bound(A, B, xh, name)[:, 0], UNIT[dtype], 64, name)
