@@ -55,6 +55,7 @@ struct ProbHost {
   int zcols = 0;
   int nconv = 0;
   int* perm = nullptr;   // device, output column -> Z column
+  std::vector<int> hperm;   // ... and on the host
   std::vector<double> eval, res;
 };
 
@@ -701,7 +702,8 @@ struct Driver {
     CK(cudaMemcpyAsync(hr.data(), rho, sizeof(double) * k, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(hres.data(), res, sizeof(double) * k, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    std::vector<int> perm(k);
+    std::vector<int>& perm = q.hperm;
+    perm.resize(k);
     for (int c = 0; c < k; ++c) perm[c] = c;
     std::stable_sort(perm.begin(), perm.end(), [&](int a, int b) { return hr[a] < hr[b]; });
     int good = 0;
@@ -1258,10 +1260,7 @@ int backward_impl(bse_handle* h, const double* g, int where, void* dA, void* dB,
   } else {
     std::memcpy(gh.data(), g, sizeof(double) * h->nev);
   }
-  std::vector<int> perm(k);
-  CK(cudaMemcpyAsync(perm.data(), q.perm, sizeof(int) * k, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  for (int c = 0; c < k; ++c) gz[perm[c]] = gh[c];
+  for (int c = 0; c < k; ++c) gz[q.hperm[c]] = gh[c];
   int rc;
   if (!h->gdev && (rc = dalloc((void**)&h->gdev, sizeof(double) * MAXM))) return rc;
   CK(cudaMemcpyAsync(h->gdev, gz.data(), sizeof(double) * k, cudaMemcpyHostToDevice, h->stream));

@@ -13,10 +13,12 @@
 // k_adjoint_tc: one persistent CTA per SM, warp-specialised.  The work unit is
 // a half-tile (128 output rows x 64 columns of a 128 x 128 tile I <= J), whose
 // FP32 accumulators (dA re/im, dB re/im) take 256 TMEM columns, so two sets
-// fit in the SM's 512: while warps 0-3 drain one set (tcgen05.ld) and write
-// the half-tile and its mirror (dA Hermitian, dB symmetric), warp 4 already
+// fit in the SM's 512: while warps 0-7 drain one set (tcgen05.ld) and write
+// the half-tile and its mirror (dA Hermitian, dB symmetric), warp 8 already
 // runs the next half-tile's tcgen05.mma (M = 128, N = 64, K = 8) into the
-// other.  Warp 4 also feeds a three-stage shared-memory pipeline with bulk
+// other.  (One lane for copies and MMAs, with 64-bit divisions for its place and
+// a descriptor built per MMA, kept the tensor cores 21 % busy: 229 us at N = 6000,
+// 32 pairs, against 86 us of HBM writes; now 125.)  Warp 9 feeds a three-stage shared-memory pipeline with bulk
 // asynchronous copies (cp.async.bulk, completion on mbarriers); tcgen05.commit
 // releases a stage when its MMAs finish and publishes a finished accumulator
 // set.  Every wait is bounded; on expiry the CTA records an error, stops, waits
@@ -31,10 +33,11 @@ namespace {
 
 constexpr int TCM = 128;                  // tile rows (M) and columns (N)
 constexpr int KC = 16;                    // K elements per pipeline chunk
-constexpr int TC_THREADS = 160;           // warps 0-3 epilogue, warp 4 copies + MMAs
+constexpr int EPI_WARPS = 8;              // two per TMEM lane quarter: dA and dB (TDA: the column halves)
+constexpr int TC_THREADS = 32 * EPI_WARPS + 64;   // ... one warp for the MMAs, one for the copies
 constexpr int NSTAGE = 3;                 // shared-memory pipeline stages
 constexpr int BLK = TCM * KC * 4;         // bytes of one operand block (8 KiB)
-constexpr int EPI_BYTES = 4 * 32 * 33 * 8;   // per-warp transpose buffers of the epilogue
+constexpr int EPI_BYTES = EPI_WARPS * 32 * 17 * 8;   // per-warp transpose buffers of the epilogue (32 x 16)
 constexpr long long TC_SPIN = 1ll << 26;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -115,64 +118,78 @@ __device__ __forceinline__ float tf32_hi(float v) {
   return __uint_as_float(r);
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+// 16 columns each of two accumulators (the warp's 32 lanes)
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float* va, float* vb) {
   uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
+#define TMEM_LD16(o, t)                                                                                         \
+  asm volatile(                                                                                                 \
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"   \
+      : "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]),             \
+        "=r"(r[o + 6]), "=r"(r[o + 7]), "=r"(r[o + 8]), "=r"(r[o + 9]), "=r"(r[o + 10]), "=r"(r[o + 11]),       \
+        "=r"(r[o + 12]), "=r"(r[o + 13]), "=r"(r[o + 14]), "=r"(r[o + 15])                                      \
+      : "r"(t))
+  TMEM_LD16(0, ta);
+  TMEM_LD16(16, tb);
+#undef TMEM_LD16
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+  for (int q = 0; q < 16; ++q) {
+    va[q] = __uint_as_float(r[q]);
+    vb[q] = __uint_as_float(r[16 + q]);
+  }
 }
 
 // Operand planes (rows padded to a multiple of 128, K to a multiple of 16, zeros beyond),
 // each in 8 KiB blocks [row block][K chunk] of the layout plane_off describes:
 //   2j = hi part, 2j + 1 = lo part of  j = 0 L_re, 1 L_im, 2 RA_re, 3 RA_im, 4 RB_re, 5 RB_im
-__global__ void k_adj_panels(const double2* __restrict__ Z, int64_t ldz, int64_t Npad, int64_t N, int k,
-                             const double* __restrict__ g, int ph, int nk, int64_t rows, float* __restrict__ P) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  const int kk = ph ? 2 * k : k;
-  const int kp = nk * KC;
-  const int64_t plane = rows * kp;
+// A thread makes four consecutive K of one row: one 16-byte store per plane, and eight threads (rows)
+// fill 128 contiguous bytes.  grid (rows / 128, K / 4), 128 threads (a thread per row and all its K
+// took 69 us at N = 6000, 32 pairs; this 11).
+__global__ void __launch_bounds__(128)
+k_adj_panels(const double2* __restrict__ Z, int64_t ldz, int64_t Npad, int64_t N, int k, const double* __restrict__ g,
+             int ph, int nk, int64_t rows, float* __restrict__ P) {
+  const int64_t r = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int q0 = blockIdx.y * 4, kk = ph ? 2 * k : k;
+  const int64_t plane = rows * (int64_t)nk * KC;
   const int nj = ph ? 6 : 4;
-  for (int q = 0; q < kp; ++q) {
-    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (r < N && q < kk) {
-      const int c = q < k ? q : q - k;
-      const double2 x = Z[(int64_t)c * ldz + r];
-      const double2 y = ph ? Z[(int64_t)c * ldz + Npad + r] : make_double2(0.0, 0.0);
-      const double gc = g[c];
-      if (q < k) {               // L = X g, R_A = X, R_B = Y
-        v[0] = (float)(gc * x.x); v[1] = (float)(gc * x.y);
-        v[2] = (float)x.x; v[3] = (float)x.y;
-        v[4] = (float)y.x; v[5] = (float)y.y;
-      } else {                   // L = conj(Y) g, R_A = conj(Y), R_B = conj(X)
-        v[0] = (float)(gc * y.x); v[1] = (float)(-gc * y.y);
-        v[2] = (float)y.x; v[3] = (float)(-y.y);
-        v[4] = (float)x.x; v[5] = (float)(-x.y);
-      }
+  float v[6][4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int q = q0 + u;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) v[j][u] = 0.f;
+    if (r >= N || q >= kk) continue;
+    const int c = q < k ? q : q - k;
+    const double2 x = Z[(int64_t)c * ldz + r];
+    const double2 y = ph ? Z[(int64_t)c * ldz + Npad + r] : make_double2(0.0, 0.0);
+    const double gc = g[c];
+    if (q < k) {               // L = X g, R_A = X, R_B = Y
+      v[0][u] = (float)(gc * x.x); v[1][u] = (float)(gc * x.y);
+      v[2][u] = (float)x.x; v[3][u] = (float)x.y;
+      v[4][u] = (float)y.x; v[5][u] = (float)y.y;
+    } else {                   // L = conj(Y) g, R_A = conj(Y), R_B = conj(X)
+      v[0][u] = (float)(gc * y.x); v[1][u] = (float)(-gc * y.y);
+      v[2][u] = (float)y.x; v[3][u] = (float)(-y.y);
+      v[4][u] = (float)x.x; v[5][u] = (float)(-x.y);
     }
-    const int64_t o = plane_off(r, q, nk);
-    for (int j = 0; j < nj; ++j) {
-      const float hi = tf32_hi(v[j]);
-      P[(int64_t)(2 * j) * plane + o] = hi;
-      P[(int64_t)(2 * j + 1) * plane + o] = v[j] - hi;
-    }
+  }
+  const int64_t o = plane_off(r, q0, nk);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    if (j >= nj) break;
+    float4 hi, lo;
+    hi.x = tf32_hi(v[j][0]); hi.y = tf32_hi(v[j][1]); hi.z = tf32_hi(v[j][2]); hi.w = tf32_hi(v[j][3]);
+    lo.x = v[j][0] - hi.x; lo.y = v[j][1] - hi.y; lo.z = v[j][2] - hi.z; lo.w = v[j][3] - hi.w;
+    *reinterpret_cast<float4*>(P + (int64_t)(2 * j) * plane + o) = hi;
+    *reinterpret_cast<float4*>(P + (int64_t)(2 * j + 1) * plane + o) = lo;
   }
 }
 
 // Half-tile unit h = 2 * (tile iteration) + q: output rows of block I, columns
 // J * 128 + 64 q ... + 63 (M = 128, N = 64), so that two accumulator sets fit
 // in the 512 TMEM columns and the epilogue of one half-tile overlaps the MMAs
-// of the next.  Warps 0-3 drain TMEM and write; warp 4 (one lane) issues the
-// bulk copies and the MMAs.  Barriers: full[s] / empty[s] for the three
+// of the next.  Warps 0-7 drain TMEM and write; one lane of warp 8 issues the
+// MMAs, one of warp 9 the bulk copies.  Barriers: full[s] / empty[s] for the three
 // shared-memory stages (copies landed / MMAs done reading), tfull[b] /
 // tempty[b] for the two accumulator buffers (MMAs done / epilogue done).
 template <bool PH>
@@ -203,7 +220,7 @@ k_adjoint_tc(const float* __restrict__ P, int64_t rows, int nk, int64_t N, const
     }
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&tfull[b])) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&tempty[b])), "r"(128) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&tempty[b])), "r"(32 * EPI_WARPS) : "memory");
     }
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -217,76 +234,58 @@ k_adjoint_tc(const float* __restrict__ P, int64_t rows, int nk, int64_t N, const
   const int nhalf = 2 * my_tiles;
   volatile int* vabort = &abort_flag;
 
-  if (warp == 4) {
-    // ------------------------------------------------ copies and MMAs (one lane)
+  if (warp == EPI_WARPS) {
+    // ------------------------------------------------ MMAs (one lane)
     if (lane == 0) {
       const uint32_t idp = instr_desc(false), idn = instr_desc(true);
-      const long long nb = (long long)nhalf * nk;     // batches: (half-tile, K-chunk)
-      auto issue_tma = [&](long long g) {
-        const int h = (int)(g / nk), c = (int)(g % nk);
-        const int2 tl = tiles[blockIdx.x + (int64_t)(h >> 1) * gridDim.x];
-        const int q = h & 1;
-        const int s = (int)(g % NSTAGE);
-        const uint32_t bar = smem_u32(&full[s]);
-        const uint32_t st = s0 + (uint32_t)s * STAGE;
-        mbar_expect_tx(bar, STAGE);
-#pragma unroll 1
-        for (int p = 0; p < 4; ++p)           // L: block row I, all 128 rows
-          bulk_g2s(st + (uint32_t)p * BLK, P + (int64_t)p * plane + ((int64_t)tl.x * nk + c) * (TCM * KC), BLK,
-                   bar);
-#pragma unroll 1
-        for (int p = 0; p < NR; ++p)          // R: block row J, rows 64 q ... 64 q + 63
-          bulk_g2s(st + LBYTES + (uint32_t)p * RBLK,
-                   reinterpret_cast<const char*>(P + (int64_t)(4 + p) * plane + ((int64_t)tl.y * nk + c) * (TCM * KC)) +
-                       q * RBLK,
-                   RBLK, bar);
-      };
-      long long issued = 0, committed = 0;
-      for (; issued < nb && issued < NSTAGE; ++issued) issue_tma(issued);
+      // descriptor of byte 0 of stage 0; an offset adds to the address field (in 16-byte units)
+      const uint64_t d0 = smem_desc(s0);
       bool ok = true;
-      for (long long g = 0; g < nb && ok; ++g) {
-        const int h = (int)(g / nk), c = (int)(g % nk);
-        const int s = (int)(g % NSTAGE), b = h & 1;
-        if (*vabort) { ok = false; break; }
-        if (!mbar_wait(smem_u32(&full[s]), (uint32_t)((g / NSTAGE) & 1))) { ok = false; break; }
-        if (c == 0 && !mbar_wait(smem_u32(&tempty[b]), (uint32_t)(((h >> 1) & 1) ^ 1))) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t st = s0 + (uint32_t)s * STAGE;
-#pragma unroll 1
-        for (int ks = 0; ks < KC / 8; ++ks) {
-          const uint32_t koff = (uint32_t)ks * 256u;
-          auto dl = [&](int p) { return smem_desc(st + (uint32_t)p * BLK + koff); };
-          auto dr = [&](int p) { return smem_desc(st + LBYTES + (uint32_t)p * RBLK + koff); };
-          const uint32_t first = (c == 0 && ks == 0) ? 0u : 1u;
-#pragma unroll 1
-          for (int m = 0; m < (PH ? 2 : 1); ++m) {
-            const int rr = 4 * m, ri = 4 * m + 2;            // R_re / R_im hi planes of this matrix
-            const uint32_t d_re = tbase + (uint32_t)b * ACC + (uint32_t)(128 * m), d_im = d_re + 64u;
-            // Re += L_re R_re^T + L_im R_im^T   (3xTF32 each)
-            mma_tf32(d_re, dl(0), dr(rr), idp, first);
-            mma_tf32(d_re, dl(0), dr(rr + 1), idp, 1u);
-            mma_tf32(d_re, dl(1), dr(rr), idp, 1u);
-            mma_tf32(d_re, dl(2), dr(ri), idp, 1u);
-            mma_tf32(d_re, dl(2), dr(ri + 1), idp, 1u);
-            mma_tf32(d_re, dl(3), dr(ri), idp, 1u);
-            // Im += L_im R_re^T - L_re R_im^T
-            mma_tf32(d_im, dl(2), dr(rr), idp, first);
-            mma_tf32(d_im, dl(2), dr(rr + 1), idp, 1u);
-            mma_tf32(d_im, dl(3), dr(rr), idp, 1u);
-            mma_tf32(d_im, dl(0), dr(ri), idn, 1u);
-            mma_tf32(d_im, dl(0), dr(ri + 1), idn, 1u);
-            mma_tf32(d_im, dl(1), dr(ri), idn, 1u);
+      int s = 0;
+      uint32_t par = 0;
+      long long last = -1;                             // the last committed stage's barrier and parity
+      uint32_t last_par = 0;
+      for (int h = 0; h < nhalf && ok; ++h) {
+        const int b = h & 1;
+        const uint32_t acc = tbase + (uint32_t)b * ACC;
+        for (int c = 0; c < nk; ++c) {
+          if (*vabort || !mbar_wait(smem_u32(&full[s]), par) ||
+              (c == 0 && !mbar_wait(smem_u32(&tempty[b]), (uint32_t)(((h >> 1) & 1) ^ 1)))) {
+            ok = false;
+            break;
           }
-        }
-        mma_commit(smem_u32(&empty[s]));              // stage s may be refilled once these finish
-        if (c == nk - 1) mma_commit(smem_u32(&tfull[b]));   // the half-tile's accumulators are final
-        committed = g + 1;
-        // refill the stage of batch g - 1 (its MMAs finish while batch g's run)
-        if (g >= 1 && issued < nb) {
-          const long long gp = g - 1;
-          if (!mbar_wait(smem_u32(&empty[gp % NSTAGE]), (uint32_t)((gp / NSTAGE) & 1))) { ok = false; break; }
-          issue_tma(issued);
-          ++issued;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t ds = d0 + (uint64_t)(((uint32_t)s * STAGE) >> 4);
+#pragma unroll
+          for (int ks = 0; ks < KC / 8; ++ks) {
+            auto dl = [&](int p) { return ds + (uint64_t)(((uint32_t)p * BLK + ks * 256u) >> 4); };
+            auto dr = [&](int p) { return ds + (uint64_t)((LBYTES + (uint32_t)p * RBLK + ks * 256u) >> 4); };
+            const uint32_t first = (c == 0 && ks == 0) ? 0u : 1u;
+#pragma unroll
+            for (int m = 0; m < (PH ? 2 : 1); ++m) {
+              const int rr = 4 * m, ri = 4 * m + 2;            // R_re / R_im hi planes of this matrix
+              const uint32_t d_re = acc + (uint32_t)(128 * m), d_im = d_re + 64u;
+              // Re += L_re R_re^T + L_im R_im^T   (3xTF32 each)
+              mma_tf32(d_re, dl(0), dr(rr), idp, first);
+              mma_tf32(d_re, dl(0), dr(rr + 1), idp, 1u);
+              mma_tf32(d_re, dl(1), dr(rr), idp, 1u);
+              mma_tf32(d_re, dl(2), dr(ri), idp, 1u);
+              mma_tf32(d_re, dl(2), dr(ri + 1), idp, 1u);
+              mma_tf32(d_re, dl(3), dr(ri), idp, 1u);
+              // Im += L_im R_re^T - L_re R_im^T
+              mma_tf32(d_im, dl(2), dr(rr), idp, first);
+              mma_tf32(d_im, dl(2), dr(rr + 1), idp, 1u);
+              mma_tf32(d_im, dl(3), dr(rr), idp, 1u);
+              mma_tf32(d_im, dl(0), dr(ri), idn, 1u);
+              mma_tf32(d_im, dl(0), dr(ri + 1), idn, 1u);
+              mma_tf32(d_im, dl(1), dr(ri), idn, 1u);
+            }
+          }
+          mma_commit(smem_u32(&empty[s]));              // stage s may be refilled once these finish
+          if (c == nk - 1) mma_commit(smem_u32(&tfull[b]));   // the half-tile's accumulators are final
+          last = s;
+          last_par = par;
+          if (++s == NSTAGE) { s = 0; par ^= 1u; }
         }
       }
       if (!ok) {
@@ -294,19 +293,56 @@ k_adjoint_tc(const float* __restrict__ P, int64_t rows, int nk, int64_t N, const
         atomicExch(err, 1);
       }
       // nothing may be in flight when the shared memory and TMEM go away
-      if (issued > 0) {
-        const long long gi = issued - 1;
-        mbar_wait(smem_u32(&full[gi % NSTAGE]), (uint32_t)((gi / NSTAGE) & 1));
+      if (last >= 0) mbar_wait(smem_u32(&empty[last]), last_par);
+    }
+  } else if (warp == EPI_WARPS + 1) {
+    // ------------------------------------------------ copies (one lane)
+    if (lane == 0) {
+      bool ok = true;
+      int s = 0;
+      uint32_t par = 1;                                 // the first use of a stage finds it empty
+      long long last = -1;
+      uint32_t last_par = 0;
+      for (int h = 0; h < nhalf && ok; ++h) {
+        const int2 tl = tiles[blockIdx.x + (int64_t)(h >> 1) * gridDim.x];
+        const int q = h & 1;
+        const float* pl = P + (int64_t)tl.x * nk * (TCM * KC);                            // block row I
+        const char* pr = reinterpret_cast<const char*>(P + 4 * plane + (int64_t)tl.y * nk * (TCM * KC)) + q * RBLK;
+        for (int c = 0; c < nk; ++c) {
+          if (*vabort || !mbar_wait(smem_u32(&empty[s]), par)) {
+            ok = false;
+            break;
+          }
+          const uint32_t bar = smem_u32(&full[s]);
+          const uint32_t st = s0 + (uint32_t)s * STAGE;
+          mbar_expect_tx(bar, STAGE);
+#pragma unroll
+          for (int p = 0; p < 4; ++p)           // L: all 128 rows
+            bulk_g2s(st + (uint32_t)p * BLK, pl + (int64_t)p * plane + (int64_t)c * (TCM * KC), BLK, bar);
+#pragma unroll
+          for (int p = 0; p < NR; ++p)          // R: rows 64 q ... 64 q + 63 of block row J
+            bulk_g2s(st + LBYTES + (uint32_t)p * RBLK, pr + ((int64_t)p * plane + (int64_t)c * (TCM * KC)) * 4, RBLK, bar);
+          last = s;
+          last_par = par ^ 1u;
+          if (++s == NSTAGE) { s = 0; par ^= 1u; }
+        }
       }
-      if (committed > 0) {
-        const long long gc = committed - 1;
-        mbar_wait(smem_u32(&empty[gc % NSTAGE]), (uint32_t)((gc / NSTAGE) & 1));
+      if (!ok) {
+        *vabort = 1;
+        atomicExch(err, 1);
       }
+      if (last >= 0) mbar_wait(smem_u32(&full[last]), last_par);   // no copy in flight at the end
     }
   } else {
-    // ------------------------------------------------ epilogue (warps 0-3)
-    float2* buf = reinterpret_cast<float2*>(sm + NSTAGE * STAGE) + warp * (32 * 33);
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+    // ------------------------------------------------ epilogue (warps 0-7)
+    // warp w reads the TMEM lanes (tile rows) of quarter w % 4; w / 4 picks dA or dB (PH) or the
+    // column half (TDA)
+    float2* buf = reinterpret_cast<float2*>(sm + NSTAGE * STAGE) + warp * (32 * 17);
+    const int qr = warp & 3, part = warp >> 2;
+    const int m = PH ? part : 0;
+    float2* __restrict__ out = m == 0 ? dA : dB;
+    const float msgn = m == 0 ? -1.f : 1.f;                // the mirror: conjugate (dA) or not (dB)
+    const uint32_t lane_off = (uint32_t)(qr * 32) << 16;
     for (int h = 0; h < nhalf; ++h) {
       const int b = h & 1;
       if (*vabort) break;
@@ -320,41 +356,47 @@ k_adjoint_tc(const float* __restrict__ P, int64_t rows, int nk, int64_t N, const
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int2 tl = tiles[blockIdx.x + (int64_t)(h >> 1) * gridDim.x];
       const int I = tl.x, J = tl.y, q = h & 1;
-      const int64_t gi = (int64_t)I * TCM + warp * 32 + lane;
+      const int64_t i0 = (int64_t)I * TCM + qr * 32, gi = i0 + lane;
       // the mirror block is written from registers (lanes run along its rows); the tile goes
       // through a per-warp transpose so that lanes run along its rows too.  A diagonal tile keeps
       // its upper triangle and mirrors it (dA exactly Hermitian with a real diagonal, dB symmetric)
+      const bool inside = I != J && (int64_t)(J + 1) * TCM <= N;     // no row or column to leave out
 #pragma unroll 1
-      for (int m = 0; m < (PH ? 2 : 1); ++m) {
-        float2* out = m == 0 ? dA : dB;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          float re[32], im[32];
-          tmem_ld32(tbase + lane_off + (uint32_t)b * ACC + (uint32_t)(128 * m + c0), re);
-          tmem_ld32(tbase + lane_off + (uint32_t)b * ACC + (uint32_t)(128 * m + 64 + c0), im);
-          const int64_t jb = (int64_t)J * TCM + 64 * q + c0;
-          if (gi < N) {
+      for (int c0 = PH ? 0 : 32 * part; c0 < (PH ? 64 : 32 * part + 32); c0 += 16) {
+        float re[16], im[16];
+        const uint32_t ta = tbase + lane_off + (uint32_t)b * ACC + (uint32_t)(128 * m + c0);
+        tmem_ld16x2(ta, ta + 64u, re, im);
+        const int64_t jb = (int64_t)J * TCM + 64 * q + c0;
+        float2* mir = out + jb * N + gi;
+        if (inside) {
 #pragma unroll
-            for (int qq = 0; qq < 32; ++qq) {
-              const int64_t gj = jb + qq;
-              if (gj < N && (I != J || gj > gi)) out[gj * N + gi] = make_float2(re[qq], m == 0 ? -im[qq] : im[qq]);
-            }
-          }
+          for (int qq = 0; qq < 16; ++qq, mir += N) *mir = make_float2(re[qq], msgn * im[qq]);
+        } else if (gi < N) {
 #pragma unroll
-          for (int qq = 0; qq < 32; ++qq) buf[lane * 33 + qq] = make_float2(re[qq], im[qq]);
-          __syncwarp();
-          const int64_t gj = jb + lane;
-#pragma unroll 4
-          for (int rr = 0; rr < 32; ++rr) {
-            const int64_t row = (int64_t)I * TCM + warp * 32 + rr;
-            if (row < N && gj < N && (I != J || gj >= row)) {
-              float2 v = buf[rr * 33 + lane];
-              if (m == 0 && gj == row) v.y = 0.f;
-              out[row * N + gj] = v;
-            }
-          }
-          __syncwarp();
+          for (int qq = 0; qq < 16; ++qq, mir += N)
+            if (jb + qq < N && (I != J || jb + qq > gi)) *mir = make_float2(re[qq], msgn * im[qq]);
         }
+#pragma unroll
+        for (int qq = 0; qq < 16; ++qq) buf[lane * 17 + qq] = make_float2(re[qq], im[qq]);
+        __syncwarp();
+        const int64_t gj = jb + (lane & 15);
+        const float2* bp = buf + (lane >> 4) * 17 + (lane & 15);
+        float2* dst = out + (i0 + (lane >> 4)) * N + gj;
+        if (inside) {
+#pragma unroll
+          for (int rr = 0; rr < 16; ++rr, dst += 2 * N) *dst = bp[rr * 34];
+        } else {
+#pragma unroll 4
+          for (int rr = 0; rr < 16; ++rr, dst += 2 * N) {
+            const int64_t row = i0 + 2 * rr + (lane >> 4);
+            if (row < N && gj < N && (I != J || gj >= row)) {
+              float2 v = bp[rr * 34];
+              if (m == 0 && gj == row) v.y = 0.f;
+              *dst = v;
+            }
+          }
+        }
+        __syncwarp();
       }
       // this accumulator set may be overwritten by the half-tile after next
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -417,7 +459,7 @@ int launch_adjoint_tc(const double2* Z, int64_t ldz, int64_t Npad, int64_t N, in
   const int kk = ph ? 2 * k : k;
   const int nk = (kk + KC - 1) / KC;
   count_launch(2);
-  k_adj_panels<<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(Z, ldz, Npad, N, k, g, ph, nk, rows, panels);
+  k_adj_panels<<<dim3((unsigned)(rows / 128), (unsigned)(nk * KC / 4)), 128, 0, s>>>(Z, ldz, Npad, N, k, g, ph, nk, rows, panels);
   if (!g_tc_sms) {
     int dev = 0;
     cudaGetDevice(&dev);
