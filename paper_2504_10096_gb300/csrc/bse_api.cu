@@ -65,16 +65,13 @@ struct ProbHost {
 struct StepGraph {
   cudaGraphExec_t exec = nullptr;
   long long launches = 0;            // kernels per replay
-  std::vector<cudaEvent_t> ev;       // product start/stop pairs recorded by the graph
-  bool pending = false;              // replayed since the events were last read
 };
 
 constexpr int kMaxGraphLog = 10;     // 2^10 = MAXM steps
 
 // Launch-shape tuner of the structured product.  While a handle is untuned,
 // its successive products (the solver's own, no extra work) cycle through
-// the candidate shapes; each product is timed by the CUDA events that also
-// feed bse_stats.  Once every candidate has kTuneSamples timings after its
+// the candidate shapes; each product is timed by CUDA events.  Once every candidate has kTuneSamples timings after its
 // first one, the shape with the lowest mean is kept for the handle and, keyed
 // by kernel variant, tile-job count and problem count, for later handles.
 constexpr int kTuneSamples = 3;
@@ -137,10 +134,10 @@ struct bse_handle {
   int* adj_err = nullptr;
   int* prod_err = nullptr;   // raised by a product kernel whose bounded wait expired
   double* gdev = nullptr;
-  // product timing ring
+  // the tuner's product timings, and the device clock of the products (bse_stats.ms_product)
   std::vector<cudaEvent_t> ev;
   int ev_used = 0;
-  double ms_product = 0.0;
+  ProdClock* clock = nullptr;
   // product launch shape and its tuner state
   ProdShape shape{0, 0};
   bool tuned = false;
@@ -292,31 +289,19 @@ struct Driver {
   using R = typename std::conditional<std::is_same<ST, float2>::value, float, double>::type;
   bse_handle* h;
   cudaStream_t s;                          // the handle's stream, or the capture stream
-  std::vector<cudaEvent_t>* cap_ev = nullptr;   // events of the graph being captured
-  size_t cap_n = 0;
+  bool capturing = false;
   explicit Driver(bse_handle* hh) : h(hh), s(hh->stream) {}
 
   void product(int mode) {
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaEvent_t e1 = nullptr;
     ProdShape shape = h->shape;
-    int tag = -1;
-    if (!h->tuned && !cap_ev && !h->cands.empty()) {
-      tag = h->tnext++ % (int)h->cands.size();
+    if (!h->tuned && !capturing && !h->cands.empty() && h->ev_used + 2 <= (int)h->ev.size()) {
+      const int tag = h->tnext++ % (int)h->cands.size();   // the tuner times this one
       shape = h->cands[tag];
-    }
-    if (cap_ev) {
-      if (cap_n + 2 <= cap_ev->size()) {
-        e0 = (*cap_ev)[cap_n];
-        e1 = (*cap_ev)[cap_n + 1];
-        cap_n += 2;
-        cudaEventRecordWithFlags(e0, s, cudaEventRecordExternal);
-      }
-    } else if (h->ev_used + 2 <= (int)h->ev.size()) {
-      e0 = h->ev[h->ev_used];
       e1 = h->ev[h->ev_used + 1];
       h->ev_tag[h->ev_used / 2] = tag;
+      cudaEventRecord(h->ev[h->ev_used], s);
       h->ev_used += 2;
-      cudaEventRecord(e0, s);
     }
     if (h->mixed)
       launch_product_mixed(h->dprobs, h->djobs_fine, h->njobs_fine, h->djobs_coarse, h->njobs_coarse, h->count,
@@ -330,26 +315,13 @@ struct Driver {
     else
       launch_product<ST, R>(h->dprobs, h->djobs, h->njobs, h->count, h->maxnT, mode, 1, nullptr, h->ph != 0,
                             shape, s);
-    if (e1) {
-      if (cap_ev) cudaEventRecordWithFlags(e1, s, cudaEventRecordExternal);
-      else cudaEventRecord(e1, s);
-    }
-  }
-
-  static double elapsed(const std::vector<cudaEvent_t>& ev, size_t n) {
-    double sum = 0.0;
-    for (size_t i = 0; i + 1 < n; i += 2) {
-      float ms = 0.f;
-      if (cudaEventElapsedTime(&ms, ev[i], ev[i + 1]) == cudaSuccess) sum += ms;
-    }
-    return sum;
+    if (e1) cudaEventRecord(e1, s);
   }
 
   void harvest_events() {
     for (int i = 0; i + 1 < h->ev_used; i += 2) {
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, h->ev[i], h->ev[i + 1]) != cudaSuccess) continue;
-      h->ms_product += ms;
       const int tag = h->ev_tag[i / 2];
       if (tag >= 0 && !h->tuned && h->tseen[tag]++ > 0) {   // the first timing of a shape is a warm-up
         h->tsum[tag] += ms;
@@ -366,11 +338,6 @@ struct Driver {
       h->tuned = true;
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tuned[h->tkey] = h->shape;
-    }
-    for (StepGraph& g : h->sg) {
-      if (!g.pending) continue;
-      h->ms_product += elapsed(g.ev, g.ev.size());
-      g.pending = false;
     }
   }
 
@@ -411,12 +378,6 @@ struct Driver {
   bool capture(int b) {
     StepGraph& g = h->sg[b];
     const int n = 1 << b;
-    const size_t nev = (size_t)(h->ph ? 4 : 2) * n;
-    while (g.ev.size() < nev) {
-      cudaEvent_t e;
-      if (cudaEventCreate(&e) != cudaSuccess) { cudaGetLastError(); h->graphs = false; return false; }
-      g.ev.push_back(e);
-    }
     if (!h->cap && cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) {
       cudaGetLastError();
       h->cap = nullptr;
@@ -430,11 +391,10 @@ struct Driver {
     }
     const long long c0 = launch_counter();
     s = h->cap;
-    cap_ev = &g.ev;
-    cap_n = 0;
+    capturing = true;
     for (int i = 0; i < n; ++i) step();
     s = h->stream;
-    cap_ev = nullptr;
+    capturing = false;
     g.launches = launch_counter() - c0;
     launch_counter() = c0;                  // counted again at every replay
     cudaGraph_t graph = nullptr;
@@ -451,8 +411,7 @@ struct Driver {
   }
 
   // `steps` Krylov steps: graphs of 2^b steps for the binary digits of
-  // `steps` (each replayed at most once per cycle, so every event pair of a
-  // replay is read before it is recorded again), or plain launches
+  // `steps`, or plain launches
   int run_steps(int steps) {
     if (!h->tuned) {                       // shapes still being compared: one launch at a time
       for (; steps > 0; --steps) step();
@@ -474,7 +433,6 @@ struct Driver {
       StepGraph& g = h->sg[b];
       if (h->graphs && (g.exec || capture(b)) && cudaGraphLaunch(g.exec, h->stream) == cudaSuccess) {
         launch_counter() += g.launches;
-        g.pending = true;
       } else {
         cudaGetLastError();
         for (int i = 0; i < n; ++i) step();
@@ -563,7 +521,6 @@ struct Driver {
     for (StepGraph& g : h->sg) {
       if (g.exec) cudaGraphExecDestroy(g.exec);
       g.exec = nullptr;
-      g.pending = false;
     }
     if (h->rg.exec) cudaGraphExecDestroy(h->rg.exec);
     h->rg.exec = nullptr;
@@ -847,6 +804,7 @@ int upload_probs(bse_handle* h) {
     d.Afx = q.Afx; d.Bfx = q.Bfx; d.texp = q.texp;
     d.nq = h->nq;
     d.err = h->prod_err;
+    d.clock = h->clock;
   }
   CK(cudaMemcpyAsync(h->dprobs, h->hprobs.data(), sizeof(Prob) * h->count, cudaMemcpyHostToDevice,
                      h->stream));
@@ -998,12 +956,12 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
                      h->stream));
   if ((rc = upload_probs(h))) return rc;
   if (h->ev.empty()) {
-    h->ev.resize(4 * MAXM + 8);
+    h->ev.resize(128);               // for the tuner: a few products per candidate
     for (auto& e : h->ev) cudaEventCreate(&e);
     h->ev_tag.assign(h->ev.size() / 2, -1);
   }
   h->ev_used = 0;
-  h->ms_product = 0.0;
+  CK(cudaMemsetAsync(h->clock, 0, sizeof(ProdClock), h->stream));
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -1039,7 +997,9 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
     if (st == BSE_ENOTPD || st == BSE_ENOTFINITE) worst = st;
   }
   cudaEventRecord(e1, h->stream);
-  cudaEventSynchronize(e1);
+  ProdClock pc{};
+  cudaMemcpyAsync(&pc, h->clock, sizeof(ProdClock), cudaMemcpyDeviceToHost, h->stream);
+  cudaStreamSynchronize(h->stream);
   float ms = 0.f;
   cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
@@ -1051,7 +1011,7 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
   h->stats.nconv = nconv_total;
   h->stats.max_residual = maxres;
   h->stats.ms_total = ms;
-  h->stats.ms_product = h->ms_product;
+  h->stats.ms_product = 1e-6 * (double)(pc.sum + (pc.end > pc.start ? pc.end - pc.start : 0));
   h->stats.launches = launch_counter() - launches0;
   h->stats.shape_ctas_per_sm = h->shape.ctas_per_sm;
   h->stats.shape_strided = h->shape.strided;
@@ -1595,6 +1555,8 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
     rc = BSE_ECUDA;
   if (rc == BSE_OK) rc = dalloc((void**)&h->dprobs, sizeof(Prob) * count);
   if (rc == BSE_OK) rc = dalloc((void**)&h->dstate, sizeof(KState) * count);
+  if (rc == BSE_OK) rc = dalloc((void**)&h->clock, sizeof(ProdClock));
+  if (rc == BSE_OK && cudaMemsetAsync(h->clock, 0, sizeof(ProdClock), h->stream) != cudaSuccess) rc = BSE_ECUDA;
   if (rc == BSE_OK && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = BSE_ECUDA;
   if (rc == BSE_OK) setup_tuner(h);
   if (rc != BSE_OK) {
@@ -1800,6 +1762,7 @@ int bse_destroy(bse_handle* h) {
   dfreet(h->prod_err);
   dfreet(h->dprobs);
   dfreet(h->dstate);
+  dfreet(h->clock);
   dfreet(h->djobs);
   dfree(h->post);
   dfree(h->blk);
@@ -1814,7 +1777,6 @@ int bse_destroy(bse_handle* h) {
   for (auto& e : h->ev) cudaEventDestroy(e);
   for (StepGraph& g : h->sg) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
-    for (auto& e : g.ev) cudaEventDestroy(e);
   }
   if (h->rg.exec) cudaGraphExecDestroy(h->rg.exec);
   if (h->cap) cudaStreamDestroy(h->cap);

@@ -108,6 +108,8 @@ __device__ __forceinline__ bool restart_ready(const KState* st) {
 // dense structure-preserving method of Sec. 2.1.1.
 enum Variant : int { VAR_SHAO = 0, VAR_GRUNING = 1, VAR_PROJECTED = 2 };
 
+struct ProdClock;
+
 // Static description of one problem (device resident, read-only in kernels).
 struct Prob {
   int64_t N;
@@ -177,6 +179,7 @@ struct Prob {
   const int* texp;
   int nq;
   int* err;           // raised by a product kernel whose bounded wait expired
+  ProdClock* clock;   // of the handle
 };
 
 // Jobs of the tiled product: problem, tile row I, tile column J, tile index.
@@ -198,6 +201,55 @@ struct GenericIO {     // explicit operands for PM_GENERIC (single problem)
   double sB;           // sign of the B term (0 disables it)
   void* y; int ldy;    // output (compute type) Npad x K
 };
+
+// Programmatic dependent launch.  The kernels of a Krylov step are short (3 to 50 us), so the time
+// between one's end and the next one's start counts: a kernel launched with launch_dep may be set up
+// while its predecessor still runs.  Every such kernel calls dep_begin() first: it waits until
+// the predecessor has completed and its writes are visible, then lets its own dependent start.  (Data
+// that a predecessor writes is never read through the non-coherent path.)
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_begin() {
+  dep_wait();
+  dep_launch();
+}
+
+template <typename... KA, typename... A>
+inline void launch_dep(void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, KA(a)...);
+}
+
+// Device time inside the products of a handle's solves, by the device's own clock (event records
+// between the kernels would keep them from overlapping): the first kernel of a product stamps its
+// start and books the previous one, every CTA of the closing reduction moves the end.
+struct ProdClock {
+  unsigned long long start, end, sum;   // nanoseconds
+};
+__device__ __forceinline__ unsigned long long dev_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ void clock_start(ProdClock* c) {
+  if (!c || threadIdx.x || blockIdx.x || blockIdx.y) return;
+  const unsigned long long t = dev_ns(), e = c->end, b = c->start;
+  if (e > b) c->sum += e - b;
+  c->end = 0;
+  c->start = t;
+}
+__device__ __forceinline__ void clock_end(ProdClock* c) {
+  if (c && threadIdx.x == 0) atomicMax(&c->end, dev_ns());
+}
 
 // Kernel launches issued by this process (reported per solve in bse_stats).
 inline long long& launch_counter() {
@@ -273,7 +325,7 @@ int fx_bands(int ntiles);      // bands per tile for a handle of that many tiles
 void launch_prod_reduce_f64(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s);
 // the FP64 tile kernel alone (k_product.cu)
 void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, GenericIO io, bool hasB,
-                      ProdShape shape, cudaStream_t s);
+                      ProdShape shape, int first, cudaStream_t s);
 int num_sms();
 
 // blocks of columns in FP64 accuracy with fixed-point tiles (k_block_fx.cu): Y = A XA + sB B XB

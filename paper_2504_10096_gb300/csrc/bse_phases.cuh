@@ -5,7 +5,7 @@
 // the phases separated by a grid barrier).  A body computes the same bits in either setting:
 // it takes its work unit and shared memory as arguments and keeps the summation order of the
 // unit fixed.  Loads of data that a persistent launch rewrites between its phases (the Krylov
-// basis, the work vectors, the partial sums) go through ldv / ldp<COH>: L2 loads (ordered by
+// basis, the work vectors, the partial sums) go through ldv / ldv<COH>: L2 loads (ordered by
 // the barrier's fences, and never served from a stale L1 line) when COH.
 #pragma once
 
@@ -18,15 +18,8 @@ namespace bse {
 template <bool COH, typename T>
 __device__ __forceinline__ T ldv(const T* p) {
   if constexpr (COH) return __ldcg(p);
-  else return __ldg(p);
-}
-// the same for loads that take the ordinary path outside a persistent launch
-template <bool COH, typename T>
-__device__ __forceinline__ T ldp(const T* p) {
-  if constexpr (COH) return __ldcg(p);
   else return *p;
 }
-
 template <typename R> struct Acc;
 template <> struct Acc<float> { using T = float2; };
 template <> struct Acc<double> { using T = double2; };
@@ -155,8 +148,8 @@ __device__ __forceinline__ void prod_tiles_body(const Prob* __restrict__ probs, 
     if (!prod_operands<ST, R>(p, mode, io, x, yout, sB)) continue;   // uniform per CTA
     const bool diag = (jb.I == jb.J);
     __syncthreads();                       // smem of the previous tile is free
-    if (tid < TS) xc[tid] = ccvt<CT>(ldp<COH>(x + (int64_t)jb.J * TS + tid));
-    else xr[tid - TS] = ccvt<CT>(ldp<COH>(x + (int64_t)jb.I * TS + tid - TS));
+    if (tid < TS) xc[tid] = ccvt<CT>(ldv<COH>(x + (int64_t)jb.J * TS + tid));
+    else xr[tid - TS] = ccvt<CT>(ldv<COH>(x + (int64_t)jb.I * TS + tid - TS));
     __syncthreads();
     // PH: M_s u = A u + s B conj(u) is real-linear; in (Re, Im) form its block
     // row is [[U_re, -V_im], [U_im, V_re]] with U = A + s B, V = A - s B (the
@@ -307,18 +300,18 @@ __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs,
   for (; J + 3 * REDUCE_GROUPS < p.nT; J += 4 * REDUCE_GROUPS) {   // four loads in flight, then the sums
     CT v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = ldp<COH>(part + (int64_t)(J + k * REDUCE_GROUPS) * TS + r);
+    for (int k = 0; k < 4; ++k) v[k] = ldv<COH>(part + (int64_t)(J + k * REDUCE_GROUPS) * TS + r);
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc = cadd(acc, v[k]);
   }
-  for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, ldp<COH>(part + (int64_t)J * TS + r));
+  for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, ldv<COH>(part + (int64_t)J * TS + r));
   if constexpr (std::is_same<CT, double2>::value) {
     // fixed-point tiles: the column sums of a tile's further bands, planes 1 ... nq - 1
     const int nb = p.nq - 1;
     for (int k = g; k < nb * I; k += REDUCE_GROUPS) {
       const int q = 1 + k / I, Jq = k - (q - 1) * I;
       if (p.texp[(int64_t)Jq * p.nT - (int64_t)Jq * (Jq - 1) / 2 + (I - Jq)] < 0) continue;
-      acc = cadd(acc, ldp<COH>(part + ((int64_t)q * p.nT * p.nT + Jq) * TS + r));
+      acc = cadd(acc, ldv<COH>(part + ((int64_t)q * p.nT * p.nT + Jq) * TS + r));
     }
   }
   grp[g][lane] = acc;
@@ -332,7 +325,7 @@ __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs,
       const int64_t t = (int64_t)I * p.nT - (int64_t)I * (I - 1) / 2;
       if (p.nq > 0 && p.texp[t] >= 0) {
         const int64_t d = t * (TS * TS) + r * (TS + 1);
-        const CT xv = ldp<COH>((const CT*)x + row);
+        const CT xv = ldv<COH>((const CT*)x + row);
         const CT u = ((const CT*)(p.ph && sB < (R)0 ? p.B : p.A))[d];
         const CT v = p.ph ? ((const CT*)(sB < (R)0 ? p.A : p.B))[d] : u;
         acc.x = fma(u.x, xv.x, acc.x); acc.x = fma(-v.y, xv.y, acc.x);
@@ -342,7 +335,7 @@ __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs,
     const ST yv = ccvt<ST>(acc);
     y[row] = yv;
     if (prod_is_norm(mode)) {          // the squared norm's partial sum Re(w^H M w)
-      const double s = norm_term(ldp<COH>(x + row), yv);
+      const double s = norm_term(ldv<COH>(x + row), yv);
       const double t = warp_sum_d(s);
       if (lane == 0) p.npart[u] = t;
     }
@@ -423,12 +416,12 @@ __device__ __forceinline__ double2 cgs_coef(const Prob& p, int ph, int c, int nc
   if (ph) {
     double v[DOT_CHUNKS];
 #pragma unroll
-    for (int k = 0; k < DOT_CHUNKS; ++k) v[k] = k < nch ? ldp<COH>(p.cpart + (int64_t)k * p.ncol + c) : 0.0;
+    for (int k = 0; k < DOT_CHUNKS; ++k) v[k] = k < nch ? ldv<COH>(p.cpart + (int64_t)k * p.ncol + c) : 0.0;
     sc.x = v[0];
     for (int k = 1; k < nch; ++k) sc.x += v[k];
   } else {
     const double2* cp = (const double2*)p.cpart;
-    for (int k = 0; k < nch; ++k) sc = cadd(sc, ldp<COH>(cp + (int64_t)k * p.ncol + c));
+    for (int k = 0; k < nch; ++k) sc = cadd(sc, ldv<COH>(cp + (int64_t)k * p.ncol + c));
   }
   return sc;
 }
@@ -511,7 +504,7 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
     for (int m = 1; m < 8; m <<= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
     if ((v & 7) == 0) {
       const int64_t o = ((int64_t)bx * RS + r) * 2 + comp;
-      const R nw = ldp<COH>((const R*)x + o) - t;
+      const R nw = ldv<COH>((const R*)x + o) - t;
       ((R*)w)[o] = nw;
       nrm += (double)nw * (double)nw;
     }
@@ -552,7 +545,7 @@ template <bool COH>
 __device__ __forceinline__ double norm_sum(const Prob& p, int ph) {
   const int n = norm_parts(p, ph);
   double s = 0.0;
-  for (int i = threadIdx.x & 31; i < n; i += 32) s += ldp<COH>(p.npart + i);
+  for (int i = threadIdx.x & 31; i < n; i += 32) s += ldv<COH>(p.npart + i);
   return warp_sum_d(s);
 }
 
@@ -587,10 +580,10 @@ __device__ __forceinline__ void normalize_row(const Prob& p, const KState* st, i
                                               typename RealOf<ST>::T inv) {
   ST *X, *Y;
   norm_dest<ST>(p, st, half, X, Y);
-  const ST xv = cscale(ldp<COH>((const ST*)p.w + row), inv);
+  const ST xv = cscale(ldv<COH>((const ST*)p.w + row), inv);
   X[row] = xv;
   ST yv = czero<ST>();
-  if (ph) Y[row] = yv = cscale(ldp<COH>((const ST*)p.pw + row), inv);
+  if (ph) Y[row] = yv = cscale(ldv<COH>((const ST*)p.pw + row), inv);
   shadow_store<ST>(p, st, half, row, xv, yv);
 }
 
@@ -604,7 +597,7 @@ __device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh
   const int j = st->j;
   if (!fresh) {
     const double2* coef = (const double2*)p.coef;
-    const double a = ldp<COH>(&coef[j].x) + ldp<COH>(&coef[p.ncol + j].x);
+    const double a = ldv<COH>(&coef[j].x) + ldv<COH>(&coef[p.ncol + j].x);
     if (!isfinite(a) || !isfinite(b2)) { st->status = ST_NOTFINITE; return; }
     if (writer) p.alpha[j] = a;
     st->passes += ph ? 2 : 1;
@@ -612,7 +605,7 @@ __device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh
     // scale of the projected matrix for the breakdown test
     double scale = fabs(a);
     scale = fmax(scale, st->theta_scale);   // max |theta| of the kept Ritz values
-    if (j > 0) scale = fmax(scale, fabs(ldp<COH>(p.beta + j - 1)));
+    if (j > 0) scale = fmax(scale, fabs(ldv<COH>(p.beta + j - 1)));
     const double tiny = 1e-26 * scale * scale + 1e-300;
     if (ph && b2 < -1e6 * tiny) { st->status = ST_NOTPD; return; }
     if (b2 <= tiny) {                 // invariant subspace: the chain restarts

@@ -197,7 +197,7 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
     return u;
   };
   auto x_value = [&](const TileJob& jb) {
-    return ldp<COH>(x + (int64_t)(tid < TS ? jb.J : jb.I) * TS + (tid & (TS - 1)));
+    return ldv<COH>(x + (int64_t)(tid < TS ? jb.J : jb.I) * TS + (tid & (TS - 1)));
   };
   TileJob jb{}, jn{}, jp{};
   int un = next_unit(u0, jn);

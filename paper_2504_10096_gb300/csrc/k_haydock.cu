@@ -23,8 +23,8 @@ namespace {
 constexpr int HD_THREADS = 256;
 
 template <typename ST>
-__global__ void __launch_bounds__(HD_THREADS) k_hd_dot(const ST* __restrict__ x, const ST* __restrict__ y,
-                                                       int64_t n, double* __restrict__ partial) {
+__global__ void __launch_bounds__(HD_THREADS) k_hd_dot(const ST* x, const ST* y, int64_t n, double* partial) {
+  dep_begin();
   __shared__ double red[HD_THREADS / 32];
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -42,12 +42,16 @@ __global__ void __launch_bounds__(HD_THREADS) k_hd_dot(const ST* __restrict__ x,
   }
 }
 
-// which = 0: <d, d>_K (start); 1: alpha_j; 2: beta_j and the step advance
-__global__ void k_hd_scalar(HdState* __restrict__ st, const double* __restrict__ partial, int np,
-                            double* __restrict__ alpha, double* __restrict__ beta, int which) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// which = 0: <d, d>_K (start); 1: alpha_j; 2: beta_j and the step advance.  One warp: FP64 adds are
+// 64 clocks each, so a thread alone took 16 us over the 256 partial sums
+__global__ void __launch_bounds__(32) k_hd_scalar(HdState* st, const double* partial, int np, double* alpha, double* beta,
+                                                  int which) {
+  dep_begin();
   double s = 0.0;
-  for (int i = 0; i < np; ++i) s += partial[i];
+  for (int i = threadIdx.x; i < np; i += 32) s += partial[i];
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+  if (threadIdx.x != 0) return;
   if (which == 0) {
     st->n2 = s;
     st->j = 0;
@@ -75,9 +79,9 @@ __global__ void k_hd_scalar(HdState* __restrict__ st, const double* __restrict__
 
 // r = w - alpha_j q - beta_{j-1} q_prev
 template <typename ST>
-__global__ void k_hd_axpy(const HdState* __restrict__ st, const double* __restrict__ alpha,
-                          const double* __restrict__ beta, const ST* __restrict__ w, const ST* __restrict__ q,
-                          const ST* __restrict__ qprev, ST* __restrict__ r, int64_t n) {
+__global__ void k_hd_axpy(const HdState* st, const double* alpha, const double* beta, const ST* w, const ST* q,
+                          const ST* qprev, ST* r, int64_t n) {
+  dep_begin();
   if (st->done || st->j >= st->m) return;
   const int j = st->j;
   using R = decltype(w[0].x);
@@ -94,9 +98,9 @@ __global__ void k_hd_axpy(const HdState* __restrict__ st, const double* __restri
 // start (init = 1): q = r / sqrt(n2), p = pr / sqrt(n2), q_prev = 0;
 // step: q_prev = q, q = r / beta_{j-1}, p = pr / beta_{j-1} (j already advanced)
 template <typename ST>
-__global__ void k_hd_scale(const HdState* __restrict__ st, const double* __restrict__ beta, const ST* __restrict__ r,
-                           const ST* __restrict__ pr, ST* __restrict__ q, ST* __restrict__ qprev, ST* __restrict__ p,
+__global__ void k_hd_scale(const HdState* st, const double* beta, const ST* r, const ST* pr, ST* q, ST* qprev, ST* p,
                            int64_t n, int init) {
+  dep_begin();
   if (st->done) return;
   double s;
   if (init) {
@@ -166,26 +170,26 @@ int haydock_partials() { return hd_grid(); }
 template <typename ST>
 void launch_hd_dot(const ST* x, const ST* y, int64_t n, double* partial, cudaStream_t s) {
   count_launch();
-  k_hd_dot<ST><<<hd_grid(), HD_THREADS, 0, s>>>(x, y, n, partial);
+  launch_dep(k_hd_dot<ST>, hd_grid(), HD_THREADS, 0, s, x, y, n, partial);
 }
 
 void launch_hd_scalar(HdState* st, const double* partial, double* alpha, double* beta, int which, cudaStream_t s) {
   count_launch();
-  k_hd_scalar<<<1, 32, 0, s>>>(st, partial, hd_grid(), alpha, beta, which);
+  launch_dep(k_hd_scalar, 1, 32, 0, s, st, partial, hd_grid(), alpha, beta, which);
 }
 
 template <typename ST>
 void launch_hd_axpy(const HdState* st, const double* alpha, const double* beta, const ST* w, const ST* q,
                     const ST* qprev, ST* r, int64_t n, cudaStream_t s) {
   count_launch();
-  k_hd_axpy<ST><<<hd_grid(), HD_THREADS, 0, s>>>(st, alpha, beta, w, q, qprev, r, n);
+  launch_dep(k_hd_axpy<ST>, hd_grid(), HD_THREADS, 0, s, st, alpha, beta, w, q, qprev, r, n);
 }
 
 template <typename ST>
 void launch_hd_scale(const HdState* st, const double* beta, const ST* r, const ST* pr, ST* q, ST* qprev, ST* p,
                      int64_t n, int init, cudaStream_t s) {
   count_launch();
-  k_hd_scale<ST><<<hd_grid(), HD_THREADS, 0, s>>>(st, beta, r, pr, q, qprev, p, n, init);
+  launch_dep(k_hd_scale<ST>, hd_grid(), HD_THREADS, 0, s, st, beta, r, pr, q, qprev, p, n, init);
 }
 
 template <typename ST>

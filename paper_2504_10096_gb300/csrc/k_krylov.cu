@@ -53,6 +53,7 @@ namespace bse {
 template <typename ST>
 __global__ void __launch_bounds__(256)
 k_cgs_dot(const Prob* __restrict__ probs, int ph, int newvec, int half, int pass) {
+  dep_begin();
   const Prob& p = probs[blockIdx.z];
   const KState* st = p.st;
   if (!kphase(st, newvec) || (int)blockIdx.y >= dot_chunks(p.nT)) return;
@@ -66,6 +67,7 @@ k_cgs_dot(const Prob* __restrict__ probs, int ph, int newvec, int half, int pass
 template <typename ST>
 __global__ void __launch_bounds__(256, 3)
 k_cgs_update(const Prob* __restrict__ probs, int ph, int pass, int newvec, int half) {
+  dep_begin();
   __shared__ ST cf[2 * MAXM + 2];
   __shared__ ST red[8][32];
   const Prob& p = probs[blockIdx.y];
@@ -102,6 +104,7 @@ __device__ __forceinline__ void df_add(float& sh, float& sl, float bh, float bl)
 // tasks and output as k_cgs_dot (folded step, half 0: Re(P^H w) and Im(V^H w))
 __global__ void __launch_bounds__(256)
 k_cgs_dot_dfs(const Prob* __restrict__ probs, int newvec) {
+  dep_begin();
   const Prob& p = probs[blockIdx.z];
   const KState* st = p.st;
   if (!kphase(st, newvec) || (int)blockIdx.y >= dot_chunks(p.nT)) return;
@@ -119,8 +122,8 @@ k_cgs_dot_dfs(const Prob* __restrict__ probs, int newvec) {
     float4 q[4], x[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      q[u] = __ldg(Q + r + 32 * u);
-      x[u] = __ldg(w + r + 32 * u);
+      q[u] = Q[r + 32 * u];
+      x[u] = w[r + 32 * u];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -163,7 +166,7 @@ __device__ __forceinline__ void cgs_update_dfs_slab(const Prob& p, int nj, int p
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int c = c0 + G * u;
-      if (c < nset) v[u] = __ldg((c >= nj ? p.Ps : p.Vs) + (int64_t)(c >= nj ? c - nj : c) * p.Npad + row);
+      if (c < nset) v[u] = ((c >= nj ? p.Ps : p.Vs) + (int64_t)(c >= nj ? c - nj : c) * p.Npad)[row];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -202,6 +205,7 @@ __device__ __forceinline__ void cgs_update_dfs_slab(const Prob& p, int nj, int p
 
 __global__ void __launch_bounds__(256, 3)
 k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
+  dep_begin();
   __shared__ float2 cf[2 * MAXM + 2];
   __shared__ float4 red[8][32];
   const Prob& p = probs[blockIdx.y];
@@ -221,6 +225,7 @@ k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
 template <typename ST>
 __global__ void __launch_bounds__(256)
 k_normalize(const Prob* __restrict__ probs, int ph, int start, int half) {
+  dep_begin();
   using R = typename RealOf<ST>::T;
   __shared__ unsigned int last;
   const Prob& p = probs[blockIdx.y];
@@ -287,6 +292,7 @@ __global__ void k_start_fill(const Prob* __restrict__ probs, uint64_t seed, cons
 template <typename ST>
 __global__ void __launch_bounds__(256)
 k_restart_gemm(const Prob* __restrict__ probs, int which) {
+  dep_begin();
   using R = typename RealOf<ST>::T;
   __shared__ ST sv[32][64];
   __shared__ R ss[32][16];
@@ -359,6 +365,7 @@ __device__ __forceinline__ void df_acc(float& ah, float& al, float vh, float vl,
 
 __global__ void __launch_bounds__(256)
 k_restart_gemm_df(const Prob* __restrict__ probs, int which) {
+  dep_begin();
   __shared__ float4 sv[32][64];      // {re_hi, im_hi, re_lo, im_lo}
   __shared__ float2 ss[32][16];      // {hi, lo}
   const Prob& p = probs[blockIdx.z];
@@ -423,6 +430,7 @@ k_restart_gemm_df(const Prob* __restrict__ probs, int which) {
 // follow.  grid (rows / 256, ncv + 1, nprob): a column per CTA row, none reads what another writes.
 template <typename ST>
 __global__ void k_restart_copy(const Prob* __restrict__ probs, int ph, int gk) {
+  dep_begin();
   const Prob& p = probs[blockIdx.z];
   const KState* st = p.st;
   if (st->status != ST_OK || !st->r_go) return;   // decided in this restart only
@@ -453,6 +461,7 @@ __global__ void k_restart_copy(const Prob* __restrict__ probs, int ph, int gk) {
 
 // one warp per problem
 __global__ void __launch_bounds__(32) k_restart_commit(const Prob* __restrict__ probs) {
+  dep_begin();
   const Prob& p = probs[blockIdx.x];
   KState* st = p.st;
   if (st->status != ST_OK || !st->r_go) return;   // decided in this restart only
@@ -485,12 +494,12 @@ void launch_step_cgs(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int
   const unsigned nch = nprob > 1 ? DOT_CHUNKS : (unsigned)dot_chunks((int)(maxNpad / TS));
   const dim3 gd((ncol + 7) / 8, nch, nprob), gu((unsigned)(maxNpad / slab), nprob);
   if (dfs && ph && half == 0) {        // the double-FP32 shadows of the mixed path
-    k_cgs_dot_dfs<<<gd, 256, 0, s>>>(dprobs, newvec);
-    k_cgs_update_dfs<<<gu, 256, 0, s>>>(dprobs, ps, newvec);
+    launch_dep(k_cgs_dot_dfs, gd, 256, 0, s, dprobs, newvec);
+    launch_dep(k_cgs_update_dfs, gu, 256, 0, s, dprobs, ps, newvec);
     return;
   }
-  k_cgs_dot<ST><<<gd, 256, 0, s>>>(dprobs, ph, newvec, half, ps);
-  k_cgs_update<ST><<<gu, 256, 0, s>>>(dprobs, ph, ps, newvec, half);
+  launch_dep(k_cgs_dot<ST>, gd, 256, 0, s, dprobs, ph, newvec, half, ps);
+  launch_dep(k_cgs_update<ST>, gu, 256, 0, s, dprobs, ph, ps, newvec, half);
 }
 
 template <typename ST>
@@ -498,7 +507,7 @@ void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int64_t maxNpa
                            cudaStream_t s) {
   count_launch();
   // start: 0 regular step, 1 fresh (first or replacement) vector
-  k_normalize<ST><<<dim3((unsigned)((maxNpad + 255) / 256), nprob), 256, 0, s>>>(dprobs, ph, start, half);
+  launch_dep(k_normalize<ST>, dim3((unsigned)((maxNpad + 255) / 256), nprob), 256, 0, s, dprobs, ph, start, half);
 }
 
 template <typename ST>
@@ -518,13 +527,13 @@ void launch_restart(const Prob* dprobs, int nprob, int ph, int64_t maxNpad, int 
   const unsigned gx = (unsigned)((maxNpad + 63) / 64);
   for (int which = 0; which < ngemm; ++which) {
     if (df && std::is_same<ST, double2>::value)
-      k_restart_gemm_df<<<dim3(gx, (ncv + 15) / 16, nprob), 256, 0, s>>>(dprobs, which);
+      launch_dep(k_restart_gemm_df, dim3(gx, (ncv + 15) / 16, nprob), 256, 0, s, dprobs, which);
     else
-      k_restart_gemm<ST><<<dim3(gx, (ncv + 15) / 16, nprob), 256, 0, s>>>(dprobs, which);
+      launch_dep(k_restart_gemm<ST>, dim3(gx, (ncv + 15) / 16, nprob), 256, 0, s, dprobs, which);
   }
   const unsigned gr = (unsigned)((maxNpad + 255) / 256);
-  k_restart_copy<ST><<<dim3(gr, ncv + 1, nprob), 256, 0, s>>>(dprobs, ph, gruning ? 1 : 0);
-  k_restart_commit<<<nprob, 32, 0, s>>>(dprobs);
+  launch_dep(k_restart_copy<ST>, dim3(gr, ncv + 1, nprob), 256, 0, s, dprobs, ph, gruning ? 1 : 0);
+  launch_dep(k_restart_commit, nprob, 32, 0, s, dprobs);
 }
 
 #define INST(ST)                                                                                        \

@@ -35,7 +35,9 @@ __device__ __forceinline__ void unpack_pq(CT& a, CT& b) {
 template <typename ST, typename R, bool HASB>
 __global__ void __launch_bounds__(PROD_THREADS, sizeof(R) == 4 ? 2 : 1)
 k_prod_tiles(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs,
-             int mode, GenericIO io, int strided) {
+             int mode, GenericIO io, int strided, int first) {
+  dep_begin();
+  if (first) clock_start(probs[0].clock);
   using CT = typename Acc<R>::T;
   __shared__ CT xc[TS];      // column block J of x
   __shared__ CT xr[TS];      // row block I of x
@@ -49,15 +51,35 @@ __global__ void __launch_bounds__(REDUCE_GROUPS * REDUCE_ROWS)
 k_prod_reduce(const Prob* __restrict__ probs, int mode, GenericIO io) {
   using CT = typename Acc<R>::T;
   __shared__ CT grp[REDUCE_GROUPS][REDUCE_ROWS];
+  dep_begin();
   prod_reduce_body<ST, R>(probs, mode, io, blockIdx.x, blockIdx.y, grp);
+  clock_end(probs[0].clock);
 }
 
 // Same reduction for the double-FP32 kernels, whose slots hold (hi, lo) float
-// pairs {re_hi, re_lo, im_hi, im_lo}: each slot is widened to FP64 and the slots
-// are summed in FP64 in the fixed order above.
+// pairs {re_hi, re_lo, im_hi, im_lo}.  Widening and adding a slot in FP64 is four FP64 adds of 64
+// clocks (92 us at N = 2e4, twelve times the slots' traffic); here a warp adds its slots as
+// triple-FP32 sums (TwoSum down the three parts: 70 bits, 40 FP32 adds) and widens once.
+struct F3 {
+  float a, b, c;
+};
+__device__ __forceinline__ void f3_two_sum(float& a, float& b) {   // (a, b) -> (fl(a + b), error)
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  b = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  a = s;
+}
+__device__ __forceinline__ void f3_add(F3& s, float h, float l) {
+  f3_two_sum(s.a, h);          // h: what is left of it
+  f3_two_sum(s.b, h);
+  f3_two_sum(s.b, l);
+  s.c = __fadd_rn(s.c, __fadd_rn(h, l));
+}
+__device__ __forceinline__ double f3_wide(const F3& s) { return (double)s.a + ((double)s.b + (double)s.c); }
+
 __global__ void __launch_bounds__(REDUCE_GROUPS * REDUCE_ROWS)
 k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
   __shared__ double2 grp[REDUCE_GROUPS][REDUCE_ROWS];
+  dep_begin();
   const Prob& p = probs[blockIdx.y];
   const int I = blockIdx.x / REDUCE_UNITS;
   if (I >= p.nT) return;
@@ -66,17 +88,19 @@ k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int r = (blockIdx.x % REDUCE_UNITS) * REDUCE_ROWS + lane;
   const float4* part = (const float4*)p.part + (int64_t)I * p.nT * TS;
-  double2 acc = make_double2(0.0, 0.0);
-  auto wide = [](float4 v) { return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w); };
-  int J = g;
-  for (; J + 3 * REDUCE_GROUPS < p.nT; J += 4 * REDUCE_GROUPS) {
+  F3 re{0.f, 0.f, 0.f}, im{0.f, 0.f, 0.f};
+  for (int J = g; J < p.nT; J += 4 * REDUCE_GROUPS) {
     float4 v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = part[(int64_t)(J + u * REDUCE_GROUPS) * TS + r];
+    for (int u = 0; u < 4; ++u)
+      v[u] = J + u * REDUCE_GROUPS < p.nT ? part[(int64_t)(J + u * REDUCE_GROUPS) * TS + r] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc = cadd(acc, wide(v[u]));
+    for (int u = 0; u < 4; ++u) {
+      f3_add(re, v[u].x, v[u].y);
+      f3_add(im, v[u].z, v[u].w);
+    }
   }
-  for (; J < p.nT; J += REDUCE_GROUPS) acc = cadd(acc, wide(part[(int64_t)J * TS + r]));
+  double2 acc = make_double2(f3_wide(re), f3_wide(im));
   grp[g][lane] = acc;
   __syncthreads();
   if (g == 0) {
@@ -89,6 +113,7 @@ k_prod_reduce_dfc(const Prob* __restrict__ probs, int mode, GenericIO io) {
       if (lane == 0) p.npart[blockIdx.x] = t;
     }
   }
+  clock_end(p.clock);
 }
 
 // ---------------------------------------------------------------- wide blocks
@@ -334,30 +359,31 @@ void launch_product(const Prob* dprobs, const TileJob* jobs, int njobs, int npro
   // registers bound the FP64 variant to one CTA per SM and the FP32 one to two
   const int grid = product_grid(product_occupancy<ST, R>(hasB), shape, njobs);
   if (hasB)
-    k_prod_tiles<ST, R, true><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+    launch_dep(k_prod_tiles<ST, R, true>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, 1);
   else
-    k_prod_tiles<ST, R, false><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
-  k_prod_reduce<ST, R><<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode, io);
+    launch_dep(k_prod_tiles<ST, R, false>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, 1);
+  launch_dep(k_prod_reduce<ST, R>, dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s, dprobs, mode,
+             io);
 }
 
 void launch_prod_reduce_d(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s) {
-  k_prod_reduce_dfc<<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode, io);
+  launch_dep(k_prod_reduce_dfc, dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s, dprobs, mode, io);
 }
 
 void launch_prod_reduce_f64(const Prob* dprobs, int nprob, int maxnT, int mode, GenericIO io, cudaStream_t s) {
   count_launch();
-  k_prod_reduce<double2, double><<<dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s>>>(dprobs, mode,
-                                                                                                      io);
+  launch_dep(k_prod_reduce<double2, double>, dim3(REDUCE_UNITS * maxnT, nprob), REDUCE_GROUPS * REDUCE_ROWS, 0, s, dprobs,
+             mode, io);
 }
 
 void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, GenericIO io, bool hasB,
-                      ProdShape shape, cudaStream_t s) {
+                      ProdShape shape, int first, cudaStream_t s) {
   count_launch();
   const int grid = product_grid(product_occupancy<double2, double>(hasB), shape, njobs);
   if (hasB)
-    k_prod_tiles<double2, double, true><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+    launch_dep(k_prod_tiles<double2, double, true>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, first);
   else
-    k_prod_tiles<double2, double, false><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+    launch_dep(k_prod_tiles<double2, double, false>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, first);
 }
 
 template void launch_product<double2, double>(const Prob*, const TileJob*, int, int, int, int, int,

@@ -176,6 +176,8 @@ template <bool HASB, bool SPLIT>
 __global__ void __launch_bounds__(PROD_THREADS, 2)
 k_prod_tiles_df(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
                 GenericIO io, int strided) {
+  dep_begin();
+  clock_start(probs[0].clock);
   static_assert(!HASB || SPLIT, "complex64 PH tiles go through k_prod_tiles_df2");
   __shared__ float4 xc[TS], xr[TS];
   // per-thread row partial sums (own slots only); after a barrier the same
@@ -374,7 +376,9 @@ __device__ __forceinline__ XPack xpack(double2 v, bool row) {
 
 __global__ void __launch_bounds__(PROD_THREADS, 2)
 k_prod_tiles_df2(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
-                 GenericIO io, int strided) {
+                 GenericIO io, int strided, int first) {
+  dep_begin();
+  if (first) clock_start(probs[0].clock);
   __shared__ XPack xc[TS], xr[TS];
   __shared__ DFC rpark[8][PROD_THREADS];
   DFC(*red)[TS] = reinterpret_cast<DFC(*)[TS]>(&rpark[0][0]);
@@ -566,6 +570,8 @@ __device__ __forceinline__ void regrid(float S, float l, float gs, float& g, flo
 // and xmax[I] = max |hi| over chunk I; grid (maxnT, nprob), TS threads
 __global__ void __launch_bounds__(TS)
 k_mx_stage_x(const Prob* __restrict__ probs, int mode, GenericIO io) {
+  dep_begin();
+  clock_start(probs[0].clock);
   __shared__ float sm[TS / 32];
   const Prob& p = probs[blockIdx.y];
   const int I = blockIdx.x;
@@ -652,7 +658,12 @@ __device__ __forceinline__ void mx_copy(uint32_t dst, const void* src, uint32_t 
 template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT)
 k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
-                GenericIO io, int strided, int* __restrict__ err) {
+                GenericIO io, int strided, int beside, int* __restrict__ err) {
+  // beside = 1: the kernel before it in the stream runs the fine tiles; it waited for the staged
+  // vector before it let this one start, so the two run side by side, and this one waits for it at
+  // its end (whoever waits for this kernel finds both done)
+  if (!beside) dep_wait();
+  dep_launch();
   using C = Mx<NT>;
   extern __shared__ __align__(128) unsigned char smx[];
   __shared__ uint64_t full[C::NST], empty[C::NST];
@@ -895,6 +906,7 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
       mx_wait(mx_s32(&full[g % C::NST]), (uint32_t)((g / C::NST) & 1));
   }
   __syncthreads();
+  if (beside) dep_wait();
 }
 
 // records {U_re, V_re, U_im, V_im} of U = fl(A + B), V = fl(A - B) for every packed element
@@ -968,9 +980,9 @@ void launch_df(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, con
   // complex128 tiles: the scalar kernel (its float4 rows leave the packed one no registers for
   // latency hiding: 0.274 vs 0.250 ms at N = 8000)
   if constexpr (HASB && !SPLIT)
-    k_prod_tiles_df2<<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+    launch_dep(k_prod_tiles_df2, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, 1);
   else
-    k_prod_tiles_df<HASB, SPLIT><<<grid, PROD_THREADS, 0, s>>>(dprobs, jobs, njobs, mode, io, shape.strided);
+    launch_dep(k_prod_tiles_df<HASB, SPLIT>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided);
 }
 
 void launch_product_df(const Prob* dprobs, const TileJob* jobs, int njobs, int nprob, int maxnT, int mode,
@@ -992,7 +1004,7 @@ int product_mx_occupancy() { return 2; }   // shapes: 1 (512 threads) or 2 (256 
 
 template <int NT>
 void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode, const GenericIO& io,
-               ProdShape shape, int* err, cudaStream_t s) {
+               ProdShape shape, int beside, int* err, cudaStream_t s) {
   using C = Mx<NT>;
   static bool attr = false;
   if (!attr) {
@@ -1001,8 +1013,8 @@ void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode,
     attr = true;
   }
   const ProdShape ms{shape.ctas_per_sm < 0 ? -1 : C::CTAS, shape.strided};
-  k_prod_tiles_mx<NT><<<product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s>>>(dprobs, coarse, ncoarse, mode, io,
-                                                                            shape.strided, err);
+  launch_dep(k_prod_tiles_mx<NT>, product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s, dprobs, coarse, ncoarse, mode, io,
+             shape.strided, beside, err);
 }
 
 void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, const TileJob* coarse, int ncoarse,
@@ -1010,19 +1022,23 @@ void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, co
                           cudaStream_t s) {
   GenericIO io{};
   if (io_host) io = *io_host;
+  if (ncoarse > 0) {
+    count_launch();
+    launch_dep(k_mx_stage_x, dim3(maxnT, nprob), TS, 0, s, dprobs, mode, io);
+  }
   if (nfine > 0) {
     count_launch();
     const ProdShape fs{0, 1};
-    k_prod_tiles_df2<<<product_grid(df_occupancy<true, false>(), fs, nfine), PROD_THREADS, 0, s>>>(
-        dprobs, fine, nfine, mode, io, 1);
+    launch_dep(k_prod_tiles_df2, product_grid(df_occupancy<true, false>(), fs, nfine), PROD_THREADS, 0, s, dprobs, fine,
+               nfine, mode, io, 1, ncoarse > 0 ? 0 : 1);
   }
   if (ncoarse > 0) {
-    count_launch(2);
-    k_mx_stage_x<<<dim3(maxnT, nprob), TS, 0, s>>>(dprobs, mode, io);
+    count_launch();
     // shape.ctas_per_sm: 1 -> the 512-thread kernel, otherwise the 256-thread one (two CTAs per
     // SM; -1: one CTA per tile)
-    if (shape.ctas_per_sm == 1) launch_mx<512>(dprobs, coarse, ncoarse, mode, io, shape, err, s);
-    else launch_mx<256>(dprobs, coarse, ncoarse, mode, io, shape, err, s);
+    const int beside = nfine > 0;
+    if (shape.ctas_per_sm == 1) launch_mx<512>(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s);
+    else launch_mx<256>(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s);
   }
   count_launch();
   launch_prod_reduce_d(dprobs, nprob, maxnT, mode, io, s);

@@ -17,6 +17,8 @@ k_prod_tiles_fx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
   FxShared<FX_RING>& sh = *reinterpret_cast<FxShared<FX_RING>*>(fxsm);
   fx_init(sh);
   __syncthreads();
+  dep_begin();
+  clock_start(probs[0].clock);
   FxPipe pipe;
   fx_tiles_body<HASB, false>(probs, jobs, njobs, nq, mode, io, strided, blockIdx.x, gridDim.x, sh, pipe, probs[0].err);
 }
@@ -117,10 +119,10 @@ void launch_product_fx(const Prob* dprobs, const TileJob* jobs, int njobs, int n
   if (nfx > 0) {
     count_launch();
     const int grid = product_grid(product_fx_occupancy(), shape, nfx * nq);
-    if (hasB) k_prod_tiles_fx<true><<<grid, FX_THREADS, sizeof(FxShared<FX_RING>), s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
-    else k_prod_tiles_fx<false><<<grid, FX_THREADS, sizeof(FxShared<FX_RING>), s>>>(dprobs, jobs, nfx, nq, mode, io, shape.strided);
+    if (hasB) launch_dep(k_prod_tiles_fx<true>, grid, FX_THREADS, sizeof(FxShared<FX_RING>), s, dprobs, jobs, nfx, nq, mode, io, shape.strided);
+    else launch_dep(k_prod_tiles_fx<false>, grid, FX_THREADS, sizeof(FxShared<FX_RING>), s, dprobs, jobs, nfx, nq, mode, io, shape.strided);
   }
-  if (njobs > nfx) launch_tiles_f64(dprobs, jobs + nfx, njobs - nfx, mode, io, hasB, shape, s);
+  if (njobs > nfx) launch_tiles_f64(dprobs, jobs + nfx, njobs - nfx, mode, io, hasB, shape, nfx == 0, s);
   launch_prod_reduce_f64(dprobs, nprob, maxnT, mode, io, s);
 }
 

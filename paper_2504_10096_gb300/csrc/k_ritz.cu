@@ -62,6 +62,7 @@ __device__ __forceinline__ double* ritz_vec(const Prob& p, int i) {
 
 // Gruning path: the tree arrays of the active block (one thread per problem)
 __global__ void k_gk_form(const Prob* __restrict__ probs, int nprob) {
+  dep_begin();
   const int ip = blockIdx.x * blockDim.x + threadIdx.x;
   if (ip >= nprob) return;
   const Prob& p = probs[ip];
@@ -126,6 +127,7 @@ __device__ void gersh(const TV& T, double& lo, double& hi, double& tnorm, int la
 // four warps (128 shifts) per wanted eigenvalue; grid (ncv, nprob); dynamic shared memory: the
 // tree's entries in FP64 and in double-FP32 (scaled by a power of two to norm 1)
 __global__ void __launch_bounds__(RV_THREADS) k_ritz_values(const Prob* __restrict__ probs) {
+  dep_begin();
   extern __shared__ double sm[];
   __shared__ double s_g[3];
   __shared__ double s_sig[RV_THREADS];
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(RV_THREADS) k_ritz_values(const Prob* __restri
 // ---------------------------------------------------------------- inverse iteration
 // one warp per cluster leader; grid (ncv, nprob), block 32, dynamic smem.
 __global__ void __launch_bounds__(32) k_ritz_vectors(const Prob* __restrict__ probs) {
+  dep_begin();
   extern __shared__ double sm[];
   const Prob& p = probs[blockIdx.y];
   const KState* st = p.st;
@@ -259,6 +262,7 @@ __global__ void __launch_bounds__(32) k_ritz_vectors(const Prob* __restrict__ pr
 // Lock the leading converged Ritz pairs, choose what to keep, and write the
 // restarted arrow (theta, b).  One warp per problem.
 __global__ void __launch_bounds__(32) k_lock_decide(const Prob* __restrict__ probs, int ph) {
+  dep_begin();
   const Prob& p = probs[blockIdx.x];
   KState* st = p.st;
   if (!restart_ready(st)) return;
@@ -307,20 +311,20 @@ __global__ void __launch_bounds__(32) k_lock_decide(const Prob* __restrict__ pro
 void launch_ritz(const Prob* dprobs, int nprob, int ncv, bool gruning, cudaStream_t s) {
   if (gruning) {
     count_launch();
-    k_gk_form<<<(nprob + 127) / 128, 128, 0, s>>>(dprobs, nprob);
+    launch_dep(k_gk_form, (nprob + 127) / 128, 128, 0, s, dprobs, nprob);
   }
   count_launch(2);
   const size_t M = gruning ? (size_t)(2 * ncv + 2) : (size_t)ncv;
   const size_t sv = M * 2 * (sizeof(double) + sizeof(float2)), sm = M * 5 * sizeof(double) + M + 16;
   if (sv > 48 * 1024) cudaFuncSetAttribute(k_ritz_values, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv);
   if (sm > 48 * 1024) cudaFuncSetAttribute(k_ritz_vectors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_ritz_values<<<dim3(ncv, nprob), RV_THREADS, sv, s>>>(dprobs);
-  k_ritz_vectors<<<dim3(ncv, nprob), 32, sm, s>>>(dprobs);
+  launch_dep(k_ritz_values, dim3(ncv, nprob), RV_THREADS, sv, s, dprobs);
+  launch_dep(k_ritz_vectors, dim3(ncv, nprob), 32, sm, s, dprobs);
 }
 
 void launch_lock_decide_form(const Prob* dprobs, int nprob, int ph, cudaStream_t s) {
   count_launch();
-  k_lock_decide<<<nprob, 32, 0, s>>>(dprobs, ph);
+  launch_dep(k_lock_decide, nprob, 32, 0, s, dprobs, ph);
 }
 
 }  // namespace bse
