@@ -437,6 +437,21 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
   const int nm = cs.nm;
   const int nset = nm + cs.nt;
   const int nch = dot_chunks(p.nT);
+  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
+  const ST* vb = (const ST*)cs.um + row;
+  const ST* pb = ph ? (const ST*)cs.ut + row : nullptr;
+  // Loads in flight per thread, the first of them beside the sums of the coefficients.  A TDA cycle at
+  // N = 2000 took 31.2 ms of steps and restarts with 4, 32.4 with 6, 33.1 with 8 (32.5 with the loads
+  // behind the coefficients); a pseudo-Hermitian one at 3000 243.7, 246.6, 247.2 (251).
+  constexpr int U = 4;
+  const int64_t ld = p.Npad;
+  // entry cc of the set: Um[:, cc] for cc < nm, else the twin's Ut[:, cc - nm]
+  auto load = [&](int cc) -> ST { return ldv<COH>(cc < nm ? vb + (int64_t)cc * ld : pb + (int64_t)(cc - nm) * ld); };
+  const int c0 = tid / RS;
+  ST v[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)                 // the first round does not wait for the coefficients
+    if (c0 + G * u < nset) v[u] = load(c0 + G * u);
   // coefficients; the first slab also stores them for the step's end
   double2* coef = (double2*)p.coef + (int64_t)(pass & 1) * p.ncol;
   for (int c = tid; c < nset; c += 256) {
@@ -445,46 +460,25 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
     if (bx == 0) coef[c] = sc;
   }
   __syncthreads();
-  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
-  const ST* vb = (const ST*)cs.um + row;
-  const ST* pb = ph ? (const ST*)cs.ut + row : nullptr;
-  constexpr int U = sizeof(ST) == 16 ? 6 : 8;   // loads in flight per thread
-  const int64_t ld = p.Npad;
-  // entry cc of the set: Um[:, cc] for cc < nm, else the twin i Ut[:, cc - nm] (as (-t.y, t.x))
-  auto colval = [&](int cc) -> ST {
-    if (cc < nm) return ldv<COH>(vb + (int64_t)cc * ld);
-    const ST q = ldv<COH>(pb + (int64_t)(cc - nm) * ld);
-    ST t;
-    t.x = -q.y;
-    t.y = q.x;
-    return t;
-  };
   ST part = czero<ST>();
-  int c = tid / RS;
-  // all U loads of a round are issued before any of their arithmetic
-  if (ph) {                                 // real coefficients (K-inner products, twin projections)
-    for (; c < nset; c += G * U) {
-      ST v[U];
+  for (int c = c0; c < nset; c += G * U) {
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (c + G * u < nset) v[u] = colval(c + G * u);
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (c + G * u < nset) {
-          const R f = cf[c + G * u].x;
-          part.x = fma(v[u].x, f, part.x);
-          part.y = fma(v[u].y, f, part.y);
-        }
+    for (int u = 0; u < U; ++u) {
+      const int cc = c + G * u;
+      if (cc >= nset) continue;
+      if (ph) {                               // real coefficients; the twin i t = (-t.y, t.x)
+        const R f = cf[cc].x;
+        const bool tw = cc >= nm;
+        part.x = fma(tw ? -v[u].y : v[u].x, f, part.x);
+        part.y = fma(tw ? v[u].x : v[u].y, f, part.y);
+      } else {
+        cfma(part, v[u], cf[cc]);
+      }
     }
-  } else {
-    for (; c < nset; c += G * U) {
-      ST v[U];
+    if (c + G * U < nset) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (c + G * u < nset) v[u] = ldv<COH>(vb + (int64_t)(c + G * u) * ld);
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (c + G * u < nset) cfma(part, v[u], cf[c + G * u]);
+        if (c + G * (U + u) < nset) v[u] = load(c + G * (U + u));
     }
   }
 #pragma unroll
@@ -589,8 +583,8 @@ __device__ __forceinline__ void normalize_row(const Prob& p, const KState* st, i
 
 // Record alpha_j, beta_j, advance j, given beta^2 = b2 of the new vector.  fresh = 0:
 // regular step; fresh = 1: a first or replacement vector was just normalised.
-// In a persistent launch every CTA keeps its own copy of the state and runs this on it; one of
-// them (`writer`) also stores alpha and beta.
+// p.st is a copy of the state that is not yet in use (k_normalize) or each CTA's own (k_persist.cu);
+// one of the CTAs (`writer`) also stores alpha and beta.
 template <bool COH>
 __device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh, double b2, bool writer) {
   KState* st = p.st;
@@ -630,7 +624,7 @@ __device__ __forceinline__ void step_finish_one(const Prob& p, int ph, int fresh
 // squared M-norm b2 of the new vector; fresh = 1: a first or replacement even vector.
 // An odd vector cannot vanish when M+ is positive definite (M+ maps the j + 1 even
 // vectors onto j + 1 independent odd ones), so a vanishing alpha means not definite.
-__device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh, double b2) {
+__device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh, double b2, bool writer) {
   KState* st = p.st;
   const int j = st->j;
   if (!isfinite(b2)) { st->status = ST_NOTFINITE; return; }
@@ -648,18 +642,18 @@ __device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh
     if (b2 < -1e6 * tiny) { st->status = ST_NOTPD; return; }
     if (half == 1) {
       if (b2 <= tiny) { st->status = ST_NOTPD; return; }
-      p.alpha[j] = sqrt(b2);
+      if (writer) p.alpha[j] = sqrt(b2);
       return;                           // the even half follows in the same step
     }
     st->passes += 2;
     st->steps += 1;
     if (b2 <= tiny) {                   // invariant subspace: the chain restarts
-      p.beta[j] = 0.0;                  // with a fresh vector (host-driven), unless the subspace is full
+      if (writer) p.beta[j] = 0.0;      // with a fresh vector (host-driven), unless the subspace is full
       if (j + 1 < st->m) st->breakdown = 1;
       else st->j = j + 1;
       return;
     }
-    p.beta[j] = sqrt(b2);
+    if (writer) p.beta[j] = sqrt(b2);
     st->j = j + 1;
   }
   if (st->steps >= st->maxit && !st->done) { st->done = 1; st->status = ST_NOCONV; }
@@ -667,7 +661,7 @@ __device__ __forceinline__ void gk_finish_one(const Prob& p, int half, int fresh
 
 template <bool COH>
 __device__ __forceinline__ void finish_one(const Prob& p, int ph, int fresh, int half, double b2, bool writer) {
-  if (half) gk_finish_one(p, half, fresh, b2);
+  if (half) gk_finish_one(p, half, fresh, b2, writer);
   else step_finish_one<COH>(p, ph, fresh, b2, writer);
 }
 

@@ -150,6 +150,15 @@ __device__ __forceinline__ void cgs_update_dfs_slab(const Prob& p, int nj, int p
   constexpr int G = 256 / RS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bx = blockIdx.x;
   const int nset = 2 * nj, nch = dot_chunks(p.nT);
+  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
+  // entry cc: V[:, cc] (cc < nj) or the twin i P[:, cc - nj] = (-P_im, P_re)
+  auto load = [&](int c) { return ((c >= nj ? p.Ps : p.Vs) + (int64_t)(c >= nj ? c - nj : c) * p.Npad)[row]; };
+  constexpr int U = 8;
+  const int c0 = tid / RS;
+  float4 v[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)                 // the first round does not wait for the coefficients
+    if (c0 + G * u < nset) v[u] = load(c0 + G * u);
   double2* coef = (double2*)p.coef + (int64_t)(pass & 1) * p.ncol;
   for (int c = tid; c < nset; c += 256) {
     const double sc = cgs_coef<false>(p, 1, c, nch).x;
@@ -158,24 +167,21 @@ __device__ __forceinline__ void cgs_update_dfs_slab(const Prob& p, int nj, int p
     if (bx == 0) coef[c] = mk(sc, 0.0);
   }
   __syncthreads();
-  const int64_t row = (int64_t)bx * RS + (tid & (RS - 1));
-  // entry cc: V[:, cc] (cc < nj) or the twin i P[:, cc - nj] = (-P_im, P_re)
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-  for (int c0 = tid / RS; c0 < nset; c0 += 4 * G) {
-    float4 v[4];
+  for (int c = c0; c < nset; c += G * U) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + G * u;
-      if (c < nset) v[u] = ((c >= nj ? p.Ps : p.Vs) + (int64_t)(c >= nj ? c - nj : c) * p.Npad)[row];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + G * u;
-      if (c >= nset) continue;
-      const float2 f = cf[c];
-      const float4 t = c >= nj ? make_float4(-v[u].y, v[u].x, -v[u].w, v[u].z) : v[u];
+    for (int u = 0; u < U; ++u) {
+      const int cc = c + G * u;
+      if (cc >= nset) continue;
+      const float2 f = cf[cc];
+      const float4 t = cc >= nj ? make_float4(-v[u].y, v[u].x, -v[u].w, v[u].z) : v[u];
       df_madd(rh, rl, t.x, t.z, f.x, f.y);
       df_madd(ih, il, t.y, t.w, f.x, f.y);
+    }
+    if (c + G * U < nset) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (c + G * (U + u) < nset) v[u] = load(c + G * (U + u));
     }
   }
 #pragma unroll
@@ -220,29 +226,40 @@ k_cgs_update_dfs(const Prob* __restrict__ probs, int pass, int newvec) {
 }
 
 // The new basis vector and the step's end in one launch: every warp sums the norm's partial sums
-// itself, scales its rows, and the last CTA of a problem to finish (a ticket) updates its state,
-// which all the others have read by then.
+// itself and scales its rows; meanwhile a ninth warp works out the state after the step, and the last
+// CTA of a problem to finish (a ticket) stores it, when all the others have read the old one.
 template <typename ST>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(288)
 k_normalize(const Prob* __restrict__ probs, int ph, int start, int half) {
   dep_begin();
   using R = typename RealOf<ST>::T;
   __shared__ unsigned int last;
+  __shared__ KState ns;
+  __shared__ Prob np;
   const Prob& p = probs[blockIdx.y];
   const KState* st = p.st;
   const unsigned int nblk = (unsigned int)((p.Npad + 255) / 256);
   if (blockIdx.x >= nblk || !kphase(st, start)) return;
   const int64_t row = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const double b2 = norm_sum<false>(p, ph);
-  // a beta^2 that is no positive number is recorded by the step's end
-  if (row < p.Npad && b2 > 0.0 && isfinite(b2)) normalize_row<ST, false>(p, st, ph, half, row, (R)rsqrt(b2));
+  if (threadIdx.x >= 256) {
+    if (threadIdx.x == 256) {
+      ns = *st;
+      np = p;
+      np.st = &ns;
+      // (alpha and beta are the same from every CTA: the first one stores them)
+      finish_one<false>(np, ph, start, half, b2, blockIdx.x == 0);
+    }
+  } else if (row < p.Npad && b2 > 0.0 && isfinite(b2)) {   // else the step's end records it
+    normalize_row<ST, false>(p, st, ph, half, row, (R)rsqrt(b2));
+  }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(p.tick, 1u);
   __syncthreads();
   if (last != nblk - 1 || threadIdx.x != 0) return;
   *p.tick = 0u;
-  finish_one<false>(p, ph, start, half, b2, true);
+  *p.st = ns;
 }
 
 // ---------------------------------------------------------------- start vector
@@ -507,7 +524,7 @@ void launch_step_normalize(const Prob* dprobs, int nprob, int ph, int64_t maxNpa
                            cudaStream_t s) {
   count_launch();
   // start: 0 regular step, 1 fresh (first or replacement) vector
-  launch_dep(k_normalize<ST>, dim3((unsigned)((maxNpad + 255) / 256), nprob), 256, 0, s, dprobs, ph, start, half);
+  launch_dep(k_normalize<ST>, dim3((unsigned)((maxNpad + 255) / 256), nprob), 288, 0, s, dprobs, ph, start, half);
 }
 
 template <typename ST>

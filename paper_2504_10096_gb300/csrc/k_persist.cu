@@ -108,17 +108,21 @@ k_steps_persist(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
         if (!grid_sync(gb, nblk, gen, &s_ok)) return;
       }
     }
-    // the new basis vector and the end of the step: warps with rows of their own and warp 0
-    const int64_t r0 = ((int64_t)bid + (int64_t)nblk * warp) * 32;
+    // the new basis vector by the warps that have rows, and beside it the end of the step by the last
+    // warp: the rows go by a copy of the index the step's end advances
+    KState now;
+    now.j = st->j;
+    __syncthreads();
+    const bool endw = warp == PS_THREADS / 32 - 1;
     double b2 = 0.0;
-    if (warp == 0 || r0 < p.Npad) b2 = norm_sum<true>(p, ph);
+    const int64_t r0 = ((int64_t)bid + (int64_t)nblk * warp) * 32;
+    if (endw || r0 < p.Npad) b2 = norm_sum<true>(p, ph);
     if (r0 < p.Npad && b2 > 0.0 && isfinite(b2)) {
       const R inv = (R)rsqrt(b2);
       for (int64_t r = r0; r < p.Npad; r += (int64_t)nblk * PS_THREADS)
-        normalize_row<ST, true>(p, st, ph, 0, r + lane, inv);
+        normalize_row<ST, true>(p, &now, ph, 0, r + lane, inv);
     }
-    __syncthreads();                                  // every warp has read the state
-    if (tid == 0) finish_one<true>(s_p, ph, 0, 0, b2, bid == 0);
+    if (endw && lane == 0) finish_one<true>(s_p, ph, 0, 0, b2, bid == 0);
     if (!grid_sync(gb, nblk, gen, &s_ok)) return;
   }
   __syncthreads();
