@@ -132,7 +132,7 @@ struct bse_handle {
   void* adj_panels = nullptr;
   size_t adj_panel_bytes = 0;
   int* adj_err = nullptr;
-  int* prod_err = nullptr;   // raised by a product kernel whose bounded wait expired
+  int* prod_err = nullptr;   // [0] raised by a product kernel whose bounded wait expired, [1] the coarse tiles' ticket
   double* gdev = nullptr;
   // the tuner's product timings, and the device clock of the products (bse_stats.ms_product)
   std::vector<cudaEvent_t> ev;
@@ -1543,8 +1543,8 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
   if (rc == BSE_OK && h->tiles64) rc = setup_scales64(h);
   if (rc == BSE_OK && h->mixed) h->hjobs = jobs;
   if (rc == BSE_OK && (h->mixed || h->nfx > 0)) {
-    rc = dalloc((void**)&h->prod_err, sizeof(int));
-    if (rc == BSE_OK && cudaMemsetAsync(h->prod_err, 0, sizeof(int), h->stream) != cudaSuccess) rc = BSE_ECUDA;
+    rc = dalloc((void**)&h->prod_err, 2 * sizeof(int));
+    if (rc == BSE_OK && cudaMemsetAsync(h->prod_err, 0, 2 * sizeof(int), h->stream) != cudaSuccess) rc = BSE_ECUDA;
   }
   if (rc == BSE_OK) {
     h->njobs = (int)jobs.size();

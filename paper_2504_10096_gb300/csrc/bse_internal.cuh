@@ -301,7 +301,8 @@ void launch_product_df(const Prob* dprobs, const TileJob* jobs, int njobs, int n
 void launch_split_tiles(const double2* packed, int64_t nelem, float4* split, cudaStream_t s);
 // mixed path (complex64 PH tiles, FP64 vectors): exact double-FP32 products on the
 // "fine" tiles (k_prod_tiles_df2), fixed-point-grid accumulation with rounded U, V on
-// the "coarse" ones (k_prod_tiles_mx), then the FP64 reduction (k_product_df.cu)
+// the "coarse" ones (k_prod_tiles_mx), then the FP64 reduction (k_product_df.cu); err: the error
+// flag and the coarse tiles' ticket
 void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, const TileJob* coarse, int ncoarse,
                           int nprob, int maxnT, int mode, const GenericIO* io_host, ProdShape shape, int* err,
                           cudaStream_t s);

@@ -182,6 +182,12 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
   const int u0 = strided ? bid : bid * per;
   const int u1 = strided ? nunit : min(nunit, u0 + per);
   const int du = strided ? nblk : 1;
+  // Unit of position u.  The plus halves of a chain take a CTA's units in the opposite order: what it
+  // read last is then what it wants first, while it may still be in the L2 (60 Haydock steps at
+  // N = 8000: 23.4 ms against 23.8; nothing in the persistent kernel, whose problems nearly fit).
+  const bool turned = !COH && (mode == PM_STEP_MPLUS || (mode == PM_GENERIC && io.sB > 0.0));
+  const int usum = 2 * u0 + (u1 > u0 ? (u1 - 1 - u0) / du * du : 0);
+  auto unit = [&](int u) { return turned ? usum - u : u; };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nrow = TS >> lq, npr = nrow / FX_WARPS;   // rows of a unit and of a warp: row0 + warp + 8 a
   const uint32_t ring = fx_s32(sh.ring[warp]), bars = fx_s32(sh.bar[warp]);
@@ -191,7 +197,7 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
   // the next unit from u on whose problem takes part, and its operand
   auto next_unit = [&](int u, TileJob& jb) {
     for (; u < u1; u += du) {
-      jb = jobs[u >> lq];
+      jb = jobs[unit(u) >> lq];
       if (prod_operands<double2, double>(probs[jb.prob], mode, io, x, y, sB)) break;
     }
     return u;
@@ -210,7 +216,7 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
   auto source = [&]() {
     if (pu >= u1) return;
     const Prob& p = probs[jp.prob];
-    const int64_t off = (int64_t)jp.t * (TS * TS) + ((pu & (nq - 1)) * nrow + warp) * TS;
+    const int64_t off = (int64_t)jp.t * (TS * TS) + ((unit(pu) & (nq - 1)) * nrow + warp) * TS;
     const bool pos = sB > 0.0;           // U, V = P, Q for the plus half, Q, P for the minus half
     srcA = (HASB && !pos ? p.Bfx : p.Afx) + off;
     if (HASB) srcB = (pos ? p.Bfx : p.Afx) + off;
@@ -244,7 +250,7 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
     jb = jn;
     const Prob& p = probs[jb.prob];
     const bool diag = jb.I == jb.J;
-    const int q = u & (nq - 1), row0 = q * nrow;
+    const int q = unit(u) & (nq - 1), row0 = q * nrow;
     const double2 xv = xn;
     un = next_unit(u + du, jn);
     if (un < u1) xn = x_value(jn);       // arrives under this unit's arithmetic

@@ -567,11 +567,12 @@ __device__ __forceinline__ void regrid(float S, float l, float gs, float& g, flo
 // x of every active problem, split once per product into chunks of 128 entries, one float4
 // record {hi_re, hi_im, lo_re, lo_im} per entry (2 KiB a chunk, so one bulk copy stages it),
 // with re and im exchanged in both pairs for the minus half (s = -1; see k_prod_tiles_mx),
-// and xmax[I] = max |hi| over chunk I; grid (maxnT, nprob), TS threads
+// and xmax[I] = max |hi| over chunk I; it also resets the ticket of the tiles' kernel; grid (maxnT, nprob), TS threads
 __global__ void __launch_bounds__(TS)
-k_mx_stage_x(const Prob* __restrict__ probs, int mode, GenericIO io) {
+k_mx_stage_x(const Prob* __restrict__ probs, int mode, GenericIO io, int* __restrict__ ticket) {
   dep_begin();
   clock_start(probs[0].clock);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;   // k_prod_tiles_mx's
   __shared__ float sm[TS / 32];
   const Prob& p = probs[blockIdx.y];
   const int I = blockIdx.x;
@@ -655,10 +656,17 @@ __device__ __forceinline__ void mx_copy(uint32_t dst, const void* src, uint32_t 
 // c_b = tx + 16 b, b < 8: one 16-byte shared load brings one record (UV and x alike), and the
 // 16 lanes of a row read 256 contiguous bytes.  Stage release: each warp arrives on empty[s]
 // when it is done with stage s; the producer (thread 0) waits for all warps before refilling.
-template <int NT>
+//
+// Who takes which tile.  One problem: CTA b takes b, b + gridDim.x, ... (or a block of them), and in
+// every other product of a chain (the plus halves) in the opposite order: what it read last is what
+// it wants first, and of 200 MB (N = 5000) a part is then still in the L2 (58.3 us a product, 59.4
+// without the turn, 63 with tickets).  Several problems end one by one, and a fixed share of the
+// tiles then leaves CTAs idle: they draw tickets (TICKET; 12 problems of 700 to 3000: 166 ms of
+// products against 177).  A tile's sums go to its own slots, whichever CTA forms them.
+template <int NT, bool TICKET>
 __global__ void __launch_bounds__(NT, 512 / NT)
 k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
-                GenericIO io, int strided, int beside, int* __restrict__ err) {
+                GenericIO io, int strided, int beside, int* __restrict__ ticket, int* __restrict__ err) {
   // beside = 1: the kernel before it in the stream runs the fine tiles; it waited for the staged
   // vector before it let this one start, so the two run side by side, and this one waits for it at
   // its end (whoever waits for this kernel finds both done)
@@ -673,6 +681,10 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
   const int t0 = strided ? blockIdx.x : blockIdx.x * per;
   const int t1 = strided ? njobs : min(njobs, t0 + per);
   const int dt = strided ? gridDim.x : 1;
+  // !TICKET: the job of position t is t, or, in the opposite order, tsum - t
+  const int tsum = 2 * t0 + (t1 > t0 ? (t1 - 1 - t0) / dt * dt : 0);
+  auto job_at = [&](int t) { return !TICKET && mode == PM_STEP_MPLUS ? tsum - t : t; };
+  __shared__ int sjob[TICKET ? 4 : 1];  // TICKET: job of tile ordinal n in sjob[n % 4]; -1: no more
   if (tid == 0) {
     for (int s = 0; s < C::NST; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mx_s32(&full[s])) : "memory");
@@ -686,16 +698,26 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
     double sb;
     return df_operands(probs[jobs[t].prob], mode, io, xx, sb);
   };
-  // producer cursor (thread 0): the next (job, slab) to copy, and the active-tile ordinal
-  int pt = t0, pa = 0, ptile = 0;
+  // producer cursor (thread 0): the next (position, slab) to copy, and the active-tile ordinal.
+  // TICKET: pa = -1 until the problem of ticket pt has been looked at; the ticket of the next tile is
+  // drawn two slabs ahead, so that nobody waits for it
+  int pt = t0, pa = TICKET ? -1 : 0, ptile = 0, nxt = 0;
+  if (TICKET && tid == 0) pt = atomicAdd(ticket, 1);
   long long issued = 0;
   bool pok = true;
   // issue every slab below `must` (waiting, bounded, for its stage to be released), then more
   // while stages happen to be free
   auto produce = [&](long long must) {
     while (pok) {
-      if (pa == 0) {
-        while (pt < t1 && !active(pt)) pt += dt;
+      if constexpr (TICKET) {
+        if (pa < 0) {
+          while (pt < njobs && !active(pt)) pt = atomicAdd(ticket, 1);
+          sjob[ptile & 3] = pt < njobs ? pt : -1;
+          pa = 0;
+        }
+        if (pt >= njobs) return;
+      } else if (pa == 0) {
+        while (pt < t1 && !active(job_at(pt))) pt += dt;
         if (pt >= t1) return;
       }
       const int s = (int)(issued % C::NST);
@@ -708,7 +730,7 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
           return;
         }
       }
-      const TileJob jb = jobs[pt];
+      const TileJob jb = jobs[job_at(pt)];
       const Prob& p = probs[jb.prob];
       const uint32_t bar = mx_s32(&full[s]);
       const uint32_t st = mx_s32(smx) + (uint32_t)s * C::STAGE;
@@ -723,25 +745,30 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
         mx_copy(xb + C::XBYTES, xs + (int64_t)jb.I * TS, C::XBYTES, bar);
       }
       ++issued;
-      if (++pa == C::SLABS) {
-        pa = 0;
-        pt += dt;
+      ++pa;
+      if (TICKET && pa == C::SLABS - 2) nxt = atomicAdd(ticket, 1);
+      if (pa == C::SLABS) {
+        pa = TICKET ? -1 : 0;
+        pt = TICKET ? nxt : pt + dt;
         ++ptile;
       }
     }
   };
   if (tid == 0) produce(0);
+  if (TICKET) __syncthreads();
   DFC(*red)[TS] = reinterpret_cast<DFC(*)[TS]>(smx + C::REDOFF);
   const f2 zero = pk(0.f, 0.f);
   long long consumed = 0;
   int ctile = 0;
   bool ok = true;
-  for (int t = t0; t < t1 && ok; t += dt) {
-    const TileJob jb = jobs[t];
+  for (int t = t0; ok; t += dt) {
+    const int jt = TICKET ? sjob[ctile & 3] : t < t1 ? job_at(t) : -1;
+    if (jt < 0) break;
+    const TileJob jb = jobs[jt];
     const Prob& p = probs[jb.prob];
     const double2* x;
     double sB;
-    if (!df_operands(p, mode, io, x, sB)) continue;   // uniform per CTA
+    if (!df_operands(p, mode, io, x, sB)) continue;   // uniform per CTA (TICKET: never)
     const bool diag = jb.I == jb.J;
     const float4* xc4 = reinterpret_cast<const float4*>(smx + C::XOFF + (ctile & 1) * 2 * C::XBYTES) + tx;
     const float4* xr4 = xc4 - tx + TS;                                       // row chunk I
@@ -845,7 +872,11 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
         part[((int64_t)jb.I * p.nT + jb.J) * TS + ty + C::ROWS * as] = dfc_pack(racc[0]);
       }
     }
-    if (__syncthreads_or(ok ? 0 : 1)) {
+    if (TICKET && tid == 0) {                  // the next tile's job is known to all behind the barrier
+      produce(consumed + 1);
+      if (!pok) atomicExch(err, 1);
+    }
+    if (__syncthreads_or(ok && (!TICKET || pok) ? 0 : 1)) {
       ok = false;
       break;
     }
@@ -1002,19 +1033,19 @@ void launch_product_df(const Prob* dprobs, const TileJob* jobs, int njobs, int n
 
 int product_mx_occupancy() { return 2; }   // shapes: 1 (512 threads) or 2 (256 threads) CTAs per SM
 
-template <int NT>
+template <int NT, bool TICKET>
 void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode, const GenericIO& io,
                ProdShape shape, int beside, int* err, cudaStream_t s) {
   using C = Mx<NT>;
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_prod_tiles_mx<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    cudaFuncSetAttribute(k_prod_tiles_mx<NT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncSetAttribute(k_prod_tiles_mx<NT, TICKET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    cudaFuncSetAttribute(k_prod_tiles_mx<NT, TICKET>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     attr = true;
   }
   const ProdShape ms{shape.ctas_per_sm < 0 ? -1 : C::CTAS, shape.strided};
-  launch_dep(k_prod_tiles_mx<NT>, product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s, dprobs, coarse, ncoarse, mode, io,
-             shape.strided, beside, err);
+  launch_dep(k_prod_tiles_mx<NT, TICKET>, product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s, dprobs, coarse, ncoarse,
+             mode, io, shape.strided, beside, err + 1, err);
 }
 
 void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, const TileJob* coarse, int ncoarse,
@@ -1024,7 +1055,7 @@ void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, co
   if (io_host) io = *io_host;
   if (ncoarse > 0) {
     count_launch();
-    launch_dep(k_mx_stage_x, dim3(maxnT, nprob), TS, 0, s, dprobs, mode, io);
+    launch_dep(k_mx_stage_x, dim3(maxnT, nprob), TS, 0, s, dprobs, mode, io, err + 1);
   }
   if (nfine > 0) {
     count_launch();
@@ -1037,8 +1068,9 @@ void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, co
     // shape.ctas_per_sm: 1 -> the 512-thread kernel, otherwise the 256-thread one (two CTAs per
     // SM; -1: one CTA per tile)
     const int beside = nfine > 0;
-    if (shape.ctas_per_sm == 1) launch_mx<512>(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s);
-    else launch_mx<256>(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s);
+    auto run = [&](auto launch) { launch(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s); };
+    if (nprob > 1) shape.ctas_per_sm == 1 ? run(launch_mx<512, true>) : run(launch_mx<256, true>);
+    else shape.ctas_per_sm == 1 ? run(launch_mx<512, false>) : run(launch_mx<256, false>);
   }
   count_launch();
   launch_prod_reduce_d(dprobs, nprob, maxnT, mode, io, s);
