@@ -187,9 +187,9 @@ def _config(ncv=0):
 
 
 # ------------------------------------------------------------------ GPU arm
-# dram__bytes_read.sum + dram__bytes_write.sum of one k_prod_tiles(+_df) launch at N = 8000
-# (profiles/k_prod_tiles_*_n8000.md); None until the current kernel has been captured
-TRAFFIC_N8000 = {"fp64": 1.057860e9 + 10.361088e6, "df": 1.067138e9 + 22.040064e6}
+# dram__bytes_read.sum + dram__bytes_write.sum of one k_prod_tiles_df launch at N = 8000
+# (profiles/k_prod_tiles_df_n8000.md); None until the current kernel has been captured
+TRAFFIC_N8000 = {"fp64": None, "df": 1.067138e9 + 22.040064e6}
 
 
 def run_gpu(args):
@@ -313,9 +313,9 @@ def run_gpu(args):
         return
     cpu_v, cpu_raw = cpu_baseline_sample()
     value = ms_max / 1e3
-    # DRAM traffic per launch from the ncu captures at N = 8000 (profiles/k_prod_tiles_c128_n8000.md,
-    # profiles/k_prod_tiles_df_n8000.md): bytes per stored 128x128 tile pair, scaled by the tile
-    # count of this workload (traffic grows with the number of tiles streamed)
+    # DRAM traffic per launch from the ncu captures at N = 8000 (profiles/k_prod_tiles_df_n8000.md):
+    # bytes per stored 128x128 tile pair, scaled by the tile count of this workload (traffic grows
+    # with the number of tiles streamed)
     n_tiles_8000 = 63 * 64 // 2
     captured = TRAFFIC_N8000.get("df" if args.df else "fp64")
     traffic = None if captured is None else captured / (2 * n_tiles_8000) * 2 * (n_tiles * (n_tiles + 1) // 2)
@@ -326,15 +326,16 @@ def run_gpu(args):
                           "split complex128 tiles, 16 B per element)",
                 "peak_kind": peak_kind, "achieved_fp64_equiv_tflops": achieved_tf}
     else:
-        roof = {"bound": "alu", "achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s",
-                "frac": achieved_tf / fp64_peak, "traffic": traffic,
+        # the products run in fixed point on the integer pipe, above the FP64 FMA rate: HBM is the bound
+        roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": peaks.get("hbm_gbs"), "unit": "GB/s",
+                "frac": achieved_gbs / peaks.get("hbm_gbs", 6800.0), "traffic": traffic,
                 "algorithmic_bytes": per_launch_bytes,
-                "kernel": "k_prod_tiles + k_prod_reduce (one folded product M+/M- over packed A and B)",
-                "peak_note": "FP64 FMA peak measured in this run (bse_measure_fp64_peak: 8 independent FMA "
+                "kernel": "k_prod_tiles_fx + k_prod_reduce (one folded product M+/M- over packed A and B)",
+                "fp64_equiv_tflops": achieved_tf, "fp64_fma_peak": fp64_peak,
+                "fp64_frac": achieved_tf / fp64_peak,
+                "peak_note": "fp64_fma_peak: measured in this run (bse_measure_fp64_peak: 8 independent FMA "
                              f"chains per thread on every SM, {fp64_ms:.1f} ms launch, CUDA events)",
-                "peak_kind": "measured", "peak_clocks": clocks64,
-                "achieved_hbm_gbs": achieved_gbs, "hbm_peak_gbs": peaks.get("hbm_gbs"),
-                "hbm_frac": achieved_gbs / peaks.get("hbm_gbs", 6800.0), "hbm_peak_kind": peak_kind}
+                "peak_kind": peak_kind, "peak_clocks": clocks64}
     line = {
         "metric": METRIC, "value": value, "unit": "s", "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": False, "scaling": "weak",

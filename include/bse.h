@@ -62,7 +62,10 @@ typedef enum bse_dtype {
      FP64 projected eigenproblem, Ritz coefficients, final residuals and
      Rayleigh-quotient refinement (the mixed-precision path) */
   BSE_C64 = 0,
-  /* complex128 storage; FP64 products (the FP64 path) */
+  /* complex128 storage; products to FP64 accuracy or better (the FP64 path):
+     60-bit fixed point on a second copy of the packed tiles, made when it
+     fits in a third of the free memory; FP64 FMAs otherwise, and on tiles
+     whose entries fixed point does not suit */
   BSE_C128 = 1,
   /* complex64 input and storage of A and B (half the bytes of BSE_C128);
      FP64 Krylov basis; the Lanczos products in double-FP32 arithmetic on

@@ -30,3 +30,26 @@ def test_batched_uneven(dtype, tol, rtol):
         assert res.max() < (1e-10 if dtype == "c128" else 1e-5)   # complex64 vectors as returned
         assert bs.residuals(i).max() <= tol                        # the solver's FP64 check
     bs.close()
+
+
+@pytest.mark.parametrize("sizes", [[129, 257], [2300, 129, 1000, 2300]])
+def test_batched_tiles_by_ticket(sizes):
+    """A mixed batch hands its coarse tiles out by ticket (fewer tiles than CTAs, and more), a single
+    problem in fixed shares: both solve to the same values within the tolerance of the solve."""
+    from paper_2504_10096_gb300 import bse
+    probs = []
+    for i, n in enumerate(sizes):
+        g = torch.Generator(device="cuda").manual_seed(70 + i)
+        rnd = lambda: torch.randn(n, n, generator=g, device="cuda") * 1e-4
+        A, B = torch.complex(rnd(), rnd()), torch.complex(rnd(), rnd())
+        A = (A + A.mH) / 2 + torch.diag(torch.linspace(1.0, 12.0, n, device="cuda")).to(A.dtype)
+        probs.append((A.contiguous(), ((B + B.mT) / 2).contiguous()))
+    bs = bse.BatchedSolver([a for a, _ in probs], [b for _, b in probs], mixed=True)
+    vals, _, nconv = bs.solve(4, tol=1e-6)
+    bs.close()
+    for i, (a, b) in enumerate(probs):
+        s = bse.Solver(a, b, mixed=True)
+        ref = s.solve(4, tol=1e-6)[0]
+        s.close()
+        assert nconv[i] == 4
+        np.testing.assert_allclose(vals[i], ref, rtol=2e-6, atol=0)   # each within tol of the exact value
