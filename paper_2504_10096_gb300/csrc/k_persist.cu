@@ -11,6 +11,11 @@
 // KState: the step loop stops when the subspace is full, a breakdown asks the host for a fresh
 // vector, or the problem is done; the restart itself stays with the per-phase kernels.
 //
+// What bounds it: the latency of a phase's loads and of its barrier (1.1-2 us), and in larger problems
+// the integer pipe in the tiles.  Per step: TDA N = 2000, complex128, 36 us (tiles 14, reduction 2.3, dots
+// 2 x 2.5, updates 2 x 4.5, normalisation 2.6, the rest barriers), 82 us with FP64-pipe tiles; PH
+// N = 3000 99 us (tiles 2 x 30), 225 before.
+//
 // The grid barrier counts arrivals; every wait is bounded (about a second of polling), after
 // which the CTA raises the barrier's error flag and returns, and the others' waits expire in turn,
 // so a wait can never hang the device.  The launch is
