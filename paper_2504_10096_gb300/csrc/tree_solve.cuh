@@ -231,9 +231,11 @@ __device__ inline void solve_tree(const TV& T, const Fact& F, double* x, int lan
   double s = 0.0;
   for (int i = lane; i < h; i += 32) s = fma(T.b[i] * x[i], F.invd[i], s);
   s = warp_sum(s);
+  // every lane runs the recurrence, one of them stores: each entry is read by all before it is rewritten
   double cur = y[0] - s;
   for (int t = 0; t + 1 < q; ++t) {
     const double nx = y[t + 1];
+    __syncwarp();
     if (F.piv[t] == 0) {
       if (lane == 0) y[t] = cur;
       cur = fma(-F.dl[t], cur, nx);
