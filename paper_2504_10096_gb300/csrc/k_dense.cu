@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(256) k_dn_panel(double* __restrict__ M, int64_
   for (int c = 0; c < kb; ++c) {
     if (warp == 0) {
       double d = a[c][c];
+      __syncwarp();                    // lane c rewrites it below
       const bool bad = !(d > 0.0);     // M_r not positive definite: flag it, keep the numbers finite
       if (bad) d = 1.0;
       const double r = rsqrt(d);

@@ -66,3 +66,46 @@ int main() {{
     assert up == down
     # backward stable: ||T x - r|| <= c n u ||T|| ||x||
     assert np.linalg.norm(m @ up - r) <= 64 * n * 2.0 ** -53 * np.linalg.norm(m, 2) * np.linalg.norm(up)
+
+
+PANEL = r"""
+#include "simt.h"
+#define __restrict__
+namespace bse {
+constexpr int DNB = 32;
+%s
+}
+using namespace bse;
+int main(int, char** argv) {
+  const int n = atoi(argv[1]), ld = (n + 31) / 32 * 32, kb = std::min(n, DNB), nt = std::max(1, (n - kb + 31) / 32);
+  for (int desc = 0; desc < 2; ++desc) {
+    std::vector<double> M(ld * n), D(DNB * DNB);
+    int notpd = 0;
+    for (int j = 0; j < n; ++j)
+      for (int i = 0; i < n; ++i) M[j * ld + i] = (i == j ? n + 1.0 : 0.0) + std::cos(0.7 * (i - j) * (i - j));
+    for (int b = 0; b < nt; ++b) {
+      blockIdx.x = b;
+      if (!simt::run_block(256, desc, [&] { k_dn_panel(M.data(), ld, n, 0, kb, D.data(), &notpd); })) return 1;
+    }
+    for (int c = 0; c < kb; ++c)
+      for (int r = c; r < kb; ++r) M[c * ld + r] = D[c * DNB + r];
+    for (int c = 0; c < kb; ++c)
+      for (int r = 0; r < n; ++r) printf("%%.17g ", r < c ? 0.0 : M[c * ld + r]);
+    printf("%%d\n", notpd);
+  }
+}
+"""
+
+
+@pytest.mark.parametrize("n", [1, 17, 32, 33, 75])
+def test_cholesky_panel_does_not_depend_on_the_order_of_threads(tmp_path, n):
+    """The first panel of the dense method's Cholesky factorisation, both orders of a CTA's threads."""
+    src = PANEL % cut("k_dense.cu", "__global__ void __launch_bounds__(256) k_dn_panel", "// trailing update")
+    up, down = run(tmp_path, src, n)
+    assert up == down
+    k = min(n, 32)
+    i = np.arange(n)
+    m = np.cos(0.7 * (i[:, None] - i[None, :]) ** 2) + (n + 1.0) * np.eye(n)
+    ref = np.linalg.cholesky(m)[:, :k]
+    assert up[-1] == 0
+    np.testing.assert_allclose(np.reshape(up[:-1], (k, n)).T, ref, rtol=0, atol=64 * n * 2.0 ** -53 * np.sqrt(n + 2))
