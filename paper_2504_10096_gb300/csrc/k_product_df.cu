@@ -124,10 +124,12 @@ __device__ __forceinline__ bool df_operands(const Prob& p, int mode, const Gener
 // Cross-lane reduction of a tile's partial sums into the two partial-sum
 // slots (I, J) and (J, I): racc[a] = this thread's sum of row ty + 16a over
 // its 8 columns, cacc[b] = its sum of column tx + 16b over its 8 rows.
-// `red` is shared scratch of 8 x TS DFC (callers alias it with their row park).
+// `red` is shared scratch of 8 x TS DFC (callers alias it with their row park); 256 threads tid, which
+// meet at sync().
+template <typename Sync>
 __device__ __forceinline__ void df_tile_reduce(DFC (&racc)[8], DFC (&cacc)[8], DFC (*red)[TS], bool diag,
-                                               const Prob& p, const TileJob& jb) {
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+                                               const Prob& p, const TileJob& jb, int tid, Sync sync) {
+  const int tx = tid & 15, ty = tid >> 4;
   const int lane = tid & 31, warp = tid >> 5;
   {
     const bool u8 = tx & 8;
@@ -160,7 +162,7 @@ __device__ __forceinline__ void df_tile_reduce(DFC (&racc)[8], DFC (&cacc)[8], D
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) red[warp][tx + 16 * (q + (up ? 4 : 0))] = cacc[q];
-    __syncthreads();
+    sync();
     if (tid < TS) {
       DFC s = red[0][tid];
 #pragma unroll
@@ -283,7 +285,7 @@ k_prod_tiles_df(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
 #pragma unroll
     for (int a = 0; a < 8; ++a) racc[a] = rpark[a][tid];
     __syncthreads();   // rpark is reused below as the column-reduction buffer
-    df_tile_reduce(racc, cacc, red, diag, p, jb);
+    df_tile_reduce(racc, cacc, red, diag, p, jb, tid, [] { __syncthreads(); });
   }
 }
 
@@ -374,35 +376,36 @@ __device__ __forceinline__ XPack xpack(double2 v, bool row) {
   return o;
 }
 
-__global__ void __launch_bounds__(PROD_THREADS, 2)
-k_prod_tiles_df2(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
-                 GenericIO io, int strided, int first) {
-  dep_begin();
-  if (first) clock_start(probs[0].clock);
-  __shared__ XPack xc[TS], xr[TS];
-  __shared__ DFC rpark[8][PROD_THREADS];
+struct Df2Shared {
+  XPack xc[TS], xr[TS];
+  DFC rpark[8][PROD_THREADS];
+};
+
+// The tiles t0, t0 + dt, ... of `jobs` by 256 threads tid, which meet at sync().
+template <typename Sync>
+__device__ __forceinline__ void df2_tiles(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int t0,
+                                          int t1, int dt, int mode, const GenericIO& io, int tid, Df2Shared& sh,
+                                          Sync sync) {
+  XPack *xc = sh.xc, *xr = sh.xr;
+  DFC(*rpark)[PROD_THREADS] = sh.rpark;
   DFC(*red)[TS] = reinterpret_cast<DFC(*)[TS]>(&rpark[0][0]);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int per = strided ? 1 : (njobs + gridDim.x - 1) / gridDim.x;
-  const int t0 = strided ? blockIdx.x : blockIdx.x * per;
-  const int t1 = strided ? njobs : min(njobs, t0 + per);
-  const int dt = strided ? gridDim.x : 1;
+  const int tx = tid & 15, ty = tid >> 4;
   const f2 zero = pk(0.f, 0.f);
   for (int t = t0; t < t1; t += dt) {
     const TileJob jb = jobs[t];
     const Prob& p = probs[jb.prob];
     const double2* x;
     double sB;
-    if (!df_operands(p, mode, io, x, sB)) continue;   // uniform per CTA
+    if (!df_operands(p, mode, io, x, sB)) continue;   // the same for all threads
     const bool diag = jb.I == jb.J;
-    __syncthreads();
+    sync();
     {
       const int r = tid & (TS - 1);
       const double2 v = x[(int64_t)(tid < TS ? jb.J : jb.I) * TS + r];
       if (tid < TS) xc[r] = xpack(v, false);
       else xr[r] = xpack(v, true);
     }
-    __syncthreads();
+    sync();
     using TT = float2;                              // exact complex64 A and B
     const TT* At = (const TT*)p.A + (int64_t)jb.t * (TS * TS);
     const TT* Bt = (const TT*)p.B + (int64_t)jb.t * (TS * TS);
@@ -483,9 +486,22 @@ k_prod_tiles_df2(const Prob* __restrict__ probs, const TileJob* __restrict__ job
     }
 #pragma unroll
     for (int a = 0; a < 8; ++a) racc[a] = rpark[a][tid];
-    __syncthreads();   // rpark is reused below as the column-reduction buffer
-    df_tile_reduce(racc, cacc, red, diag, p, jb);
+    sync();   // rpark is reused below as the column-reduction buffer
+    df_tile_reduce(racc, cacc, red, diag, p, jb, tid, sync);
   }
+}
+
+// every tile exact (no coarse ones beside them)
+__global__ void __launch_bounds__(PROD_THREADS, 2)
+k_prod_tiles_df2(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
+                 GenericIO io, int strided) {
+  dep_begin();
+  clock_start(probs[0].clock);
+  __shared__ Df2Shared sh;
+  const int per = strided ? 1 : (njobs + gridDim.x - 1) / gridDim.x;
+  const int t0 = strided ? blockIdx.x : blockIdx.x * per;
+  df2_tiles(probs, jobs, t0, strided ? njobs : min(njobs, t0 + per), strided ? gridDim.x : 1, mode, io, threadIdx.x, sh,
+            [] { __syncthreads(); });
 }
 
 // ---------------------------------------------------------------------------
@@ -663,24 +679,34 @@ __device__ __forceinline__ void mx_copy(uint32_t dst, const void* src, uint32_t 
 // without the turn, 63 with tickets).  Several problems end one by one, and a fixed share of the
 // tiles then leaves CTAs idle: they draw tickets (TICKET; 12 problems of 700 to 3000: 166 ms of
 // products against 177).  A tile's sums go to its own slots, whichever CTA forms them.
+//
+// The first nfb CTAs take the fine tiles instead (df2_tiles; NT = 512: one tile per half of the CTA), so
+// that the two kinds run side by side in one launch.
 template <int NT, bool TICKET>
 __global__ void __launch_bounds__(NT, 512 / NT)
 k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs, int njobs, int mode,
-                GenericIO io, int strided, int beside, int* __restrict__ ticket, int* __restrict__ err) {
-  // beside = 1: the kernel before it in the stream runs the fine tiles; it waited for the staged
-  // vector before it let this one start, so the two run side by side, and this one waits for it at
-  // its end (whoever waits for this kernel finds both done)
-  if (!beside) dep_wait();
-  dep_launch();
+                GenericIO io, int strided, const TileJob* __restrict__ fine, int nfine, int nfb,
+                int* __restrict__ ticket, int* __restrict__ err) {
+  dep_begin();
   using C = Mx<NT>;
   extern __shared__ __align__(128) unsigned char smx[];
+  if ((int)blockIdx.x < nfb) {
+    constexpr int W = NT / PROD_THREADS;           // tiles at a time
+    static_assert(W * sizeof(Df2Shared) <= C::SMEM, "the fine tiles' buffers");
+    const int w = threadIdx.x / PROD_THREADS;
+    Df2Shared& sh = reinterpret_cast<Df2Shared*>(smx)[w];
+    auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(w + 1), "n"(PROD_THREADS) : "memory"); };
+    df2_tiles(probs, fine, blockIdx.x * W + w, nfine, nfb * W, mode, io, threadIdx.x % PROD_THREADS, sh, sync);
+    return;
+  }
+  const int bid = blockIdx.x - nfb, nblk = gridDim.x - nfb;
   __shared__ uint64_t full[C::NST], empty[C::NST];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int lane = tid & 31, warp = tid >> 5;
-  const int per = strided ? 1 : (njobs + gridDim.x - 1) / gridDim.x;
-  const int t0 = strided ? blockIdx.x : blockIdx.x * per;
+  const int per = strided ? 1 : (njobs + nblk - 1) / nblk;
+  const int t0 = strided ? bid : bid * per;
   const int t1 = strided ? njobs : min(njobs, t0 + per);
-  const int dt = strided ? gridDim.x : 1;
+  const int dt = strided ? nblk : 1;
   // !TICKET: the job of position t is t, or, in the opposite order, tsum - t
   const int tsum = 2 * t0 + (t1 > t0 ? (t1 - 1 - t0) / dt * dt : 0);
   auto job_at = [&](int t) { return !TICKET && mode == PM_STEP_MPLUS ? tsum - t : t; };
@@ -937,7 +963,6 @@ k_prod_tiles_mx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
       mx_wait(mx_s32(&full[g % C::NST]), (uint32_t)((g / C::NST) & 1));
   }
   __syncthreads();
-  if (beside) dep_wait();
 }
 
 // records {U_re, V_re, U_im, V_im} of U = fl(A + B), V = fl(A - B) for every packed element
@@ -1011,7 +1036,7 @@ void launch_df(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, con
   // complex128 tiles: the scalar kernel (its float4 rows leave the packed one no registers for
   // latency hiding: 0.274 vs 0.250 ms at N = 8000)
   if constexpr (HASB && !SPLIT)
-    launch_dep(k_prod_tiles_df2, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided, 1);
+    launch_dep(k_prod_tiles_df2, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided);
   else
     launch_dep(k_prod_tiles_df<HASB, SPLIT>, grid, PROD_THREADS, 0, s, dprobs, jobs, njobs, mode, io, shape.strided);
 }
@@ -1035,7 +1060,7 @@ int product_mx_occupancy() { return 2; }   // shapes: 1 (512 threads) or 2 (256 
 
 template <int NT, bool TICKET>
 void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode, const GenericIO& io,
-               ProdShape shape, int beside, int* err, cudaStream_t s) {
+               ProdShape shape, const TileJob* fine, int nfine, int* err, cudaStream_t s) {
   using C = Mx<NT>;
   static bool attr = false;
   if (!attr) {
@@ -1044,8 +1069,10 @@ void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode,
     attr = true;
   }
   const ProdShape ms{shape.ctas_per_sm < 0 ? -1 : C::CTAS, shape.strided};
-  launch_dep(k_prod_tiles_mx<NT, TICKET>, product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s, dprobs, coarse, ncoarse,
-             mode, io, shape.strided, beside, err + 1, err);
+  constexpr int W = NT / PROD_THREADS;
+  const int nfb = std::min((nfine + W - 1) / W, C::CTAS * num_sms());
+  launch_dep(k_prod_tiles_mx<NT, TICKET>, nfb + product_grid(C::CTAS, ms, ncoarse), NT, C::SMEM, s, dprobs, coarse, ncoarse,
+             mode, io, shape.strided, fine, nfine, nfb, err + 1, err);
 }
 
 void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, const TileJob* coarse, int ncoarse,
@@ -1053,22 +1080,16 @@ void launch_product_mixed(const Prob* dprobs, const TileJob* fine, int nfine, co
                           cudaStream_t s) {
   GenericIO io{};
   if (io_host) io = *io_host;
-  if (ncoarse > 0) {
+  if (ncoarse == 0) {
     count_launch();
+    launch_dep(k_prod_tiles_df2, product_grid(df_occupancy<true, false>(), ProdShape{0, 1}, nfine), PROD_THREADS, 0, s,
+               dprobs, fine, nfine, mode, io, 1);
+  } else {
+    count_launch(2);
     launch_dep(k_mx_stage_x, dim3(maxnT, nprob), TS, 0, s, dprobs, mode, io, err + 1);
-  }
-  if (nfine > 0) {
-    count_launch();
-    const ProdShape fs{0, 1};
-    launch_dep(k_prod_tiles_df2, product_grid(df_occupancy<true, false>(), fs, nfine), PROD_THREADS, 0, s, dprobs, fine,
-               nfine, mode, io, 1, ncoarse > 0 ? 0 : 1);
-  }
-  if (ncoarse > 0) {
-    count_launch();
     // shape.ctas_per_sm: 1 -> the 512-thread kernel, otherwise the 256-thread one (two CTAs per
     // SM; -1: one CTA per tile)
-    const int beside = nfine > 0;
-    auto run = [&](auto launch) { launch(dprobs, coarse, ncoarse, mode, io, shape, beside, err, s); };
+    auto run = [&](auto launch) { launch(dprobs, coarse, ncoarse, mode, io, shape, fine, nfine, err, s); };
     if (nprob > 1) shape.ctas_per_sm == 1 ? run(launch_mx<512, true>) : run(launch_mx<256, true>);
     else shape.ctas_per_sm == 1 ? run(launch_mx<512, false>) : run(launch_mx<256, false>);
   }
