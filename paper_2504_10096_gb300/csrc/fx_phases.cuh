@@ -88,12 +88,12 @@ __device__ __forceinline__ void fx_copy(uint32_t dst, const void* src, uint32_t 
 
 __device__ __forceinline__ unsigned int hi_abs(double v) { return (unsigned int)__double2hiint(v) & 0x7fffffffu; }
 
-// round(v 2^59 / 2^(e - 1022)): v's magnitude is below 2^(e - 1022), e a biased exponent >= 64
+// round(v 2^59 / 2^(e - 1022)): v's magnitude is below 2^(e - 1022), e a biased exponent >= 1
 __device__ __forceinline__ long long fx_fixed(double v, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   const int ev = (int)(b >> 52) & 0x7ff;
-  const int d = e - ev;
-  unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 6;
+  const int d = e - max(ev, 1);
+  unsigned long long m = ((b & 0xfffffffffffffull) | (ev ? 0x10000000000000ull : 0ull)) << 6;
   m = d > 0 ? ((m >> (min(d, 63) - 1)) + 1) >> 1 : m;
   const long long f = d < 62 ? (long long)m : 0ll;
   return (long long)b < 0 ? -f : f;
@@ -145,10 +145,11 @@ __device__ __forceinline__ double fx_pack_double(long long h, unsigned long long
     m = l << n;
     q = -n;
   }
-  const unsigned long long r = (m >> 11) + ((m >> 10) & 1);      // 53 bits, rounded
   const int e = q + 63 + (eu + ex - 2044 - 72) + 1023;
-  unsigned long long b = ((unsigned long long)(e - 1) << 52) + r;
-  if (e < 1 || m == 0) b = 0;
+  const int sub = max(0, min(1 - e, 52));                        // bits a subnormal result loses
+  const unsigned long long r = (m >> (11 + sub)) + ((m >> (10 + sub)) & 1);      // 53 bits or fewer, rounded
+  unsigned long long b = ((unsigned long long)(max(e, 1) - 1) << 52) + r;
+  if (m == 0 || e < -52) b = 0;
   if (e > 2046) b = 0x7ff0000000000000ull;
   if (ex == 2047) b = 0x7ff8000000000000ull;
   return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
@@ -262,7 +263,7 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
     __syncthreads();
     auto chunk_exp = [&](int k) {
       const unsigned int m = max(max(sh.mx[k][0], sh.mx[k][1]), max(sh.mx[k][2], sh.mx[k][3]));
-      return max(64, (int)(m >> 20));
+      return max(1, (int)(m >> 20));
     };
     const int ec = chunk_exp(0), er = chunk_exp(1);
     sh.x[tid >> 7][tid & (TS - 1)] = fx_entry(xv, tid < TS ? ec : er);

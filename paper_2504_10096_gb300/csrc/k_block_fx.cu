@@ -46,7 +46,9 @@ k_block_stage(const double2* __restrict__ xa, const double2* __restrict__ xb, in
     b = xb ? xb[c * ldx + r] : conjc(a);
     b = cscale(b, sB);
     if (PQ) {
-      const double2 s = cscale(cadd(a, b), 0.5), d = cscale(csub(a, b), 0.5);
+      a = cscale(a, 0.5);                // halves first: the sum of two large entries stays finite
+      b = cscale(b, 0.5);
+      const double2 s = cadd(a, b), d = csub(a, b);
       a = s;
       b = d;
     }
@@ -57,7 +59,7 @@ k_block_stage(const double2* __restrict__ xa, const double2* __restrict__ xb, in
   if ((tid & 31) == 0) smx[tid >> 5] = m;
   __syncthreads();
   m = max(max(smx[0], smx[1]), max(smx[2], smx[3]));
-  const int e = max(64, (int)(m >> 20));
+  const int e = max(1, (int)(m >> 20));
   F0[c * Npad + r] = fx_entry(a, e);
   if (HASB) F1[c * Npad + r] = fx_entry(b, e);
   if (tid == 0) E[(int64_t)c * nT + blockIdx.x] = e;

@@ -149,11 +149,22 @@ inline T warp_fold(T v, F f) {
 
 inline void __syncwarp(unsigned = 0xffffffffu) { simt::wait_at(simt::AT_WARP); }
 inline void __syncthreads() { simt::wait_at(simt::AT_BLOCK); }
+inline int __syncthreads_or(int v) {
+  static int any;
+  any = 0;
+  __syncthreads();
+  any |= v;
+  __syncthreads();
+  return any != 0;
+}
 template <typename T> inline T __shfl_xor_sync(unsigned, T v, int m) { return simt::exchange(v, (threadIdx.x & 31) ^ m); }
 template <typename T> inline T __shfl_sync(unsigned, T v, int src) { return simt::exchange(v, src); }
 inline int __reduce_add_sync(unsigned, int v) { return simt::warp_fold(v, [](int a, int b) { return a + b; }); }
 inline unsigned __reduce_max_sync(unsigned, unsigned v) {
   return simt::warp_fold(v, [](unsigned a, unsigned b) { return a > b ? a : b; });
+}
+inline unsigned __reduce_min_sync(unsigned, unsigned v) {
+  return simt::warp_fold(v, [](unsigned a, unsigned b) { return a < b ? a : b; });
 }
 inline long long __double_as_longlong(double v) { long long u; std::memcpy(&u, &v, 8); return u; }
 inline double __longlong_as_double(long long u) { double v; std::memcpy(&v, &u, 8); return v; }

@@ -1,0 +1,58 @@
+"""complex128 products on matrices and vectors whose entries differ by many orders of magnitude, element
+by element against |M||x|: a product that is accurate only against the largest entry of a tile or of a
+chunk of the vector does not pass.  The constant is that of the other product tests (a few tens of
+roundings per entry), also where one entry of x is far above the others."""
+import numpy as np
+import pytest
+
+from tests.gpu_common import UNIT, assert_elementwise, product_bound
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _matrices(rng, n):
+    """Dense Hermitian A with a small diagonal, dense symmetric B."""
+    g = lambda: rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))        # noqa: E731
+    a, b = g(), g()
+    return (a + a.conj().T) / 2, (b + b.T) / 4
+
+
+def _graded(a, b, d):
+    return a * d[:, None] * d[None, :], b * d[:, None] * d[None, :]
+
+
+def _cases(n):
+    rng = np.random.default_rng(n)
+    a, b = _matrices(rng, n)
+    x = rng.standard_normal((n, 1)) + 1j * rng.standard_normal((n, 1))
+    yield "x of 1e-300", a, b, 1e-300 * x
+    yield "x near the smallest normal number", 2.0 ** 40 * a, 2.0 ** 40 * b, 2.0 ** -1015 * x
+    yield "x of 1e300", 2.0 ** -40 * a, 2.0 ** -40 * b, 1e300 * x
+
+
+NAMES = [c[0] for c in _cases(3)]
+
+
+@pytest.mark.parametrize("form", ["ph", "tda"])
+@pytest.mark.parametrize("n", [96, 300])
+@pytest.mark.parametrize("name", NAMES)
+def test_every_entry(name, n, form):
+    from paper_2504_10096_gb300 import bse
+    _, a, b, x = next(c for c in _cases(n) if c[0] == name)
+    s = bse.Solver(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda() if form == "ph" else None)
+    L = np.clongdouble
+    al, bl, xl = a.astype(L), b.astype(L), x.astype(L)
+    ops = [(bse.BSE_OP_A, "a", al @ xl)]
+    if form == "ph":
+        ops += [(bse.BSE_OP_MPLUS, "mplus", al @ xl + bl @ xl.conj()),
+                (bse.BSE_OP_MMINUS, "mminus", al @ xl - bl @ xl.conj())]
+    for op, kind, ref in ops:
+        # scaled to keep the checks' own squares and sums in range
+        f = 2.0 ** np.round(-np.log2(np.abs(ref).max().astype(float)))
+        bound = product_bound(a, b, x * f, kind)
+        for k in (1, 3):
+            y = s.apply(op, torch.from_numpy(np.repeat(x, k, 1)).cuda()).cpu().numpy()
+            for c in range(k):
+                assert_elementwise(y[:, c:c + 1] * f, (ref * f).astype(complex), bound, UNIT["c128"], 64, f"{name}, {kind}, k = {k}")
+    s.close()
