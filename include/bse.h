@@ -62,10 +62,15 @@ typedef enum bse_dtype {
      FP64 projected eigenproblem, Ritz coefficients, final residuals and
      Rayleigh-quotient refinement (the mixed-precision path) */
   BSE_C64 = 0,
-  /* complex128 storage; products to FP64 accuracy or better (the FP64 path):
+  /* complex128 storage; products to FP64 accuracy (the FP64 path): each entry
+     of Y = M X is off by at most a few tens of 2^-53 (|M||X|)_i.  They run in
      60-bit fixed point on a second copy of the packed tiles, made when it
-     fits in a third of the free memory; FP64 FMAs otherwise, and on tiles
-     whose entries fixed point does not suit */
+     fits in a third of the free memory, on every 128 x 128 tile whose entries
+     lie within a factor 2^14 of one another (entries of X may differ by any
+     factor), and in FP64 FMAs otherwise.  Where X has one entry far above all
+     others of its 128-entry chunk, an entry of Y that couples to it by 2^-s
+     of the tile's largest element may be off by 2^(s - 59) of that coupling
+     (s <= 14) */
   BSE_C128 = 1,
   /* complex64 input and storage of A and B (half the bytes of BSE_C128);
      FP64 Krylov basis; the Lanczos products in double-FP32 arithmetic on

@@ -15,11 +15,15 @@
 // value per tile, row and column, built with integer instructions.
 //
 // Accuracy.  Each entry of U and of x is off by at most 2^-60 of its tile's or chunk's 2^E, each
-// product by 2^-60 (the dropped term); the sums add nothing.  An FP64 dot product rounds every
-// partial sum at 2^-53, so the fixed-point one is the more accurate of the two as long as the
-// tile's largest entry is not far above its typical one.  Where it is -- peak^2 above
-// FX_PEAK^2 mean square, an infinity, a NaN, or exponents near the ends of the FP64 range -- the
-// tile stays on the FP64 kernel (k_fx_pack writes the decision).  The diagonal of the matrix,
+// product by 2^-60 (the dropped term); the sums add nothing.  So what a tile adds to a row is off by
+// some 2^-57 max|U| max|x| (about 2^-59 when one entry of x is far above the others), where an FP64 dot
+// product is off by 2^-53 of the row's own sum of magnitudes |U||x|.  That sum is at least min|U| max|x|:
+// a tile runs in fixed point only when every entry of the matrix in it is within 2^FX_SPREAD of its
+// largest (k_fx_pack; in the diagonal tiles the diagonal counts as one of the entries), whatever x is.
+// Sparse tiles, graded rows or columns, a peak, an infinity, a NaN, or exponents near the ends of the
+// FP64 range keep a tile on the FP64 kernel.  2^14 lets complex tiles without structure pass (the
+// spread of 16384 complex Gaussian entries is 2^9 to 2^13 for one matrix, 2^5 to 2^10 for the pair A, B);
+// x may have any exponent, subnormals included.  The diagonal of the matrix,
 // which holds the transition energies far above everything else in its tiles, is left out of the
 // tiles (zeros there) and added in FP64 by the block-row reduction.
 //
@@ -37,7 +41,7 @@ namespace bse {
 
 constexpr int FX_THREADS = 256;
 constexpr int FX_WARPS = FX_THREADS / 32;
-constexpr float FX_PEAK = 64.f;
+constexpr int FX_SPREAD = 14;        // largest over smallest entry of a fixed-point tile, log2
 
 constexpr long long FX_SPIN = 1ll << 24;      // polls of one wait for a row
 

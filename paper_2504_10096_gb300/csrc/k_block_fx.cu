@@ -72,31 +72,31 @@ k_block_scale64(const float2* __restrict__ A, const float2* __restrict__ B, int6
   const int I = blockIdx.y, J = blockIdx.x;
   if (J < I) return;
   const int64_t t = (int64_t)I * nT - (int64_t)I * (I - 1) / 2 + (J - I);
-  __shared__ float smx[8], ssq[8];
+  __shared__ float smx[8], smn[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float m = 0.f, s = 0.f;
+  const int nr = (int)min((int64_t)TS, N - (int64_t)I * TS), nc = (int)min((int64_t)TS, N - (int64_t)J * TS);
+  float m = 0.f, mn = INFINITY;
   bool bad = false;
   for (int e = tid; e < TS * TS; e += 256) {
-    if (I == J && (e >> 7) == (e & (TS - 1))) continue;
     const float2 a = A[t * (TS * TS) + e], b = HASB ? B[t * (TS * TS) + e] : make_float2(0.f, 0.f);
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y))));
-    s += a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y;
+    const float v = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
+    if ((e >> 7) < nr && (e & (TS - 1)) < nc) mn = fminf(mn, v);
+    if (I == J && (e >> 7) == (e & (TS - 1))) continue;
+    m = fmaxf(m, v);
     bad |= !(isfinite(a.x) && isfinite(a.y) && isfinite(b.x) && isfinite(b.y));
   }
 #pragma unroll
   for (int k = 16; k >= 1; k >>= 1) {
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
-    s += __shfl_xor_sync(0xffffffffu, s, k);
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, k));
   }
-  if (lane == 0) { smx[warp] = m; ssq[warp] = s; }
+  if (lane == 0) { smx[warp] = m; smn[warp] = mn; }
   const bool any_bad = __syncthreads_or(bad ? 1 : 0);
   if (tid == 0) {
-    for (int w = 1; w < 8; ++w) { m = fmaxf(m, smx[w]); s += ssq[w]; }
-    const int64_t nr = min((int64_t)TS, N - (int64_t)I * TS), nc = min((int64_t)TS, N - (int64_t)J * TS);
-    const float count = (float)(nr * nc) * (HASB ? 4.f : 2.f);
+    for (int w = 1; w < 8; ++w) { m = fmaxf(m, smx[w]); mn = fminf(mn, smn[w]); }
     const int ex = (int)((__float_as_uint(m) >> 23) & 0xffu) + 896;      // FP64 bias
-    // squares of entries below 2^-50 leave the FP32 range too early to be judged
-    const bool ok = !any_bad && (m == 0.f || (m > 1e-15f && m < 1e15f && count * m * m <= FX_PEAK * FX_PEAK * s));
+    // (entries far below 2^-100 would leave the FP32 range of the limbs' conversion)
+    const bool ok = !any_bad && (m == 0.f || (m > 1e-25f && m < 1e25f && m <= (float)(1 << FX_SPREAD) * mn));
     texp[t] = !ok ? -1 : (m == 0.f ? 64 : ex);
   }
 }

@@ -23,16 +23,8 @@ k_prod_tiles_fx(const Prob* __restrict__ probs, const TileJob* __restrict__ jobs
   fx_tiles_body<HASB, false>(probs, jobs, njobs, nq, mode, io, strided, blockIdx.x, gridDim.x, sh, pipe, probs[0].err);
 }
 
-// v / 2^(e - 1022) as a float (magnitude below 1, truncated; small values flush to zero)
-__device__ __forceinline__ float fx_ratio(double v, int e) {
-  const unsigned int h = (unsigned int)__double2hiint(v), l = (unsigned int)__double2loint(v);
-  const int ev = (int)((h >> 20) & 0x7ffu) - e + 126;
-  const unsigned int m = ((h & 0xfffffu) << 3) | (l >> 29);
-  return ev > 0 ? __uint_as_float(((unsigned int)ev << 23) | m) : 0.f;
-}
-
 // One CTA per tile (I, J >= I): the scale from the largest component, the choice between the
-// fixed-point and the FP64 kernel, and the limbs (zeros on the matrix diagonal).  The tile's
+// fixed-point and the FP64 kernel (FX_SPREAD), and the limbs (zeros on the matrix diagonal).  The tile's
 // second reading comes from L2.
 template <bool HASB>
 __global__ void __launch_bounds__(256)
@@ -43,47 +35,45 @@ k_fx_pack(const double2* __restrict__ A, const double2* __restrict__ B, int64_t 
   const int64_t t = (int64_t)I * nT - (int64_t)I * (I - 1) / 2 + (J - I);
   const double2* a = A + t * (TS * TS);
   const double2* b = HASB ? B + t * (TS * TS) : nullptr;
-  __shared__ unsigned int smx[8];
-  __shared__ float ssq[8];
+  __shared__ unsigned int smx[8], smn[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto off_diag = [&](int e) { return I != J || (e >> 7) != (e & (TS - 1)); };
   // high words of the magnitudes; 1 for a subnormal that has none
   auto mag = [](double v) { return max(hi_abs(v), __double2loint(v) ? 1u : 0u); };
-  unsigned int m = 0;
+  const int nr = (int)min((int64_t)TS, N - (int64_t)I * TS), nc = (int)min((int64_t)TS, N - (int64_t)J * TS);
+  unsigned int m = 0, mn = 0xffffffffu;
   for (int e = tid; e < TS * TS; e += 256) {
-    if (!off_diag(e)) continue;
     const double2 v = a[e];
-    m = max(m, max(mag(v.x), mag(v.y)));
+    unsigned int t = max(mag(v.x), mag(v.y));
     if (HASB) {
       const double2 w = b[e];
-      m = max(m, max(mag(w.x), mag(w.y)));
+      t = max(t, max(mag(w.x), mag(w.y)));
     }
+    if (off_diag(e)) m = max(m, t);
+    if ((e >> 7) < nr && (e & (TS - 1)) < nc) mn = min(mn, t);
   }
   m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) smx[warp] = m;
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  if (lane == 0) {
+    smx[warp] = m;
+    smn[warp] = mn;
+  }
   __syncthreads();
-  for (int w = 0; w < 8; ++w) m = max(m, smx[w]);
-  const int ex = max(64, (int)(m >> 20));
-  float s = 0.f;
+  for (int w = 0; w < 8; ++w) {
+    m = max(m, smx[w]);
+    mn = min(mn, smn[w]);
+  }
+  const int ex = max(1, (int)(m >> 20));
   for (int e = tid; e < TS * TS; e += 256) {
     double2 v = a[e], w = HASB ? b[e] : make_double2(0.0, 0.0);
     if (!off_diag(e)) v = w = make_double2(0.0, 0.0);
     Af[t * (TS * TS) + e] = fx_entry(v, ex);
     if (HASB) Bf[t * (TS * TS) + e] = fx_entry(w, ex);
-    const float f0 = fx_ratio(v.x, ex), f1 = fx_ratio(v.y, ex), f2 = fx_ratio(w.x, ex), f3 = fx_ratio(w.y, ex);
-    s += f0 * f0 + f1 * f1 + f2 * f2 + f3 * f3;
   }
-#pragma unroll
-  for (int k = 16; k >= 1; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-  if (lane == 0) ssq[warp] = s;
-  __syncthreads();
+  // (a tile of zeros adds nothing; high words compare magnitudes to a few units of 2^-20)
   if (tid == 0) {
-    for (int w = 1; w < 8; ++w) s += ssq[w];
-    // entries inside the matrix; the peak is at least half the scale, 2^-2 of it squared
-    const int64_t nr = min((int64_t)TS, N - (int64_t)I * TS), nc = min((int64_t)TS, N - (int64_t)J * TS);
-    const float count = (float)(nr * nc) * (HASB ? 4.f : 2.f);
     const bool in_range = ex >= 256 && ex <= 1792;
-    texp[t] = m == 0 || (in_range && count <= FX_PEAK * FX_PEAK * s) ? ex : -1;
+    texp[t] = m == 0 || (in_range && m <= mn + (FX_SPREAD << 20)) ? ex : -1;
   }
 }
 

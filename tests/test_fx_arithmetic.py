@@ -66,7 +66,7 @@ int main(int, char** argv) {
 def _product(tmp_path, u, x, n=256, tile=(0, 1)):
     """(tile exponent or -1, U x by the kernel's arithmetic); tile (I, J) of a matrix of order n"""
     a = cut("fx_phases.cuh", "__device__ __forceinline__ unsigned int hi_abs", "// A warp's place")
-    k = cut("k_product_fx.cu", "// v / 2", "}  // namespace")
+    k = cut("k_product_fx.cu", "template <bool HASB>\n__global__ void __launch_bounds__(256)", "}  // namespace")
     c = cut("fx_phases.cuh", "constexpr int FX_THREADS", "constexpr long long FX_SPIN")
     fu, fx = tmp_path / "u", tmp_path / "x"
     fu.write_bytes(np.ascontiguousarray(u, np.complex128).tobytes())
@@ -95,3 +95,99 @@ def test_vector_of_any_exponent(tmp_path, scale):
     err, mag = _err(u, x, y / big / scale if scale >= 2.0 ** -900 else y * 2.0 ** 1015)
     assert ex > 0
     assert np.all(err <= 2.0 ** -53 * mag + (2.0 ** -50 if scale == 2.0 ** -1015 else 0.0))
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_outlier_in_the_vector(tmp_path, seed):
+    """An entry of x 1e10 above the others, every row's own magnitude as the measure."""
+    rng = np.random.default_rng(seed)
+    u, x = _gauss(rng, 128, 128), _gauss(rng, 128)
+    x[rng.integers(128)] *= 1e10
+    ex, y = _product(tmp_path, u, x)
+    err, mag = _err(u, x, y)
+    assert ex > 0 and np.all(err <= 64 * 2.0 ** -53 * mag)
+
+
+def test_unit_vector(tmp_path):
+    """x = e_j gives the column of U to the rounding of its entries, 2^-60 of the scale."""
+    rng = np.random.default_rng(5)
+    u, x = _gauss(rng, 128, 128), np.zeros(128)
+    x[17] = 1.0
+    ex, y = _product(tmp_path, u, x)
+    assert ex > 0 and np.all(np.abs(y - u[:, 17]) <= 2.0 ** -59 * np.maximum(np.abs(u.real), np.abs(u.imag)).max() + 2.0 ** -52 * np.abs(u[:, 17]))
+
+
+def _tiles():
+    rng = np.random.default_rng(7)
+    g = _gauss(rng, 128, 128)
+    half = np.arange(128) >= 64
+    yield "dense", g, True
+    yield "zero", 0 * g, True
+    yield "two uncoupled blocks", np.where(half[:, None] == half[None, :], g, 0), False
+    yield "graded rows", np.where(half[:, None], 1e-10 * g, g), False
+    yield "graded columns", np.where(half[None, :], 1e-10 * g, g), False
+    one = np.where(np.arange(128)[:, None] == 5, g, 1e-12 * g)
+    yield "one large row", one, False
+    hole = g.copy()
+    hole[100, 3] = 0
+    yield "one zero", hole, False
+    peak = g.copy()
+    peak[4, 99] *= 1e5
+    yield "a peak", peak, False
+    bad = g.copy()
+    bad[9, 9] = np.inf
+    yield "an infinity", bad, False
+    yield "tiny", g * 2.0 ** -900, False
+
+
+SRC32 = r"""
+#include "simt.h"
+#define __restrict__
+namespace bse {
+constexpr int TS = 128;
+%s
+%s
+}
+using namespace bse;
+int main(int, char** argv) {
+  std::vector<double2> u(TS * TS);
+  fread(u.data(), 16, TS * TS, fopen(argv[1], "rb"));
+  std::vector<float2> A(3 * TS * TS), B(3 * TS * TS);
+  for (int e = 0; e < TS * TS; ++e) {
+    A[TS * TS + e] = make_float2((float)u[e].x, 0.f);        // tile (0, 1); the parts over A and B
+    B[TS * TS + e] = make_float2(0.f, (float)u[e].y);
+  }
+  int texp[3] = {0, 0, 0};
+  blockIdx.x = 1;
+  if (!simt::run_block(256, false, [&] { k_block_scale64<true>(A.data(), B.data(), 256, 2, texp); })) return 1;
+  printf("%%d\n", texp[1]);
+}
+"""
+
+
+@pytest.mark.parametrize("name,u,fixed", list(_tiles())[:-1], ids=[t[0] for t in list(_tiles())[:-1]])
+def test_choice_of_complex64_tiles(tmp_path, name, u, fixed):
+    """The same rule for the residual products of complex64 tiles (k_block_scale64)."""
+    c = cut("fx_phases.cuh", "constexpr int FX_THREADS", "constexpr long long FX_SPIN")
+    k = cut("k_block_fx.cu", "template <bool HASB>\n__global__ void __launch_bounds__(256)", "// limbs of a float")
+    (tmp_path / "u").write_bytes(np.ascontiguousarray(u).tobytes())
+    assert (run(tmp_path, SRC32 % (c, k), tmp_path / "u")[0][0] >= 0) == fixed
+
+
+@pytest.mark.parametrize("name,u,fixed", list(_tiles()), ids=[t[0] for t in _tiles()])
+def test_choice_of_tiles(tmp_path, name, u, fixed):
+    """Tiles in which some row's magnitude may be far below max|u| max|x| stay with the FP64 kernel."""
+    ex, _ = _product(tmp_path, u, np.ones(128))
+    assert (ex >= 0) == fixed
+
+
+def test_edges_of_the_matrix(tmp_path):
+    """The zeros beyond the order of the matrix do not count, the diagonal does (but not as the scale)."""
+    rng = np.random.default_rng(8)
+    g = _gauss(rng, 128, 128)
+    g = g + g.conj().T
+    cutoff = np.where((np.arange(128)[:, None] < 100) & (np.arange(128)[None, :] < 100), g, 0)
+    for d, fixed in ((30.0, True), (1e9, True), (1e-9, False)):
+        m = cutoff.copy()
+        np.fill_diagonal(m[:100, :100], d)
+        assert (_product(tmp_path, m, np.ones(128), 228, (1, 1))[0] >= 0) == fixed, d

@@ -26,6 +26,23 @@ def _cases(n):
     rng = np.random.default_rng(n)
     a, b = _matrices(rng, n)
     x = rng.standard_normal((n, 1)) + 1j * rng.standard_normal((n, 1))
+    half = np.arange(n) % 128 >= 64
+    same = half[:, None] == half[None, :]
+    yield "two uncoupled blocks, one part of x at 1e-12", a * same, b * same, np.where(half[:, None], 1e-12 * x, x)
+    yield "two uncoupled blocks, one part of x at 1e-19", a * same, b * same, np.where(half[:, None], 1e-19 * x, x)
+    yield ("graded rows and columns", *_graded(a, b, np.where(half, 1e-10, 1.0)), x)
+    yield ("one row far above the others", *_graded(a, b, np.where(np.arange(n) == 5 % n, 1.0, 1e-6)), x)
+    out = x.copy()
+    out[n // 3] *= 1e10
+    yield "an entry of x far above the others", a, b, out
+    hole = np.ones((n, n))
+    hole[n // 2:, n // 3] = hole[n // 3, n // 2:] = 0
+    yield "... that some rows do not see", a * hole, b * hole, out
+    peak = np.ones((n, n))
+    peak[0, n - 1] = peak[n - 1, 0] = 1e5
+    z = x.copy()
+    z[[0, n - 1]] = 0
+    yield "a peak that x does not see", a * peak, b * peak, z
     yield "x of 1e-300", a, b, 1e-300 * x
     yield "x near the smallest normal number", 2.0 ** 40 * a, 2.0 ** 40 * b, 2.0 ** -1015 * x
     yield "x of 1e300", 2.0 ** -40 * a, 2.0 ** -40 * b, 1e300 * x
