@@ -21,8 +21,12 @@
 // a tile runs in fixed point only when every entry of the matrix in it is within 2^FX_SPREAD of its
 // largest (k_fx_pack; in the diagonal tiles the diagonal counts as one of the entries), whatever x is.
 // Sparse tiles, graded rows or columns, a peak, an infinity, a NaN, or exponents near the ends of the
-// FP64 range keep a tile on the FP64 kernel.  2^14 lets complex tiles without structure pass (the
-// spread of 16384 complex Gaussian entries is 2^9 to 2^13 for one matrix, 2^5 to 2^10 for the pair A, B);
+// FP64 range keep a tile on the FP64 kernel.  Why 2^16: 16384 entries without structure spread by
+// themselves (2^5 to 2^10 for a complex pair A, B; 2^8 to 2^14 for a complex A alone, one tile in 600
+// above that and about one in 50000 above 2^16), a tile left over costs a persistent step 20 us, and
+// graded rows or blocks add their own factor to that spread.  Without an outlier in x a row is then
+// within a few 2^-53 of its |U||x|; with one, an entry that couples to it by 2^-s max|U| is off by
+// 2^(s - 59) of that coupling.
 // x may have any exponent, subnormals included.  The diagonal of the matrix,
 // which holds the transition energies far above everything else in its tiles, is left out of the
 // tiles (zeros there) and added in FP64 by the block-row reduction.
@@ -41,7 +45,7 @@ namespace bse {
 
 constexpr int FX_THREADS = 256;
 constexpr int FX_WARPS = FX_THREADS / 32;
-constexpr int FX_SPREAD = 14;        // largest over smallest entry of a fixed-point tile, log2
+constexpr int FX_SPREAD = 16;        // largest over smallest entry of a fixed-point tile, log2
 
 constexpr long long FX_SPIN = 1ll << 24;      // polls of one wait for a row
 

@@ -6,7 +6,7 @@ Bound.  u and x are off by at most 2^-60 of 2^E (twice the largest component at 
 product by 2^-60: 3 2^-58 max|u| max|x| per real multiply-add.  A row has two per entry; their signs are
 as good as random, so a sum over 128 entries is within 6 sigma of sqrt(2 128) times a third of that:
 96 2^-58 max|u| max|x| < 2^-51 max|u| max|x|, and 2^-53 of the result.  In a tile that qualifies max|u| is
-at most 2^14 times any entry, so this is at most 2^-37 |U||x|, whatever x; for x without
+at most 2^16 times any entry, so this is at most 2^-35 |U||x|, whatever x; for x without
 outliers, |U||x| is some 128 / 8 max|u| max|x|, and the bound 2^-53 |U||x| holds."""
 import numpy as np
 import pytest
