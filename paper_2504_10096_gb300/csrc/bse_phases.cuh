@@ -348,7 +348,9 @@ __device__ __forceinline__ void prod_reduce_body(const Prob* __restrict__ probs,
 // Im(conj(Dt[row, c']) x[row]) for c = nm + c' (the twin coefficients), nm + nt in all;
 // TDA: the complex conj(V[row, c]) x[row], c <= j.  A warp-wide FP64 instruction takes 64 clocks
 // of its scheduler, so the work is cut into one-warp tasks (a column on a chunk of rows) that
-// spread evenly over all schedulers of the GPU; at most DOT_CHUNKS chunks, whole tiles each.
+// spread evenly over all schedulers of the GPU; at most DOT_CHUNKS chunks, whole tiles each.  A lane's
+// FP32 sums go to FP64 every DOT_RUN rounds of four rows, so their rounding does not grow with N.
+constexpr int DOT_RUN = 4;
 __host__ __device__ __forceinline__ int dot_chunk_tiles(int nT) { return (nT + DOT_CHUNKS - 1) / DOT_CHUNKS; }
 __host__ __device__ __forceinline__ int dot_chunks(int nT) {
   return (nT + dot_chunk_tiles(nT) - 1) / dot_chunk_tiles(nT);
@@ -369,7 +371,8 @@ __device__ __forceinline__ void cgs_dot_task(const Prob& p, const KState* st, co
   int64_t r = r0 + lane;
   if (ph) {   // real coefficients: Re(conj(q) x), or Im(conj(q) x) = Re(conj(q) (-i x)) for twins
     R a1 = 0, a2 = 0;   // two chains (x and y products)
-    for (; r < r1; r += 4 * 32) {                       // whole tiles: four rows per lane and round
+    double s = 0.0;
+    for (int n = 1; r < r1; r += 4 * 32, ++n) {                       // whole tiles: four rows per lane and round
       ST q[4], x[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -381,12 +384,17 @@ __device__ __forceinline__ void cgs_dot_task(const Prob& p, const KState* st, co
         a1 = fma(q[u].x, twin ? x[u].y : x[u].x, a1);
         a2 = fma(q[u].y, twin ? -x[u].x : x[u].y, a2);
       }
+      if (sizeof(R) == 4 && n % DOT_RUN == 0) {
+        s += (double)a1 + (double)a2;
+        a1 = a2 = 0;
+      }
     }
-    const double t = warp_sum_d((double)a1 + (double)a2);
+    const double t = warp_sum_d(sizeof(R) == 4 ? s + ((double)a1 + (double)a2) : (double)a1 + (double)a2);
     if (lane == 0) p.cpart[(int64_t)k * p.ncol + c] = t;
   } else {
     ST acc = czero<ST>();
-    for (; r < r1; r += 4 * 32) {
+    double2 a = mk(0.0, 0.0);
+    for (int n = 1; r < r1; r += 4 * 32, ++n) {
       ST q[4], x[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -395,8 +403,12 @@ __device__ __forceinline__ void cgs_dot_task(const Prob& p, const KState* st, co
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) cfmac(acc, q[u], x[u]);
+      if (sizeof(R) == 4 && n % DOT_RUN == 0) {
+        a = cadd(a, mk((double)acc.x, (double)acc.y));
+        acc = czero<ST>();
+      }
     }
-    double2 a = mk((double)acc.x, (double)acc.y);
+    a = sizeof(R) == 4 ? cadd(a, mk((double)acc.x, (double)acc.y)) : mk((double)acc.x, (double)acc.y);
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) a = cadd(a, dshfl(a, m));
     if (lane == 0) ((double2*)p.cpart)[(int64_t)k * p.ncol + c] = a;
@@ -443,7 +455,8 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
   // Loads in flight per thread, the first of them beside the sums of the coefficients.  A TDA cycle at
   // N = 2000 took 31.2 ms of steps and restarts with 4, 32.4 with 6, 33.1 with 8 (32.5 with the loads
   // behind the coefficients); a pseudo-Hermitian one at 3000 243.7, 246.6, 247.2 (251).
-  constexpr int U = 4;
+  // FP32 has a sum for each of eight loads: one sum alone would be a chain of nset / 8 roundings.
+  constexpr int U = sizeof(R) == 4 ? 8 : 4, NA = sizeof(R) == 4 ? U : 1;
   const int64_t ld = p.Npad;
   // entry cc of the set: Um[:, cc] for cc < nm, else the twin's Ut[:, cc - nm]
   auto load = [&](int cc) -> ST { return ldv<COH>(cc < nm ? vb + (int64_t)cc * ld : pb + (int64_t)(cc - nm) * ld); };
@@ -460,12 +473,15 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
     if (bx == 0) coef[c] = sc;
   }
   __syncthreads();
-  ST part = czero<ST>();
+  ST acc[NA];
+#pragma unroll
+  for (int u = 0; u < NA; ++u) acc[u] = czero<ST>();
   for (int c = c0; c < nset; c += G * U) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int cc = c + G * u;
       if (cc >= nset) continue;
+      ST& part = acc[u % NA];
       if (ph) {                               // real coefficients; the twin i t = (-t.y, t.x)
         const R f = cf[cc].x;
         const bool tw = cc >= nm;
@@ -481,6 +497,9 @@ __device__ __forceinline__ void cgs_update_slab(const Prob& p, const KState* st,
         if (c + G * (U + u) < nset) v[u] = load(c + G * (U + u));
     }
   }
+  ST part = acc[0];
+#pragma unroll
+  for (int u = 1; u < NA; ++u) part = cadd(part, acc[u]);
 #pragma unroll
   for (int m = RS; m < 32; m <<= 1) part = cadd(part, shfl_xor_c(part, m));   // the warp's groups
   if (lane < RS) red[warp][lane] = part;

@@ -118,7 +118,9 @@ k_cgs_dot_dfs(const Prob* __restrict__ probs, int newvec) {
   const int64_t rows = (int64_t)dot_chunk_tiles(p.nT) * TS;
   const int64_t r0 = blockIdx.y * rows, r1 = min(p.Npad, r0 + rows);
   float sh = 0.f, sl = 0.f;
-  for (int64_t r = r0 + lane; r < r1; r += 4 * 32) {
+  double s = 0.0;
+  int n = 1;
+  for (int64_t r = r0 + lane; r < r1; r += 4 * 32, ++n) {
     float4 q[4], x[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -135,13 +137,18 @@ k_cgs_dot_dfs(const Prob* __restrict__ probs, int newvec) {
         df_madd(sh, sl, q[u].y, q[u].w, x[u].y, x[u].w);
       }
     }
+    if (n % DOT_RUN == 0 && r + 4 * 32 < r1) {     // longer chains would round more than FP64 sums of them
+      s += (double)sh + (double)sl;
+      sh = sl = 0.f;
+    }
   }
 #pragma unroll
   for (int m = 16; m >= 1; m >>= 1) {
     const float oh = __shfl_xor_sync(0xffffffffu, sh, m), ol = __shfl_xor_sync(0xffffffffu, sl, m);
     df_add(sh, sl, oh, ol);
   }
-  if (lane == 0) p.cpart[(int64_t)blockIdx.y * p.ncol + c] = (double)sh + (double)sl;
+  if (r1 - r0 > DOT_RUN * 4 * 32) s = warp_sum_d(s);
+  if (lane == 0) p.cpart[(int64_t)blockIdx.y * p.ncol + c] = s + ((double)sh + (double)sl);
 }
 
 // units as k_cgs_update: w = w - V c - i P d (c, d the pass's real coefficients), and ws
