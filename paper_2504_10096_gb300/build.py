@@ -36,7 +36,7 @@ def _stale(obj, src):
     t = os.path.getmtime(obj)
     deps = [src, os.path.join(CSRC, "bse_internal.cuh"), os.path.join(CSRC, "bse_phases.cuh"),
             os.path.join(CSRC, "fx_phases.cuh"), os.path.join(CSRC, "tree_solve.cuh"),
-            os.path.join(CSRC, "grid_sync.cuh"),
+            os.path.join(CSRC, "grid_sync.cuh"), os.path.join(CSRC, "per_device.h"),
             os.path.join(HERE, "..", "include", "bse.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "per_device.h"
+
 namespace bse {
 
 constexpr int TS = 128;            // tile edge of the packed storage
@@ -251,6 +253,12 @@ __device__ __forceinline__ void clock_end(ProdClock* c) {
   if (c && threadIdx.x == 0) atomicMax(&c->end, dev_ns());
 }
 
+inline int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+
 // Kernel launches issued by this process (reported per solve in bse_stats).
 inline long long& launch_counter() {
   static long long c = 0;
@@ -327,7 +335,7 @@ void launch_prod_reduce_f64(const Prob* dprobs, int nprob, int maxnT, int mode, 
 // the FP64 tile kernel alone (k_product.cu)
 void launch_tiles_f64(const Prob* dprobs, const TileJob* jobs, int njobs, int mode, GenericIO io, bool hasB,
                       ProdShape shape, int first, cudaStream_t s);
-int num_sms();
+int num_sms();                 // of the current device
 
 // blocks of columns in FP64 accuracy with fixed-point tiles (k_block_fx.cu): Y = A XA + sB B XB
 // (XB null: conj(XA)), Npad rows; `work` holds block_fx_bytes

@@ -24,6 +24,7 @@
 // set.  Every wait is bounded; on expiry the CTA records an error, stops, waits
 // (bounded) for what it has in flight and releases its TMEM, and the host
 // returns a timeout.
+#include <algorithm>
 #include <cstdint>
 
 #include "bse_internal.cuh"
@@ -426,8 +427,6 @@ __global__ void k_wait_selftest(int arrive, long long spins, int* __restrict__ e
   *expired = ok ? 0 : 1;
 }
 
-int g_tc_sms = 0;
-
 }  // namespace
 
 int selftest_bounded_wait(int arrive, int* expired_host) {
@@ -460,16 +459,10 @@ int launch_adjoint_tc(const double2* Z, int64_t ldz, int64_t Npad, int64_t N, in
   const int nk = (kk + KC - 1) / KC;
   count_launch(2);
   k_adj_panels<<<dim3((unsigned)(rows / 128), (unsigned)(nk * KC / 4)), 128, 0, s>>>(Z, ldz, Npad, N, k, g, ph, nk, rows, panels);
-  if (!g_tc_sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_tc_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_tc_sms <= 0) g_tc_sms = 1;
-  }
   // stage: L (4 planes x 8 KiB) + R (8 or 4 planes x 4 KiB)
   const size_t smem = (size_t)NSTAGE * (4 * BLK + (ph ? 8 : 4) * (BLK / 2)) + EPI_BYTES;
   cudaMemsetAsync(derr, 0, sizeof(int), s);
-  const int grid = (int)(ntiles < g_tc_sms ? ntiles : g_tc_sms);
+  const int grid = (int)std::min<int64_t>(ntiles, num_sms());
   if (ph) {
     cudaFuncSetAttribute(k_adjoint_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_adjoint_tc<true><<<grid, TC_THREADS, smem, s>>>(panels, rows, nk, N, tiles128, (int)ntiles, dA, dB, derr);

@@ -147,20 +147,19 @@ size_t persist_smem() {
 
 template <typename ST, typename R, bool HASB>
 int persist_grid() {
-  static int grid = -1;
-  if (grid < 0) {
+  static PerDevice<int> grid;
+  const int dev = current_device();
+  return grid.get(dev, [&] {
     const size_t sm = persist_smem<ST, R, HASB>();
     if (sm > 48 * 1024)
       cudaFuncSetAttribute(k_steps_persist<ST, R, HASB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int occ = 0, dev = 0, nsm = 0, coop = 0;
-    cudaGetDevice(&dev);
+    int occ = 0, nsm = 0, coop = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_steps_persist<ST, R, HASB>, PS_THREADS, sm);
-    grid = (coop && occ >= 1) ? nsm : 0;    // one CTA per SM: every CTA resident
     cudaGetLastError();
-  }
-  return grid;
+    return (coop && occ >= 1) ? nsm : 0;    // one CTA per SM: every CTA resident
+  });
 }
 
 template <typename ST, typename R, bool HASB>

@@ -314,15 +314,14 @@ void launch_pq_combine(double2* a, double2* b, int64_t n, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- launchers
-static int g_num_sms = 0;
 int num_sms() {
-  if (!g_num_sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_num_sms <= 0) g_num_sms = 1;
-  }
-  return g_num_sms;
+  static PerDevice<int> sms;
+  const int dev = current_device();
+  return sms.get(dev, [&] {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+  });
 }
 
 int product_grid(int occ, ProdShape shape, int njobs) {
@@ -336,17 +335,15 @@ int product_grid(int occ, ProdShape shape, int njobs) {
 
 template <typename ST, typename R>
 int product_occupancy(bool hasB) {
-  static int occ[2] = {0, 0};
-  const int ib = hasB ? 1 : 0;
-  if (!occ[ib]) {
+  static PerDevice<int> occ[2];
+  return occ[hasB ? 1 : 0].get(current_device(), [&] {
     int o = 0;
     if (hasB)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles<ST, R, true>, PROD_THREADS, 0);
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles<ST, R, false>, PROD_THREADS, 0);
-    occ[ib] = o > 0 ? o : 1;
-  }
-  return occ[ib];
+    return o > 0 ? o : 1;
+  });
 }
 
 template <typename ST, typename R>

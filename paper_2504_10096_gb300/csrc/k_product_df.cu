@@ -1011,16 +1011,15 @@ __global__ void k_split_tiles(const double2* __restrict__ in, int64_t n, float4*
 
 template <bool HASB, bool SPLIT>
 int df_occupancy() {
-  static int occ = 0;
-  if (!occ) {
+  static PerDevice<int> occ;
+  return occ.get(current_device(), [] {
     int o = 0;
     if constexpr (HASB && !SPLIT)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_df2, PROD_THREADS, 0);
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_prod_tiles_df<HASB, SPLIT>, PROD_THREADS, 0);
-    occ = o > 0 ? o : 1;
-  }
-  return occ;
+    return o > 0 ? o : 1;
+  });
 }
 
 int product_df_occupancy(bool hasB, bool split) {
@@ -1062,12 +1061,12 @@ template <int NT, bool TICKET>
 void launch_mx(const Prob* dprobs, const TileJob* coarse, int ncoarse, int mode, const GenericIO& io,
                ProdShape shape, const TileJob* fine, int nfine, int* err, cudaStream_t s) {
   using C = Mx<NT>;
-  static bool attr = false;
-  if (!attr) {
+  static PerDevice<bool> opt_in;
+  opt_in.get(current_device(), [] {
     cudaFuncSetAttribute(k_prod_tiles_mx<NT, TICKET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     cudaFuncSetAttribute(k_prod_tiles_mx<NT, TICKET>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    attr = true;
-  }
+    return true;
+  });
   const ProdShape ms{shape.ctas_per_sm < 0 ? -1 : C::CTAS, shape.strided};
   constexpr int W = NT / PROD_THREADS;
   const int nfb = std::min((nfine + W - 1) / W, C::CTAS * num_sms());

@@ -93,12 +93,12 @@ int fx_bands(int ntiles) {
 
 // two CTAs per SM (96 KiB of shared memory and 128 registers a thread each)
 int product_fx_occupancy() {
-  static const bool set = [] {
+  static PerDevice<bool> opt_in;
+  opt_in.get(current_device(), [] {
     cudaFuncSetAttribute(k_prod_tiles_fx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared<FX_RING>));
     cudaFuncSetAttribute(k_prod_tiles_fx<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared<FX_RING>));
     return true;
-  }();
-  (void)set;
+  });
   return 2;
 }
 
