@@ -315,9 +315,18 @@ void launch_ritz(const Prob* dprobs, int nprob, int ncv, bool gruning, cudaStrea
   }
   count_launch(2);
   const size_t M = gruning ? (size_t)(2 * ncv + 2) : (size_t)ncv;
-  const size_t sv = M * 2 * (sizeof(double) + sizeof(float2)), sm = M * 5 * sizeof(double) + M + 16;
-  if (sv > 48 * 1024) cudaFuncSetAttribute(k_ritz_values, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv);
-  if (sm > 48 * 1024) cudaFuncSetAttribute(k_ritz_vectors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  auto values_bytes = [](size_t m) { return m * 2 * (sizeof(double) + sizeof(float2)); };
+  auto vectors_bytes = [](size_t m) { return m * 5 * sizeof(double) + m + 16; };
+  const size_t sv = values_bytes(M), sm = vectors_bytes(M);
+  // opt in to what the largest subspace takes: the 48 KiB without it include the static arrays, and
+  // another thread's launch may need more than this one
+  static PerDevice<bool> opt_in;
+  opt_in.get(current_device(), [&] {
+    const size_t top = 2 * MAXM + 2;
+    cudaFuncSetAttribute(k_ritz_values, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)values_bytes(top));
+    cudaFuncSetAttribute(k_ritz_vectors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vectors_bytes(top));
+    return true;
+  });
   launch_dep(k_ritz_values, dim3(ncv, nprob), RV_THREADS, sv, s, dprobs);
   launch_dep(k_ritz_vectors, dim3(ncv, nprob), 32, sm, s, dprobs);
 }

@@ -189,3 +189,18 @@ def test_variant_config4_recipe_n4000(variant):
     print(f"config-4 recipe N=4000 {variant}: steps {st['steps']}, restarts {st['restarts']}, "
           f"{st['ms_total']:.1f} ms")
     s.close()
+
+
+@pytest.mark.parametrize("ncv", [748, 752, 767, 769])
+def test_gruning_subspaces_around_48_kib_of_scratch(ncv):
+    """Subspaces whose projected problem (2 ncv + 2 entries of 32 bytes) takes just less than 48 KiB of
+    dynamic shared memory beside the static one."""
+    from paper_2504_10096_gb300 import bse
+    n = 800
+    A, B = problem(n, "c128", seed=5, n_g=40)
+    s = bse.Solver(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda())
+    ref, _, _ = s.solve(4, tol=1e-11, vectors=False)
+    vals, _, nconv = s.solve(4, tol=1e-11, ncv=ncv, vectors=False, variant=bse.BSE_VARIANT_GRUNING)
+    assert nconv == 4
+    np.testing.assert_allclose(vals, ref, rtol=1e-10, atol=0)
+    s.close()
