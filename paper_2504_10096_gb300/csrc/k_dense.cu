@@ -681,16 +681,24 @@ int dense_run(int64_t N, int64_t Npad, int nev, double* work, int* dflag, double
   k_dn_mirror<<<dim3(ng, ng), b2, 0, s>>>(M, ld, n);
   k_dn_wgemm<<<dim3(ng, ng), 256, 0, s>>>(W, M, ld, n);
   k_dn_skew<<<g2, b2, 0, s>>>(W, ld, n);
+  // the opt-ins below are to DN_SMEM for all orders: another thread's solve may need more than this one
+  constexpr size_t DN_SMEM = 200 * 1024;
+  static PerDevice<bool> opt_in;
+  opt_in.get(current_device(), [] {
+    cudaFuncSetAttribute(k_dn_tridiag<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DN_SMEM);
+    cudaFuncSetAttribute(k_dn_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DN_SMEM);
+    cudaFuncSetAttribute(k_dn_back<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DN_SMEM);
+    return true;
+  });
   // 4. skew-tridiagonalisation
   {
     int nn = (int)n;
     int64_t lda = ld;
     const int grid = (int)std::min<int64_t>(num_sms(), n);
     const size_t cols = sizeof(double) * (size_t)n * ((n + grid - 1) / grid + 2);
-    const bool smc = cols <= 200 * 1024;
+    const bool smc = cols <= DN_SMEM;
     void* args[] = {(void*)&W, (void*)&lda, (void*)&nn, (void*)&E, (void*)&T, (void*)&Pv, (void*)&gb};
     const void* fn = smc ? (const void*)k_dn_tridiag<true> : (const void*)k_dn_tridiag<false>;
-    if (smc) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
     count_launch();
     if (cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(256), args, smc ? cols : 0, s) != cudaSuccess) {
       cudaGetLastError();
@@ -702,8 +710,7 @@ int dense_run(int64_t N, int64_t Npad, int nev, double* work, int* dflag, double
   k_dn_prepare<<<1, 1024, 0, s>>>(E, n, S);
   k_dn_bisect<<<nev, RV_THREADS, 0, s>>>(S, n, N, lam);
   const size_t fs = sizeof(double) * (size_t)(4 * n) + (size_t)n;
-  if (fs <= 200 * 1024) {
-    cudaFuncSetAttribute(k_dn_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs);
+  if (fs <= DN_SMEM) {
     k_dn_inverse<true><<<nev, 32, fs, s>>>(S, n, nev, lam, inv, Sv);
   } else {
     k_dn_inverse<false><<<nev, 32, 0, s>>>(S, n, nev, lam, inv, Sv);
@@ -711,8 +718,7 @@ int dense_run(int64_t N, int64_t Npad, int nev, double* work, int* dflag, double
   // 6.
   count_launch();
   const size_t qs = sizeof(double2) * (size_t)n;
-  if (qs <= 200 * 1024) {
-    cudaFuncSetAttribute(k_dn_back<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
+  if (qs <= DN_SMEM) {
     k_dn_back<true><<<nev, 256, qs, s>>>(W, M, ld, n, E, T, Sv, qb, Npad, Z);
   } else {
     k_dn_back<false><<<nev, 256, 0, s>>>(W, M, ld, n, E, T, Sv, qb, Npad, Z);

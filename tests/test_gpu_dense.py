@@ -93,3 +93,32 @@ def test_dense_not_positive_definite_and_invalid():
     rc, _, _ = bse.bse_solve_dense(t.h, 4, 1e-10)
     assert rc == bse.BSE_EINVAL
     t.close()
+
+
+def test_dense_orders_in_several_threads():
+    """Solves of different orders by several threads: a kernel's opt-in to shared memory belongs to the
+    device, not to the call (their launches share a stream, so they run one after another)."""
+    import threading
+    from paper_2504_10096_gb300 import bse
+    probs = {n: problem(n, "c128", seed=n, n_g=16) for n in (40, 130, 300, 520)}
+    refs, wrong = {}, []
+    for n, (A, B) in probs.items():
+        s = _solver(A, B)
+        refs[n] = s.solve_dense(4, vectors=False)[0]
+        s.close()
+
+    def work(n):
+        s = _solver(*probs[n])
+        for _ in range(12):
+            try:
+                if not np.array_equal(s.solve_dense(4, vectors=False)[0], refs[n]):
+                    wrong.append((n, "differs"))
+            except bse.BSEError as e:
+                wrong.append((n, str(e)))
+        s.close()
+    t = [threading.Thread(target=work, args=(n,)) for n in probs]
+    for x in t:
+        x.start()
+    for x in t:
+        x.join()
+    assert not wrong, wrong
