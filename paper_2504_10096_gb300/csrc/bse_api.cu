@@ -241,12 +241,18 @@ int pack_matrix(bse_handle* h, const T* src, int64_t N, int nT, int herm, int wh
   return BSE_OK;
 }
 
-// Y = A XA + sB B XB (FP64 blocks of K columns, Npad rows) with the stored tiles of problem i
+// Y = A XA + sB B XB (FP64 blocks of K columns, Npad rows) with the stored tiles of problem i.  The
+// fixed-point kernels take the columns in groups: their workspace (2 + splits times the group) stays
+// below kBlkBytes whatever K is, and the grid's second dimension below its limit.
+constexpr size_t kBlkBytes = (size_t)256 << 20;
+
 int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB) {
   ProbHost& q = h->p[i];
   // (complex128 PH tiles hold P and Q, so they always go through the two-matrix form)
   if (hasB == (h->ph != 0) && q.block_fx) {
-    const size_t need = block_fx_bytes(q.nT, K, hasB);
+    int kg = std::min(K, 32768);
+    while (kg > 16 && block_fx_bytes(q.nT, kg, hasB) > kBlkBytes) kg = (kg + 1) / 2;
+    const size_t need = block_fx_bytes(q.nT, kg, hasB);
     if (need > h->blk_bytes) {
       dfree(h->blk);
       h->blk_bytes = dalloc(&h->blk, need) == BSE_OK ? need : 0;
@@ -259,7 +265,11 @@ int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, do
       b.A = q.A;
       b.B = q.B;
       b.nT = q.nT;
-      launch_block_fx(b, hasB, h->tiles64, xa, xb, q.Npad, sB, y, q.Npad, K, h->blk, h->stream);
+      for (int c = 0; c < K; c += kg) {
+        const int64_t o = (int64_t)c * q.Npad;
+        launch_block_fx(b, hasB, h->tiles64, xa + o, xb ? xb + o : nullptr, q.Npad, sB, y + o, q.Npad,
+                        std::min(kg, K - c), h->blk, h->stream);
+      }
       CK(cudaGetLastError());
       return BSE_OK;
     }

@@ -73,3 +73,19 @@ def test_every_entry(name, n, form):
             for c in range(k):
                 assert_elementwise(y[:, c:c + 1] * f, (ref * f).astype(complex), bound, UNIT["c128"], 64, f"{name}, {kind}, k = {k}")
     s.close()
+
+
+@pytest.mark.parametrize("n,k", [(3, 40000), (1100, 2900)])
+def test_more_columns_than_one_launch_takes(n, k):
+    """H on blocks that the block kernels take in several groups of columns."""
+    from paper_2504_10096_gb300 import bse
+    rng = np.random.default_rng(k)
+    a, b = _matrices(rng, n)
+    X = torch.randn(2 * n, k, dtype=torch.complex128, device="cuda")
+    s = bse.Solver(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda())
+    Y = s.apply(bse.BSE_OP_H, X)
+    s.close()
+    at, bt = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    ref = torch.cat([at @ X[:n] + bt @ X[n:], -(bt.conj() @ X[:n] + at.conj() @ X[n:])])
+    mag = torch.cat([at.abs() @ X[:n].abs() + bt.abs() @ X[n:].abs(), bt.abs() @ X[:n].abs() + at.abs() @ X[n:].abs()])
+    assert bool(((Y - ref).abs() <= 64 * UNIT["c128"] * 2 * mag).all())       # both sides are off by as much
