@@ -65,7 +65,8 @@ typedef enum bse_dtype {
   /* complex128 storage; products to FP64 accuracy (the FP64 path): each entry
      of Y = M X is off by at most a few tens of 2^-53 (|M||X|)_i.  They run in
      60-bit fixed point on a second copy of the packed tiles, made when it
-     fits in a third of the free memory, on every 128 x 128 tile whose entries
+     fits in a third of the free memory and given up when a later allocation
+     of this library needs its memory, on every 128 x 128 tile whose entries
      lie within a factor 2^16 of one another (entries of X may differ by any
      factor), and in FP64 FMAs otherwise.  Where X has one entry far above all
      others of its 128-entry chunk, an entry of Y that couples to it by 2^-s

@@ -90,6 +90,7 @@ std::map<TuneKey, ProdShape> g_tuned;
 }  // namespace
 
 struct bse_handle {
+  std::mutex busy;       // held by the call that works with the handle (Use), or by one that takes its copy
   int count = 0, form = 0, dtype = 0, ph = 0;
   bool df = false;       // Lanczos products in double-FP32 arithmetic
   bool split = false;    // ... on split complex128 tiles (else on complex64 tiles)
@@ -174,7 +175,7 @@ namespace {
     if (e_ != cudaSuccess) return BSE_ECUDA;          \
   } while (0)
 
-int dalloc(void** ptr, size_t bytes) {
+int dalloc_plain(void** ptr, size_t bytes) {
   *ptr = nullptr;
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(ptr, bytes);
@@ -184,6 +185,52 @@ int dalloc(void** ptr, size_t bytes) {
     return e == cudaErrorMemoryAllocation ? BSE_ENOMEM : BSE_ECUDA;
   }
   return BSE_OK;
+}
+
+// The fixed-point copies are the one thing a handle can do without, so memory that another
+// allocation of this library needs is taken from them (drop_fx): from the handle the thread works
+// with and from every handle that no thread is working with.
+std::mutex g_fx_mu;
+std::vector<bse_handle*> g_fx_handles;       // that hold a copy
+thread_local bse_handle* t_handle = nullptr; // the handle this thread works with
+
+// one per call that works with a handle
+struct Use {
+  bse_handle* h;
+  explicit Use(bse_handle* hh) : h(hh) {
+    h->busy.lock();
+    t_handle = h;
+  }
+  ~Use() {
+    t_handle = nullptr;
+    h->busy.unlock();
+  }
+  Use(const Use&) = delete;
+  Use& operator=(const Use&) = delete;
+};
+
+void drop_fx(bse_handle* h);
+
+bool release_copies() {
+  std::lock_guard<std::mutex> lk(g_fx_mu);
+  const size_t had = g_fx_handles.size();
+  for (size_t i = 0; i < g_fx_handles.size();) {
+    bse_handle* o = g_fx_handles[i];
+    const bool own = o == t_handle;
+    if (!own && !o->busy.try_lock()) {
+      ++i;
+      continue;
+    }
+    drop_fx(o);
+    if (!own) o->busy.unlock();
+    g_fx_handles.erase(g_fx_handles.begin() + (ptrdiff_t)i);
+  }
+  return g_fx_handles.size() < had;
+}
+
+int dalloc(void** ptr, size_t bytes) {
+  const int rc = dalloc_plain(ptr, bytes);
+  return rc == BSE_ENOMEM && release_copies() ? dalloc_plain(ptr, bytes) : rc;
 }
 
 void dfree(void*& ptr) {
@@ -257,7 +304,7 @@ int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, do
       dfree(h->blk);
       h->blk_bytes = dalloc(&h->blk, need) == BSE_OK ? need : 0;
     }
-    if (h->blk) {
+    if (h->blk && q.block_fx) {          // (the allocation may have taken the copy)
       BlockFx b{};
       b.M0 = h->tiles64 ? (const void*)q.A : q.Afx;
       b.M1 = hasB ? (h->tiles64 ? (const void*)q.B : q.Bfx) : nullptr;
@@ -862,8 +909,8 @@ int split_mixed_jobs(bse_handle* h, double tol, double tau_opt) {
 
 // The fixed-point copy of a complex128 handle's tiles (fx_phases.cuh), which doubles its packed
 // storage: made when it takes at most a third of the device memory that is free (a handle that
-// nearly fills the GPU, or one that finds it nearly full, keeps the FP64 product alone), and
-// dropped again when any allocation fails.  The jobs are reordered: fixed-point tiles first.
+// nearly fills the GPU, or one that finds it nearly full, keeps the FP64 product alone), and given
+// back when an allocation needs its memory (drop_fx).  The jobs are reordered: fixed-point tiles first.
 int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
   size_t need = 0, freeb = 0, totalb = 0;
   for (const ProbHost& q : h->p) need += (size_t)q.ntiles * TS * TS * sizeof(int4) * (h->ph ? 2 : 1);
@@ -874,8 +921,8 @@ int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
   for (int i = 0; i < h->count && rc == BSE_OK; ++i) {
     ProbHost& q = h->p[i];
     const size_t bytes = (size_t)q.ntiles * TS * TS * sizeof(int4);
-    if ((rc = dalloc((void**)&q.Afx, bytes)) || (h->ph && (rc = dalloc((void**)&q.Bfx, bytes))) ||
-        (rc = dalloc((void**)&q.texp, sizeof(int) * (size_t)q.ntiles)))
+    if ((rc = dalloc_plain((void**)&q.Afx, bytes)) || (h->ph && (rc = dalloc_plain((void**)&q.Bfx, bytes))) ||
+        (rc = dalloc_plain((void**)&q.texp, sizeof(int) * (size_t)q.ntiles)))
       break;
     launch_fx_pack((const double2*)q.A, (const double2*)q.B, q.N, q.nT, q.Afx, q.Bfx, q.texp, h->stream);
     ex[i].resize(q.ntiles);
@@ -893,6 +940,7 @@ int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
   h->nq = fx_bands(h->nfx);
   return BSE_OK;
 }
+
 
 // The scales of complex64 tiles, for the fixed-point block products (residuals in FP64 accuracy).
 int setup_scales64(bse_handle* h) {
@@ -1073,6 +1121,31 @@ void setup_tuner(bse_handle* h) {
   auto it = g_tuned.find(h->tkey);
   h->tuned = it != g_tuned.end();
   if (h->tuned) h->shape = it->second;
+}
+
+// The handle without its fixed-point copy: from here on its products run on the FP64 kernels.  The
+// calls of a handle end synchronised, and cudaFree waits for the device, so nothing reads the copy.
+void drop_fx(bse_handle* h) {
+  for (ProbHost& q : h->p) {
+    dfreet(q.Afx);
+    dfreet(q.Bfx);
+    dfreet(q.texp);
+    q.block_fx = false;
+  }
+  h->nfx = h->nq = 0;
+  for (StepGraph& g : h->sg) {               // captured with the fixed-point kernels
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    g.exec = nullptr;
+  }
+  for (Prob& d : h->hprobs) {
+    d.Afx = d.Bfx = nullptr;
+    d.texp = nullptr;
+    d.nq = 0;
+  }
+  if (!h->hprobs.empty())
+    cudaMemcpy(h->dprobs, h->hprobs.data(), sizeof(Prob) * h->hprobs.size(), cudaMemcpyHostToDevice);
+  h->ev_used = 0;
+  setup_tuner(h);
 }
 
 // ------------------------------------------------------------------ apply helpers
@@ -1573,6 +1646,10 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
     bse_destroy(h);
     return rc;
   }
+  if (h->nq > 0) {
+    std::lock_guard<std::mutex> lk(g_fx_mu);
+    g_fx_handles.push_back(h);
+  }
   *out = h;
   return BSE_OK;
 }
@@ -1588,6 +1665,7 @@ int bse_solve_ex(bse_handle* h, int nev, double tol, int which, const bse_solve_
                  void* evec_out, int* nconv_out) {
   if (!h || which != BSE_LOWEST) return BSE_EINVAL;
   if (h->count != 1) return BSE_EINVAL;
+  const Use use(h);
   void* const ev[1] = {evec_out};
   if (h->vs == sizeof(float2)) return solve_impl<float2>(h, nev, tol, opts, eval_out, ev, nconv_out);
   return solve_impl<double2>(h, nev, tol, opts, eval_out, ev, nconv_out);
@@ -1600,6 +1678,7 @@ int bse_solve(bse_handle* h, int nev, double tol, int which, double* eval_out, v
 int bse_solve_batched(bse_handle* h, int nev, double tol, int which, const bse_solve_opts* opts,
                       double* eval_out, void* const* evec_out, int* nconv_out) {
   if (!h || which != BSE_LOWEST) return BSE_EINVAL;
+  const Use use(h);
   if (h->vs == sizeof(float2)) return solve_impl<float2>(h, nev, tol, opts, eval_out, evec_out, nconv_out);
   return solve_impl<double2>(h, nev, tol, opts, eval_out, evec_out, nconv_out);
 }
@@ -1612,6 +1691,7 @@ int bse_backward_ex(bse_handle* h, const double* dL_dlambda, int where, void* dA
   if (h->count != 1) return BSE_EINVAL;
   if (h->ph && !dB) return BSE_EINVAL;
   if (!h->ph && dB) return BSE_EINVAL;
+  const Use use(h);
   if (!h->solved) return BSE_ESTATE;
   if (is_c64(h->dtype)) return backward_impl<float2>(h, dL_dlambda, where, dA, dB, impl);
   return backward_impl<double2>(h, dL_dlambda, where, dA, dB, impl);
@@ -1624,12 +1704,14 @@ int bse_backward(bse_handle* h, const double* dL_dlambda, int where, void* dA, v
 int bse_apply(bse_handle* h, int op, int k, const void* X, void* Y) {
   if (!h || !X || !Y || k < 1 || h->count != 1) return BSE_EINVAL;
   if (op < BSE_OP_A || op > BSE_OP_H) return BSE_EINVAL;
+  const Use use(h);
   if (is_c64(h->dtype)) return apply_impl<float2>(h, op, k, X, Y);
   return apply_impl<double2>(h, op, k, X, Y);
 }
 
 int bse_solve_dense(bse_handle* h, int nev, double tol, double* eval_out, void* evec_out, int* nconv_out) {
   if (!h || h->count != 1 || !h->ph || !eval_out || !(tol > 0.0)) return BSE_EINVAL;
+  const Use use(h);
   ProbHost& q = h->p[0];
   if (nev < 1 || nev > q.N) return BSE_EINVAL;
   int rc;
@@ -1695,6 +1777,7 @@ int bse_apply_mixed(bse_handle* h, int op, double tile_tau, const void* X, void*
   if (!h || !X || !Y || h->count != 1 || !h->mixed) return BSE_EINVAL;
   if (op != BSE_OP_MPLUS && op != BSE_OP_MMINUS) return BSE_EINVAL;
   if (!std::isfinite(tile_tau)) return BSE_EINVAL;
+  const Use use(h);
   ProbHost& q = h->p[0];
   int rc;
   if (!q.w || q.ncv == 0) {
@@ -1725,6 +1808,7 @@ int bse_haydock(bse_handle* h, const void* d, int where, int m, int sign, int nw
   if (where != BSE_HOST && where != BSE_DEVICE) return BSE_EINVAL;
   if (m < 1 || m > 1000000 || nw < 1 || !(eta > 0.0) || !std::isfinite(eta)) return BSE_EINVAL;
   if (h->ph && sign != 1 && sign != -1) return BSE_EINVAL;
+  const Use use(h);
   if (h->vs == sizeof(float2))
     return haydock_impl<float2>(h, d, where, m, sign, nw, omega, eta, spectrum_out, response_out, coef_out,
                                 steps_out);
@@ -1753,6 +1837,10 @@ int bse_get_stats(const bse_handle* h, bse_stats* out) {
 
 int bse_destroy(bse_handle* h) {
   if (!h) return BSE_EINVAL;
+  {
+    std::lock_guard<std::mutex> lk(g_fx_mu);
+    g_fx_handles.erase(std::remove(g_fx_handles.begin(), g_fx_handles.end(), h), g_fx_handles.end());
+  }
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (auto& q : h->p) {
     free_solve_buffers(q);
