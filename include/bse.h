@@ -442,9 +442,18 @@ int bse_selftest_bounded_wait(int arrive, int* expired);
 int bse_get_residuals(const bse_handle* h, int problem, double* res_out, int n);
 
 /*
+ * bse_get_fixed_point -- which arithmetic the products of a BSE_C128 handle
+ * run in: the number of its packed tiles on the fixed-point kernels now
+ * (0 for other handles, without memory for the second copy of the tiles, and
+ * once that copy was given up), and of all its packed tiles.  The two differ
+ * in the last bits of a result.  Either output may be NULL.
+ */
+int bse_get_fixed_point(const bse_handle* h, int64_t* fixed_tiles, int64_t* tiles);
+
+/*
  * bse_measure_fp64_peak -- FP64 FMA throughput of the current device, for the
- * roofline of the FP64 path (whose structured product is bound by the FP64
- * pipe on this GPU).  One launch of `iters` iterations of 8 independent FMA
+ * roofline of the FP64 path (the bound of its products on tiles that are not in
+ * fixed point).  One launch of `iters` iterations of 8 independent FMA
  * chains per thread on every SM, timed with CUDA events after a warm-up;
  * *tflops_out = 2 x FMAs / time.  The paper has no counterpart.  Allocates a
  * small output buffer; BSE_EINVAL for iters outside [1, 2^24].

@@ -28,7 +28,8 @@ BSE_OP_A, BSE_OP_MPLUS, BSE_OP_MMINUS, BSE_OP_H = 0, 1, 2, 3
 EXPORTED = ["bse_strerror", "bse_create", "bse_create_batched", "bse_solve", "bse_solve_ex",
             "bse_solve_batched", "bse_backward", "bse_apply", "bse_get_stats", "bse_destroy",
             "bse_apply_noalloc", "bse_backward_ex", "bse_haydock", "bse_selftest_bounded_wait",
-            "bse_get_residuals", "bse_apply_mixed", "bse_measure_fp64_peak", "bse_solve_dense"]
+            "bse_get_residuals", "bse_apply_mixed", "bse_measure_fp64_peak", "bse_solve_dense",
+            "bse_get_fixed_point"]
 BSE_IMPL_AUTO, BSE_IMPL_CUDA_CORES, BSE_IMPL_TENSOR_CORES = 0, 1, 2
 BSE_VARIANT_SHAO, BSE_VARIANT_GRUNING, BSE_VARIANT_PROJECTED = 0, 1, 2
 BSE_NOALLOC_MAX_N = 4096
@@ -86,6 +87,7 @@ def load_library(path: str | None = None):
     lib.bse_apply.argtypes = [H, c_int, c_int, c_vp, c_vp]
     lib.bse_get_stats.argtypes = [H, ctypes.POINTER(bse_stats)]
     lib.bse_get_residuals.argtypes = [H, c_int, ctypes.POINTER(c_dbl), c_int]
+    lib.bse_get_fixed_point.argtypes = [H, ctypes.POINTER(c_i64), ctypes.POINTER(c_i64)]
     lib.bse_apply_mixed.argtypes = [H, c_int, c_dbl, c_vp, c_vp]
     lib.bse_solve_dense.argtypes = [H, c_int, c_dbl, ctypes.POINTER(c_dbl), c_vp, ctypes.POINTER(c_int)]
     lib.bse_measure_fp64_peak.argtypes = [c_int, ctypes.POINTER(c_dbl), ctypes.POINTER(c_dbl)]
@@ -219,6 +221,13 @@ def bse_get_residuals(h, n, problem=0):
     r = (ctypes.c_double * max(n, 1))()
     _check(load_library().bse_get_residuals(h, int(problem), r, int(n)), "bse_get_residuals")
     return np.array(r[:n], dtype=np.float64)
+
+
+def bse_get_fixed_point(h):
+    """(tiles whose products run in fixed point, all packed tiles) of a handle."""
+    f, t = ctypes.c_int64(), ctypes.c_int64()
+    _check(load_library().bse_get_fixed_point(h, ctypes.byref(f), ctypes.byref(t)), "bse_get_fixed_point")
+    return f.value, t.value
 
 
 def bse_measure_fp64_peak(iters=1 << 16):

@@ -1829,6 +1829,13 @@ int bse_get_residuals(const bse_handle* h, int problem, double* res_out, int n) 
   return BSE_OK;
 }
 
+int bse_get_fixed_point(const bse_handle* h, int64_t* fixed_tiles, int64_t* tiles) {
+  if (!h) return BSE_EINVAL;
+  if (fixed_tiles) *fixed_tiles = h->nfx;
+  if (tiles) *tiles = h->njobs;
+  return BSE_OK;
+}
+
 int bse_get_stats(const bse_handle* h, bse_stats* out) {
   if (!h || !out) return BSE_EINVAL;
   *out = h->stats;

@@ -73,3 +73,23 @@ def test_new_handle_takes_the_memory_of_an_idle_one():
     np.testing.assert_allclose(r2, r0, rtol=1e-10, atol=0)
     first.close()
     second.close()
+
+
+def test_handle_reports_its_arithmetic():
+    """How many tiles run in fixed point: all of a dense matrix (3 x 3 blocks), none of a graded one, none
+    after the copy was given up, none of a complex64 handle."""
+    from paper_2504_10096_gb300 import bse
+    A, B = _matrices(300)
+    d = torch.logspace(0, -12, 300, dtype=torch.float64, device="cuda").to(A.dtype)
+    for a, b, fixed in ((A, B, 6), (A * d[:, None] * d[None, :], B * d[:, None] * d[None, :], 0),
+                        (A.to(torch.complex64), B.to(torch.complex64), 0)):
+        s = bse.Solver(a, b)
+        assert bse.bse_get_fixed_point(s.h) == (fixed, 6)
+        s.close()
+    A, B = _matrices(4000)
+    s = bse.Solver(A, B)
+    assert bse.bse_get_fixed_point(s.h) == (528, 528)
+    with _Filled(200 * MB):
+        s.solve(4, tol=1e-9, ncv=1000, vectors=False)
+    assert bse.bse_get_fixed_point(s.h) == (0, 528)
+    s.close()
