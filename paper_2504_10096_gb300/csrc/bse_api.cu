@@ -329,6 +329,22 @@ int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, do
   return BSE_OK;
 }
 
+// BSE_ETIMEOUT when perr, the flag of the product kernels, was raised by an expired wait; the flag is
+// lowered, so only the call that ran into it fails
+int expired_wait(bse_handle* h, int perr) {
+  if (!perr) return BSE_OK;
+  CK(cudaMemsetAsync(h->prod_err, 0, sizeof(int), h->stream));
+  return BSE_ETIMEOUT;
+}
+
+// waits for the handle's stream and reads that flag
+int sync_product(bse_handle* h) {
+  int perr = 0;
+  if (h->prod_err) CK(cudaMemcpyAsync(&perr, h->prod_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return expired_wait(h, perr);
+}
+
 int map_status(int st) {
   switch (st) {
     case ST_OK: return BSE_OK;
@@ -567,6 +583,7 @@ struct Driver {
     if (!h->gbar) {
       const int rc = dalloc((void**)&h->gbar, sizeof(GridBar));
       if (rc) return rc;
+      CK(cudaMemsetAsync(h->gbar, 0, sizeof(GridBar), h->stream));
     }
     const int r = launch_steps_persist<ST, R>(h->dprobs, h->djobs, h->njobs, h->nfx, h->ph != 0, steps, h->gbar,
                                               h->stream);
@@ -603,7 +620,12 @@ struct Driver {
     CK(cudaStreamSynchronize(h->stream));
     CK(cudaGetLastError());
     harvest_events();
-    return (perr || gb.err) ? BSE_ETIMEOUT : BSE_OK;
+    if (gb.err) {
+      expired_wait(h, perr);
+      CK(cudaMemsetAsync(h->gbar, 0, sizeof(GridBar), h->stream));
+      return BSE_ETIMEOUT;
+    }
+    return expired_wait(h, perr);
   }
 
   int iterate(uint64_t seed, const void* v0) {
@@ -1200,14 +1222,6 @@ __global__ void k_cvt_pad(const ST* __restrict__ X, int64_t N, int64_t Npad, int
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= Npad) return;
   out[(int64_t)c * Npad + r] = r < N ? ccvt<CT>(X[(int64_t)c * N + r]) : czero<CT>();
-}
-
-// waits for the handle's stream; BSE_ETIMEOUT if a product kernel's bounded wait expired
-int sync_product(bse_handle* h) {
-  int perr = 0;
-  if (h->prod_err) CK(cudaMemcpyAsync(&perr, h->prod_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  return perr ? BSE_ETIMEOUT : BSE_OK;
 }
 
 template <typename ST>
