@@ -124,6 +124,7 @@ struct bse_handle {
   void* post = nullptr;
   size_t post_bytes = 0;
   void* blk = nullptr;       // workspace of the fixed-point block product
+  bool scaled64 = false;     // complex64 tiles: their scales have been worked out
   size_t blk_bytes = 0;
   // adjoint tile list
   int2* adj_tiles = nullptr;
@@ -293,8 +294,15 @@ int pack_matrix(bse_handle* h, const T* src, int64_t N, int nT, int herm, int wh
 // below kBlkBytes whatever K is, and the grid's second dimension below its limit.
 constexpr size_t kBlkBytes = (size_t)256 << 20;
 
+int setup_scales64(bse_handle* h);
+
 int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB) {
   ProbHost& q = h->p[i];
+  if (h->tiles64 && !h->scaled64) {
+    const int rc = setup_scales64(h);
+    if (rc != BSE_OK && rc != BSE_ENOMEM) return rc;
+    h->scaled64 = true;
+  }
   // (complex128 PH tiles hold P and Q, so they always go through the two-matrix form)
   if (hasB == (h->ph != 0) && q.block_fx) {
     int kg = std::min(K, 32768);
@@ -964,18 +972,20 @@ int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
 }
 
 
-// The scales of complex64 tiles, for the fixed-point block products (residuals in FP64 accuracy).
+// The scales of complex64 tiles, for the fixed-point block products (residuals in FP64 accuracy): made by
+// the first of them, so a handle that never asks for one does not read its tiles for it.
 int setup_scales64(bse_handle* h) {
   std::vector<std::vector<int>> ex(h->count);
+  int rc = BSE_OK;
   for (int i = 0; i < h->count; ++i) {
     ProbHost& q = h->p[i];
-    const int rc = dalloc((void**)&q.texp, sizeof(int) * (size_t)q.ntiles);
-    if (rc) return rc;
+    if ((rc = dalloc((void**)&q.texp, sizeof(int) * (size_t)q.ntiles))) break;
     launch_block_scale64((const float2*)q.A, (const float2*)q.B, q.N, q.nT, q.texp, h->stream);
     ex[i].resize(q.ntiles);
     CK(cudaMemcpyAsync(ex[i].data(), q.texp, sizeof(int) * (size_t)q.ntiles, cudaMemcpyDeviceToHost, h->stream));
   }
   CK(cudaStreamSynchronize(h->stream));
+  if (rc) return rc;
   for (int i = 0; i < h->count; ++i) h->p[i].block_fx = *std::min_element(ex[i].begin(), ex[i].end()) >= 0;
   return BSE_OK;
 }
@@ -1637,7 +1647,6 @@ int bse_create_batched(int count, const int64_t* N, const void* const* A, const 
   for (const ProbHost& q : h->p) rows += q.Npad;
   while (h->slab > 8 && rows / (h->slab / 2) <= num_sms()) h->slab /= 2;
   if (rc == BSE_OK && dtype == BSE_C128) rc = setup_fx(h, jobs);
-  if (rc == BSE_OK && h->tiles64) rc = setup_scales64(h);
   if (rc == BSE_OK && h->mixed) h->hjobs = jobs;
   if (rc == BSE_OK && (h->mixed || h->nfx > 0)) {
     rc = dalloc((void**)&h->prod_err, 2 * sizeof(int));
