@@ -107,6 +107,7 @@ struct bse_handle {
   int njobs = 0;
   int nfx = 0;           // complex128: the first nfx jobs are fixed-point tiles, in nq bands each
   int nq = 0;            // (0: the handle has no fixed-point tiles)
+  void* fx = nullptr;    // the fixed-point copy of the tiles and its scales (ProbHost::Afx, Bfx, texp)
   std::vector<TileJob> hjobs;
   // mixed PH path: the tile jobs split by precision for the current solve
   bool mixed = false;        // BSE_C64_MIXED with B
@@ -294,15 +295,8 @@ int pack_matrix(bse_handle* h, const T* src, int64_t N, int nT, int herm, int wh
 // below kBlkBytes whatever K is, and the grid's second dimension below its limit.
 constexpr size_t kBlkBytes = (size_t)256 << 20;
 
-int setup_scales64(bse_handle* h);
-
 int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB) {
   ProbHost& q = h->p[i];
-  if (h->tiles64 && !h->scaled64) {
-    const int rc = setup_scales64(h);
-    if (rc != BSE_OK && rc != BSE_ENOMEM) return rc;
-    h->scaled64 = true;
-  }
   // (complex128 PH tiles hold P and Q, so they always go through the two-matrix form)
   if (hasB == (h->ph != 0) && q.block_fx) {
     int kg = std::min(K, 32768);
@@ -937,44 +931,68 @@ int split_mixed_jobs(bse_handle* h, double tol, double tau_opt) {
   return BSE_OK;
 }
 
+void free_fx(bse_handle* h) {
+  for (ProbHost& q : h->p) {
+    q.Afx = q.Bfx = nullptr;
+    if (!h->tiles64) q.texp = nullptr;
+    q.block_fx = false;
+  }
+  dfree(h->fx);
+}
+
+constexpr size_t kFxUnasked = (size_t)64 << 20;    // copies up to this size are made without asking for the free memory
+
 // The fixed-point copy of a complex128 handle's tiles (fx_phases.cuh), which doubles its packed
 // storage: made when it takes at most a third of the device memory that is free (a handle that
 // nearly fills the GPU, or one that finds it nearly full, keeps the FP64 product alone), and given
 // back when an allocation needs its memory (drop_fx).  The jobs are reordered: fixed-point tiles first.
 int setup_fx(bse_handle* h, std::vector<TileJob>& jobs) {
-  size_t need = 0, freeb = 0, totalb = 0;
-  for (const ProbHost& q : h->p) need += (size_t)q.ntiles * TS * TS * sizeof(int4) * (h->ph ? 2 : 1);
-  if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess) { cudaGetLastError(); return BSE_OK; }
-  if (need > freeb / 3) return BSE_OK;
-  std::vector<std::vector<int>> ex(h->count);
-  int rc = BSE_OK;
-  for (int i = 0; i < h->count && rc == BSE_OK; ++i) {
-    ProbHost& q = h->p[i];
-    const size_t bytes = (size_t)q.ntiles * TS * TS * sizeof(int4);
-    if ((rc = dalloc_plain((void**)&q.Afx, bytes)) || (h->ph && (rc = dalloc_plain((void**)&q.Bfx, bytes))) ||
-        (rc = dalloc_plain((void**)&q.texp, sizeof(int) * (size_t)q.ntiles)))
-      break;
+  // one buffer: the scales of all problems, then limbs of A (and B) problem by problem
+  const int nm = h->ph ? 2 : 1;
+  size_t ntiles = 0;
+  for (const ProbHost& q : h->p) ntiles += (size_t)q.ntiles;
+  const size_t head = (sizeof(int) * ntiles + 255) / 256 * 256, tile = (size_t)TS * TS * sizeof(int4);
+  const size_t need = head + ntiles * tile * nm;
+  if (need > kFxUnasked) {
+    size_t freeb = 0, totalb = 0;
+    if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess) { cudaGetLastError(); return BSE_OK; }
+    if (need > freeb / 3) return BSE_OK;
+  }
+  const int rc = dalloc_plain(&h->fx, need);
+  if (rc != BSE_OK) return rc == BSE_ENOMEM ? BSE_OK : rc;
+  int* texp = (int*)h->fx;
+  char* limbs = (char*)h->fx + head;
+  for (ProbHost& q : h->p) {
+    q.texp = texp;
+    texp += q.ntiles;
+    q.Afx = (int4*)limbs;
+    q.Bfx = h->ph ? (int4*)(limbs + (size_t)q.ntiles * tile) : nullptr;
+    limbs += (size_t)q.ntiles * tile * nm;
     launch_fx_pack((const double2*)q.A, (const double2*)q.B, q.N, q.nT, q.Afx, q.Bfx, q.texp, h->stream);
-    ex[i].resize(q.ntiles);
-    CK(cudaMemcpyAsync(ex[i].data(), q.texp, sizeof(int) * (size_t)q.ntiles, cudaMemcpyDeviceToHost, h->stream));
   }
+  std::vector<int> ex(ntiles);
+  CK(cudaMemcpyAsync(ex.data(), h->fx, sizeof(int) * ntiles, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  if (rc != BSE_OK) {
-    for (ProbHost& q : h->p) { dfreet(q.Afx); dfreet(q.Bfx); dfreet(q.texp); }
-    return rc == BSE_ENOMEM ? BSE_OK : rc;
+  std::vector<const int*> first(h->count);
+  const int* e = ex.data();
+  for (int i = 0; i < h->count; ++i) {
+    first[i] = e;
+    h->p[i].block_fx = *std::min_element(e, e + h->p[i].ntiles) >= 0;
+    e += h->p[i].ntiles;
   }
-  for (int i = 0; i < h->count; ++i) h->p[i].block_fx = *std::min_element(ex[i].begin(), ex[i].end()) >= 0;
   const auto mid = std::stable_partition(jobs.begin(), jobs.end(),
-                                         [&](const TileJob& j) { return ex[j.prob][j.t] >= 0; });
+                                         [&](const TileJob& j) { return first[j.prob][j.t] >= 0; });
   h->nfx = (int)(mid - jobs.begin());
-  h->nq = fx_bands(h->nfx);
+  h->nq = h->nfx > 0 ? fx_bands(h->nfx) : 0;
+  if (h->nfx == 0) free_fx(h);           // nothing would read it
   return BSE_OK;
 }
 
-
 // The scales of complex64 tiles, for the fixed-point block products (residuals in FP64 accuracy): made by
-// the first of them, so a handle that never asks for one does not read its tiles for it.
+// the first solve, so a handle that is never asked for one does not read its tiles for it.
 int setup_scales64(bse_handle* h) {
+  if (!h->tiles64 || h->scaled64) return BSE_OK;
+  h->scaled64 = true;
   std::vector<std::vector<int>> ex(h->count);
   int rc = BSE_OK;
   for (int i = 0; i < h->count; ++i) {
@@ -985,7 +1003,7 @@ int setup_scales64(bse_handle* h) {
     CK(cudaMemcpyAsync(ex[i].data(), q.texp, sizeof(int) * (size_t)q.ntiles, cudaMemcpyDeviceToHost, h->stream));
   }
   CK(cudaStreamSynchronize(h->stream));
-  if (rc) return rc;
+  if (rc) return rc == BSE_ENOMEM ? BSE_OK : rc;       // the row-block kernel takes them
   for (int i = 0; i < h->count; ++i) h->p[i].block_fx = *std::min_element(ex[i].begin(), ex[i].end()) >= 0;
   return BSE_OK;
 }
@@ -1056,10 +1074,11 @@ int solve_impl(bse_handle* h, int nev, double tol, const bse_solve_opts* opts, d
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, h->stream);
+  rc = setup_scales64(h);
   const long long launches0 = launch_counter();
   Driver<ST> drv(h);
   h->graphs = graphs;
-  rc = drv.iterate(seed, v0);
+  if (!rc) rc = drv.iterate(seed, v0);
   if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
   int worst = BSE_OK;
   double maxres = 0.0;
@@ -1158,12 +1177,7 @@ void setup_tuner(bse_handle* h) {
 // The handle without its fixed-point copy: from here on its products run on the FP64 kernels.  The
 // calls of a handle end synchronised, and cudaFree waits for the device, so nothing reads the copy.
 void drop_fx(bse_handle* h) {
-  for (ProbHost& q : h->p) {
-    dfreet(q.Afx);
-    dfreet(q.Bfx);
-    dfreet(q.texp);
-    q.block_fx = false;
-  }
+  free_fx(h);
   h->nfx = h->nq = 0;
   for (StepGraph& g : h->sg) {               // captured with the fixed-point kernels
     if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -1751,6 +1765,7 @@ int bse_solve_dense(bse_handle* h, int nev, double tol, double* eval_out, void* 
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, h->stream);
+  if ((rc = setup_scales64(h))) return rc;
   const long long launches0 = launch_counter();
   h->solved = false;
   h->nev = nev;
@@ -1879,9 +1894,7 @@ int bse_destroy(bse_handle* h) {
     dfree(q.B);
     dfree(q.Ahl);
     dfree(q.Bhl);
-    dfreet(q.Afx);
-    dfreet(q.Bfx);
-    dfreet(q.texp);
+    if (h->tiles64) dfreet(q.texp);
     dfreet(q.tmax);
     dfree(q.UV);
   }
@@ -1893,6 +1906,7 @@ int bse_destroy(bse_handle* h) {
   dfreet(h->clock);
   dfreet(h->djobs);
   dfree(h->post);
+  dfree(h->fx);
   dfree(h->blk);
   dfreet(h->pj_work);
   dfreet(h->pj_flag);
