@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(32) k_dn_inverse(DnS S, int64_t n, int nev, co
   F.du = w + 2 * n;
   F.du2 = w + 3 * n;
   F.piv = (unsigned char*)(w + 4 * n);
-  const double pivmin = eps * fmax(bound, 1e-300);
+  const double pivmin = eps * fmax(bound, 1e-290);
   double lprev = -1e300;
   for (int c = c0; c < c1; ++c) {
     double lm = lam[c];
@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(256) k_dn_back(const double* __restrict__ Wv, 
   fetch_row(n - 1);
   double dn = __ldg(L + (n - 1) * ld + n - 1);
   for (int64_t i = n - 1; i >= 0; --i) {
-    const double inv = recip(dn);
+    const double inv = recip_any(dn);
     double cur[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) cur[u] = nx[u];

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(32) k_ritz_vectors(const Prob* __restrict__ pr
   // pivot guard of the inverse iteration: a shift equal to a leaf value (a
   // converged kept Ritz value with a negligible coupling) must give a large
   // but finite growth, so tiny pivots are replaced by eps * ||T||
-  const double pivmin = eps * fmax(tnorm, 1e-300);
+  const double pivmin = eps * fmax(tnorm, 1e-290);    // normal, and its reciprocal too
   const double pert = 10.0 * eps * tnorm;
   double lam_prev = -1e300;
   for (int i = i0; i < i1; ++i) {

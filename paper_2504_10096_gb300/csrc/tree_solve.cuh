@@ -10,8 +10,8 @@
 //     arithmetic (FP32 pipes), and FP64 counts take over from there: they check that the bracket
 //     holds the wanted index (else they start from the whole interval) and finish to FP64
 //     accuracy, so the result does not rest on the FP32 counts;
-//   * reciprocals are the hardware's 20-bit one and one cubic Newton step, r (1 + e + e^2) with
-//     e = 1 - q r (three FMAs), signs and magnitudes are compared as integers;
+//   * reciprocals are the hardware's 20-bit one and one step of the third-order iteration (three
+//     FMAs, recip), signs and magnitudes are compared as integers;
 //   * in the factorisation and the solves the leaves go over the lanes, and only the path part
 //     (the new Lanczos vectors of the cycle) is sequential, with the pivots' reciprocals kept.
 #pragma once
@@ -31,12 +31,21 @@ struct TV {        // view of the matrix
 
 __device__ __forceinline__ int mag_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
 
-// 1 / q to FP64 rounding for a normal q: the hardware's approximation and one cubic Newton step
+// 1 / q within an ulp, for a normal q with a normal reciprocal: the hardware's approximation r (20 bits)
+// and one step of the third-order iteration r (1 + e + e^2), e = 1 - q r (the first terms of the
+// geometric series of 1 / (1 - e)): what is left of r's error is its cube, 2^-60.  The pivots below are
+// in that range: of a finite T none is smaller than its pivmin (1e-306 at least) or larger than 1e300.
 __device__ __forceinline__ double recip(double q) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
   const double e = fma(-q, r, 1.0);
   return fma(r, fma(e, e, e), r);
+}
+// ... for any q: zero, a subnormal, one above 2^1022, an infinity or a NaN goes to the division (which
+// costs the loops of the counts and factorisations 1 % where it is not needed)
+__device__ __forceinline__ double recip_any(double q) {
+  const unsigned ex = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
+  return ex - 1u < 2044u ? recip(q) : 1.0 / q;
 }
 
 // a pivot of the Sturm count: tiny ones become -pivmin (their high words compared); the sign adds
