@@ -89,3 +89,37 @@ def test_more_columns_than_one_launch_takes(n, k):
     ref = torch.cat([at @ X[:n] + bt @ X[n:], -(bt.conj() @ X[:n] + at.conj() @ X[n:])])
     mag = torch.cat([at.abs() @ X[:n].abs() + bt.abs() @ X[n:].abs(), bt.abs() @ X[:n].abs() + at.abs() @ X[n:].abs()])
     assert bool(((Y - ref).abs() <= 64 * UNIT["c128"] * 2 * mag).all())       # both sides are off by as much
+
+
+@pytest.mark.parametrize("form", ["ph", "tda"])
+@pytest.mark.parametrize("n", [140, 520, 1300])
+def test_solve_with_tiles_of_both_kinds(n, form):
+    """A matrix with holes in every other off-diagonal tile and one graded stripe: the tiles divide between
+    fixed point (in bands at these orders) and FP64, in the persistent launch, the replayed graphs and the
+    single launches alike."""
+    from paper_2504_10096_gb300 import bse
+    rng = np.random.default_rng(n)
+    a, b = _matrices(rng, n)
+    a, b = 1e-3 * a, 1e-3 * b
+    for m in (a, b):
+        for i in range(0, n, 256):
+            if i + 130 < n:
+                m[i + 3, i + 130] = m[i + 130, i + 3] = 0
+        m[:5] *= 1e-9
+        m[:, :5] *= 1e-9
+    np.fill_diagonal(a, np.linspace(1.0, 9.0, n))
+    s = bse.Solver(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda() if form == "ph" else None)
+    fixed, tiles = bse.bse_get_fixed_point(s.h)
+    assert 0 < fixed < tiles
+    out = [s.solve(8, tol=1e-12, **kw) for kw in ({}, {"persistent": False}, {"graphs": False})]
+    for vals, vecs, nconv in out:
+        assert nconv == 8 and s.residuals().max() <= 1e-12
+        assert np.array_equal(vals, out[0][0]) and torch.equal(vecs, out[0][1])
+    s.close()
+    if form == "tda":
+        ref = np.linalg.eigvalsh(a)[:8]
+    else:
+        real = lambda t: np.block([[a.real + t * b.real, -a.imag + t * b.imag], [a.imag + t * b.imag, a.real - t * b.real]])  # noqa: E731
+        low = np.linalg.cholesky(real(-1.0))
+        ref = np.sqrt(np.linalg.eigvalsh(low.T @ real(1.0) @ low)[:16:2])
+    np.testing.assert_allclose(out[0][0], ref, rtol=1e-11, atol=0)
