@@ -5,7 +5,7 @@
 // the phases separated by a grid barrier).  A body computes the same bits in either setting:
 // it takes its work unit and shared memory as arguments and keeps the summation order of the
 // unit fixed.  Loads of data that a persistent launch rewrites between its phases (the Krylov
-// basis, the work vectors, the partial sums) go through ldv / ldv<COH>: L2 loads (ordered by
+// basis, the work vectors, the partial sums) go through ldv<COH>: L2 loads (ordered by
 // the barrier's fences, and never served from a stale L1 line) when COH.
 #pragma once
 

@@ -237,7 +237,8 @@ k_block_fx(const void* __restrict__ M0, const void* __restrict__ M1, const int* 
             }
           }
         }
-        // after 8 (hl) or 16 (hh) products a sum is below 2^63 with the 2^38 left before
+        // after 16 products of two limbs (2^58 each at most; hl takes eight per q, hh four) a sum is below
+        // 2^63 with the 2^38 left before
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll

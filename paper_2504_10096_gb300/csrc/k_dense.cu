@@ -410,13 +410,6 @@ __global__ void __launch_bounds__(RV_THREADS) k_dn_bisect(DnS S, int64_t n, int6
   if (threadIdx.x == 0) lam[blockIdx.x] = v;
 }
 
-__device__ __forceinline__ uint64_t dn_mix(uint64_t x) {
-  x += 0x9e3779b97f4a7c15ull;
-  x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
-  x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
-  return x ^ (x >> 31);
-}
-
 // inverse iteration for the eigenvectors of S, one warp per cluster of close eigenvalues
 // (Gram-Schmidt inside a cluster); the factorisation in shared memory (SM) or in 5 n doubles of
 // scratch; vectors s_c (n doubles each, unit 2-norm) go to Sv[c * n ...]
@@ -453,7 +446,7 @@ __global__ void __launch_bounds__(32) k_dn_inverse(DnS S, int64_t n, int nev, co
     factor_tree(tv, lm, pivmin, F, lane);
     double* x = Sv + (int64_t)c * n;
     for (int64_t t = lane; t < n; t += 32)
-      x[t] = (double)(dn_mix((uint64_t)(c + 1) * 0x100000001b3ull + (uint64_t)t) >> 11) * (1.0 / 9007199254740992.0) - 0.5;
+      x[t] = (double)(mix64((uint64_t)(c + 1) * 0x100000001b3ull + (uint64_t)t) >> 11) * (1.0 / 9007199254740992.0) - 0.5;
     __syncwarp();
     for (int it = 0; it < 4; ++it) {
       for (int rep = 0; rep < 2; ++rep)

@@ -77,7 +77,7 @@ __device__ __forceinline__ CT na_elem(const CT* M, int64_t N, int64_t gi, int64_
 // solver's streaming product: y_I += A_IJ x_J + s B_IJ conj(x_J), y_J += A_IJ^H x_I + s B_IJ^T conj(x_I).
 // A band's column sums go to plane q of the slots.  Small problems are cut into bands because a
 // whole tile takes a CTA's time whatever the number of tiles: N = 600 (15 tiles), complex64, 28 us a
-// call without bands, 16 with eight.
+// call without bands, 16 to 18 with eight (by the machine).
 template <typename R, bool HASB, int NR>
 __global__ void __launch_bounds__(256)
 k_na_tiles(int64_t N, int nT, const typename NAC<R>::T* __restrict__ A, const typename NAC<R>::T* __restrict__ B,

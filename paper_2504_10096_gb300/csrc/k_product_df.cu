@@ -557,12 +557,6 @@ __device__ __forceinline__ void gacc(f2& H, f2& L, f2 u, f2 xh, f2 xl) {
   H = t;
 }
 
-__device__ __forceinline__ void two_sum1(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bp = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
-}
-
 // (grid part, tail) pairs of the coarse kernel's cross-lane sums: the grid parts of all lanes
 // lie on one grid coarse enough that their sums are exact, so the pairs add with plain adds
 __device__ __forceinline__ DFC gadd(DFC a, const DFC& b) {
