@@ -187,9 +187,10 @@ def _config(ncv=0):
 
 
 # ------------------------------------------------------------------ GPU arm
-# dram__bytes_read.sum + dram__bytes_write.sum of one k_prod_tiles_df launch at N = 8000
-# (profiles/k_prod_tiles_df_n8000.md); None until the current kernel has been captured
-TRAFFIC_N8000 = {"fp64": None, "df": 1.067138e9 + 22.040064e6}
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the product's tile kernel and the packed
+# tiles it streams (per matrix): k_prod_tiles_fx at N = 6000 (profiles/k_prod_tiles_fx_n6000.md),
+# k_prod_tiles_df at N = 8000 (profiles/k_prod_tiles_df_n8000.md)
+TRAFFIC = {"fp64": (591.759e6 + 4.631e6, 47 * 48 // 2), "df": (1.067138e9 + 22.040064e6, 63 * 64 // 2)}
 
 
 def run_gpu(args):
@@ -313,12 +314,10 @@ def run_gpu(args):
         return
     cpu_v, cpu_raw = cpu_baseline_sample()
     value = ms_max / 1e3
-    # DRAM traffic per launch from the ncu captures at N = 8000 (profiles/k_prod_tiles_df_n8000.md):
-    # bytes per stored 128x128 tile pair, scaled by the tile count of this workload (traffic grows
-    # with the number of tiles streamed)
-    n_tiles_8000 = 63 * 64 // 2
-    captured = TRAFFIC_N8000.get("df" if args.df else "fp64")
-    traffic = None if captured is None else captured / (2 * n_tiles_8000) * 2 * (n_tiles * (n_tiles + 1) // 2)
+    # DRAM traffic per launch from the ncu captures: bytes per stored 128x128 tile pair, scaled by the
+    # tile count of this workload (traffic grows with the number of tiles streamed)
+    captured, tiles = TRAFFIC["df" if args.df else "fp64"]
+    traffic = captured / tiles * (n_tiles * (n_tiles + 1) // 2)
     if args.df:
         roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": peaks.get("hbm_gbs"), "unit": "GB/s",
                 "frac": achieved_gbs / peaks.get("hbm_gbs", 6800.0), "traffic": traffic,
