@@ -63,15 +63,14 @@ typedef enum bse_dtype {
      Rayleigh-quotient refinement (the mixed-precision path) */
   BSE_C64 = 0,
   /* complex128 storage; products to FP64 accuracy (the FP64 path): each entry
-     of Y = M X is off by at most a few tens of 2^-53 (|M||X|)_i.  They run in
+     of Y = M X is off by a few 2^-53 (|M||X|)_i, whatever X is (by some tens
+     where an entry of X far above the others couples weakly).  They run in
      60-bit fixed point on a second copy of the packed tiles, made when it
      fits in a third of the free memory and given up when a later allocation
      of this library needs its memory, on every 128 x 128 tile whose entries
-     lie within a factor 2^16 of one another (entries of X may differ by any
-     factor), and in FP64 FMAs otherwise.  Where X has one entry far above all
-     others of its 128-entry chunk, an entry of Y that couples to it by 2^-s
-     of the tile's largest element may be off by 2^(s - 59) of that coupling
-     (s <= 16) */
+     lie within a factor 2^16 of one another (sums that may be too small for
+     the scales of tile and vector are formed again in FP64), and in FP64 FMAs
+     otherwise */
   BSE_C128 = 1,
   /* complex64 input and storage of A and B (half the bytes of BSE_C128);
      FP64 Krylov basis; the Lanczos products in double-FP32 arithmetic on

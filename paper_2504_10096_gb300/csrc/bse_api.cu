@@ -292,10 +292,12 @@ int pack_matrix(bse_handle* h, const T* src, int64_t N, int nT, int herm, int wh
 
 // Y = A XA + sB B XB (FP64 blocks of K columns, Npad rows) with the stored tiles of problem i.  The
 // fixed-point kernels take the columns in groups: their workspace (2 + splits times the group) stays
-// below kBlkBytes whatever K is, and the grid's second dimension below its limit.
+// below kBlkBytes whatever K is, and the grid's second dimension below its limit.  each: every entry to
+// FP64 accuracy against |M||x| (else in norm, which is what a residual needs).
 constexpr size_t kBlkBytes = (size_t)256 << 20;
 
-int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB) {
+int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, double sB, double2* y, int K, bool hasB,
+                  bool each) {
   ProbHost& q = h->p[i];
   // (complex128 PH tiles hold P and Q, so they always go through the two-matrix form)
   if (hasB == (h->ph != 0) && q.block_fx) {
@@ -313,6 +315,8 @@ int block_product(bse_handle* h, int i, const double2* xa, const double2* xb, do
       b.texp = q.texp;
       b.A = q.A;
       b.B = q.B;
+      b.N = q.N;
+      b.each = each;
       b.nT = q.nT;
       for (int c = 0; c < K; c += kg) {
         const int64_t o = (int64_t)c * q.Npad;
@@ -733,7 +737,7 @@ struct Driver {
     const void* xb = h->ph ? (const void*)XB : nullptr;
     const double sgn = h->ph ? 1.0 : 0.0;
     if (h->ph) launch_prepare_hz2(q.Z, ldz, Npad, k, XA, XB, h->stream);
-    if ((rc = block_product(h, i, (const double2*)xa, (const double2*)xb, sgn, U, kc, h->ph != 0))) return rc;
+    if ((rc = block_product(h, i, (const double2*)xa, (const double2*)xb, sgn, U, kc, h->ph != 0, false))) return rc;
     launch_residuals2(q.Z, ldz, U, Npad, k, h->ph, part4, nrb, rho, z2, res, h->stream);
     CK(cudaGetLastError());
     std::vector<double> hr(k), hres(k);
@@ -1317,7 +1321,7 @@ int apply_impl(bse_handle* h, int op, int k, const void* X, void* Y) {
   // P, Q tiles always go through the unpacking variant (sB = 0 drops the B half)
   const bool two = hasB && (op != BSE_OP_A || !h->tiles64);
   if constexpr (std::is_same<ST, double2>::value) {
-    if ((rc = block_product(h, 0, XA, (const double2*)xb, sB, U, kc, two))) return rc;
+    if ((rc = block_product(h, 0, XA, (const double2*)xb, sB, U, kc, two, true))) return rc;
   } else {
     launch_rowblock<ST, R>(h->dprobs, 0, q.nT, XA, xb, (int)Npad, sB, U, (int)Npad, kc, two, h->stream);
   }

@@ -174,7 +174,7 @@ struct Prob {
   float4* ws;
   // complex128 tiles in fixed point (fx_phases.cuh; null where the FP64 product runs alone):
   // int4 limbs {re_hi, re_lo, im_hi, im_lo} per packed element of A and B (P and Q on PH
-  // handles), diagonal left out; the biased exponent of each tile's scale (-1: the tile is on
+  // handles), diagonal left out; the biased exponent of each tile's scale and its weak entries (-1: the tile is on
   // the FP64 kernel); and the bands per tile, whose column sums take nq planes of `part`
   const int4* Afx;
   const int4* Bfx;
@@ -342,10 +342,12 @@ int num_sms();                 // of the current device
 struct BlockFx {
   const void* M0;     // limbs of A (P on PH handles), or complex64 A
   const void* M1;     // ... of B (Q), or complex64 B; null without B
-  const int* texp;    // scale exponents of the tiles, all >= 0
+  const int* texp;    // scale exponents (and weak entries) of the tiles, all >= 0
   const void* A;      // the packed tiles themselves (the diagonal's part is FP64)
   const void* B;
+  int64_t N;
   int nT;
+  bool each;          // accurate entry by entry (|M||x|), not only in norm
 };
 int block_fx_splits(int nT, int K);
 size_t block_fx_bytes(int nT, int K, bool hasB);

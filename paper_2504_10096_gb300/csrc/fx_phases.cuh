@@ -15,18 +15,22 @@
 // value per tile, row and column, built with integer instructions.
 //
 // Accuracy.  Each entry of U and of x is off by at most 2^-60 of its tile's or chunk's 2^E, each
-// product by 2^-60 (the dropped term); the sums add nothing.  So what a tile adds to a row is off by
-// some 2^-57 max|U| max|x| (about 2^-59 when one entry of x is far above the others), where an FP64 dot
-// product is off by 2^-53 of the row's own sum of magnitudes |U||x|.  That sum is at least min|U| max|x|:
-// a tile runs in fixed point only when every entry of the matrix in it is within 2^FX_SPREAD of its
-// largest (k_fx_pack; in the diagonal tiles the diagonal counts as one of the entries), whatever x is.
-// Sparse tiles, graded rows or columns, a peak, an infinity, a NaN, or exponents near the ends of the
+// product by 2^-60 (the dropped term); the sums add nothing.  So a sum over a tile is off by some
+// 2^-57.6 of 2^(E_u + E_x) (root mean square over its 256 multiply-adds; 2^-59 where one entry of x is far
+// above the others), where an FP64 one is off by 2^-53 of its own sum of magnitudes |U||x|.  So a sum is
+// good to a few tens of 2^-53 |U||x| if |U||x| is at least 2^-10 or 2^-11 of 2^(E_u + E_x).  That is sure when
+//   * the chunk has FX_MASS strong entries more than any row (column) of the tile has weak ones: FX_MASS pairs
+//     of 2^-2 FX_STRONG max|U| max|x| each.  Almost every sum is certified that way, before it is formed; or
+//   * the sum itself is that large (2^-FX_SURE; less for the few terms of the matrix's last rows and columns).
+// Any other sum -- x with a few entries far above the rest of its chunk, mostly -- is formed again in FP64 by
+// a warp.  For these to be rare a tile runs in fixed point only when every entry of the matrix in
+// it is within 2^FX_SPREAD of its largest (k_fx_pack; in the diagonal tiles the diagonal counts as one
+// of the entries).  Sparse tiles, graded rows or columns, a peak, an infinity, a NaN, or exponents near the ends of the
 // FP64 range keep a tile on the FP64 kernel.  Why 2^16: 16384 entries without structure spread by
 // themselves (2^5 to 2^10 for a complex pair A, B; 2^8 to 2^14 for a complex A alone, one tile in 600
-// above that and about one in 50000 above 2^16), a tile left over costs a persistent step 20 us, and
-// graded rows or blocks add their own factor to that spread.  Without an outlier in x a row is then
-// within a few 2^-53 of its |U||x|; with one, an entry that couples to it by 2^-s max|U| is off by
-// 2^(s - 59) of that coupling.
+// above that and about one in 50000 above 2^16), and a tile left over costs a persistent step 20 us.
+// (Without the count, sums that are small by cancellation were formed again too: N = 900, PH, 53 ms a solve
+// and its gradients instead of 42.)
 // x may have any exponent, subnormals included.  The diagonal of the matrix,
 // which holds the transition energies far above everything else in its tiles, is left out of the
 // tiles (zeros there) and added in FP64 by the block-row reduction.
@@ -46,6 +50,14 @@ namespace bse {
 constexpr int FX_THREADS = 256;
 constexpr int FX_WARPS = FX_THREADS / 32;
 constexpr int FX_SPREAD = 16;        // largest over smallest entry of a fixed-point tile, log2
+// What tells whether a sum's own magnitude |U||x| may be far below its scales (see above).  An entry of a
+// tile or a chunk is strong when it is within 2^-FX_STRONG of the largest.  texp[t] holds the tile's scale
+// exponent, then the largest number of entries in one of its rows or columns that are not strong: those
+// where neither matrix has a strong element, and those where one of the two has not.
+constexpr int FX_STRONG = 6, FX_EBITS = 11, FX_EMASK = (1 << FX_EBITS) - 1;
+constexpr int FX_WEAK = FX_EBITS, FX_WEAK2 = FX_EBITS + 8, FX_WMASK = 0xff;
+constexpr int FX_MASS = 16;          // strong pairs that make a sum sure
+constexpr int FX_SURE = 11;          // a sum of 128 terms is sure above 2^-FX_SURE of its scales, too
 
 constexpr long long FX_SPIN = 1ll << 24;      // polls of one wait for a row
 
@@ -61,6 +73,7 @@ struct FxShared {
   int rows[TS][6];                     // three words of (re, im) per row of the unit
   int cols[FX_WARPS][6][TS];           // ... per column, one partial sum per warp
   unsigned int mx[2][TS / 32];
+  int4 strong[2];                      // strong entries of the two chunks, by warp
 };
 
 __device__ __forceinline__ uint32_t fx_s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -175,6 +188,61 @@ struct FxPipe {
   bool ok = true;                        // no wait has expired
 };
 
+// A sum of n terms, its larger component's high word h, under the scales eu and ex (1: a tile or a chunk of
+// zeros) that has to be formed again in FP64; an infinity or a NaN in the chunk (ex = 2047) asks for it too.
+// (Its error goes with the square root of the terms.)
+__device__ __forceinline__ bool fx_weak(unsigned int h, int eu, int ex, int n) {
+  const int sure = FX_SURE + ((__clz(n) - 24) >> 1);
+  return eu > 1 && ex > 1 && ((int)(h >> 20) < eu + ex - 1021 - sure || ex == 2047);
+}
+
+// One sum of a unit in FP64, by a warp (in every lane): row idx of the tile times x_J, or its rows
+// [r0, r0 + n) of column idx times x_I; the matrix diagonal left out.  U, V: the tile's elements.
+template <bool HASB, bool COH>
+__device__ __forceinline__ double2 fx_exact(const double2* U, const double2* V, const double2* x, int idx, int r0, int n,
+                                         bool col, bool diag) {
+  const int lane = threadIdx.x & 31;
+  double re = 0.0, im = 0.0;
+  for (int k = r0 + lane; k < r0 + n; k += 32) {
+    if (diag && k == idx) continue;
+    const int e = col ? k * TS + idx : idx * TS + k;
+    const double2 u = U[e], v = HASB ? V[e] : u, z = ldv<COH>(x + k);
+    if (col) {
+      re = fma(u.x, z.x, fma(u.y, z.y, re));
+      im = fma(v.x, z.y, fma(-v.y, z.x, im));
+    } else {
+      re = fma(u.x, z.x, fma(-v.y, z.y, re));
+      im = fma(u.y, z.x, fma(v.x, z.y, im));
+    }
+  }
+  return make_double2(warp_sum_d(re), warp_sum_d(im));
+}
+
+// The row sums (or the column sums) of a unit that nothing answers for, again in FP64: those of the mask
+// `todo` (a warp's lanes; sum threadIdx.x / 2 goes to the thread's `out`).  Out of line: it is rare.
+template <bool HASB, bool COH>
+__device__ __noinline__ void fx_settle(const Prob& p, int I, int J, int t, int mode, const void* io_x, double io_sB,
+                                       double* out, unsigned int todo, int row0, int nrow, bool col) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const double2* x;
+  double2* y;
+  double sB;
+  GenericIO io{};
+  io.xa = io_x;
+  io.sB = io_sB;
+  prod_operands<double2, double>(p, mode, io, x, y, sB);
+  const double2* U = (const double2*)(HASB && !(sB > 0.0) ? p.B : p.A) + (int64_t)t * (TS * TS);
+  const double2* V = HASB ? (const double2*)(sB > 0.0 ? p.B : p.A) + (int64_t)t * (TS * TS) : nullptr;
+  x += (int64_t)(col ? I : J) * TS;
+  while (todo) {
+    const int l = __ffs(todo) - 1, i = (tid - lane + l) >> 1;
+    todo &= ~(3u << l);
+    const double2 s = col ? fx_exact<HASB, COH>(U, V, x, i, row0, nrow, true, I == J)
+                          : fx_exact<HASB, COH>(U, V, x, row0 + i, 0, TS, false, I == J);
+    if ((lane >> 1) == (l >> 1)) *out = tid & 1 ? s.y : s.x;
+  }
+}
+
 // Units of the fixed-point product: a tile, or a band of TS / nq of its rows.  A band's row sums
 // are whole rows of slot (I, J); its column sums go to plane q of the slots, which the reduction
 // adds.  Bands exist so that a problem of few tiles still occupies every SM.
@@ -274,6 +342,11 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
       return max(1, (int)(m >> 20));
     };
     const int ec = chunk_exp(0), er = chunk_exp(1);
+    {
+      const unsigned int m = max(max(sh.mx[warp >> 2][0], sh.mx[warp >> 2][1]), max(sh.mx[warp >> 2][2], sh.mx[warp >> 2][3]));
+      const unsigned int b = __ballot_sync(0xffffffffu, max(hi_abs(xv.x), hi_abs(xv.y)) + (FX_STRONG << 20) >= m);
+      if (lane == 0) reinterpret_cast<int*>(sh.strong)[warp] = __popc(b);
+    }
     sh.x[tid >> 7][tid & (TS - 1)] = fx_entry(xv, tid < TS ? ec : er);
     __syncthreads();
     int4 xc[4];
@@ -350,21 +423,36 @@ __device__ __forceinline__ void fx_tiles_body(const Prob* __restrict__ probs, co
       }
     }
     __syncthreads();
-    const int eu = p.texp[jb.t];
+    const int te = p.texp[jb.t], eu = te & FX_EMASK;
     double* part = (double*)p.part;
     const int i = tid >> 1, c = tid & 1;
+    auto settle = [&](double v, double* out, bool live, int k, int ex) {
+      const int4 ns = sh.strong[k];
+      if (ns.x + ns.y + ns.z + ns.w >= ((te >> FX_WEAK) & FX_WMASK) + FX_MASS && ex != 2047) return;
+      unsigned int h = hi_abs(v);
+      h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+      const int n = (int)min((int64_t)TS, p.N - (int64_t)(k ? jb.I : jb.J) * TS);
+      const unsigned int todo = __ballot_sync(0xffffffffu, live && fx_weak(h, eu, ex, n));
+      if (todo) fx_settle<HASB, COH>(p, jb.I, jb.J, jb.t, mode, io.xa, io.sB, out, todo, row0, nrow, k != 0);
+    };
+    double v = 0.0;
+    double* out = part + (((int64_t)jb.I * p.nT + jb.J) * TS + row0 + i) * 2 + c;
     if (i < nrow) {
       const int* w = sh.rows[i] + 3 * c;
-      part[(((int64_t)jb.I * p.nT + jb.J) * TS + row0 + i) * 2 + c] = fx_double(w[0], w[1], w[2], eu, ec);
+      v = fx_double(w[0], w[1], w[2], eu, ec);
+      *out = v;
     }
+    settle(v, out, i < nrow && (int64_t)jb.I * TS + row0 + i < p.N, 0, ec);
     if (!diag) {
       int w[3] = {0, 0, 0};
 #pragma unroll
       for (int wp = 0; wp < FX_WARPS; ++wp)
 #pragma unroll
         for (int k = 0; k < 3; ++k) w[k] += sh.cols[wp][3 * c + k][i];
-      part[(((int64_t)q * p.nT * p.nT + (int64_t)jb.J * p.nT + jb.I) * TS + i) * 2 + c] =
-          fx_double(w[0], w[1], w[2], eu, er);
+      out = part + (((int64_t)q * p.nT * p.nT + (int64_t)jb.J * p.nT + jb.I) * TS + i) * 2 + c;
+      v = fx_double(w[0], w[1], w[2], eu, er);
+      *out = v;
+      settle(v, out, (int64_t)jb.J * TS + i < p.N, 1, er);
     }
   }
   if (!pipe.ok && lane == 0)             // leave no copy in flight

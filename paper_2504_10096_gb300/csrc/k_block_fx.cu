@@ -17,7 +17,8 @@
 //
 // Unit: 64 rows x 16 columns, 256 threads of 2 x 2 outputs; 8 steps of q staged at a time.  Every
 // two (hl) or four (hh) q a sum's bits above 2^38 move to a 32-bit counter, so it stays exact over a whole tile; then
-// it becomes one FP64 number (integer instructions) and is added.  Measured against
+// it becomes one FP64 number (integer instructions; formed again in FP64 where it is too small for the error
+// of its scales, fx_weak) and is added.  Measured against
 // k_prod_rowblock: H on 20 vectors at N = 1500, complex128, 6.8 -> 0.50 ms a call; the residuals of 32
 // pairs at N = 5000, complex64 storage, 42.7 -> 6.4 ms; of 20 pairs at N = 2000, TDA, 4.3 -> 0.28 ms.
 #include <algorithm>
@@ -33,12 +34,13 @@ constexpr int BQ = 8;        // inner indices staged at a time
 constexpr int BRP = BR + 1;  // padded row stride of the staged tile (conflict-free both ways)
 
 // limbs of a block of columns: F0 (s or XA) and F1 (d or XB), column c at c Npad, and the scale
-// exponent of chunk I at E[c nT + I]; grid (nT, K), TS threads
+// exponent of chunk I (and its strong entries, as in texp) at E[c nT + I]; grid (nT, K), TS threads
 template <bool HASB, bool PQ>
 __global__ void __launch_bounds__(TS)
 k_block_stage(const double2* __restrict__ xa, const double2* __restrict__ xb, int64_t ldx, double sB, int64_t Npad,
               int nT, int4* __restrict__ F0, int4* __restrict__ F1, int* __restrict__ E) {
   __shared__ unsigned int smx[TS / 32];
+  __shared__ int sst[TS / 32];
   const int c = blockIdx.y, tid = threadIdx.x;
   const int64_t r = (int64_t)blockIdx.x * TS + tid;
   double2 a = xa[c * ldx + r], b = make_double2(0.0, 0.0);
@@ -62,7 +64,13 @@ k_block_stage(const double2* __restrict__ xa, const double2* __restrict__ xb, in
   const int e = max(1, (int)(m >> 20));
   F0[c * Npad + r] = fx_entry(a, e);
   if (HASB) F1[c * Npad + r] = fx_entry(b, e);
-  if (tid == 0) E[(int64_t)c * nT + blockIdx.x] = e;
+  // strong entries: both vectors' (a sum P s + Q d is only as large as its smaller pairing)
+  unsigned int h = max(hi_abs(a.x), hi_abs(a.y));
+  if (HASB) h = min(h, max(hi_abs(b.x), hi_abs(b.y)));
+  const unsigned int st = __ballot_sync(0xffffffffu, h + (FX_STRONG << 20) >= m);
+  if ((tid & 31) == 0) sst[tid >> 5] = __popc(st);
+  __syncthreads();
+  if (tid == 0) E[(int64_t)c * nT + blockIdx.x] = e | ((sst[0] + sst[1] + sst[2] + sst[3]) << FX_EBITS);
 }
 
 // scales of complex64 tiles, -1 for those a fixed-point product must not take (as k_fx_pack)
@@ -97,7 +105,7 @@ k_block_scale64(const float2* __restrict__ A, const float2* __restrict__ B, int6
     const int ex = (int)((__float_as_uint(m) >> 23) & 0xffu) + 896;      // FP64 bias
     // (entries far below 2^-100 would leave the FP32 range of the limbs' conversion)
     const bool ok = !any_bad && (m == 0.f || (m > 1e-25f && m < 1e25f && m <= (float)(1 << FX_SPREAD) * mn));
-    texp[t] = !ok ? -1 : (m == 0.f ? 64 : ex);
+    texp[t] = !ok ? -1 : (m == 0.f ? 1 : ex);
   }
 }
 
@@ -109,6 +117,22 @@ __device__ __forceinline__ void fx_limbs32(float v, int e, int& hi, int& lo) {
   m = d > 0 ? ((m >> (min(d, 63) - 1)) + 1) >> 1 : m;
   const long long f = d < 62 ? ((int)b < 0 ? -(long long)m : (long long)m) : 0ll;
   fx_limbs(f, hi, lo);
+}
+
+// (A, B) of a packed element
+template <int MODE>
+__device__ __forceinline__ void block_element(const void* A, const void* B, int64_t o, double2& a, double2& b) {
+  if (MODE & 1) {
+    a = ccvt<double2>(((const float2*)A)[o]);
+    if (MODE < 2) b = ccvt<double2>(((const float2*)B)[o]);
+  } else {
+    a = ((const double2*)A)[o];
+    if (MODE < 2) {                      // stored P = A + B, Q = A - B
+      const double2 p = a, q = ((const double2*)B)[o];
+      a = cscale(cadd(p, q), 0.5);
+      b = cscale(csub(p, q), 0.5);
+    }
+  }
 }
 
 // an exact sum over a tile: value = (x 2^38 + v), |v| < 2^63
@@ -127,13 +151,41 @@ __device__ __forceinline__ double fx_acc_double(const FxAcc& hh, const FxAcc& hl
   return fx_pack_double((long long)(t >> 68), (unsigned long long)(t >> 16) & 0xfffffffffffffull, eu, ex);
 }
 
+// what the sums in FP64 read (A null: none are formed)
+struct BlockExact {
+  const void* A;
+  const void* B;
+  const double2* xa;
+  const double2* xb;
+  int64_t ldx, N;
+  double sB;
+};
+
+// One output of a tile in FP64, by a warp (in every lane): row r of block row I times chunk J of a column;
+// A, B, xa, xb as for k_block_sum, the matrix diagonal left out
+template <int MODE>
+__device__ __noinline__ double2 block_exact(const void* A, const void* B, int64_t t, bool upper, bool diag, int r,
+                                            const double2* xa, const double2* xb, double sB) {
+  constexpr bool HASB = MODE < 2;
+  double2 y = make_double2(0.0, 0.0);
+  for (int q = threadIdx.x & 31; q < TS; q += 32) {
+    if (diag && q == r) continue;
+    const int64_t o = t * (TS * TS) + (upper ? r * TS + q : q * TS + r);
+    double2 a, b = make_double2(0.0, 0.0);
+    block_element<MODE>(A, B, o, a, b);
+    cfma(y, upper ? a : conjc(a), xa[q]);
+    if (HASB) cfma(y, b, cscale(xb ? xb[q] : conjc(xa[q]), sB));
+  }
+  return make_double2(warp_sum_d(y.x), warp_sum_d(y.y));
+}
+
 // MODE 0: complex128 PH (P, Q limbs); 1: complex64 PH (A, B); 2: complex128 TDA (A limbs);
 // 3: complex64 TDA.  grid (2 nT, ceil(K / BC), splits); part: splits x K x Npad
 template <int MODE>
 __global__ void __launch_bounds__(256, 2)
 k_block_fx(const void* __restrict__ M0, const void* __restrict__ M1, const int* __restrict__ texp, int nT, int64_t Npad,
            const int4* __restrict__ F0, const int4* __restrict__ F1, const int* __restrict__ E, int K,
-           double2* __restrict__ part) {
+           double2* __restrict__ part, const BlockExact ax) {
   constexpr bool HASB = MODE < 2, F32 = MODE & 1;
   constexpr int NZ = HASB ? 4 : 2;
   __shared__ int4 sm0[BQ * BRP];
@@ -153,7 +205,7 @@ k_block_fx(const void* __restrict__ M0, const void* __restrict__ M1, const int* 
     const bool upper = J >= I;
     const int ti = upper ? I : J, tj = upper ? J : I;
     const int64_t t = (int64_t)ti * nT - (int64_t)ti * (ti - 1) / 2 + (tj - ti);
-    const int eu = texp[t];
+    const int te = texp[t], eu = te & FX_EMASK;
     FxAcc hh[2][2][2], hl[2][2][2];      // [row][column][re, im]
 #pragma unroll
     for (int i = 0; i < 2; ++i)
@@ -253,11 +305,25 @@ k_block_fx(const void* __restrict__ M0, const void* __restrict__ M1, const int* 
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int c = c0 + 2 * cp + j;
-      const int ex = c < K ? E[(int64_t)c * nT + J] : 64;
+      const int xe = c < K ? E[(int64_t)c * nT + J] : 64, ex = xe & FX_EMASK;
+      // sums that nothing answers for are formed again in FP64, the warp's rows one by one (its columns are the
+      // same); not for the residuals (ax.A null), which are a norm
+      const bool check = !F32 && ax.A && c < K && ((xe >> FX_EBITS) < ((te >> FX_WEAK2) & FX_WMASK) + FX_MASS || ex == 2047);
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        y[i][j].x += fx_acc_double(hh[i][j][0], hl[i][j][0], eu, ex);
-        y[i][j].y += fx_acc_double(hh[i][j][1], hl[i][j][1], eu, ex);
+        double2 v = make_double2(fx_acc_double(hh[i][j][0], hl[i][j][0], eu, ex),
+                                 fx_acc_double(hh[i][j][1], hl[i][j][1], eu, ex));
+        if (check) {
+          const bool weak = (int64_t)I * TS + rh + rp + 32 * i < ax.N && fx_weak(max(hi_abs(v.x), hi_abs(v.y)), eu, ex, (int)min((int64_t)TS, ax.N - (int64_t)J * TS));
+          for (unsigned int todo = __ballot_sync(0xffffffffu, weak); todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            const int64_t o = c * ax.ldx + (int64_t)J * TS;
+            const double2 e = block_exact<MODE>(ax.A, ax.B, t, upper, I == J, rh + l + 32 * i, ax.xa + o,
+                                                ax.xb ? ax.xb + o : nullptr, ax.sB);
+            if (rp == l) v = e;
+          }
+        }
+        y[i][j] = cadd(y[i][j], v);
       }
     }
   }
@@ -277,7 +343,7 @@ __global__ void __launch_bounds__(256)
 k_block_sum(const double2* __restrict__ part, int nsplit, const void* __restrict__ A, const void* __restrict__ B,
             int nT, int64_t Npad, const double2* __restrict__ xa, const double2* __restrict__ xb, int64_t ldx, double sB,
             int K, double2* __restrict__ Y, int64_t ldy) {
-  constexpr bool HASB = MODE < 2, F32 = MODE & 1;
+  constexpr bool HASB = MODE < 2;
   const int c = blockIdx.y;
   const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (r >= Npad) return;
@@ -287,17 +353,7 @@ k_block_sum(const double2* __restrict__ part, int nsplit, const void* __restrict
   const int64_t o = ((int64_t)I * nT - (int64_t)I * (I - 1) / 2) * (TS * TS) + (int64_t)d * (TS + 1);
   const double2 va = xa[c * ldx + r];
   double2 a, b = make_double2(0.0, 0.0);
-  if (F32) {
-    a = ccvt<double2>(((const float2*)A)[o]);
-    if (HASB) b = ccvt<double2>(((const float2*)B)[o]);
-  } else {
-    a = ((const double2*)A)[o];
-    if (HASB) {                          // stored P = A + B, Q = A - B
-      const double2 p = a, q = ((const double2*)B)[o];
-      a = cscale(cadd(p, q), 0.5);
-      b = cscale(csub(p, q), 0.5);
-    }
-  }
+  block_element<MODE>(A, B, o, a, b);
   cfma(y, a, va);
   if (HASB) cfma(y, b, cscale(xb ? xb[c * ldx + r] : conjc(va), sB));
   Y[c * ldy + r] = y;
@@ -315,7 +371,8 @@ void run_block(const BlockFx& q, const double2* xa, const double2* xb, int64_t l
   int* E = (int*)(part + (size_t)ns * K * Npad);
   count_launch(3);
   k_block_stage<(MODE < 2), MODE == 0><<<dim3(nT, K), TS, 0, s>>>(xa, xb, ldx, sB, Npad, nT, F0, F1, E);
-  k_block_fx<MODE><<<dim3(2 * nT, (K + BC - 1) / BC, ns), 256, 0, s>>>(q.M0, q.M1, q.texp, nT, Npad, F0, F1, E, K, part);
+  k_block_fx<MODE><<<dim3(2 * nT, (K + BC - 1) / BC, ns), 256, 0, s>>>(q.M0, q.M1, q.texp, nT, Npad, F0, F1, E, K, part,
+                                                                 BlockExact{q.each ? q.A : nullptr, q.B, xa, xb, ldx, q.N, sB});
   k_block_sum<MODE><<<dim3((unsigned)((Npad + 255) / 256), K), 256, 0, s>>>(part, ns, q.A, q.B, nT, Npad, xa, xb, ldx,
                                                                             sB, K, y, ldy);
 }

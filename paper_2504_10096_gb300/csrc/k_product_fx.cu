@@ -36,10 +36,12 @@ k_fx_pack(const double2* __restrict__ A, const double2* __restrict__ B, int64_t 
   const double2* a = A + t * (TS * TS);
   const double2* b = HASB ? B + t * (TS * TS) : nullptr;
   __shared__ unsigned int smx[8], smn[8];
+  __shared__ int weak[2][2][TS];       // of the rows and columns: neither matrix strong, not both
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto off_diag = [&](int e) { return I != J || (e >> 7) != (e & (TS - 1)); };
   // high words of the magnitudes; 1 for a subnormal that has none
   auto mag = [](double v) { return max(hi_abs(v), __double2loint(v) ? 1u : 0u); };
+  weak[0][tid >> 7][tid & (TS - 1)] = weak[1][tid >> 7][tid & (TS - 1)] = 0;
   const int nr = (int)min((int64_t)TS, N - (int64_t)I * TS), nc = (int)min((int64_t)TS, N - (int64_t)J * TS);
   unsigned int m = 0, mn = 0xffffffffu;
   for (int e = tid; e < TS * TS; e += 256) {
@@ -69,11 +71,36 @@ k_fx_pack(const double2* __restrict__ A, const double2* __restrict__ B, int64_t 
     if (!off_diag(e)) v = w = make_double2(0.0, 0.0);
     Af[t * (TS * TS) + e] = fx_entry(v, ex);
     if (HASB) Bf[t * (TS * TS) + e] = fx_entry(w, ex);
+    // entries that are not strong (the matrix diagonal never is)
+    const unsigned int hv = max(hi_abs(v.x), hi_abs(v.y)), hw = HASB ? max(hi_abs(w.x), hi_abs(w.y)) : hv;
+    const int r = e >> 7, c = e & (TS - 1);
+    if (r < nr && c < nc && min(hv, hw) + (FX_STRONG << 20) < m) {
+      atomicAdd(&weak[1][0][r], 1);
+      atomicAdd(&weak[1][1][c], 1);
+      if (max(hv, hw) + (FX_STRONG << 20) < m) {
+        atomicAdd(&weak[0][0][r], 1);
+        atomicAdd(&weak[0][1][c], 1);
+      }
+    }
   }
+  __syncthreads();
+  const int top = __reduce_max_sync(0xffffffffu, weak[0][tid >> 7][tid & (TS - 1)]);
+  const int top2 = __reduce_max_sync(0xffffffffu, weak[1][tid >> 7][tid & (TS - 1)]);
+  __syncthreads();
+  if (lane == 0) {
+    smx[warp] = top;
+    smn[warp] = top2;
+  }
+  __syncthreads();
   // (a tile of zeros adds nothing; high words compare magnitudes to a few units of 2^-20)
   if (tid == 0) {
     const bool in_range = ex >= 256 && ex <= 1792;
-    texp[t] = m == 0 || (in_range && m <= mn + (FX_SPREAD << 20)) ? ex : -1;
+    unsigned int w = 0, w2 = 0;
+    for (int k = 0; k < 8; ++k) {
+      w = max(w, smx[k]);
+      w2 = max(w2, smn[k]);
+    }
+    texp[t] = m == 0 ? 1 : (in_range && m <= mn + (FX_SPREAD << 20) ? ex | (int)(w << FX_WEAK | w2 << FX_WEAK2) : -1);
   }
 }
 

@@ -174,6 +174,10 @@ inline float __uint_as_float(unsigned u) { float v; std::memcpy(&v, &u, 4); retu
 inline unsigned __float_as_uint(float v) { unsigned u; std::memcpy(&u, &v, 4); return u; }
 inline int __clzll(long long v) { return v ? __builtin_clzll((unsigned long long)v) : 64; }
 inline int atomicExch(int* p, int v) { const int o = *p; *p = v; return o; }
+inline int atomicAdd(int* p, int v) { const int o = *p; *p += v; return o; }
+inline int __reduce_max_sync(unsigned, int v) {
+  return simt::warp_fold(v, [](int a, int b) { return a > b ? a : b; });
+}
 inline double rsqrt(double v) { return 1.0 / std::sqrt(v); }
 using std::max;
 using std::min;

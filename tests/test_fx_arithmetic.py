@@ -36,8 +36,9 @@ int main(int, char** argv) {
   blockIdx.x = J;
   blockIdx.y = I;
   if (!simt::run_block(256, false, [&] { k_fx_pack<false>(A.data(), nullptr, N, nT, Af.data(), nullptr, texp); })) return 1;
-  printf("%%d\n", texp[t]);
-  const int eu = texp[t] < 0 ? 1 : texp[t];
+  printf("%%d %%d %%d\n", texp[t] < 0 ? -1 : texp[t] & FX_EMASK, (texp[t] >> FX_WEAK) & FX_WMASK,
+         (texp[t] >> FX_WEAK2) & FX_WMASK);
+  const int eu = texp[t] < 0 ? 1 : texp[t] & FX_EMASK;
   unsigned m = 0;
   for (auto v : x) m = max(m, max(hi_abs(v.x), hi_abs(v.y)));
   const int ex = max(1, (int)(m >> 20));
@@ -72,6 +73,7 @@ def _product(tmp_path, u, x, n=256, tile=(0, 1)):
     fu.write_bytes(np.ascontiguousarray(u, np.complex128).tobytes())
     fx.write_bytes(np.ascontiguousarray(x, np.complex128).tobytes())
     out = run(tmp_path, SRC % (c, a, k), fu, fx, n, *tile)
+    _product.weak = out[0][1:]
     return int(out[0][0]), np.array([complex(*v) for v in out[1:]])
 
 
@@ -179,6 +181,26 @@ def test_choice_of_tiles(tmp_path, name, u, fixed):
     """Tiles in which some row's magnitude may be far below max|u| max|x| stay with the FP64 kernel."""
     ex, _ = _product(tmp_path, u, np.ones(128))
     assert (ex >= 0) == fixed
+
+
+@pytest.mark.parametrize("n,tile", [(256, (0, 1)), (228, (1, 1)), (133, (0, 1))])
+def test_count_of_weak_entries(tmp_path, n, tile):
+    """The most entries of a row or column that are not within 2^-6 of the tile's largest (high words, so to
+    2^-20); a diagonal tile's diagonal counts as one of them."""
+    rng = np.random.default_rng(n)
+    nr, nc = min(128, n - 128 * tile[0]), min(128, n - 128 * tile[1])
+    u = np.zeros((128, 128), complex)
+    u[:nr, :nc] = _gauss(rng, nr, nc)
+    u[3, :nc // 2] *= 2.0 ** -4
+    if tile[0] == tile[1]:
+        u[np.arange(nr), np.arange(nr)] = 5.0
+    ex, _ = _product(tmp_path, u, np.ones(128), n, tile)
+    m = np.maximum(np.abs(u.real), np.abs(u.imag))[:nr, :nc]
+    if tile[0] == tile[1]:
+        np.fill_diagonal(m, 0)
+    weak = m < 2.0 ** -6 * m.max()
+    top = max(weak.sum(0).max(), weak.sum(1).max())
+    assert ex > 0 and _product.weak == [top, top]
 
 
 def test_edges_of_the_matrix(tmp_path):

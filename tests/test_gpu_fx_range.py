@@ -75,6 +75,47 @@ def test_every_entry(name, n, form):
     s.close()
 
 
+@pytest.mark.parametrize("form", ["ph", "tda"])
+@pytest.mark.parametrize("n", [100, 300, 1300])
+def test_weak_couplings_to_an_outlier(n, form):
+    """Entries of size one, some rows coupled by 2^-15 to the one entry of x that counts: every tile is in
+    fixed point, and its sums for those rows are far below the scales.  Bands at the smaller orders."""
+    from paper_2504_10096_gb300 import bse
+    rng = np.random.default_rng(n)
+    ph = np.exp(2j * np.pi * rng.random((n, n)))
+    a = np.triu(ph, 1)
+    a = a + a.conj().T + np.eye(n)
+    b = 0.3 * np.exp(2j * np.pi * rng.random((n, n)))
+    b = np.triu(b) + np.triu(b, 1).T
+    out, weak = n // 3, np.concatenate([np.arange(n // 2, n // 2 + 9), [n - 1]])
+    for m in (a, b):
+        m[weak, out] *= 2.0 ** -15
+        m[out, weak] *= 2.0 ** -15
+    x = rng.standard_normal((n, 1)) + 1j * rng.standard_normal((n, 1))
+    x[out] *= 1e10
+    s = bse.Solver(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda() if form == "ph" else None)
+    nt = -(-n // 128)
+    assert bse.bse_get_fixed_point(s.h) == (nt * (nt + 1) // 2,) * 2
+    L = np.clongdouble
+    al, bl, xl = a.astype(L), b.astype(L), x.astype(L)
+    ops = [(bse.BSE_OP_A, "a", al @ xl)]
+    if form == "ph":
+        ops += [(bse.BSE_OP_MPLUS, "mplus", al @ xl + bl @ xl.conj()), (bse.BSE_OP_MMINUS, "mminus", al @ xl - bl @ xl.conj())]
+    for op, kind, ref in ops:
+        for k in (1, 3, 17):
+            y = s.apply(op, torch.from_numpy(np.repeat(x, k, 1)).cuda()).cpu().numpy()
+            for c in (0, k - 1):
+                assert_elementwise(y[:, c:c + 1], ref.astype(complex), product_bound(a, b, x, kind), UNIT["c128"], 64, f"{kind}, k = {k}")
+    # an infinite entry: what FP64 arithmetic gives, infinities and no NaN (on blocks of the PH form A x and
+    # B conj(x) meet with opposite signs, inf - inf)
+    x[out] = np.inf
+    op = bse.BSE_OP_MPLUS if form == "ph" else bse.BSE_OP_A
+    for k in (1, 2) if form == "tda" else (1,):
+        y = s.apply(op, torch.from_numpy(np.repeat(x, k, 1)).cuda()).cpu().numpy()
+        assert np.isinf(y[:, 0].real).all() and np.isinf(y[:, 0].imag[np.arange(n) != out]).all()
+    s.close()
+
+
 @pytest.mark.parametrize("n,k", [(3, 40000), (1100, 2900)])
 def test_more_columns_than_one_launch_takes(n, k):
     """H on blocks that the block kernels take in several groups of columns."""
